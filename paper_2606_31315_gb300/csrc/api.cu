@@ -137,7 +137,7 @@ int bp_block_attention(const void* q, const void* k, const void* v, void* o, flo
     a.scratch = scratch(workspace);
     a.scratch_bytes = workspace_bytes - sizeof(WorkspaceHeader);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    rc = dtype == BP_BF16 ? launch_attention_bf16(a, dev, st) : launch_attention_f32(a, st);
+    rc = dtype == BP_BF16 ? launch_attention_bf16(a, dev, st) : launch_attention_f32(a, dev, st);
     if (rc == BP_ERR_CUDA) cudaGetLastError();
     return rc;
 }

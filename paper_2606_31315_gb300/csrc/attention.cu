@@ -21,7 +21,7 @@
 //   16 lanes of each TMEM sub-partition and each half-warp takes one 64-key half of a row, so
 //   all four softmax warps share the exp2 work.
 //
-// fp32 path: a plain SIMT kernel (one warp per output row, online softmax).
+// fp32 path (CUDA cores): register-tiled online softmax, keys split over a thread-block cluster.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
@@ -903,80 +903,285 @@ __global__ void __launch_bounds__(kCombThreads) attn_combine_kernel(const AttnPa
     if (p.lse && c4 == 0) p.lse[orow] = (M + __log2f(Lsum)) * 0.6931471805599453f;
 }
 
-// --------------------------------------------------------------------------- fp32 SIMT path
-// One warp per (query row, query head): online softmax over the row's visible keys in
-// chunks of 32 (lane = key), lane d-slices of the output.
+// --------------------------------------------------------------------------- fp32 path
+// Unit = (sequence, KV head, tile of kFR of the block's query rows x the head group's heads).  A cluster of
+// CS CTAs splits the unit's keys into runs of 64-key chunks; a CTA streams its chunks' K and V rows through
+// two shared-memory stages (16-byte cp.async, zero-filled past the sequence and past D) and runs the online
+// softmax on register tiles: a thread owns 2 rows x 4 keys of the scores and 2 rows x DP / 16 columns of the
+// output, the 16 threads of a row pair sit in one half-warp, so the row statistics are shuffles and the
+// weights cross through shared memory without a CTA barrier.  The CS partial (m, l, O) are merged through
+// distributed shared memory.  Everything is fp32 (FFMA and expf).
+// What bounds it: these shapes hold a few MB, so latency: the number of chunks in a CTA's chain and the one
+// merge.  Within a chunk, the 10 shared-memory wavefronts a warp needs for its 32 FFMAs.  The kernel it
+// replaces (a warp per output row, a key per lane, each lane walking its key row alone) read 32 rows per load
+// instruction and put the whole context into one warp's chain: 4 sequences x 1008 keys x 8 positions, 4 / 2
+// heads of 64, took 322.7 us a call and takes 13.9 us here; the error against 64-bit sums went from 6.3e-7
+// to 3.3e-7 (shorter chains).
 constexpr int kF32MaxD = 128;
+constexpr int kFR = 32;         // query rows per tile
+constexpr int kFK = 64;         // keys per chunk
+constexpr int kFThreads = 256;  // 16 row pairs x 16 key / column groups
+constexpr int kFPadP = kFK + 4;
 
-__global__ void __launch_bounds__(128) attn_f32_simt_kernel(const float* __restrict__ q, const float* __restrict__ k,
-                                                            const float* __restrict__ v, float* __restrict__ o,
-                                                            float* __restrict__ lse, const int32_t* __restrict__ cu_q,
-                                                            const int32_t* __restrict__ cu_kv, int num_seqs,
-                                                            int total_q, int hq, int hkv, int D, int causal,
-                                                            float scale) {
-    __shared__ float qs[4][kF32MaxD];
+struct F32Params {
+    const float* q;
+    const float* k;
+    const float* v;
+    float* o;
+    float* lse;
+    const int32_t* cu_q;
+    const int32_t* cu_kv;
+    int hq, hkv, D, m_tiles, causal;
+    float scale;
+};
+
+template <int DP>
+constexpr size_t f32_smem_bytes() {
+    return sizeof(float) * ((size_t)kFR * (DP + 4) + 2 * (size_t)kFK * (DP + 4) + 2 * (size_t)kFK * DP +
+                            (size_t)kFR * kFPadP + 2 * kFR);
+}
+
+// ROWS rows of D floats, row_stride apart, into shared memory rows of DP floats, ld apart; rows from `valid`
+// on and columns from D on become zero.
+template <int ROWS, int DP, bool VEC>
+__device__ __forceinline__ void f32_load_rows(float* dst, int ld, const float* src, size_t row_stride, int valid,
+                                              int D, int tid) {
+    if (VEC) {
+        for (int idx = tid; idx < ROWS * (DP / 4); idx += kFThreads) {
+            const int r = idx / (DP / 4), c = 4 * (idx % (DP / 4));
+            const bool ok = r < valid && c < D;
+            cp_async16(dst + r * ld + c, ok ? src + r * row_stride + c : src, ok);
+        }
+    } else {
+        for (int idx = tid; idx < ROWS * DP; idx += kFThreads) {
+            const int r = idx / DP, c = idx % DP;
+            dst[r * ld + c] = r < valid && c < D ? __ldg(src + r * row_stride + c) : 0.f;
+        }
+    }
+}
+
+template <int DP, bool VEC>
+__global__ void __launch_bounds__(kFThreads) attn_f32_kernel(const F32Params p) {
+    extern __shared__ float4 f32_smem[];
+    float* sQ = reinterpret_cast<float*>(f32_smem);  // [kFR][DP + 4]
+    float* sK = sQ + kFR * (DP + 4);                 // [2][kFK][DP + 4]
+    float* sV = sK + 2 * kFK * (DP + 4);             // [2][kFK][DP]
+    float* sP = sV + 2 * kFK * DP;                   // [kFR][kFPadP] weights of the current chunk
+    float2* sML = reinterpret_cast<float2*>(sP + kFR * kFPadP);  // [kFR] the CTA's (m, l)
+    constexpr int kLdK = DP + 4;  // 16-byte reads of 8 consecutive keys fall on distinct banks
+    constexpr int kCols = DP / 64;  // 16-byte column groups per thread
+
     griddep_launch_dependents();
     griddep_wait();
-    const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long row = (long long)blockIdx.x * 4 + wib;
-    if (row >= (long long)total_q * hq) return;
-    const int t = (int)(row / hq), h = (int)(row % hq);
-    const int g = hq / hkv, kvh = h / g;
-    int lo = 0, hi = num_seqs;  // sequence containing query t: cu_q[s] <= t < cu_q[s+1]
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (cu_q[mid] <= t) lo = mid; else hi = mid;
-    }
-    const int s = lo;
-    const int B = cu_q[s + 1] - cu_q[s];
-    const int i = t - cu_q[s];
-    const int kv0 = cu_kv[s];
-    const int n = cu_kv[s + 1] - kv0;
-    const int L = n - B;
-    const int nk = causal ? L + i + 1 : n;
-    for (int d = lane; d < D; d += 32) qs[wib][d] = q[((size_t)t * hq + h) * D + d];
-    __syncwarp();
-    float m = -INFINITY, l = 0.f;
-    float acc[kF32MaxD / 32];
-#pragma unroll
-    for (int e = 0; e < kF32MaxD / 32; ++e) acc[e] = 0.f;
-    for (int j0 = 0; j0 < nk; j0 += 32) {
-        const int j = j0 + lane;
-        float sc = -INFINITY;
-        if (j < nk) {
-            const float* kr = k + ((size_t)(kv0 + j) * hkv + kvh) * D;
-            float dot = 0.f;
-            for (int d = 0; d < D; ++d) dot = fmaf(qs[wib][d], kr[d], dot);
-            sc = dot * scale;
-        }
-        float cm = sc;
-        for (int off = 16; off; off >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, off));
-        const float m_new = fmaxf(m, cm);
-        const float alpha = (m == -INFINITY) ? 0.f : expf(m - m_new);
-        const float pj = (j < nk) ? expf(sc - m_new) : 0.f;
-        float ps = pj;
-        for (int off = 16; off; off >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, off);
-        l = l * alpha + ps;
-#pragma unroll
-        for (int e = 0; e < kF32MaxD / 32; ++e) acc[e] *= alpha;
-        const int cnt = min(32, nk - j0);
-        for (int jj = 0; jj < cnt; ++jj) {
-            const float pjj = __shfl_sync(0xffffffffu, pj, jj);
-            const float* vr = v + ((size_t)(kv0 + j0 + jj) * hkv + kvh) * D;
-#pragma unroll
-            for (int e = 0; e < kF32MaxD / 32; ++e) {
-                const int d = lane + e * 32;
-                if (d < D) acc[e] = fmaf(pjj, vr[d], acc[e]);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int CS = (int)cluster_size(), crank = (int)cluster_rank();
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int unit = blockIdx.x / CS;
+    const int G = p.hq / p.hkv, D = p.D;
+    const int mt = unit % p.m_tiles, kvh = (unit / p.m_tiles) % p.hkv, s = unit / (p.m_tiles * p.hkv);
+    const int q0 = __ldg(p.cu_q + s), B = __ldg(p.cu_q + s + 1) - q0;
+    const int kv0 = __ldg(p.cu_kv + s), n = __ldg(p.cu_kv + s + 1) - kv0;
+    const int L = n - B, rows = B * G;
+    const size_t kvstride = (size_t)p.hkv * D;
+    const float* kbase = p.k + ((size_t)kv0 * p.hkv + kvh) * D;
+    const float* vbase = p.v + ((size_t)kv0 * p.hkv + kvh) * D;
+
+    // (one pass, unless a block is longer than max_q_len; the bounds are the same in every CTA of the cluster)
+    for (int row0 = mt * kFR; row0 < rows; row0 += p.m_tiles * kFR) {
+        const int nr = min(kFR, rows - row0);
+        const int visible = p.causal ? L + (row0 + nr - 1) / G + 1 : n;  // keys the tile's last row sees
+        const int chunks = cdiv(visible, kFK);
+        const int c0 = (int)((long long)crank * chunks / CS), c1 = (int)((long long)(crank + 1) * chunks / CS);
+        auto load_chunk = [&](int c, int st) {
+            const int key0 = c * kFK, valid = min(kFK, n - key0);
+            f32_load_rows<kFK, DP, VEC>(sK + st * kFK * kLdK, kLdK, kbase + key0 * kvstride, kvstride, valid, D, tid);
+            f32_load_rows<kFK, DP, VEC>(sV + st * kFK * DP, DP, vbase + key0 * kvstride, kvstride, valid, D, tid);
+            cp_async_commit();
+        };
+        // row r of the tile: block position (row0 + r) / G, head (row0 + r) % G of the group
+        auto row_offset = [&](int r) {
+            const int lr = row0 + r;
+            return ((size_t)(q0 + lr / G) * p.hq + kvh * G + lr % G) * D;
+        };
+        if (VEC) {
+            for (int idx = tid; idx < kFR * (DP / 4); idx += kFThreads) {
+                const int r = idx / (DP / 4), c = 4 * (idx % (DP / 4));
+                const bool ok = r < nr && c < D;
+                cp_async16(sQ + r * kLdK + c, ok ? p.q + row_offset(r) + c : p.q, ok);
+            }
+        } else {
+            for (int idx = tid; idx < kFR * DP; idx += kFThreads) {
+                const int r = idx / DP, c = idx % DP;
+                sQ[r * kLdK + c] = r < nr && c < D ? __ldg(p.q + row_offset(r) + c) : 0.f;
             }
         }
-        m = m_new;
-    }
+        if (c0 < c1) load_chunk(c0, 0);
+
+        int limit[2];  // keys rows 2 ty and 2 ty + 1 see (0 past the tile)
+        float m[2], l[2], acc[2][4 * kCols];
 #pragma unroll
-    for (int e = 0; e < kF32MaxD / 32; ++e) {
-        const int d = lane + e * 32;
-        if (d < D) o[((size_t)t * hq + h) * D + d] = acc[e] / l;
+        for (int a = 0; a < 2; ++a) {
+            const int r = 2 * ty + a;
+            limit[a] = r < nr ? (p.causal ? L + (row0 + r) / G + 1 : n) : 0;
+            m[a] = -INFINITY;
+            l[a] = 0.f;
+#pragma unroll
+            for (int e = 0; e < 4 * kCols; ++e) acc[a][e] = 0.f;
+        }
+        for (int c = c0; c < c1; ++c) {
+            const int st = (c - c0) & 1;
+            if (c + 1 < c1) {
+                load_chunk(c + 1, st ^ 1);
+                cp_async_wait_group<1>();
+            } else {
+                cp_async_wait_group<0>();
+            }
+            __syncthreads();
+            const float* kk = sK + st * kFK * kLdK;
+            const float* vv = sV + st * kFK * DP;
+            float x[2][4];
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) x[a][j] = 0.f;
+#pragma unroll 4
+            for (int d = 0; d < DP; d += 4) {
+                const float4 qa = *reinterpret_cast<const float4*>(sQ + (2 * ty) * kLdK + d);
+                const float4 qb = *reinterpret_cast<const float4*>(sQ + (2 * ty + 1) * kLdK + d);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float4 kv = *reinterpret_cast<const float4*>(kk + (tx + 16 * j) * kLdK + d);
+                    x[0][j] = fmaf(qa.w, kv.w, fmaf(qa.z, kv.z, fmaf(qa.y, kv.y, fmaf(qa.x, kv.x, x[0][j]))));
+                    x[1][j] = fmaf(qb.w, kv.w, fmaf(qb.z, kv.z, fmaf(qb.y, kv.y, fmaf(qb.x, kv.x, x[1][j]))));
+                }
+            }
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                float mx = -INFINITY;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    x[a][j] = c * kFK + tx + 16 * j < limit[a] ? x[a][j] * p.scale : -INFINITY;
+                    mx = fmaxf(mx, x[a][j]);
+                }
+#pragma unroll
+                for (int o = 8; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                const float mn = fmaxf(m[a], mx);
+                const bool any = mn != -INFINITY;  // some key of this CTA is visible to the row so far
+                const float alpha = m[a] == -INFINITY ? 0.f : expf(m[a] - mn);
+                float sum = 0.f;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float w = any ? expf(x[a][j] - mn) : 0.f;
+                    sum += w;
+                    sP[(2 * ty + a) * kFPadP + tx + 16 * j] = w;
+                }
+                l[a] = l[a] * alpha + sum;  // this thread's keys; joined over the row below
+#pragma unroll
+                for (int e = 0; e < 4 * kCols; ++e) acc[a][e] *= alpha;
+                m[a] = mn;
+            }
+            __syncwarp();  // a row pair's weights are written and read by one half-warp
+#pragma unroll 2
+            for (int k4 = 0; k4 < kFK; k4 += 4) {
+                const float4 pa = *reinterpret_cast<const float4*>(sP + (2 * ty) * kFPadP + k4);
+                const float4 pb = *reinterpret_cast<const float4*>(sP + (2 * ty + 1) * kFPadP + k4);
+                const float wa[4] = {pa.x, pa.y, pa.z, pa.w}, wb[4] = {pb.x, pb.y, pb.z, pb.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+#pragma unroll
+                    for (int cc = 0; cc < kCols; ++cc) {
+                        const float4 z = *reinterpret_cast<const float4*>(vv + (k4 + e) * DP + 64 * cc + 4 * tx);
+                        acc[0][4 * cc] = fmaf(wa[e], z.x, acc[0][4 * cc]);
+                        acc[0][4 * cc + 1] = fmaf(wa[e], z.y, acc[0][4 * cc + 1]);
+                        acc[0][4 * cc + 2] = fmaf(wa[e], z.z, acc[0][4 * cc + 2]);
+                        acc[0][4 * cc + 3] = fmaf(wa[e], z.w, acc[0][4 * cc + 3]);
+                        acc[1][4 * cc] = fmaf(wb[e], z.x, acc[1][4 * cc]);
+                        acc[1][4 * cc + 1] = fmaf(wb[e], z.y, acc[1][4 * cc + 1]);
+                        acc[1][4 * cc + 2] = fmaf(wb[e], z.z, acc[1][4 * cc + 2]);
+                        acc[1][4 * cc + 3] = fmaf(wb[e], z.w, acc[1][4 * cc + 3]);
+                    }
+            }
+            __syncthreads();  // the stage and the weights are free
+        }
+        if (c0 >= c1) {  // no chunk: the query rows' copies still have to land before the memory is used again
+            cp_async_wait_group<0>();
+            __syncthreads();
+        }
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int o = 8; o >= 1; o >>= 1) l[a] += __shfl_xor_sync(0xffffffffu, l[a], o);
+
+        // four output columns of a row: any D and any alignment of o
+        auto store = [&](int r, int col, float4 val) {
+            float* dst = p.o + row_offset(r) + col;
+            if (VEC && col < D) {
+                *reinterpret_cast<float4*>(dst) = val;
+            } else if (!VEC) {
+                if (col < D) dst[0] = val.x;
+                if (col + 1 < D) dst[1] = val.y;
+                if (col + 2 < D) dst[2] = val.z;
+                if (col + 3 < D) dst[3] = val.w;
+            }
+        };
+        if (CS == 1) {
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                const int r = 2 * ty + a;
+                if (r >= nr) continue;
+#pragma unroll
+                for (int cc = 0; cc < kCols; ++cc)
+                    store(r, 64 * cc + 4 * tx,
+                          make_float4(acc[a][4 * cc] / l[a], acc[a][4 * cc + 1] / l[a], acc[a][4 * cc + 2] / l[a],
+                                      acc[a][4 * cc + 3] / l[a]));
+                if (p.lse && tx == 0) p.lse[row_offset(r) / D] = m[a] + logf(l[a]);
+            }
+            continue;
+        }
+        // ---- merge of the cluster's partials: each CTA leaves its own in the first K stage and (m, l) beside
+        // it; the tile's 16-byte output chunks are dealt out over the cluster's threads
+        float* opart = sK;  // [kFR][DP]
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            const int r = 2 * ty + a;
+#pragma unroll
+            for (int cc = 0; cc < kCols; ++cc)
+                *reinterpret_cast<float4*>(opart + r * DP + 64 * cc + 4 * tx) =
+                    make_float4(acc[a][4 * cc], acc[a][4 * cc + 1], acc[a][4 * cc + 2], acc[a][4 * cc + 3]);
+            if (tx == 0) sML[r] = make_float2(m[a], l[a]);
+        }
+        cluster.sync();
+        for (int item = crank * kFThreads + tid; item < nr * (DP / 4); item += CS * kFThreads) {
+            const int r = item / (DP / 4), col = 4 * (item % (DP / 4));
+            float2 ml[kMaxCluster];
+            float4 z[kMaxCluster];
+#pragma unroll
+            for (int pr = 0; pr < kMaxCluster; ++pr) {  // every peer's loads in flight together
+                ml[pr] = make_float2(-INFINITY, 0.f);
+                z[pr] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (pr < CS) {
+                    ml[pr] = *cluster.map_shared_rank(sML + r, pr);
+                    z[pr] = *cluster.map_shared_rank(reinterpret_cast<const float4*>(opart + r * DP + col), pr);
+                }
+            }
+            float M = -INFINITY, sum = 0.f;
+#pragma unroll
+            for (int pr = 0; pr < kMaxCluster; ++pr) M = fmaxf(M, ml[pr].x);
+            float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int pr = 0; pr < kMaxCluster; ++pr) {
+                const float w = ml[pr].x == -INFINITY ? 0.f : expf(ml[pr].x - M);
+                sum = fmaf(w, ml[pr].y, sum);
+                out.x = fmaf(w, z[pr].x, out.x);
+                out.y = fmaf(w, z[pr].y, out.y);
+                out.z = fmaf(w, z[pr].z, out.z);
+                out.w = fmaf(w, z[pr].w, out.w);
+            }
+            store(r, col, make_float4(out.x / sum, out.y / sum, out.z / sum, out.w / sum));
+            if (p.lse && col == 0) p.lse[row_offset(r) / D] = M + logf(sum);
+        }
+        cluster.sync();  // no CTA reuses or leaves its shared memory while a peer may still read it
     }
-    if (lse && lane == 0) lse[(size_t)t * hq + h] = m + logf(l);
 }
 
 }  // namespace
@@ -1198,24 +1403,87 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
     return BP_OK;
 }
 
-int launch_attention_f32(const AttentionArgs& a, cudaStream_t stream) {
-    if (a.head_dim > kF32MaxD) return BP_ERR_UNSUPPORTED;
-    const long long rows = (long long)a.total_q * a.num_q_heads;
-    if (rows == 0) return BP_OK;
+namespace {
+// One instantiation of the fp32 kernel: its shared-memory opt-in and how many clusters of each size the
+// device holds at once, found once per device (from any host thread).
+template <int DP, bool VEC>
+int run_attention_f32(const F32Params& p, int units, int chunks, const DeviceInfo& dev, cudaStream_t stream) {
+    static std::mutex mu;
+    static bool configured[64] = {};
+    static int max_active[64][kMaxCluster + 1];
+    constexpr size_t smem = f32_smem_bytes<DP>();
+    auto kern = attn_f32_kernel<DP, VEC>;
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    cfg.gridDim = dim3((unsigned)((rows + 3) / 4), 1, 1);
-    cfg.blockDim = dim3(128, 1, 1);
-    cfg.stream = stream;
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    cfg.blockDim = dim3(kFThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(
-        &cfg, attn_f32_simt_kernel, static_cast<const float*>(a.q), static_cast<const float*>(a.k),
-        static_cast<const float*>(a.v), static_cast<float*>(a.o), a.lse, a.cu_q, a.cu_kv, a.num_seqs, a.total_q,
-        a.num_q_heads, a.num_kv_heads, a.head_dim, (int)(a.mask == BP_MASK_CAUSAL_BLOCK), a.scale);
-    return e == cudaSuccess ? BP_OK : BP_ERR_CUDA;
+    if (dev.device < 0 || dev.device >= 64) return BP_ERR_UNSUPPORTED;
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        if (!configured[dev.device]) {
+            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+                cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+                return BP_ERR_CUDA;
+            for (int c = 1; c <= kMaxCluster; ++c) {
+                cfg.gridDim = dim3((unsigned)c, 1, 1);
+                attr[0].val.clusterDim.x = (unsigned)c;
+                int n = 0;
+                if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+                    cudaGetLastError();
+                    n = 0;
+                }
+                max_active[dev.device][c] = n;
+            }
+            configured[dev.device] = true;
+        }
+    }
+    // the widest split of the keys (a chunk per CTA at least) whose clusters are all resident at once
+    int cs = 1;
+    for (int c = 2; c <= kMaxCluster && c <= chunks; ++c)
+        if (units <= max_active[dev.device][c] && (long long)units * c <= dev.sm_count) cs = c;
+    cfg.gridDim = dim3((unsigned)(units * cs), 1, 1);
+    cfg.stream = stream;
+    attr[0].val.clusterDim.x = (unsigned)cs;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kern, p) == cudaSuccess ? BP_OK : BP_ERR_CUDA;
+}
+}  // namespace
+
+int launch_attention_f32(const AttentionArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
+    if (a.head_dim > kF32MaxD) return BP_ERR_UNSUPPORTED;
+    if (a.total_q == 0) return BP_OK;
+    const int G = a.num_q_heads / a.num_kv_heads;
+    F32Params p;
+    p.q = static_cast<const float*>(a.q);
+    p.k = static_cast<const float*>(a.k);
+    p.v = static_cast<const float*>(a.v);
+    p.o = static_cast<float*>(a.o);
+    p.lse = a.lse;
+    p.cu_q = a.cu_q;
+    p.cu_kv = a.cu_kv;
+    p.hq = a.num_q_heads;
+    p.hkv = a.num_kv_heads;
+    p.D = a.head_dim;
+    p.m_tiles = (int)std::max<long long>(1, ((long long)a.max_q_len * G + kFR - 1) / kFR);
+    p.causal = a.mask == BP_MASK_CAUSAL_BLOCK;
+    p.scale = a.scale;
+    const long long units = (long long)a.num_seqs * a.num_kv_heads * p.m_tiles;
+    if (units > INT32_MAX) return BP_ERR_UNSUPPORTED;
+    const int chunks = (a.max_kv_len + kFK - 1) / kFK;
+    const auto aligned16 = [](const void* x) { return (reinterpret_cast<uintptr_t>(x) & 15) == 0; };
+    const bool vec = a.head_dim % 4 == 0 && aligned16(a.q) && aligned16(a.k) && aligned16(a.v) && aligned16(a.o);
+    if (a.head_dim <= 64)
+        return vec ? run_attention_f32<64, true>(p, (int)units, chunks, dev, stream)
+                   : run_attention_f32<64, false>(p, (int)units, chunks, dev, stream);
+    return vec ? run_attention_f32<128, true>(p, (int)units, chunks, dev, stream)
+               : run_attention_f32<128, false>(p, (int)units, chunks, dev, stream);
 }
 
 // --------------------------------------------------------------------------- paged KV append

@@ -90,7 +90,7 @@ struct KvAppendArgs {
     int pages_per_seq, page_size, num_seqs, total_new, num_kv_heads, row_bytes;  // row_bytes = head_dim * elt
 };
 int launch_kv_append(const KvAppendArgs& a, cudaStream_t stream);
-int launch_attention_f32(const AttentionArgs& a, cudaStream_t stream);
+int launch_attention_f32(const AttentionArgs& a, const DeviceInfo& dev, cudaStream_t stream);
 
 struct AcceptArgs {
     const float* target;

@@ -178,3 +178,40 @@ def test_invalid_arguments_are_rejected_on_the_host():
         bp.block_attention(to_dev(a64["q"], "bf16"), to_dev(a64["k"], "bf16"), to_dev(a64["v"], "bf16"),
                            to_dev(a64["cu_q"]), to_dev(a64["cu_kv"]), 4, 14)
     assert e.value.status == 2
+
+
+@pytest.mark.parametrize("ctx,block,hq,hkv,d", [
+    ((0, 1, 63, 64, 65), (1, 8, 16, 2, 33), 4, 2, 64),     # chunk edges; 66 rows: three row tiles, the last of 2
+    ((1000, 7, 0), (8, 0, 24), 8, 1, 128),                 # a wide group (192 rows), an empty block, no context
+    ((2047,), (64,), 4, 4, 128),                           # one long unit per head: the widest cluster split
+    ((500, 129), (9, 16), 6, 2, 80),                       # D padded to the 128-column tile
+    ((300, 40), (5, 12), 3, 1, 33),                        # D not a multiple of 4: scalar loads and stores
+    ((40,) * 90, (4,) * 90, 4, 2, 64),                     # more units than SMs: no clusters
+])
+def test_fp32_shapes(ctx, block, hq, hkv, d):
+    """fp32 sums of at most 2111 keys and 128 columns: the error of a dot and of a weighted sum is a few
+    sqrt(length) roundings of 2^-24, well inside 1e-5 of the slice's largest value."""
+    w = wl.custom(seed=d + len(ctx), ctx=ctx, block=block, num_q_heads=hq, num_kv_heads=hkv, head_dim=d, dtype="f32")
+    a = wl.attention_inputs(w)
+    for mask in (CAUSAL, BIDIR):
+        o, lse = run_attention(a, mask)
+        err, lerr = attention_errors(o, lse, a, mask, range(len(ctx)))
+        assert err <= 1e-5 and lerr <= 1e-5, (err, lerr)
+
+
+def test_fp32_unaligned_bases():
+    """Tensors that start off a 16-byte boundary give the same values as aligned ones (same order of sums)."""
+    a = wl.attention_inputs(wl.custom(seed=3, ctx=(200, 30), block=(8, 5), num_q_heads=4, num_kv_heads=2, head_dim=64,
+                                      dtype="f32"))
+    cu_q, cu_kv = to_dev(a["cu_q"]), to_dev(a["cu_kv"])
+
+    def shifted(x):
+        flat = torch.zeros(x.numel() + 1, device="cuda")
+        flat[1:] = x.reshape(-1)
+        return flat[1:].view(x.shape)
+
+    q, k, v = to_dev(a["q"]), to_dev(a["k"]), to_dev(a["v"])
+    o, _ = bp.block_attention(q, k, v, cu_q, cu_kv, a["max_q_len"], a["max_kv_len"])
+    o1, _ = bp.block_attention(shifted(q), shifted(k), shifted(v), cu_q, cu_kv, a["max_q_len"], a["max_kv_len"],
+                               out=shifted(torch.zeros_like(q)))
+    assert torch.equal(o, o1)
