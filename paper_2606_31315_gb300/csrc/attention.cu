@@ -51,7 +51,7 @@ constexpr int kStageBytes = 2 * kKVBytes;       // 64 KB
 constexpr int kDynSmem = kQBytes + kStages * kStageBytes + 1024;
 constexpr int kThreads = 192;
 constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kColO = 256;
+constexpr uint32_t kColO = 384;
 constexpr int kMaxOrderedSeqs = 256;  // longest-first ordering for batches up to this size
 constexpr int kMaxCluster = 16;
 
@@ -81,7 +81,7 @@ struct AttnParams {
 };
 constexpr int kMaxSub = kTileN / 16;  // sub-boxes per K/V tile at the smallest page size (16 keys)
 
-__device__ __forceinline__ uint32_t col_s(int sb) { return sb ? 128u : 0u; }  // TMEM column of S buffer sb
+__device__ __forceinline__ uint32_t col_s(int st) { return (uint32_t)st * 128u; }  // TMEM column of stage st's S (then P)
 
 __device__ __forceinline__ float fast_exp2(float x) {
     float y;
@@ -201,8 +201,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint8_t* sQ = smem;
     uint8_t* sKV = smem + kQBytes;  // stage s: K at s*64KB, V at s*64KB + 32KB
 
-    __shared__ uint64_t bar_kv_full[kStages], bar_kv_empty[kStages];
-    __shared__ uint64_t bar_s_full[2], bar_p_full[2], bar_pv_done[2], bar_o_done, bar_q_full, bar_q_empty;
+    // one set per ring stage; the tile's S and P have a tensor-memory buffer of the same index.  done: the
+    // tile's P V is complete, so its K, V and P are read (the stage may be refilled, the buffer overwritten).
+    // With two S buffers Q K^T of a tile waited for the P V two tiles before it, which the same thread had just
+    // issued, and each tile took four commits; three buffers leave two commits and no such wait (25 sequences
+    // of up to 10412 keys: 100.7 -> 96.5 us, the ragged 32 90.5 -> 89.1 us, 1 x 2064 keys 8.35 -> 8.23 us).
+    __shared__ uint64_t bar_kv_full[kStages], bar_s_full[kStages], bar_p_full[kStages], bar_done[kStages];
+    __shared__ uint64_t bar_o_done, bar_q_full, bar_q_empty;
     __shared__ uint32_t tmem_base_sh;
     __shared__ int unit_seq_sh;
     // cluster split: the sequences' key offsets (longest-first order); flat split: their tile prefix sums
@@ -371,12 +376,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (tid == 0) {
         for (int i = 0; i < kStages; ++i) {
             mbar_init(&bar_kv_full[i], 1);
-            mbar_init(&bar_kv_empty[i], 1);
-        }
-        for (int i = 0; i < 2; ++i) {
             mbar_init(&bar_s_full[i], 1);
             mbar_init(&bar_p_full[i], 128);
-            mbar_init(&bar_pv_done[i], 1);
+            mbar_init(&bar_done[i], 1);
         }
         mbar_init(&bar_o_done, 1);
         mbar_init(&bar_q_full, 1);
@@ -407,7 +409,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     int rows[kMaxSub];
                     tile_rows(g, jl, rows);  // page lookups in flight while the stage drains
                     if (J >= kStages &&
-                        !mbar_wait(&bar_kv_empty[J % kStages], ((J / kStages) - 1) & 1, kWaitBudget)) {
+                        !mbar_wait(&bar_done[J % kStages], ((J / kStages) - 1) & 1, kWaitBudget)) {
                         ok = false;
                         break;
                     }
@@ -439,16 +441,16 @@ __global__ void __launch_bounds__(kThreads, 1)
             int J = 0, nq = 0;
             bool ok = true;
             auto issue_pv = [&](int Jx, bool first) {
-                const int sb = Jx & 1, st = Jx % kStages;
-                if (!mbar_wait(&bar_p_full[sb], (Jx >> 1) & 1, kWaitBudget)) return false;
+                const int st = Jx % kStages;
+                if (!mbar_wait(&bar_p_full[st], (Jx / kStages) & 1, kWaitBudget)) return false;
                 tc_fence_after();
                 const uint32_t v_addr = smem_addr(sKV + st * kStageBytes + kKVBytes);
+#pragma unroll
                 for (int kk = 0; kk < kTileN / 16; ++kk) {
                     const uint64_t bdesc = smem_desc(v_addr + kk * 2048, kHalf, 1024, kSwizzle128B);
-                    umma_ts(tmem + kColO, tmem + col_s(sb) + kk * 8, bdesc, id_o, (!first || kk > 0) ? 1u : 0u);
+                    umma_ts(tmem + kColO, tmem + col_s(st) + kk * 8, bdesc, id_o, (!first || kk > 0) ? 1u : 0u);
                 }
-                umma_commit(&bar_pv_done[sb]);
-                umma_commit(&bar_kv_empty[st]);
+                umma_commit(&bar_done[st]);
                 return true;
             };
             for (int t = t_begin; t < t_end && ok;) {
@@ -460,18 +462,19 @@ __global__ void __launch_bounds__(kThreads, 1)
                     break;
                 }
                 for (int jl = 0; jl < g.nt; ++jl, ++J) {
-                    const int sb = J & 1, st = J % kStages;
+                    // (the stage was refilled after the P V of tile J - kStages, so its S buffer is free too)
+                    const int st = J % kStages;
                     if (!mbar_wait(&bar_kv_full[st], (J / kStages) & 1, kWaitBudget)) { ok = false; break; }
-                    if (J >= 2 && !mbar_wait(&bar_pv_done[sb], ((J - 2) >> 1) & 1, kWaitBudget)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t k_addr = smem_addr(sKV + st * kStageBytes);
+#pragma unroll
                     for (int kk = 0; kk < kD / 16; ++kk) {
                         const uint32_t off = (kk >> 2) * kHalf + (kk & 3) * 32;
                         const uint64_t adesc = smem_desc(q_addr + off, 16, 1024, kSwizzle128B);
                         const uint64_t bdesc = smem_desc(k_addr + off, 16, 1024, kSwizzle128B);
-                        umma_ss(tmem + col_s(sb), adesc, bdesc, id_s, kk > 0 ? 1u : 0u);
+                        umma_ss(tmem + col_s(st), adesc, bdesc, id_s, kk > 0 ? 1u : 0u);
                     }
-                    umma_commit(&bar_s_full[sb]);
+                    umma_commit(&bar_s_full[st]);
                     if (jl == g.nt - 1) umma_commit(&bar_q_empty);  // the last read of this stretch's Q
                     if (jl >= 1 && !issue_pv(J - 1, jl == 1)) { ++J; ok = false; break; }
                 }
@@ -543,8 +546,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             m_run = -INFINITY;
             l_run = 0.f;
             for (int jl = 0; jl < g.nt; ++jl, ++J) {
-                const int sb = J & 1;
-                if (!__all_sync(0xffffffffu, mbar_wait(&bar_s_full[sb], (J >> 1) & 1, kWaitBudget))) {
+                const int st = J % kStages;
+                if (!__all_sync(0xffffffffu, mbar_wait(&bar_s_full[st], (J / kStages) & 1, kWaitBudget))) {
                     failed = true;
                     break;
                 }
@@ -556,8 +559,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     uint32_t x[kCols / 32][32];
 #pragma unroll
                     for (int c = 0; c < kCols / 32; ++c) {
-                        if (SPREAD) tmem_ld16x2_32<kTileN / 2>(tmem + lane_base + col_s(sb) + c * 32, x[c]);
-                        else tmem_ld32(tmem + lane_base + col_s(sb) + c * 32, x[c]);
+                        if (SPREAD) tmem_ld16x2_32<kTileN / 2>(tmem + lane_base + col_s(st) + c * 32, x[c]);
+                        else tmem_ld32(tmem + lane_base + col_s(st) + c * 32, x[c]);
                     }
                     tmem_ld_wait();
                     if (!__all_sync(0xffffffffu, nvalid >= kTileN)) {
@@ -587,7 +590,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // rescale the TMEM accumulator of rows whose max grew (warp-uniform TMEM access)
                     if (__any_sync(0xffffffffu, need && jl > 0 && m_run != -INFINITY)) {
                         if (!__all_sync(0xffffffffu,
-                                        mbar_wait(&bar_pv_done[(J - 1) & 1], ((J - 1) >> 1) & 1, kWaitBudget))) {
+                                        mbar_wait(&bar_done[(J - 1) % kStages], ((J - 1) / kStages) & 1, kWaitBudget))) {
                             failed = true;
                         } else {
                             tc_fence_after();
@@ -636,14 +639,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                         uint32_t pk[32];
 #pragma unroll
                         for (int e = 0; e < 32; ++e) pk[e] = weights(x[e / 16][2 * e % 32], x[e / 16][2 * e % 32 + 1], e & 1);
-                        tmem_st16x2_32<kTileN / 4>(tmem + lane_base + col_s(sb), pk);
+                        tmem_st16x2_32<kTileN / 4>(tmem + lane_base + col_s(st), pk);
                     } else {
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
                             uint32_t pk[16];
 #pragma unroll
                             for (int e = 0; e < 16; ++e) pk[e] = weights(x[c % (kCols / 32)][2 * e], x[c % (kCols / 32)][2 * e + 1], e & 1);
-                            tmem_st16(tmem + lane_base + col_s(sb) + c * 16, pk);
+                            tmem_st16(tmem + lane_base + col_s(st) + c * 16, pk);
                         }
                     }
                     float s0, s1, s2, s3;
@@ -654,7 +657,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     tmem_st_wait();
                 }
                 tc_fence_before();
-                mbar_arrive(&bar_p_full[sb]);
+                mbar_arrive(&bar_p_full[st]);
                 if (failed) break;
             }
             // the stretch's accumulator
