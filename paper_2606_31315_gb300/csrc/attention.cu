@@ -192,7 +192,11 @@ __device__ __forceinline__ Seg flat_seg(const AttnParams& p, const int32_t* pre,
 // to the output, a partial stretch to its workspace slot for attn_combine_kernel.  Otherwise the
 // cluster split: a unit per cluster, its tiles cut into CS ranges, partials merged through
 // distributed shared memory.
-template <bool PAGED, bool SPREAD, bool FLAT>
+// AHEAD (cluster split): K and V are separate rings.  K's stage is free after Q K^T, a softmax and a P V before
+// V's, and refills then, V a tile behind (the order in which the stages come free); with the rings joined both
+// wait for the tile's P V and only one of the three stages is in flight.  Where the line lies:
+// launch_attention_bf16.
+template <bool PAGED, bool SPREAD, bool FLAT, bool AHEAD>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_bf16_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
                         const __grid_constant__ CUtensorMap vmap, const AttnParams p) {
@@ -207,6 +211,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // issued, and each tile took four commits; three buffers leave two commits and no such wait (25 sequences
     // of up to 10412 keys: 100.7 -> 96.5 us, the ragged 32 90.5 -> 89.1 us, 1 x 2064 keys 8.35 -> 8.23 us).
     __shared__ uint64_t bar_kv_full[kStages], bar_s_full[kStages], bar_p_full[kStages], bar_done[kStages];
+    __shared__ uint64_t bar_k_full[kStages], bar_k_empty[kStages];  // AHEAD: the K ring's; bar_kv_full is the V ring's then
     __shared__ uint64_t bar_o_done, bar_q_full, bar_q_empty;
     __shared__ uint32_t tmem_base_sh;
     __shared__ int unit_seq_sh;
@@ -330,30 +335,35 @@ __global__ void __launch_bounds__(kThreads, 1)
                 row[sb] = __ldg(bt + pi) * (1 << p.page_shift) + (key & ((1 << p.page_shift) - 1));
             }
     };
-    // K/V tile jl of stretch g -> ring stage J % kStages (J counts the CTA's tiles; producer thread only)
-    auto issue_kv = [&](int J, const Seg& g, int jl, const int (&row)[kMaxSub]) {
-        const int st = J % kStages;
-        uint8_t* sK = sKV + st * kStageBytes;
-        uint8_t* sV = sK + kKVBytes;
-        mbar_arrive_expect_tx(&bar_kv_full[st], kStageBytes);
+    // the K rows (or the V rows) of tile jl of stretch g -> stage J % kStages of the ring (J counts the CTA's
+    // tiles; producer thread only)
+    auto load_rows = [&](uint8_t* dst, const CUtensorMap* map, uint64_t* bar, const Seg& g, int jl,
+                         const int (&row)[kMaxSub]) {
         if (!paged) {
             const int key = g.kv0 + (g.jt0 + jl) * kTileN;
-            tma_load_3d(sK, &kmap, &bar_kv_full[st], 0, g.h, key);
-            tma_load_3d(sK + kHalf, &kmap, &bar_kv_full[st], 64, g.h, key);
-            tma_load_3d(sV, &vmap, &bar_kv_full[st], 0, g.h, key);
-            tma_load_3d(sV + kHalf, &vmap, &bar_kv_full[st], 64, g.h, key);
+            tma_load_3d(dst, map, bar, 0, g.h, key);
+            tma_load_3d(dst + kHalf, map, bar, 64, g.h, key);
         } else {
 #pragma unroll
             for (int sb = 0; sb < kMaxSub; ++sb) {  // sub-box sb lands at row sb * sub_rows of the tile
                 if (sb < nsub) {
                     const int off = sb * sub_rows * 128;
-                    tma_load_3d(sK + off, &kmap, &bar_kv_full[st], 0, g.h, row[sb]);
-                    tma_load_3d(sK + kHalf + off, &kmap, &bar_kv_full[st], 64, g.h, row[sb]);
-                    tma_load_3d(sV + off, &vmap, &bar_kv_full[st], 0, g.h, row[sb]);
-                    tma_load_3d(sV + kHalf + off, &vmap, &bar_kv_full[st], 64, g.h, row[sb]);
+                    tma_load_3d(dst + off, map, bar, 0, g.h, row[sb]);
+                    tma_load_3d(dst + kHalf + off, map, bar, 64, g.h, row[sb]);
                 }
             }
         }
+    };
+    auto issue_k = [&](int J, const Seg& g, int jl, const int (&row)[kMaxSub]) {
+        const int st = J % kStages;
+        uint64_t* bar = AHEAD ? &bar_k_full[st] : &bar_kv_full[st];
+        mbar_arrive_expect_tx(bar, AHEAD ? kKVBytes : kStageBytes);  // not AHEAD: V's bytes too
+        load_rows(sKV + st * kStageBytes, &kmap, bar, g, jl, row);
+    };
+    auto issue_v = [&](int J, const Seg& g, int jl, const int (&row)[kMaxSub]) {
+        const int st = J % kStages;
+        if (AHEAD) mbar_arrive_expect_tx(&bar_kv_full[st], kKVBytes);
+        load_rows(sKV + st * kStageBytes + kKVBytes, &vmap, &bar_kv_full[st], g, jl, row);
     };
     // the Q tile of stretch g (producer thread only)
     auto issue_q = [&](const Seg& g) {
@@ -379,6 +389,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(&bar_s_full[i], 1);
             mbar_init(&bar_p_full[i], 128);
             mbar_init(&bar_done[i], 1);
+            if (AHEAD) {
+                mbar_init(&bar_k_full[i], 1);
+                mbar_init(&bar_k_empty[i], 1);
+            }
         }
         mbar_init(&bar_o_done, 1);
         mbar_init(&bar_q_full, 1);
@@ -401,6 +415,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) {
             int J = 0, nq = 0;
             bool ok = true;
+            int jv = 0, rows_v[kMaxSub];  // AHEAD: tiles whose V is issued, the pool rows of the next one
             for (int t = t_begin; t < t_end && ok;) {
                 const Seg g = seg_at(t, t == t_begin);
                 t += seg_len(g);
@@ -408,12 +423,30 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int jl = 0; jl < g.nt; ++jl, ++J) {
                     int rows[kMaxSub];
                     tile_rows(g, jl, rows);  // page lookups in flight while the stage drains
-                    if (J >= kStages &&
-                        !mbar_wait(&bar_done[J % kStages], ((J / kStages) - 1) & 1, kWaitBudget)) {
+                    if (J >= kStages && !mbar_wait(AHEAD ? &bar_k_empty[J % kStages] : &bar_done[J % kStages],
+                                                   ((J / kStages) - 1) & 1, kWaitBudget)) {
                         ok = false;
                         break;
                     }
-                    issue_kv(J, g, jl, rows);
+                    issue_k(J, g, jl, rows);
+                    if (AHEAD) {  // one stretch: tile J - 1's V, once its stage is free
+                        if (J > 0) {
+                            if (jv >= kStages &&
+                                !mbar_wait(&bar_done[jv % kStages], ((jv / kStages) - 1) & 1, kWaitBudget)) {
+                                ++J;
+                                ok = false;
+                                break;
+                            }
+                            issue_v(jv, g, jv, rows_v);
+                            ++jv;
+                        }
+                        if (paged) {
+#pragma unroll
+                            for (int sb = 0; sb < kMaxSub; ++sb) rows_v[sb] = rows[sb];
+                        }
+                    } else {
+                        issue_v(J, g, jl, rows);
+                    }
                     if (jl == 0 && p.q_tma) {
                         // the stretch's Q, once the MMAs of the previous stretch no longer read the buffer
                         if (nq > 0 && !mbar_wait(&bar_q_empty, (nq - 1) & 1, kWaitBudget)) {
@@ -425,11 +458,22 @@ __global__ void __launch_bounds__(kThreads, 1)
                         ++nq;
                     }
                 }
+                if (AHEAD && ok) {  // the last tile's V
+                    ok = jv < kStages || mbar_wait(&bar_done[jv % kStages], ((jv / kStages) - 1) & 1, kWaitBudget);
+                    if (ok) {
+                        issue_v(jv, g, jv, rows_v);
+                        ++jv;
+                    }
+                }
             }
             if (!ok) raise_error(p.err, kErrTimeout);
             // no copy may still be in flight when the CTA leaves
-            for (int j = max(0, J - kStages); j < J; ++j)
+            const int nv = AHEAD ? jv : J;
+            for (int j = max(0, nv - kStages); j < nv; ++j)
                 if (!mbar_wait(&bar_kv_full[j % kStages], (j / kStages) & 1, kDrainBudget)) raise_error(p.err, kErrTimeout);
+            if (AHEAD)
+                for (int j = max(0, J - kStages); j < J; ++j)
+                    if (!mbar_wait(&bar_k_full[j % kStages], (j / kStages) & 1, kDrainBudget)) raise_error(p.err, kErrTimeout);
             if (nq > 0 && !mbar_wait(&bar_q_full, (nq - 1) & 1, kDrainBudget)) raise_error(p.err, kErrTimeout);
         }
     } else if (warp == 1) {
@@ -442,6 +486,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             bool ok = true;
             auto issue_pv = [&](int Jx, bool first) {
                 const int st = Jx % kStages;
+                if (AHEAD && !mbar_wait(&bar_kv_full[st], (Jx / kStages) & 1, kWaitBudget)) return false;
                 if (!mbar_wait(&bar_p_full[st], (Jx / kStages) & 1, kWaitBudget)) return false;
                 tc_fence_after();
                 const uint32_t v_addr = smem_addr(sKV + st * kStageBytes + kKVBytes);
@@ -464,7 +509,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int jl = 0; jl < g.nt; ++jl, ++J) {
                     // (the stage was refilled after the P V of tile J - kStages, so its S buffer is free too)
                     const int st = J % kStages;
-                    if (!mbar_wait(&bar_kv_full[st], (J / kStages) & 1, kWaitBudget)) { ok = false; break; }
+                    if (!mbar_wait(AHEAD ? &bar_k_full[st] : &bar_kv_full[st], (J / kStages) & 1, kWaitBudget)) { ok = false; break; }
+                    if (AHEAD && J >= kStages && !mbar_wait(&bar_done[st], ((J / kStages) - 1) & 1, kWaitBudget)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t k_addr = smem_addr(sKV + st * kStageBytes);
 #pragma unroll
@@ -475,6 +521,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         umma_ss(tmem + col_s(st), adesc, bdesc, id_s, kk > 0 ? 1u : 0u);
                     }
                     umma_commit(&bar_s_full[st]);
+                    if (AHEAD) umma_commit(&bar_k_empty[st]);
                     if (jl == g.nt - 1) umma_commit(&bar_q_empty);  // the last read of this stretch's Q
                     if (jl >= 1 && !issue_pv(J - 1, jl == 1)) { ++J; ok = false; break; }
                 }
@@ -1222,6 +1269,18 @@ size_t attention_flat_scratch_bytes(int max_q_len, int group) {
            (size_t)2 * kAttnFlatMaxGrid * sizeof(int4);
 }
 
+namespace {
+// The instantiations: [variant][spread][paged], variants cluster split, cluster split AHEAD, flat split.
+using AttnKernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, AttnParams);
+const AttnKernel kAttnKernels[12] = {
+    attn_bf16_tc_kernel<false, false, false, false>, attn_bf16_tc_kernel<true, false, false, false>,
+    attn_bf16_tc_kernel<false, true, false, false>,  attn_bf16_tc_kernel<true, true, false, false>,
+    attn_bf16_tc_kernel<false, false, false, true>,  attn_bf16_tc_kernel<true, false, false, true>,
+    attn_bf16_tc_kernel<false, true, false, true>,   attn_bf16_tc_kernel<true, true, false, true>,
+    attn_bf16_tc_kernel<false, false, true, false>,  attn_bf16_tc_kernel<true, false, true, false>,
+    attn_bf16_tc_kernel<false, true, true, false>,   attn_bf16_tc_kernel<true, true, true, false>};
+}  // namespace
+
 int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
     if (a.head_dim != kD) return BP_ERR_UNSUPPORTED;
     const int G = a.num_q_heads / a.num_kv_heads;
@@ -1293,10 +1352,7 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
     int max_active[kMaxCluster + 1];
     std::unique_lock<std::mutex> cfg_lock(cfg_mu);
     if (!configured[dev.device]) {
-        for (auto kern : {attn_bf16_tc_kernel<false, false, false>, attn_bf16_tc_kernel<true, false, false>,
-                          attn_bf16_tc_kernel<false, true, false>, attn_bf16_tc_kernel<true, true, false>,
-                          attn_bf16_tc_kernel<false, false, true>, attn_bf16_tc_kernel<true, false, true>,
-                          attn_bf16_tc_kernel<false, true, true>, attn_bf16_tc_kernel<true, true, true>})
+        for (AttnKernel kern : kAttnKernels)
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem) != cudaSuccess ||
                 cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
                 cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -1315,7 +1371,7 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
             probe.attrs = pa;
             probe.numAttrs = 1;
             int n_clusters = 0;
-            if (cudaOccupancyMaxActiveClusters(&n_clusters, attn_bf16_tc_kernel<false, false, false>, &probe) !=
+            if (cudaOccupancyMaxActiveClusters(&n_clusters, kAttnKernels[0], &probe) !=
                 cudaSuccess) {
                 cudaGetLastError();
                 n_clusters = 0;
@@ -1374,8 +1430,17 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
     const bool flat_ok = q_tma && a.num_seqs <= kMaxOrderedSeqs && a.scratch != nullptr &&
                          a.scratch_bytes >= attention_flat_scratch_bytes(a.max_q_len, G) && ngroups >= 1;
     const long long cluster_ctas = units * cs;
+    // and where whole units per CTA leave the longest one far above the average: a CTA streams a tile in about
+    // 1.35 us, 152 of them together at HBM's rate one each 1.48 us, and the flat split adds about 4.2 us for
+    // each stretch of a CTA and 8 us for the second kernel.  20 sequences of 339-5425 keys (longest unit 38
+    // tiles, 19.7 on average): 49.3 against 52.6 us; 25 of up to 10412 (73, 49.3): 90.8 against 96.5 us; the
+    // ragged 32 (62, 54.3): 99 against 89 us.
+    const double avg_tiles = (double)a.num_kv_heads * m_tiles * ((double)a.total_kv / kTileN + 0.5 * a.num_seqs) /
+                             dev.sm_count;
+    const bool uneven = cs == 1 && flat_ok &&
+                        1.35 * max_tiles > 1.48 * avg_tiles + 4.2 * (1.0 + (double)a.num_seqs / ngroups) + 8.0;
     bool flat = flat_ok && ((cluster_ctas * 10 <= 9LL * dev.sm_count && tiles_bound >= 64LL * ngroups) ||
-                            cluster_ctas >= 3LL * dev.sm_count);
+                            cluster_ctas >= 3LL * dev.sm_count || uneven);
     if (const char* force = getenv("BP_ATTENTION_SPLIT")) {
         if (strcmp(force, "flat") == 0) {
             flat = flat_ok;
@@ -1393,10 +1458,7 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
         cfg.gridDim = dim3((unsigned)flat_grid, 1, 1);
         cfg.attrs = &attr[1];
         cfg.numAttrs = 1;
-        if (paged) e = spread ? cudaLaunchKernelEx(&cfg, attn_bf16_tc_kernel<true, true, true>, qmap, kmap, vmap, p)
-                              : cudaLaunchKernelEx(&cfg, attn_bf16_tc_kernel<true, false, true>, qmap, kmap, vmap, p);
-        else e = spread ? cudaLaunchKernelEx(&cfg, attn_bf16_tc_kernel<false, true, true>, qmap, kmap, vmap, p)
-                        : cudaLaunchKernelEx(&cfg, attn_bf16_tc_kernel<false, false, true>, qmap, kmap, vmap, p);
+        e = cudaLaunchKernelEx(&cfg, kAttnKernels[8 + 2 * spread + paged], qmap, kmap, vmap, p);
         if (e != cudaSuccess) return BP_ERR_CUDA;
         if (max_tiles <= 1) return BP_OK;  // every unit is one tile: none is cut between CTAs
         cudaLaunchConfig_t cc = {};
@@ -1410,16 +1472,19 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
 
     cfg.gridDim = dim3((unsigned)(units * cs), 1, 1);
     p.early_release = units <= max_active[cs] && units * cs <= dev.sm_count;  // one wave
+    // A CTA's bandwidth is what it keeps in flight; where SMs are idle and each CTA streams a long run, refilling
+    // K's stages early (AHEAD) took 16 x 4112 keys (128 CTAs of 33 tiles) from 47.4 to 44.9 us and 4 x 8208
+    // (clusters of 4, 17 tiles a CTA) from 29.9 to 28.9 us.  With every SM streaming, HBM is the bound and the
+    // freer order of requests costs more than it hides (the ragged 32 lost 2 us); on short runs (4 tiles: 13.4
+    // against 13.2 us) and in wide clusters (1 x 32784 keys: 31.7 against 30.9 us) it loses too.
+    const bool ahead = units * cs < dev.sm_count && cs <= 4 && max_tiles >= 16 * cs;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cs;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (paged) e = spread ? cudaLaunchKernelEx(&cfg, attn_bf16_tc_kernel<true, true, false>, qmap, kmap, vmap, p)
-                          : cudaLaunchKernelEx(&cfg, attn_bf16_tc_kernel<true, false, false>, qmap, kmap, vmap, p);
-    else e = spread ? cudaLaunchKernelEx(&cfg, attn_bf16_tc_kernel<false, true, false>, qmap, kmap, vmap, p)
-                    : cudaLaunchKernelEx(&cfg, attn_bf16_tc_kernel<false, false, false>, qmap, kmap, vmap, p);
+    e = cudaLaunchKernelEx(&cfg, kAttnKernels[4 * ahead + 2 * spread + paged], qmap, kmap, vmap, p);
     if (e != cudaSuccess) return BP_ERR_CUDA;
     return BP_OK;
 }

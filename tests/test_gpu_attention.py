@@ -215,3 +215,26 @@ def test_fp32_unaligned_bases():
     o1, _ = bp.block_attention(shifted(q), shifted(k), shifted(v), cu_q, cu_kv, a["max_q_len"], a["max_kv_len"],
                                out=shifted(torch.zeros_like(q)))
     assert torch.equal(o, o1)
+
+
+@pytest.mark.parametrize("block", [(16, 1, 9, 16, 8, 12, 16, 3, 16, 5), (24, 1, 17, 20, 8, 32, 24, 3, 31, 5)])
+def test_k_ring_ahead_of_v(block):
+    """80 units of one CTA each, up to 33 key tiles: fewer CTAs than SMs and long runs, so K's ring
+    refills ahead of V's; runs of 1 to 33 tiles wrap the rings at every phase, in both row layouts."""
+    ctx = (2049, 4100, 2303, 31, 0, 900, 2176, 1, 3000, 128)
+    a = wl.attention_inputs(wl.custom(seed=len(block) + block[0], ctx=ctx, block=block, num_q_heads=32, num_kv_heads=8))
+    for mask in (CAUSAL, BIDIR):
+        _check(a, mask, split="cluster")
+
+
+def test_uneven_batch_takes_the_flat_split():
+    """One 9000-key sequence among short ones: the flat split when the library chooses (the longest unit alone
+    would take longer than every tile spread over all SMs); a batch of equal lengths keeps whole units."""
+    ctx = (9000,) + tuple(range(300, 2100, 100)) + (31, 0)
+    uneven = wl.attention_inputs(wl.custom(seed=8, ctx=ctx, block=(16, 9, 24) * 7, num_q_heads=32, num_kv_heads=8))
+    _attn_kernels(uneven, "auto")
+    assert any("attn_combine_kernel" in x for x in _attn_kernels(uneven, "auto"))
+    err, lerr = attention_errors(*run_attention(uneven, BIDIR), uneven, BIDIR, [0, 1, 10, 19, 20])
+    assert err <= ATTN_TOL and lerr <= LSE_TOL
+    even = wl.attention_inputs(wl.custom(seed=8, ctx=(1500,) * 21, block=(16,) * 21, num_q_heads=32, num_kv_heads=8))
+    assert not any("attn_combine_kernel" in x for x in _attn_kernels(even, "auto"))
