@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // of up to 10412 keys: 100.7 -> 96.5 us, the ragged 32 90.5 -> 89.1 us, 1 x 2064 keys 8.35 -> 8.23 us).
     __shared__ uint64_t bar_kv_full[kStages], bar_s_full[kStages], bar_p_full[kStages], bar_done[kStages];
     __shared__ uint64_t bar_k_full[kStages], bar_k_empty[kStages];  // AHEAD: the K ring's; bar_kv_full is the V ring's then
-    __shared__ uint64_t bar_o_done, bar_q_full, bar_q_empty;
+    __shared__ uint64_t bar_o_done, bar_drain, bar_q_full, bar_q_empty;
     __shared__ uint32_t tmem_base_sh;
     __shared__ int unit_seq_sh;
     // cluster split: the sequences' key offsets (longest-first order); flat split: their tile prefix sums
@@ -395,6 +395,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
         mbar_init(&bar_o_done, 1);
+        mbar_init(&bar_drain, 1);
         mbar_init(&bar_q_full, 1);
         mbar_init(&bar_q_empty, 1);
         fence_mbar_init();
@@ -532,9 +533,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             if (!ok) raise_error(p.err, kErrTimeout);
             if (J > 0) {
-                // no MMA may still be writing tensor memory when it is released
-                umma_commit(&bar_o_done);
-                if (!mbar_wait(&bar_o_done, nq & 1, kDrainBudget)) raise_error(p.err, kErrTimeout);
+                // no MMA may still be writing tensor memory when it is released (a barrier of its own: a second
+                // phase of bar_o_done completing right behind the first could pass a softmax warp that has not
+                // yet looked at the first, which would then wait until its budget expired)
+                umma_commit(&bar_drain);
+                if (!mbar_wait(&bar_drain, 0, kDrainBudget)) raise_error(p.err, kErrTimeout);
             }
         }
     }
