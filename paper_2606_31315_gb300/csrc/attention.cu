@@ -30,7 +30,6 @@
 
 #include <algorithm>
 #include <mutex>
-#include <type_traits>
 
 #include "common.cuh"
 #include "ptx_sm103.cuh"
@@ -410,6 +409,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tmem = tmem_base_sh;
     // inputs may be produced by the previous kernel on the stream: wait for it before any global access
     griddep_wait();
+    // the merge's first cluster barrier joins the softmax warps' row statistics; these two warps have nothing
+    // to publish there and must not hold it up
+    if (!FLAT && CS > 1 && warp < 2) cluster_arrive_relaxed();
 
     if (warp == 0) {
         // ================= TMA producer: the Q tile of each stretch, the K/V tiles through the ring
@@ -557,6 +559,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool failed = false;
     bool row_active = false;  // the cluster split's merge below needs the (one) stretch's values
     int m_valid = 0;
+    // merge of the cluster split: the CTA's (m, l) per row, in the last K stage (every Q K^T is complete before
+    // it is written)
+    float2* row_ml = reinterpret_cast<float2*>(sKV + (kStages - 1) * kStageBytes);
 
     // normalised output row r of stretch g (and its log-sum-exp)
     auto write_row = [&](const Seg& g) {
@@ -710,6 +715,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                 mbar_arrive(&bar_p_full[st]);
                 if (failed) break;
             }
+            if (SPREAD) l_run += __shfl_xor_sync(0xffffffffu, l_run, 16);  // the whole row's sum
+            if (!FLAT && CS > 1) {  // the rows' (m, l) for the merge, while the last P V runs
+                if (half == 0) row_ml[r] = make_float2(m_run, l_run);
+                __syncwarp();
+                cluster_arrive_release();
+            }
             // the stretch's accumulator
             if (g.nt > 0 && !failed && !__all_sync(0xffffffffu, mbar_wait(&bar_o_done, nq & 1, kWaitBudget)))
                 failed = true;
@@ -733,7 +744,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                     l_run = 0.f;
                 }
             }
-            if (SPREAD) l_run += __shfl_xor_sync(0xffffffffu, l_run, 16);  // the whole row's sum
             if (g.nt > 0) ++nq;
             if (FLAT && !g.whole && m_valid > p.slot_rows) {  // a block longer than max_q_len: rows past the slot are dropped
                 if (r == 0 && warp == 2) raise_error(p.err, kErrDeviceArg);
@@ -765,115 +775,76 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (CS == 1) {
             if (row_active) write_row(one);
         } else {
-            // ---- merge of the CS partial (m, l, O) triples through distributed shared memory.  After the
-            // first cluster barrier every K/V ring is idle (all of its TMA loads were consumed); each CTA
-            // leaves its partial there and pulls the rows it owns from all peers:
-            //   opart  [kM rows][kD] fp32 partial O (16-byte chunks swizzled by row)
-            //   row_ml [kM] (m, l) of each row's partial
-            //   ml_st, w_st, inv_st  the peers' (m, l) of the owned rows, their weights, 1/L
+            // ---- merge of the CS partial (m, l, O) triples through distributed shared memory.  Row r of the
+            // unit belongs to CTA r / per.  Behind the first cluster barrier (arrived at when the last weights
+            // were written, so it completes while the last P V runs) a thread reads its row's (m, l) of every
+            // CTA, scales its partial O by 2^(m - M) / L and stores it straight into the owner's slot for this
+            // CTA; behind the second the owner adds its slots, in CTA order, from its own shared memory.  Nothing
+            // reads a peer's memory after that, so CTAs leave on their own.  The slots lie where the owner's Q
+            // and K tiles were: every CTA's Q K^T is complete at the first barrier.  What bounds it: the partials
+            // cross between SMs at about 14 bytes a clock (32 KB a CTA in 2400 cycles; whole rows per store,
+            // staged through shared memory, were no faster).  Against pulling the partials row by row behind one
+            // barrier and leaving behind another: 8 x 915 keys 14.1 -> 12.8 us, 8 ragged 13.4 -> 11.8 us, 4 x 8208
+            // 28.9 -> 28.1 us, 1 x 2064 the same (8.2 us).
             m_valid = min(kM, one.B * G - one.mt * kM);
             const int row0 = one.mt * kM;
-            cg::cluster_group cluster = cg::this_cluster();
-            float* opart = reinterpret_cast<float*>(sKV);
-            float2* row_ml = reinterpret_cast<float2*>(sKV + kM * kD * sizeof(float));
-            __syncthreads();  // the producer has drained the ring (after an expired wait copies may still land)
-            if (is_softmax) {
-                if (row_active) {
-#pragma unroll
-                    for (int c = 0; c < kOCols / 4; ++c) {
-                        const int pc = (half * (kOCols / 4) + c) ^ (r & 31);
-                        *reinterpret_cast<float4*>(opart + r * kD + pc * 4) =
-                            make_float4(o_acc[c * 4], o_acc[c * 4 + 1], o_acc[c * 4 + 2], o_acc[c * 4 + 3]);
-                    }
-                }
-                if (half == 0) row_ml[r] = make_float2(m_run, l_run);
-            }
-            cluster.sync();
             const int per = (m_valid + (int)CS - 1) / (int)CS;
+            // slot j, 512 bytes: the Q buffer and K stage 0 are adjacent (128 slots), then K stage 1
+            static_assert(kStages >= 3 && kQBytes + kKVBytes == 128 * kD * 4 && kMaxCluster * kD * 4 <= kKVBytes,
+                          "slots of at most kM + kMaxCluster - 1 rows");
+            auto slot = [&](int j) {
+                return j < 128 ? sQ + j * (kD * 4) : sKV + kStageBytes + (j - 128) * (kD * 4);
+            };
+            __syncwarp();
+            cluster_wait();
+            if (is_softmax && row_active) {
+                float2 ml[kMaxCluster];
+                const uint32_t ml_addr = smem_addr(row_ml + r);
+#pragma unroll
+                for (int pr = 0; pr < kMaxCluster; ++pr) {  // every load in flight together
+                    ml[pr] = make_float2(-INFINITY, 0.f);
+                    if (pr < (int)CS) ml[pr] = ld_cluster_f32x2(mapa(ml_addr, (uint32_t)pr));
+                }
+                float M = -INFINITY, L = 0.f;
+#pragma unroll
+                for (int pr = 0; pr < kMaxCluster; ++pr) M = fmaxf(M, ml[pr].x);
+#pragma unroll
+                for (int pr = 0; pr < kMaxCluster; ++pr)
+                    if (ml[pr].x != -INFINITY) L += fast_exp2(ml[pr].x - M) * ml[pr].y;
+                const float w = m_run != -INFINITY && L > 0.f ? fast_exp2(m_run - M) * (1.f / L) : 0.f;
+                const int owner = r / per;
+                const uint32_t dst = mapa(smem_addr(slot((int)crank * per + r - owner * per)), (uint32_t)owner);
+#pragma unroll
+                for (int c = 0; c < kOCols / 4; ++c)  // 16-byte chunks swizzled by row: rows 512 bytes apart
+                    st_cluster_f32x4(dst + (((half * (kOCols / 4) + c) ^ (r & 31)) << 4), o_acc[c * 4] * w,
+                                     o_acc[c * 4 + 1] * w, o_acc[c * 4 + 2] * w, o_acc[c * 4 + 3] * w);
+                if (p.lse && half == 0 && owner == (int)crank) {
+                    const int lr = row0 + r;
+                    p.lse[(size_t)(one.q0 + lr / G) * p.num_q_heads + one.h * G + lr % G] = (M + __log2f(L)) * kLn2;
+                }
+            }
+            __syncwarp();
+            cluster_sync_all();
             const int rbeg = (int)crank * per;
             const int nmy = max(0, min(m_valid, rbeg + per) - rbeg);
-            // one round of remote loads per owned row: a warp takes the row, lane c its 16-byte chunk c of
-            // every peer's partial O and, for c below the cluster size, peer c's (m, l); the weights then
-            // go round the warp by shuffles.  With more owned rows than warps a warp takes two rows per pass
-            // (rows w and w + 6 of warp w), so up to twelve owned rows take one pass
-            static_assert(kD / 4 == 32 && kThreads % 32 == 0, "a warp's 32 items are one row");
-            const int nitems = nmy * (kD / 4);
-            // one pass: the row of `item` and (PAIR, when present) the row six further, their loads in flight
-            // together and their shuffle chains interleaved
-            auto merge_pass = [&](auto pair_tag, int item) {
-                constexpr bool PAIR = decltype(pair_tag)::value;
-                const bool two = PAIR && item + kThreads < nitems;  // warp-uniform
-                const int c = item % (kD / 4);
-                const int rowa = rbeg + item / (kD / 4), rowb = rowa + kThreads / 32;
-                float4 va[kMaxCluster], vb[kMaxCluster];
-                const float* srca = opart + rowa * kD + ((c ^ (rowa & 31)) * 4);
-                const float* srcb = opart + rowb * kD + ((c ^ (rowb & 31)) * 4);
-#pragma unroll
-                for (int pr = 0; pr < kMaxCluster; ++pr) {
-                    if (pr < (int)CS) va[pr] = *cluster.map_shared_rank(reinterpret_cast<const float4*>(srca), pr);
-                    if constexpr (PAIR) {
-                        if (pr < (int)CS && two)
-                            vb[pr] = *cluster.map_shared_rank(reinterpret_cast<const float4*>(srcb), pr);
-                        else
-                            vb[pr] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
+            for (int j = warp; j < nmy; j += kThreads / 32) {  // a warp per owned row, a 16-byte chunk per lane
+                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                const int ch = (lane ^ ((rbeg + j) & 31)) << 4;
+#pragma unroll 4
+                for (int pr = 0; pr < (int)CS; ++pr) {
+                    const float4 v = *reinterpret_cast<const float4*>(slot(pr * per + j) + ch);
+                    acc.x += v.x;
+                    acc.y += v.y;
+                    acc.z += v.z;
+                    acc.w += v.w;
                 }
-                const float2 mla = c < (int)CS ? *cluster.map_shared_rank(&row_ml[rowa], c) : make_float2(-INFINITY, 0.f);
-                float2 mlb = make_float2(-INFINITY, 0.f);
-                if constexpr (PAIR) {
-                    if (c < (int)CS && two) mlb = *cluster.map_shared_rank(&row_ml[rowb], c);
-                }
-                float Ma = mla.x, Mb = mlb.x;
-#pragma unroll
-                for (int o = 16; o >= 1; o >>= 1) {
-                    Ma = fmaxf(Ma, __shfl_xor_sync(0xffffffffu, Ma, o));
-                    if constexpr (PAIR) Mb = fmaxf(Mb, __shfl_xor_sync(0xffffffffu, Mb, o));
-                }
-                const float wla = mla.x == -INFINITY ? 0.f : fast_exp2(mla.x - Ma);
-                const float wlb = mlb.x == -INFINITY ? 0.f : fast_exp2(mlb.x - Mb);
-                float La = wla * mla.y, Lb = wlb * mlb.y;
-#pragma unroll
-                for (int o = 16; o >= 1; o >>= 1) {
-                    La += __shfl_xor_sync(0xffffffffu, La, o);
-                    if constexpr (PAIR) Lb += __shfl_xor_sync(0xffffffffu, Lb, o);
-                }
-                float4 acca = make_float4(0.f, 0.f, 0.f, 0.f), accb = acca;
-#pragma unroll
-                for (int pr = 0; pr < kMaxCluster; ++pr) {
-                    if (pr < (int)CS) {
-                        const float wa = __shfl_sync(0xffffffffu, wla, pr);
-                        acca.x += wa * va[pr].x;
-                        acca.y += wa * va[pr].y;
-                        acca.z += wa * va[pr].z;
-                        acca.w += wa * va[pr].w;
-                        if constexpr (PAIR) {
-                            const float wb = __shfl_sync(0xffffffffu, wlb, pr);
-                            accb.x += wb * vb[pr].x;
-                            accb.y += wb * vb[pr].y;
-                            accb.z += wb * vb[pr].z;
-                            accb.w += wb * vb[pr].w;
-                        }
-                    }
-                }
-                auto store = [&](int row, float4 acc, float M, float Lsum) {
-                    const float inv = Lsum > 0.f ? 1.f / Lsum : 0.f;
-                    const int lr = row0 + row;
-                    const size_t orow = (size_t)(one.q0 + lr / G) * p.num_q_heads + one.h * G + lr % G;
-                    uint2 w2;
-                    w2.x = pack_bf16x2(acc.x * inv, acc.y * inv);
-                    w2.y = pack_bf16x2(acc.z * inv, acc.w * inv);
-                    *reinterpret_cast<uint2*>(p.o + orow * kD + c * 4) = w2;
-                    if (p.lse && c == 0) p.lse[orow] = (M + __log2f(Lsum)) * kLn2;
-                };
-                store(rowa, acca, Ma, La);
-                if (two) store(rowb, accb, Mb, Lb);
-            };
-            if (nmy > kThreads / 32) {  // more owned rows than warps: two rows per warp and pass
-                for (int item = tid; item < nitems; item += 2 * kThreads) merge_pass(std::true_type{}, item);
-            } else {
-                for (int item = tid; item < nitems; item += kThreads) merge_pass(std::false_type{}, item);
+                const int lr = row0 + rbeg + j;
+                const size_t orow = (size_t)(one.q0 + lr / G) * p.num_q_heads + one.h * G + lr % G;
+                uint2 w2;
+                w2.x = pack_bf16x2(acc.x, acc.y);
+                w2.y = pack_bf16x2(acc.z, acc.w);
+                *reinterpret_cast<uint2*>(p.o + orow * kD + lane * 4) = w2;
             }
-            cluster.sync();  // no CTA leaves while peers may still read its shared memory
         }
     }
 
