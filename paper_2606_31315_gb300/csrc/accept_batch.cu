@@ -43,8 +43,9 @@ constexpr int kBSegs = kBVec;                  // 128-entry segments per warp of
 constexpr int kMaxDrawSplit = 4;               // parts a draw chunk may be cut into
 
 struct BatchParams {
-    const float* target;  // [rows_t][vocab]
-    const float* draft;   // [total_draft][vocab] (T > 0)
+    const float* target;  // [rows_t][ld], vocab entries each
+    const float* draft;   // [total_draft][ld] (T > 0)
+    int ld;               // floats from one row to the next
     const int32_t* tokens;
     const int32_t* cu_draft;
     int num_seqs, total_draft, rows_t, vocab, chunks;
@@ -71,7 +72,7 @@ __device__ __forceinline__ int ticket_acq_rel(int* addr) {
 
 // Row r of the stacked rows: target rows first, then the drafter's rows.
 __device__ __forceinline__ const float* row_ptr(const BatchParams& p, int r) {
-    return r < p.rows_t ? p.target + (size_t)r * p.vocab : p.draft + (size_t)(r - p.rows_t) * p.vocab;
+    return r < p.rows_t ? p.target + (size_t)r * p.ld : p.draft + (size_t)(r - p.rows_t) * p.ld;
 }
 
 // Entry e (16-byte group q, element k) of a chunk held by thread t: q = t + 256 j, so a warp's
@@ -226,8 +227,8 @@ __device__ __forceinline__ DecideIn decide_inputs(const BatchParams& p, int s, i
     q.tx = -INFINITY;
     q.dx = -INFINITY;
     if (!GREEDY && draft && q.x >= 0 && q.x < p.vocab) {
-        q.tx = p.target[(size_t)(q.d0 + s + lane) * p.vocab + q.x];
-        q.dx = p.draft[(size_t)(q.d0 + lane) * p.vocab + q.x];
+        q.tx = p.target[(size_t)(q.d0 + s + lane) * p.ld + q.x];
+        q.dx = p.draft[(size_t)(q.d0 + lane) * p.ld + q.x];
     }
     return q;
 }
@@ -298,8 +299,8 @@ __device__ __forceinline__ void decide_draw(const BatchParams& p, int s, int lan
                 tx = in.tx;
                 dx = in.dx;
             } else if (valid) {
-                tx = p.target[(size_t)(t0 + i) * p.vocab + x];
-                dx = p.draft[(size_t)(d0 + i) * p.vocab + x];
+                tx = p.target[(size_t)(t0 + i) * p.ld + x];
+                dx = p.draft[(size_t)(d0 + i) * p.ld + x];
             }
             // a = min(1, p(x)/q(x)) in the log domain (q(x) = 0 < p(x) gives 1, p(x) = 0 gives 0)
             float a;
@@ -678,8 +679,9 @@ int run_batch(const BatchParams& p, int sm_count, cudaStream_t stream) {
     return rc != BP_OK ? rc : run_decisions<GREEDY, VEC>(p, sm_count, stream);
 }
 
-BatchParams batch_params(const AcceptArgs& a, int* tickets, void* draw_scratch) {
+BatchParams batch_params(const AcceptArgs& a, int ld, int* tickets, void* draw_scratch) {
     BatchParams p;
+    p.ld = ld;
     p.target = a.target;
     p.draft = a.draft;
     p.tokens = a.tokens;
@@ -715,7 +717,7 @@ bool batch_vec(const AcceptArgs& a, bool greedy) {
 int launch_accept_batch(const AcceptArgs& a, int sm_count, int* tickets, void* scratch, cudaStream_t stream) {
     const size_t chunks = ((size_t)a.vocab + kBChunk - 1) / kBChunk, rows = 2 * (size_t)a.total_draft + a.num_seqs;
     uint8_t* w = static_cast<uint8_t*>(scratch);
-    BatchParams p = batch_params(a, tickets, w + align_up(rows * chunks * sizeof(float2), 256));
+    BatchParams p = batch_params(a, a.vocab, tickets, w + align_up(rows * chunks * sizeof(float2), 256));
     p.part = reinterpret_cast<float2*>(w);
     p.inputs_early = 1;  // the statistics kernel releases the decisions after its own wait
     const bool greedy = a.temperature == 0.f, vec = batch_vec(a, greedy);
@@ -723,9 +725,9 @@ int launch_accept_batch(const AcceptArgs& a, int sm_count, int* tickets, void* s
     return vec ? run_batch<false, true>(p, sm_count, stream) : run_batch<false, false>(p, sm_count, stream);
 }
 
-int launch_accept_rows(const AcceptArgs& a, const float2* row_stats, int sm_count, int* tickets, void* draw_scratch,
-                       cudaStream_t stream) {
-    BatchParams p = batch_params(a, tickets, draw_scratch);
+int launch_accept_rows(const AcceptArgs& a, int ld, const float2* row_stats, int sm_count, int* tickets,
+                       void* draw_scratch, cudaStream_t stream) {
+    BatchParams p = batch_params(a, ld, tickets, draw_scratch);
     p.part = const_cast<float2*>(row_stats);
     p.nparts = 1;
     const bool greedy = a.temperature == 0.f, vec = batch_vec(a, greedy);

@@ -284,7 +284,7 @@ int bp_spec_accept_noalloc(const float* target_logits, const float* draft_logits
 
 size_t bp_verify_epilogue_workspace_size(int num_seqs, int total_draft, int vocab) {
     if (num_seqs < 0 || total_draft < 0 || vocab < 1) return 0;
-    return sizeof(WorkspaceHeader) + verify_epilogue_scratch_bytes(num_seqs, total_draft, vocab);
+    return sizeof(WorkspaceHeader) + verify_epilogue_scratch_bytes(num_seqs, total_draft, vocab, true);
 }
 
 int bp_verify_epilogue(const void* lm_head, const void* h_target, const void* h_draft, int hidden, int vocab,
@@ -305,7 +305,7 @@ int bp_verify_epilogue(const void* lm_head, const void* h_target, const void* h_
     const long long rows = (long long)total_draft + num_seqs + (greedy ? 0 : total_draft);
     if (2LL * total_draft + num_seqs > INT_MAX / 2) return BP_ERR_UNSUPPORTED;
     int rc = check_workspace(workspace, workspace_bytes,
-                             bp_verify_epilogue_workspace_size(num_seqs, total_draft, vocab));
+                             sizeof(WorkspaceHeader) + verify_epilogue_scratch_bytes(num_seqs, total_draft, vocab, false));
     if (rc != BP_OK) return rc;
     DeviceInfo dev;
     if ((rc = device_info(&dev)) != BP_OK) return rc;
@@ -323,6 +323,7 @@ int bp_verify_epilogue(const void* lm_head, const void* h_target, const void* h_
     a.tokens = draft_tokens; a.cu_draft = cu_draft; a.u_accept = u_accept; a.u_sample = u_sample;
     a.n_accepted = n_accepted; a.out_tokens = out_tokens; a.accept_prob = accept_prob; a.logits_out = logits_out;
     a.scratch = scratch(workspace);
+    a.scratch_bytes = workspace_bytes - sizeof(WorkspaceHeader);
     a.err_word = err_word(workspace);
     rc = launch_verify_epilogue(a, dev, static_cast<cudaStream_t>(stream));
     if (rc == BP_ERR_CUDA) cudaGetLastError();

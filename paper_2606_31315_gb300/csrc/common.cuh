@@ -127,10 +127,11 @@ size_t accept_batch_scratch_bytes(int num_seqs, int total_draft, int vocab);
 int launch_accept_batch(const AcceptArgs& a, int sm_count, int* tickets, void* scratch, cudaStream_t stream);
 // The throughput path's decisions and draw alone, from statistics merged beforehand: row_stats[r] is row
 // r's (scaled max, sum of 2^(l*log2e/T - max)) over the whole vocabulary, at T = 0 its (max, lowest
-// index bits); rows in the stacked order (target rows, then the drafter's).  At T = 0 no logits are read.
+// index bits); rows in the stacked order (target rows, then the drafter's), ld floats apart.  At T = 0 no
+// logits are read.
 size_t accept_draw_scratch_bytes(int num_seqs, int vocab);
-int launch_accept_rows(const AcceptArgs& a, const float2* row_stats, int sm_count, int* tickets, void* draw_scratch,
-                       cudaStream_t stream);
+int launch_accept_rows(const AcceptArgs& a, int ld, const float2* row_stats, int sm_count, int* tickets,
+                       void* draw_scratch, cudaStream_t stream);
 // Same kernel, scratch taken from the library's own static device array (no workspace).
 int launch_accept_noalloc(const AcceptArgs& a, const DeviceInfo& dev, cudaStream_t stream);
 
@@ -170,18 +171,22 @@ struct VerifyEpilogueArgs {
     float* accept_prob;
     float* logits_out;
     void* scratch;
+    size_t scratch_bytes;
     unsigned int* err_word;
 };
 // Rows (target + drafter) above which the verify epilogue streams the LM head (verify_stream.cu)
 // instead of keeping every logit in tensor memory (verify_epilogue.cu).
 constexpr int kVerifyResidentRows = 64;
-size_t verify_epilogue_scratch_bytes(int num_seqs, int total_draft, int vocab);
+// padded: with the streamed path's logits rows padded to a multiple of 8 (what callers are told to bring);
+// without, what a call needs at least.
+size_t verify_epilogue_scratch_bytes(int num_seqs, int total_draft, int vocab, bool padded);
 // Grid size, padded row count (MMA N) and tiles per CTA; BP_ERR_UNSUPPORTED outside the limits.
 int verify_epilogue_config(int rows, int vocab, int hidden, int sm_count, int* grid, int* np, int* tiles_per_cta);
 int launch_verify_epilogue(const VerifyEpilogueArgs& a, const DeviceInfo& dev, cudaStream_t stream);
 // The streamed path's scratch, carved from the verify epilogue's workspace.
 struct VerifyStreamScratch {
-    float* logits;      // [rows][vocab] fp32: the logits at T > 0 when the caller gives no logits_out
+    float* logits;      // [rows][ld] fp32: the logits at T > 0 when the caller gives no logits_out
+    int ld;             // floats from one of those rows to the next: the vocabulary, rounded up to 8 if it fits
     float2* part;       // [rows][slices] slice statistics
     float2* row_stats;  // [rows] merged statistics
     int* tickets;       // [num_seqs], zero between calls

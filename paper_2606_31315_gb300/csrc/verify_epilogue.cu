@@ -731,7 +731,8 @@ struct VeLayout {
     size_t sync_off, part_off, xg_off, tot_off, total;
     size_t rowst_off, tickets_off, draw_off, logits_off;  // the streamed path (more than 64 rows at T > 0)
 };
-VeLayout ve_layout(int num_seqs, int total_draft, int vocab) {
+int ve_padded(int vocab) { return (int)(((long long)vocab + 7) / 8 * 8); }
+VeLayout ve_layout(int num_seqs, int total_draft, int vocab, bool padded) {
     VeLayout l;
     const int rows = 2 * total_draft + num_seqs;
     l.sync_off = 0;
@@ -745,7 +746,7 @@ VeLayout ve_layout(int num_seqs, int total_draft, int vocab) {
         l.tickets_off = l.rowst_off + align_up((size_t)rows * sizeof(float2), 256);
         l.draw_off = l.tickets_off + align_up((size_t)num_seqs * sizeof(int), 256);
         l.logits_off = l.draw_off + align_up(accept_draw_scratch_bytes(num_seqs, vocab), 256);
-        l.total = l.logits_off + align_up((size_t)rows * (size_t)vocab * sizeof(float), 256);
+        l.total = l.logits_off + align_up((size_t)rows * (size_t)(padded ? ve_padded(vocab) : vocab) * sizeof(float), 256);
     }
     return l;
 }
@@ -785,8 +786,8 @@ int ve_launch(const CUtensorMap& wmap, const VeParams& p, int grid, const Device
 
 }  // namespace
 
-size_t verify_epilogue_scratch_bytes(int num_seqs, int total_draft, int vocab) {
-    return ve_layout(num_seqs, total_draft, vocab).total;
+size_t verify_epilogue_scratch_bytes(int num_seqs, int total_draft, int vocab, bool padded) {
+    return ve_layout(num_seqs, total_draft, vocab, padded).total;
 }
 
 int verify_epilogue_config(int rows, int vocab, int hidden, int sm_count, int* grid, int* np, int* tiles_per_cta) {
@@ -807,11 +808,14 @@ int launch_verify_epilogue(const VerifyEpilogueArgs& a, const DeviceInfo& dev, c
     const bool greedy = a.temperature == 0.f;
     const int rows_t = a.total_draft + a.num_seqs;
     const int rows = rows_t + (greedy ? 0 : a.total_draft);
-    const VeLayout l = ve_layout(a.num_seqs, a.total_draft, a.vocab);
+    const VeLayout l = ve_layout(a.num_seqs, a.total_draft, a.vocab, false);
     uint8_t* ws = static_cast<uint8_t*>(a.scratch);
     if (rows > kVerifyResidentRows) {
         VerifyStreamScratch s;
         s.logits = reinterpret_cast<float*>(ws + l.logits_off);
+        // rows that start 16-byte aligned where the workspace has the room (it does when it was sized for this call)
+        const bool pad = a.vocab <= INT_MAX - 8 && ve_layout(a.num_seqs, a.total_draft, a.vocab, true).total <= a.scratch_bytes;
+        s.ld = pad ? ve_padded(a.vocab) : a.vocab;
         s.part = reinterpret_cast<float2*>(ws + l.part_off);
         s.row_stats = reinterpret_cast<float2*>(ws + l.rowst_off);
         s.tickets = reinterpret_cast<int*>(ws + l.tickets_off);

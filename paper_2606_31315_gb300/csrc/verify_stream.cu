@@ -68,7 +68,8 @@ struct VsParams {
     int ht0, hd0;                   // first target / drafter state of the group (TMA row coordinates)
     int row_t0, row_d0;             // their stacked rows (target rows first, then the drafter's)
     float c2;                       // log2(e) / T (0 at T = 0)
-    float* logits;                  // [rows][vocab] fp32, or null
+    float* logits;                  // [rows][ld] fp32, or null
+    int ld;                         // floats from one logits row to the next
     int vec;                        // logits rows start 16-byte aligned
     int tma_store;                  // the group's rows are contiguous stacked rows: chunks go out by TMA
     int grows;                      // stacked rows of the group
@@ -158,7 +159,7 @@ __device__ __forceinline__ void store_chunk(uint8_t* stage, const uint32_t (&r)[
             const int j = 4 * k + (lane >> 3);
             const int row = stacked_row(p, srow0 + j);
             const float4 x = *reinterpret_cast<const float4*>(stage + j * 128 + ((c ^ (j & 7)) << 4));
-            if (row >= 0) __stcs(reinterpret_cast<float4*>(p.logits + (size_t)row * p.vocab + v0) + c, x);
+            if (row >= 0) __stcs(reinterpret_cast<float4*>(p.logits + (size_t)row * p.ld + v0) + c, x);
         }
     } else {
 #pragma unroll 4
@@ -166,7 +167,7 @@ __device__ __forceinline__ void store_chunk(uint8_t* stage, const uint32_t (&r)[
             const int row = stacked_row(p, srow0 + j);
             const float x =
                 *reinterpret_cast<const float*>(stage + j * 128 + (((lane >> 2) ^ (j & 7)) << 4) + ((lane & 3) << 2));
-            if (row >= 0 && lane < n) __stcs(p.logits + (size_t)row * p.vocab + v0 + lane, x);
+            if (row >= 0 && lane < n) __stcs(p.logits + (size_t)row * p.ld + v0 + lane, x);
         }
     }
     __syncwarp();  // the buffer is free for the next chunk
@@ -219,11 +220,13 @@ __global__ void __launch_bounds__(kVsThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_sh;
+    griddep_wait();  // the states (and the scratch the previous call's kernels read) come from earlier kernels
 
     if (warp == kVsProducer) {
         // ---- TMA producer: stage j = (pass j / atoms, hidden atom j % atoms): 256 W rows, the group's states
         if (lane == 0) {
             int issued = 0;
+            const uint64_t pol = l2_policy_evict_first();  // W is read once: it leaves L2 to the states and the logits
             for (int j = 0; j < J; ++j) {
                 const int st = j % STG;
                 if (j >= STG && !mbar_wait(&empty[st], ((j / STG) - 1) & 1, kWaitBudget)) {
@@ -234,7 +237,7 @@ __global__ void __launch_bounds__(kVsThreads, 1)
                 uint8_t* sw = sbase + st * STAGE;
                 uint8_t* sh = sw + kVsWBytes;
                 mbar_arrive_expect_tx(&full[st], stage_tx);
-                tma_load_2d(sw, &wmap, &full[st], a * kVsAtom, (pass0 + pp) * kVsN);
+                tma_load_2d_hint(sw, &wmap, &full[st], a * kVsAtom, (pass0 + pp) * kVsN, pol);
                 if (p.nt) tma_load_2d(sh, &htmap, &full[st], a * kVsAtom, p.ht0);
                 if (p.nd) tma_load_2d(sh + p.nt8 * 128, &hdmap, &full[st], a * kVsAtom, p.hd0);
                 issued = j + 1;
@@ -397,8 +400,20 @@ int vs_launch(const CUtensorMap& wmap, const CUtensorMap& htmap, const CUtensorM
             configured[dev.device] = 1;
         }
     }
-    lm_head_stream_kernel<GREEDY, MT, WRITE><<<grid, kVsThreads, smem, stream>>>(wmap, htmap, hdmap, lmap, p);
-    return cudaGetLastError() == cudaSuccess ? BP_OK : BP_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kVsThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // the set-up overlaps the previous kernel
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, lm_head_stream_kernel<GREEDY, MT, WRITE>, wmap, htmap, hdmap, lmap, p) ==
+                   cudaSuccess
+               ? BP_OK
+               : BP_ERR_CUDA;
 }
 
 template <bool GREEDY>
@@ -446,7 +461,11 @@ int launch_verify_stream(const VerifyEpilogueArgs& a, const VerifyStreamScratch&
     p.passes_extra = passes % grid;
     p.c2 = greedy ? 0.f : 1.4426950408889634f / a.temperature;
     p.logits = logits;
-    p.vec = write && a.vocab % 4 == 0 && reinterpret_cast<uintptr_t>(logits) % 16 == 0;
+    // the path's own rows are padded to 16-byte boundaries where the workspace has the room (8 x 31 rows of a
+    // 50257-entry vocabulary: 115 -> 86 us); the caller's logits_out has rows of exactly the vocabulary
+    const int ld = a.logits_out ? a.vocab : s.ld;
+    p.ld = ld;
+    p.vec = write && ld % 4 == 0 && reinterpret_cast<uintptr_t>(logits) % 16 == 0;
     p.part = s.part;
     p.nslices = grid;
     p.err = a.err_word;
@@ -473,9 +492,9 @@ int launch_verify_stream(const VerifyEpilogueArgs& a, const VerifyStreamScratch&
         p.grows = r1 - r0;
         if (p.tma_store) {
             const cuuint64_t dims[2] = {(cuuint64_t)a.vocab, (cuuint64_t)(r1 - r0)};
-            const cuuint64_t strides[1] = {(cuuint64_t)a.vocab * 4};
+            const cuuint64_t strides[1] = {(cuuint64_t)ld * 4};
             const cuuint32_t box[2] = {32, 32};
-            if (encode_tensor_map(&lmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, logits + (size_t)r0 * a.vocab, dims,
+            if (encode_tensor_map(&lmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, logits + (size_t)r0 * ld, dims,
                                   strides, box, CU_TENSOR_MAP_SWIZZLE_128B) != BP_OK)
                 return BP_ERR_CUDA;
         }
@@ -505,7 +524,7 @@ int launch_verify_stream(const VerifyEpilogueArgs& a, const VerifyStreamScratch&
 
     AcceptArgs aa;
     aa.target = logits;
-    aa.draft = logits ? logits + (size_t)rows_t * a.vocab : nullptr;
+    aa.draft = logits ? logits + (size_t)rows_t * ld : nullptr;
     aa.tokens = a.tokens;
     aa.cu_draft = a.cu_draft;
     aa.num_seqs = a.num_seqs;
@@ -519,7 +538,7 @@ int launch_verify_stream(const VerifyEpilogueArgs& a, const VerifyStreamScratch&
     aa.accept_prob = a.accept_prob;
     aa.scratch = nullptr;
     aa.err_word = a.err_word;
-    return launch_accept_rows(aa, s.row_stats, dev.sm_count, s.tickets, s.draw, stream);
+    return launch_accept_rows(aa, ld, s.row_stats, dev.sm_count, s.tickets, s.draw, stream);
 }
 
 }  // namespace bp

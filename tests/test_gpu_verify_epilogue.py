@@ -410,3 +410,25 @@ def test_long_context_batch_full_head(qwen_weight, temp):
             exact += int(planted.sum())
             ks.update(int(k) for k, pl in zip(tref["n_accepted"], planted) if pl)
     assert exact >= 24 and len(ks) >= 3, (exact, ks)
+
+
+@pytest.mark.parametrize("vocab", [5003, 20002, 20004, 20008])
+def test_streamed_rows_padded_or_not(vocab):
+    """141 rows (two halves): the streamed path's own logits rows are padded to 8 entries where the workspace
+    has the room and are `vocab` apart in a workspace of the smallest accepted size.  The sums run over the
+    same entries in the same order, so every output is the same bit for bit; one byte less is refused."""
+    w = wl.custom(seed=vocab, ctx=(0,) * 5, block=(16, 16, 9, 16, 16), vocab=vocab)
+    inp = wl.lm_head_inputs(w, 1.0, hidden=128)
+    ref = run_oracle(inp, 1.0)
+    full = run_gpu(inp, 1.0)
+    compare(inp, 1.0, full, ref)
+    td, s = len(inp["draft_tokens"]), len(inp["cu_draft"]) - 1
+    up = lambda n: -(-n // 256) * 256  # noqa: E731
+    rows = 2 * td + s
+    least = bp.verify_epilogue_workspace_size(s, td, vocab) - up(rows * (-(-vocab // 8) * 8) * 4) + up(rows * vocab * 4)
+    small = run_gpu(inp, 1.0, ws=bp.workspace(least, dev()))
+    for a, b in zip(full[:4], small[:4]):
+        np.testing.assert_array_equal(a, b)
+    with pytest.raises(bp.BlockPilotError) as e:
+        run_gpu(inp, 1.0, ws=bp.workspace(least, dev())[:-1])
+    assert e.value.status == 4
