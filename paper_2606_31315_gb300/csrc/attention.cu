@@ -1549,7 +1549,10 @@ int launch_attention_f32(const AttentionArgs& a, const DeviceInfo& dev, cudaStre
 // --------------------------------------------------------------------------- paged KV append
 // Writes each sequence's new K/V rows (its block) into their slots of the paged cache: new row
 // i of sequence s is key L_s + i, with L_s = (cu_kv[s+1] - cu_kv[s]) - (cu_new[s+1] - cu_new[s]).
-// One warp per (new row, KV head): 16-byte copies of the K row and of the V row.
+// One warp per (new row, KV head): 16-byte copies of the K row and of the V row.  In a decoding loop this runs
+// once a layer between two attentions and is a chain of round trips to L2, not a copy: so the warp's first 32
+// copies are loaded ahead of their place, up to 32 sequences' offsets are read in one round instead of a binary
+// search, and a single sequence's page is picked from block-table entries loaded with the offsets.
 __global__ void __launch_bounds__(256) kv_append_kernel(uint8_t* __restrict__ kc, uint8_t* __restrict__ vc,
                                                         const uint8_t* __restrict__ kn,
                                                         const uint8_t* __restrict__ vn,
@@ -1563,23 +1566,47 @@ __global__ void __launch_bounds__(256) kv_append_kernel(uint8_t* __restrict__ kc
     const int warp = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (warp >= total_new * hkv) return;
     const int t = warp / hkv, hh = warp % hkv;
-    int lo = 0, hi = num_seqs;  // largest s with cu_new[s] <= t
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(cu_new + mid) <= t) lo = mid; else hi = mid;
+    // copy `item`: 16 bytes of the K row, then of the V row
+    const int n16 = row_bytes / 16;
+    const size_t src = ((size_t)t * hkv + hh) * row_bytes;
+    auto from = [&](int item) {
+        return reinterpret_cast<const uint4*>(item < n16 ? kn + src + (size_t)item * 16 : vn + src + (size_t)(item - n16) * 16);
+    };
+    uint4 first = make_uint4(0u, 0u, 0u, 0u);
+    if (lane < 2 * n16) first = *from(lane);
+    int s = 0, pos, page0 = 0, page1 = 0;
+    const bool one = num_seqs == 1;  // offsets 0 and total_new
+    if (one) {
+        if (lane < pages_per_seq) page0 = __ldg(bt + lane);
+        if (lane + 32 < pages_per_seq) page1 = __ldg(bt + lane + 32);
+        pos = __ldg(cu_kv + 1) - __ldg(cu_kv) - total_new + t;
+    } else if (num_seqs <= 32) {  // the sequences after the first that start at or before row t, counted
+        const int begin = lane < num_seqs ? __ldg(cu_new + lane) : 0, end = lane < num_seqs ? __ldg(cu_new + lane + 1) : 0;
+        const int len = lane < num_seqs ? __ldg(cu_kv + lane + 1) - __ldg(cu_kv + lane) : 0;
+        s = __popc(__ballot_sync(0xffffffffu, lane > 0 && lane < num_seqs && begin <= t));
+        pos = __shfl_sync(0xffffffffu, len - (end - begin) - begin, s) + t;
+    } else {
+        int lo = 0, hi = num_seqs;  // largest s with cu_new[s] <= t
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (__ldg(cu_new + mid) <= t) lo = mid; else hi = mid;
+        }
+        s = lo;
+        const int nb = __ldg(cu_new + s + 1) - __ldg(cu_new + s);
+        const int len = __ldg(cu_kv + s + 1) - __ldg(cu_kv + s);
+        pos = len - nb + (t - __ldg(cu_new + s));
     }
-    const int s = lo;
-    const int nb = __ldg(cu_new + s + 1) - __ldg(cu_new + s);
-    const int len = __ldg(cu_kv + s + 1) - __ldg(cu_kv + s);
-    const int pos = len - nb + (t - __ldg(cu_new + s));
-    const long long page = __ldg(bt + (size_t)s * pages_per_seq + (pos >> page_shift));
+    const int pi = pos >> page_shift;
+    long long page;
+    if (one && pi < 64) page = __shfl_sync(0xffffffffu, pi < 32 ? page0 : page1, pi & 31);
+    else page = __ldg(bt + (size_t)s * pages_per_seq + pi);
     const long long slot = (page << page_shift) + (pos & ((1 << page_shift) - 1));
     const size_t dst = ((size_t)slot * hkv + hh) * row_bytes;
-    const size_t src = ((size_t)t * hkv + hh) * row_bytes;
-    for (int b = lane * 16; b < row_bytes; b += 32 * 16) {
-        *reinterpret_cast<uint4*>(kc + dst + b) = *reinterpret_cast<const uint4*>(kn + src + b);
-        *reinterpret_cast<uint4*>(vc + dst + b) = *reinterpret_cast<const uint4*>(vn + src + b);
-    }
+    auto to = [&](int item) {
+        return reinterpret_cast<uint4*>(item < n16 ? kc + dst + (size_t)item * 16 : vc + dst + (size_t)(item - n16) * 16);
+    };
+    if (lane < 2 * n16) *to(lane) = first;
+    for (int item = lane + 32; item < 2 * n16; item += 32) *to(item) = *from(item);
 }
 
 int launch_kv_append(const KvAppendArgs& a, cudaStream_t stream) {
