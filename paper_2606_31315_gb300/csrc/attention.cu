@@ -1079,69 +1079,71 @@ __global__ void __launch_bounds__(kFThreads) attn_f32_kernel(const F32Params p) 
                 cp_async_wait_group<0>();
             }
             __syncthreads();
-            const float* kk = sK + st * kFK * kLdK;
-            const float* vv = sV + st * kFK * DP;
-            float x[2][4];
+            if (4 * (tid >> 5) < nr) {  // a warp of padding rows only leaves shared memory to the others
+                const float* kk = sK + st * kFK * kLdK;
+                const float* vv = sV + st * kFK * DP;
+                float x[2][4];
 #pragma unroll
-            for (int a = 0; a < 2; ++a)
+                for (int a = 0; a < 2; ++a)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) x[a][j] = 0.f;
+                    for (int j = 0; j < 4; ++j) x[a][j] = 0.f;
 #pragma unroll 4
-            for (int d = 0; d < DP; d += 4) {
-                const float4 qa = *reinterpret_cast<const float4*>(sQ + (2 * ty) * kLdK + d);
-                const float4 qb = *reinterpret_cast<const float4*>(sQ + (2 * ty + 1) * kLdK + d);
+                for (int d = 0; d < DP; d += 4) {
+                    const float4 qa = *reinterpret_cast<const float4*>(sQ + (2 * ty) * kLdK + d);
+                    const float4 qb = *reinterpret_cast<const float4*>(sQ + (2 * ty + 1) * kLdK + d);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float4 kv = *reinterpret_cast<const float4*>(kk + (tx + 16 * j) * kLdK + d);
-                    x[0][j] = fmaf(qa.w, kv.w, fmaf(qa.z, kv.z, fmaf(qa.y, kv.y, fmaf(qa.x, kv.x, x[0][j]))));
-                    x[1][j] = fmaf(qb.w, kv.w, fmaf(qb.z, kv.z, fmaf(qb.y, kv.y, fmaf(qb.x, kv.x, x[1][j]))));
-                }
-            }
-#pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                float mx = -INFINITY;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    x[a][j] = c * kFK + tx + 16 * j < limit[a] ? x[a][j] * p.scale : -INFINITY;
-                    mx = fmaxf(mx, x[a][j]);
-                }
-#pragma unroll
-                for (int o = 8; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                const float mn = fmaxf(m[a], mx);
-                const bool any = mn != -INFINITY;  // some key of this CTA is visible to the row so far
-                const float alpha = m[a] == -INFINITY ? 0.f : expf(m[a] - mn);
-                float sum = 0.f;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float w = any ? expf(x[a][j] - mn) : 0.f;
-                    sum += w;
-                    sP[(2 * ty + a) * kFPadP + tx + 16 * j] = w;
-                }
-                l[a] = l[a] * alpha + sum;  // this thread's keys; joined over the row below
-#pragma unroll
-                for (int e = 0; e < 4 * kCols; ++e) acc[a][e] *= alpha;
-                m[a] = mn;
-            }
-            __syncwarp();  // a row pair's weights are written and read by one half-warp
-#pragma unroll 2
-            for (int k4 = 0; k4 < kFK; k4 += 4) {
-                const float4 pa = *reinterpret_cast<const float4*>(sP + (2 * ty) * kFPadP + k4);
-                const float4 pb = *reinterpret_cast<const float4*>(sP + (2 * ty + 1) * kFPadP + k4);
-                const float wa[4] = {pa.x, pa.y, pa.z, pa.w}, wb[4] = {pb.x, pb.y, pb.z, pb.w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-#pragma unroll
-                    for (int cc = 0; cc < kCols; ++cc) {
-                        const float4 z = *reinterpret_cast<const float4*>(vv + (k4 + e) * DP + 64 * cc + 4 * tx);
-                        acc[0][4 * cc] = fmaf(wa[e], z.x, acc[0][4 * cc]);
-                        acc[0][4 * cc + 1] = fmaf(wa[e], z.y, acc[0][4 * cc + 1]);
-                        acc[0][4 * cc + 2] = fmaf(wa[e], z.z, acc[0][4 * cc + 2]);
-                        acc[0][4 * cc + 3] = fmaf(wa[e], z.w, acc[0][4 * cc + 3]);
-                        acc[1][4 * cc] = fmaf(wb[e], z.x, acc[1][4 * cc]);
-                        acc[1][4 * cc + 1] = fmaf(wb[e], z.y, acc[1][4 * cc + 1]);
-                        acc[1][4 * cc + 2] = fmaf(wb[e], z.z, acc[1][4 * cc + 2]);
-                        acc[1][4 * cc + 3] = fmaf(wb[e], z.w, acc[1][4 * cc + 3]);
+                    for (int j = 0; j < 4; ++j) {
+                        const float4 kv = *reinterpret_cast<const float4*>(kk + (tx + 16 * j) * kLdK + d);
+                        x[0][j] = fmaf(qa.w, kv.w, fmaf(qa.z, kv.z, fmaf(qa.y, kv.y, fmaf(qa.x, kv.x, x[0][j]))));
+                        x[1][j] = fmaf(qb.w, kv.w, fmaf(qb.z, kv.z, fmaf(qb.y, kv.y, fmaf(qb.x, kv.x, x[1][j]))));
                     }
+                }
+#pragma unroll
+                for (int a = 0; a < 2; ++a) {
+                    float mx = -INFINITY;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        x[a][j] = c * kFK + tx + 16 * j < limit[a] ? x[a][j] * p.scale : -INFINITY;
+                        mx = fmaxf(mx, x[a][j]);
+                    }
+#pragma unroll
+                    for (int o = 8; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                    const float mn = fmaxf(m[a], mx);
+                    const bool any = mn != -INFINITY;  // some key of this CTA is visible to the row so far
+                    const float alpha = m[a] == -INFINITY ? 0.f : expf(m[a] - mn);
+                    float sum = 0.f;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float w = any ? expf(x[a][j] - mn) : 0.f;
+                        sum += w;
+                        sP[(2 * ty + a) * kFPadP + tx + 16 * j] = w;
+                    }
+                    l[a] = l[a] * alpha + sum;  // this thread's keys; joined over the row below
+#pragma unroll
+                    for (int e = 0; e < 4 * kCols; ++e) acc[a][e] *= alpha;
+                    m[a] = mn;
+                }
+                __syncwarp();  // a row pair's weights are written and read by one half-warp
+#pragma unroll 2
+                for (int k4 = 0; k4 < kFK; k4 += 4) {
+                    const float4 pa = *reinterpret_cast<const float4*>(sP + (2 * ty) * kFPadP + k4);
+                    const float4 pb = *reinterpret_cast<const float4*>(sP + (2 * ty + 1) * kFPadP + k4);
+                    const float wa[4] = {pa.x, pa.y, pa.z, pa.w}, wb[4] = {pb.x, pb.y, pb.z, pb.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+#pragma unroll
+                        for (int cc = 0; cc < kCols; ++cc) {
+                            const float4 z = *reinterpret_cast<const float4*>(vv + (k4 + e) * DP + 64 * cc + 4 * tx);
+                            acc[0][4 * cc] = fmaf(wa[e], z.x, acc[0][4 * cc]);
+                            acc[0][4 * cc + 1] = fmaf(wa[e], z.y, acc[0][4 * cc + 1]);
+                            acc[0][4 * cc + 2] = fmaf(wa[e], z.z, acc[0][4 * cc + 2]);
+                            acc[0][4 * cc + 3] = fmaf(wa[e], z.w, acc[0][4 * cc + 3]);
+                            acc[1][4 * cc] = fmaf(wb[e], z.x, acc[1][4 * cc]);
+                            acc[1][4 * cc + 1] = fmaf(wb[e], z.y, acc[1][4 * cc + 1]);
+                            acc[1][4 * cc + 2] = fmaf(wb[e], z.z, acc[1][4 * cc + 2]);
+                            acc[1][4 * cc + 3] = fmaf(wb[e], z.w, acc[1][4 * cc + 3]);
+                        }
+                }
             }
             __syncthreads();  // the stage and the weights are free
         }
