@@ -174,12 +174,13 @@ struct VerifyEpilogueArgs {
     size_t scratch_bytes;
     unsigned int* err_word;
 };
-// Rows (target + drafter) above which the verify epilogue streams the LM head (verify_stream.cu)
-// instead of keeping every logit in tensor memory (verify_epilogue.cu).
+// Rows (target + drafter) that the verify epilogue's resident kernel (verify_epilogue.cu: every logit kept in
+// tensor memory) can take, and up to which it is chosen at T > 0; others stream (verify_stream.cu).
 constexpr int kVerifyResidentRows = 64;
-// padded: with the streamed path's logits rows padded to a multiple of 8 (what callers are told to bring);
-// without, what a call needs at least.
-size_t verify_epilogue_scratch_bytes(int num_seqs, int total_draft, int vocab, bool padded);
+constexpr int kVerifyKeepRows = 32;
+// full: what callers are told to bring (the streamed path's regions wherever it is chosen, its logits rows padded
+// to a multiple of 8); otherwise what a call needs at least.
+size_t verify_epilogue_scratch_bytes(int num_seqs, int total_draft, int vocab, bool full);
 // Grid size, padded row count (MMA N) and tiles per CTA; BP_ERR_UNSUPPORTED outside the limits.
 int verify_epilogue_config(int rows, int vocab, int hidden, int sm_count, int* grid, int* np, int* tiles_per_cta);
 int launch_verify_epilogue(const VerifyEpilogueArgs& a, const DeviceInfo& dev, cudaStream_t stream);

@@ -18,12 +18,12 @@
 //     rows, zero rows up to NP) into the stage with 16-byte cp.async copies; one thread of warp 1
 //     issues M=128 x N=NP x K=16 tcgen05 MMAs into the tile's own NP columns of tensor memory.
 //   * Warps 4-7 read each finished tile (TMEM lane = vocabulary entry, column = row) while the next
-//     one streams: every row's running max and sum of 2^(l*log2e/T - max) (T = 0: running argmax,
-//     lowest index first), and the scaled logits at the draft tokens the slice holds.
+//     one streams: every row's running max and sum of 2^(l*log2e/T - max), and the scaled logits at the
+//     draft tokens the slice holds.
 //   * Grid barrier 1.  Every CTA merges the slices' statistics of every row in the same fixed
 //     order, so all CTAs hold bit-identical normalisers, ratios a_i and first rejections k_s; CTA 0
-//     writes n_accepted, the accepted drafts and accept_prob (T = 0: the emitted argmax too).
-//   * T > 0: every CTA sums its slice's mass of max(0, p_k - q_k) (p_gamma for a bonus draw) per
+//     writes n_accepted, the accepted drafts and accept_prob.
+//   * Every CTA sums its slice's mass of max(0, p_k - q_k) (p_gamma for a bonus draw) per
 //     sequence in exact 2^-52 fixed point; grid barrier 2; the CTA whose slice holds the crossing of
 //     u_s * total recomputes its 32-entry chunks, finds the entry and writes the emitted token.
 //   * The last CTA out clears the grid-barrier counters for the next call.
@@ -74,7 +74,7 @@ struct VeParams {
     int32_t* out_tokens;
     float* accept_prob;
     float* logits_out;              // [rows][vocab] or null
-    float2* part;                   // [rows][grid] slice statistics (T = 0: value, index bits)
+    float2* part;                   // [rows][grid] slice statistics
     float2* xg;                     // [total_draft] scaled (target, drafter) logits at the draft token
     ulonglong2* tot;                // [num_seqs][grid] slice masses of r and p, 2^-52 units
     unsigned int* sync;             // [0] grid-barrier arrivals, [1] exits; zero between calls
@@ -152,25 +152,6 @@ __device__ __forceinline__ float2 lse_reduce_scatter32(float (&m)[32], float (&s
     }
     return make_float2(m[0], s[0]);
 }
-// The same for (value, index) argmax pairs.
-__device__ __forceinline__ float2 amax_reduce_scatter32(float (&v)[32], int (&ix)[32], int lane) {
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int j = 0; j < o; ++j) {
-            const float sv = up ? v[j] : v[j + o];
-            const int si = up ? ix[j] : ix[j + o];
-            float kv = up ? v[j + o] : v[j];
-            int ki = up ? ix[j + o] : ix[j];
-            amax_merge(kv, ki, __shfl_xor_sync(0xffffffffu, sv, o), __shfl_xor_sync(0xffffffffu, si, o));
-            v[j] = kv;
-            ix[j] = ki;
-        }
-    }
-    return make_float2(v[0], __int_as_float(ix[0]));
-}
-
 // Weights of this lane's entry in tile t of the slice for one sequence's draw: x.x = r = max(0, p - q)
 // (0 without a draft row), x.y = p.  The crossing search recomputes them with this same code.
 struct DrawRow {
@@ -193,7 +174,7 @@ __device__ __forceinline__ float2 entry_weights(uint32_t tmem_q, int t, const Dr
     return draw_weights(lt, ld, d, in_vocab, c2);
 }
 
-template <bool GREEDY, int NP, int APS>
+template <int NP, int APS>
 __global__ void __launch_bounds__(kVeThreads, 1)
     verify_epilogue_kernel(const __grid_constant__ CUtensorMap wmap, const VeParams p) {
     constexpr int STG = ve_stages(NP, APS);
@@ -340,28 +321,26 @@ __global__ void __launch_bounds__(kVeThreads, 1)
         for (int i = lane; i <= S; i += 32) cu_sh[i] = p.cu_draft[i];
         for (int i = lane; i < p.total_draft; i += 32) {  // inputs of the decisions, read before they are due
             tok_sh[i] = p.tokens[i];
-            ua_sh[i] = GREEDY ? 0.f : p.u_accept[i];
+            ua_sh[i] = p.u_accept[i];
         }
         __syncwarp();
-        if (!GREEDY) {
-            for (int i = lane; i < p.total_draft; i += 32) {
-                const int x = tok_sh[i];
-                if (x >= v0 && x < v1) {
-                    int lo = 0, hi = S;  // sequence of draft i: cu[lo] <= i < cu[lo + 1]
-                    while (hi - lo > 1) {
-                        const int mid = (lo + hi) >> 1;
-                        if (cu_sh[mid] <= i) lo = mid; else hi = mid;
-                    }
-                    const int o = atomicAdd(&own_n, 1);
-                    own_v[o] = x - v0;
-                    own_i[o] = i;
-                    own_ct[o] = i + lo;           // target row of draft i
-                    own_cd[o] = p.rows_t + i;     // its drafter row
+        for (int i = lane; i < p.total_draft; i += 32) {
+            const int x = tok_sh[i];
+            if (x >= v0 && x < v1) {
+                int lo = 0, hi = S;  // sequence of draft i: cu[lo] <= i < cu[lo + 1]
+                while (hi - lo > 1) {
+                    const int mid = (lo + hi) >> 1;
+                    if (cu_sh[mid] <= i) lo = mid; else hi = mid;
                 }
+                const int o = atomicAdd(&own_n, 1);
+                own_v[o] = x - v0;
+                own_i[o] = i;
+                own_ct[o] = i + lo;           // target row of draft i
+                own_cd[o] = p.rows_t + i;     // its drafter row
             }
-            __threadfence_block();
-            named_arrive(2, 160);
         }
+        __threadfence_block();
+        named_arrive(2, 160);
         if (c == 0)
             for (int i = lane; i < p.total_draft; i += 32) {
                 const int x = tok_sh[i];
@@ -372,18 +351,13 @@ __global__ void __launch_bounds__(kVeThreads, 1)
         const int q = warp & 3;
         const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
         float m[NP], s[NP];
-        int ix[NP];
 #pragma unroll
         for (int e = 0; e < NP; ++e) {
             m[e] = -INFINITY;
             s[e] = 0.f;
-            ix[e] = INT_MAX;
         }
-        int nown = 0;
-        if (!GREEDY) {
-            named_sync(2, 160);
-            nown = own_n;
-        }
+        named_sync(2, 160);
+        const int nown = own_n;
         for (int t = 0; t < ntile; ++t) {
             if (!mbar_wait(&acc_full[t], 0, kWaitBudget)) {
                 raise_error(p.err, kErrTimeout);
@@ -403,18 +377,11 @@ __global__ void __launch_bounds__(kVeThreads, 1)
                     for (int e = 0; e < 32; ++e) {
                         if (h0 + e < p.rows) {
                             const float l = __uint_as_float(r[e]);
-                            if (GREEDY) {
-                                if (l > m[h0 + e]) {  // entries arrive in increasing index: ties keep the first
-                                    m[h0 + e] = l;
-                                    ix[h0 + e] = v;
-                                }
-                            } else {
-                                const float x = __fmul_rn(l, p.c2);
-                                const float d = __fsub_rn(x, m[h0 + e]);
-                                const float w = ex2(-fabsf(d));
-                                s[h0 + e] = d > 0.f ? __fmaf_rn(s[h0 + e], w, 1.f) : __fadd_rn(s[h0 + e], w);
-                                m[h0 + e] = fmaxf(m[h0 + e], x);
-                            }
+                            const float x = __fmul_rn(l, p.c2);
+                            const float d = __fsub_rn(x, m[h0 + e]);
+                            const float w = ex2(-fabsf(d));
+                            s[h0 + e] = d > 0.f ? __fmaf_rn(s[h0 + e], w, 1.f) : __fadd_rn(s[h0 + e], w);
+                            m[h0 + e] = fmaxf(m[h0 + e], x);
                             if (p.logits_out) p.logits_out[(size_t)(h0 + e) * p.vocab + v] = l;
                         }
                     }
@@ -430,39 +397,18 @@ __global__ void __launch_bounds__(kVeThreads, 1)
         // the statistics of every row over the warp's 32 lanes, then over the four warps
 #pragma unroll
         for (int h0 = 0; h0 < NP; h0 += 32) {
-            float2 res;
-            if (GREEDY) {
-                float vv[32];
-                int ii[32];
+            float mm[32], ss[32];
 #pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    vv[e] = m[h0 + e];
-                    ii[e] = ix[h0 + e];
-                }
-                res = amax_reduce_scatter32(vv, ii, lane);
-            } else {
-                float mm[32], ss[32];
-#pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    mm[e] = m[h0 + e];
-                    ss[e] = s[h0 + e];
-                }
-                res = lse_reduce_scatter32(mm, ss, lane);
+            for (int e = 0; e < 32; ++e) {
+                mm[e] = m[h0 + e];
+                ss[e] = s[h0 + e];
             }
-            wst[q][h0 + lane] = res;
+            wst[q][h0 + lane] = lse_reduce_scatter32(mm, ss, lane);
         }
         named_sync(1, 128);
         for (int r = tid - kVeEpi * 32; r < p.rows; r += 128) {
             float2 a = wst[0][r];
-            for (int w = 1; w < 4; ++w) {
-                if (GREEDY) {
-                    int ai = __float_as_int(a.y);
-                    amax_merge(a.x, ai, wst[w][r].x, __float_as_int(wst[w][r].y));
-                    a.y = __int_as_float(ai);
-                } else {
-                    lse_merge(a.x, a.y, wst[w][r].x, wst[w][r].y);
-                }
-            }
+            for (int w = 1; w < 4; ++w) lse_merge(a.x, a.y, wst[w][r].x, wst[w][r].y);
             p.part[(size_t)r * grid + c] = a;
         }
     }
@@ -481,7 +427,7 @@ __global__ void __launch_bounds__(kVeThreads, 1)
 #pragma unroll
             for (int m = 0; m < kVeMaxGrid / 32; ++m) {
                 const int cc = m * 32 + lane;
-                const float2 none = make_float2(-INFINITY, GREEDY ? __int_as_float(INT_MAX) : 0.f);
+                const float2 none = make_float2(-INFINITY, 0.f);
                 x[b][m] = (r < p.rows && cc < grid) ? __ldcg(&p.part[(size_t)r * grid + cc]) : none;
             }
         }
@@ -489,22 +435,14 @@ __global__ void __launch_bounds__(kVeThreads, 1)
         for (int b = 0; b < 4; ++b) {
             const int r = r0 + b * (kVeThreads / 32);
             float a0 = -INFINITY, a1 = 0.f;
-            int ai = INT_MAX;
 #pragma unroll
-            for (int m = 0; m < kVeMaxGrid / 32; ++m) {
-                if (GREEDY) amax_merge(a0, ai, x[b][m].x, __float_as_int(x[b][m].y));
-                else lse_merge(a0, a1, x[b][m].x, x[b][m].y);
-            }
+            for (int m = 0; m < kVeMaxGrid / 32; ++m) lse_merge(a0, a1, x[b][m].x, x[b][m].y);
 #pragma unroll
             for (int o = 16; o >= 1; o >>= 1) {
                 const float b0 = __shfl_xor_sync(0xffffffffu, a0, o);
-                if (GREEDY) {
-                    amax_merge(a0, ai, b0, __shfl_xor_sync(0xffffffffu, ai, o));
-                } else {
-                    lse_merge(a0, a1, b0, __shfl_xor_sync(0xffffffffu, a1, o));
-                }
+                lse_merge(a0, a1, b0, __shfl_xor_sync(0xffffffffu, a1, o));
             }
-            if (lane == 0 && r < p.rows) rst[r] = GREEDY ? make_float2(a0, __int_as_float(ai)) : make_float2(a0, a1);
+            if (lane == 0 && r < p.rows) rst[r] = make_float2(a0, a1);
         }
     }
     __syncthreads();
@@ -519,9 +457,7 @@ __global__ void __launch_bounds__(kVeThreads, 1)
         const int ct = i + sq;
         const int x = tok_sh[i];
         float a;
-        if (GREEDY) {
-            a = (x == __float_as_int(rst[ct].y)) ? 1.f : 0.f;
-        } else if (x < 0 || x >= p.vocab) {
+        if (x < 0 || x >= p.vocab) {
             a = 0.f;
         } else {
             const float2 xx = __ldcg(&p.xg[i]);
@@ -531,179 +467,176 @@ __global__ void __launch_bounds__(kVeThreads, 1)
             a = fminf(1.f, ex2(lr) * __fdiv_rn(sd.y, st.y));
         }
         if (c == 0 && p.accept_prob) p.accept_prob[i] = a;
-        const bool rej = GREEDY ? (a == 0.f) : !(ua_sh[i] < a);
+        const bool rej = !(ua_sh[i] < a);
         if (rej) atomicMin(&k_sh[sq], i - cu_sh[sq]);
     }
     __syncthreads();
-    if (c == 0) {  // n_accepted, the accepted drafts, -1 past the emitted slot (T = 0: the emitted argmax)
+    if (c == 0) {  // n_accepted, the accepted drafts, -1 past the emitted slot
         for (int sq = warp; sq < S; sq += kVeThreads / 32) {
             const int d0 = cu_sh[sq], g = cu_sh[sq + 1] - d0, k = k_sh[sq], t0 = d0 + sq;
             for (int j = lane; j <= g; j += 32) {
                 if (j < k) p.out_tokens[t0 + j] = tok_sh[d0 + j];
                 else if (j > k) p.out_tokens[t0 + j] = -1;
-                else if (GREEDY) p.out_tokens[t0 + j] = __float_as_int(rst[t0 + k].y);
             }
             if (lane == 0) p.n_accepted[sq] = k;
         }
     }
 
-    if (!GREEDY) {
-        // ---- this slice's mass of each sequence's draw distribution, exact fixed point; the masses of
-        // its 32-entry chunks are kept (in the ring's shared memory, idle now) for the crossing search
-        ulonglong2* chunk = reinterpret_cast<ulonglong2*>(sW);  // [sequence][tile][lane quarter]
-        const int q = warp & 3;
-        const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
-        if (warp >= kVeEpi) {
-            for (int sq = 0; sq < S; ++sq) {
-                const int d0 = cu_sh[sq], g = cu_sh[sq + 1] - d0, k = k_sh[sq];
-                DrawRow d;
-                d.ct = d0 + sq + k;
-                d.cd = k < g ? p.rows_t + d0 + k : -1;
-                d.Mt = rst[d.ct].x;
-                d.izt = __fdiv_rn(1.f, rst[d.ct].y);
-                d.Md = d.cd >= 0 ? rst[d.cd].x : 0.f;
-                d.izd = d.cd >= 0 ? __fdiv_rn(1.f, rst[d.cd].y) : 0.f;
-                // every tile's two columns first (one wait), then the weights of this lane's entries
-                uint32_t rt[kVeMaxTiles], rd[kVeMaxTiles];
-#pragma unroll
-                for (int t = 0; t < kVeMaxTiles; ++t) {
-                    if (t < ntile) {
-                        rt[t] = tmem_ld1(tq + (uint32_t)(t * NP + d.ct));
-                        rd[t] = d.cd >= 0 ? tmem_ld1(tq + (uint32_t)(t * NP + d.cd)) : 0u;
-                    }
-                }
-                tmem_ld_wait();
-                // lane t ends with the r-mass of tile t's chunk, lane 16 + t with its p-mass (31 shuffles)
-                float v[32];
-#pragma unroll
-                for (int t = 0; t < kVeMaxTiles; ++t) {
-                    float2 w = make_float2(0.f, 0.f);
-                    if (t < ntile)
-                        w = draw_weights(__uint_as_float(rt[t]), __uint_as_float(rd[t]), d,
-                                         v0 + t * kVeM + q * 32 + lane < v1, p.c2);
-                    v[t] = w.x;
-                    v[kVeMaxTiles + t] = w.y;
-                }
-                const unsigned long long f = to_fix(reduce_scatter32(v, lane));
-                const int tl = lane & (kVeMaxTiles - 1);
-                unsigned long long* cf = reinterpret_cast<unsigned long long*>(chunk);
-                if (tl < ntile) cf[((sq * ntile + tl) * 4 + q) * 2 + (lane >> 4)] = f;  // .x = r, .y = p
-                unsigned long long tot = tl < ntile ? f : 0ull;  // lanes 0-15 sum r, lanes 16-31 sum p
-#pragma unroll
-                for (int o = kVeMaxTiles / 2; o >= 1; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-                if (lane == 0) wtot[q][sq].x = tot;
-                if (lane == kVeMaxTiles) wtot[q][sq].y = tot;
-            }
-            named_sync(1, 128);
-            for (int sq = tid - kVeEpi * 32; sq < S; sq += 128) {
-                ulonglong2 a = wtot[0][sq];
-                for (int w = 1; w < 4; ++w) {
-                    a.x += wtot[w][sq].x;
-                    a.y += wtot[w][sq].y;
-                }
-                p.tot[(size_t)sq * grid + c] = a;
-            }
-        }
-
-        // ================= grid barrier 2: every slice's masses are out
-        if (!grid_barrier(p.sync, 2u * (unsigned)grid, &ok_sh)) raise_error(p.err, kErrTimeout);
-
+    // ---- this slice's mass of each sequence's draw distribution, exact fixed point; the masses of
+    // its 32-entry chunks are kept (in the ring's shared memory, idle now) for the crossing search
+    ulonglong2* chunk = reinterpret_cast<ulonglong2*>(sW);  // [sequence][tile][lane quarter]
+    const int q = warp & 3;
+    const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
+    if (warp >= kVeEpi) {
         for (int sq = 0; sq < S; ++sq) {
             const int d0 = cu_sh[sq], g = cu_sh[sq + 1] - d0, k = k_sh[sq];
-            if (warp == 0) {
-                unsigned long long R = 0, P = 0, Rb = 0, Pb = 0;
-                for (int cc = lane; cc < grid; cc += 32) {
-                    const ulonglong2 x = __ldcg(&p.tot[(size_t)sq * grid + cc]);
-                    R += x.x;
-                    P += x.y;
-                    if (cc < c) {
-                        Rb += x.x;
-                        Pb += x.y;
-                    }
-                }
+            DrawRow d;
+            d.ct = d0 + sq + k;
+            d.cd = k < g ? p.rows_t + d0 + k : -1;
+            d.Mt = rst[d.ct].x;
+            d.izt = __fdiv_rn(1.f, rst[d.ct].y);
+            d.Md = d.cd >= 0 ? rst[d.cd].x : 0.f;
+            d.izd = d.cd >= 0 ? __fdiv_rn(1.f, rst[d.cd].y) : 0.f;
+            // every tile's two columns first (one wait), then the weights of this lane's entries
+            uint32_t rt[kVeMaxTiles], rd[kVeMaxTiles];
 #pragma unroll
-                for (int o = 16; o >= 1; o >>= 1) {
-                    R += __shfl_xor_sync(0xffffffffu, R, o);
-                    P += __shfl_xor_sync(0xffffffffu, P, o);
-                    Rb += __shfl_xor_sync(0xffffffffu, Rb, o);
-                    Pb += __shfl_xor_sync(0xffffffffu, Pb, o);
-                }
-                if (lane == 0) {
-                    const ulonglong2 own = __ldcg(&p.tot[(size_t)sq * grid + c]);
-                    const bool use_r = k < g && R > 0;  // a vanishing residual (p == q) draws from p
-                    const unsigned long long total = use_r ? R : P, below = use_r ? Rb : Pb;
-                    const unsigned long long mine = use_r ? own.x : own.y;
-                    float u = __ldg(p.u_sample + sq);
-                    if (!(u >= 0.f)) u = 0.f;
-                    u = fminf(u, 0.99999994f);  // u in [0, 1): the crossing always exists
-                    const unsigned long long thr = __umul64hi(__float2ull_rn(u * 18446744073709551616.f), total);
-                    int find = 0;
-                    if (total == 0) {  // no positive mass at all: report, emit 0
-                        if (c == 0) {
-                            raise_error(p.err, kErrDeviceArg);
-                            p.out_tokens[d0 + sq + k] = 0;
-                        }
-                    } else if (below <= thr && thr < below + mine) {
-                        find = 1;
-                        off_sh = thr - below;
-                    }
-                    find_sh = find;
-                    use_r_sh = use_r;
+            for (int t = 0; t < kVeMaxTiles; ++t) {
+                if (t < ntile) {
+                    rt[t] = tmem_ld1(tq + (uint32_t)(t * NP + d.ct));
+                    rd[t] = d.cd >= 0 ? tmem_ld1(tq + (uint32_t)(t * NP + d.cd)) : 0u;
                 }
             }
-            __syncthreads();
-            if (find_sh && warp >= kVeEpi) {
-                // ---- the crossing is in this slice: chunk masses in entry order, then the entry
-                DrawRow d;
-                d.ct = d0 + sq + k;
-                d.cd = k < g ? p.rows_t + d0 + k : -1;
-                d.Mt = rst[d.ct].x;
-                d.izt = __fdiv_rn(1.f, rst[d.ct].y);
-                d.Md = d.cd >= 0 ? rst[d.cd].x : 0.f;
-                d.izd = d.cd >= 0 ? __fdiv_rn(1.f, rst[d.cd].y) : 0.f;
-                const bool use_r = use_r_sh != 0;
-                if (warp == kVeEpi) {  // one warp scans the chunk masses in entry order (tile, then quarter)
-                    const unsigned long long off = off_sh;
-                    const int n = ntile * 4, i0 = 2 * lane;  // lane l holds chunks 2l and 2l + 1
-                    const ulonglong2 c0 = i0 < n ? chunk[sq * n + i0] : make_ulonglong2(0ull, 0ull);
-                    const ulonglong2 c1 = i0 + 1 < n ? chunk[sq * n + i0 + 1] : make_ulonglong2(0ull, 0ull);
-                    const unsigned long long x0 = use_r ? c0.x : c0.y, x1 = use_r ? c1.x : c1.y;
-                    const unsigned long long incl = warp_incl_scan(x0 + x1, lane);
-                    const unsigned long long b0 = incl - x1 - x0, b1 = incl - x1;
-                    const bool h0 = x0 > 0 && b0 <= off && off < b1, h1 = x1 > 0 && b1 <= off && off < incl;
-                    const unsigned hits = __ballot_sync(0xffffffffu, h0 || h1);  // exactly one with exact sums
-                    if (hits == 0u) {
-                        if (lane == 0) sel_sh = -1;
-                    } else if (lane == __ffs(hits) - 1) {
-                        sel_sh = h0 ? i0 : i0 + 1;
-                        base_sh = h0 ? b0 : b1;
-                    }
-                }
-                named_sync(1, 128);
-                const int sel = sel_sh;
-                if (sel < 0) {  // unreachable with exact sums: report, emit the slice's first entry
-                    if (tid == kVeEpi * 32) {
-                        raise_error(p.err, kErrDeviceArg);
-                        p.out_tokens[d0 + sq + k] = v0;
-                    }
-                } else if ((sel & 3) == q) {
-                    const int t = sel >> 2;
-                    const int v = v0 + t * kVeM + q * 32 + lane;
-                    const float2 w2 = entry_weights<NP>(tq, t, d, v < v1, p.c2);
-                    const float w = use_r ? w2.x : w2.y;
-                    // offset of the threshold inside the chunk, back in probability units
-                    const float off = __ull2float_rn(off_sh - base_sh) * 2.220446049250313e-16f;
-                    const float run = warp_incl_scan_f(w, lane);
-                    const unsigned hit = __ballot_sync(0xffffffffu, w > 0.f && run > off);
-                    const unsigned pos = __ballot_sync(0xffffffffu, w > 0.f);
-                    // fp32 rounding inside the chunk can leave the crossing just past its end: then
-                    // the chunk's last entry with positive weight
-                    const int ln = hit ? __ffs(hit) - 1 : (pos ? 31 - __clz(pos) : 0);
-                    if (lane == 0) p.out_tokens[d0 + sq + k] = v0 + t * kVeM + q * 32 + ln;
-                }
+            tmem_ld_wait();
+            // lane t ends with the r-mass of tile t's chunk, lane 16 + t with its p-mass (31 shuffles)
+            float v[32];
+#pragma unroll
+            for (int t = 0; t < kVeMaxTiles; ++t) {
+                float2 w = make_float2(0.f, 0.f);
+                if (t < ntile)
+                    w = draw_weights(__uint_as_float(rt[t]), __uint_as_float(rd[t]), d,
+                                     v0 + t * kVeM + q * 32 + lane < v1, p.c2);
+                v[t] = w.x;
+                v[kVeMaxTiles + t] = w.y;
             }
-            __syncthreads();
+            const unsigned long long f = to_fix(reduce_scatter32(v, lane));
+            const int tl = lane & (kVeMaxTiles - 1);
+            unsigned long long* cf = reinterpret_cast<unsigned long long*>(chunk);
+            if (tl < ntile) cf[((sq * ntile + tl) * 4 + q) * 2 + (lane >> 4)] = f;  // .x = r, .y = p
+            unsigned long long tot = tl < ntile ? f : 0ull;  // lanes 0-15 sum r, lanes 16-31 sum p
+#pragma unroll
+            for (int o = kVeMaxTiles / 2; o >= 1; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+            if (lane == 0) wtot[q][sq].x = tot;
+            if (lane == kVeMaxTiles) wtot[q][sq].y = tot;
         }
+        named_sync(1, 128);
+        for (int sq = tid - kVeEpi * 32; sq < S; sq += 128) {
+            ulonglong2 a = wtot[0][sq];
+            for (int w = 1; w < 4; ++w) {
+                a.x += wtot[w][sq].x;
+                a.y += wtot[w][sq].y;
+            }
+            p.tot[(size_t)sq * grid + c] = a;
+        }
+    }
+
+    // ================= grid barrier 2: every slice's masses are out
+    if (!grid_barrier(p.sync, 2u * (unsigned)grid, &ok_sh)) raise_error(p.err, kErrTimeout);
+
+    for (int sq = 0; sq < S; ++sq) {
+        const int d0 = cu_sh[sq], g = cu_sh[sq + 1] - d0, k = k_sh[sq];
+        if (warp == 0) {
+            unsigned long long R = 0, P = 0, Rb = 0, Pb = 0;
+            for (int cc = lane; cc < grid; cc += 32) {
+                const ulonglong2 x = __ldcg(&p.tot[(size_t)sq * grid + cc]);
+                R += x.x;
+                P += x.y;
+                if (cc < c) {
+                    Rb += x.x;
+                    Pb += x.y;
+                }
+            }
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) {
+                R += __shfl_xor_sync(0xffffffffu, R, o);
+                P += __shfl_xor_sync(0xffffffffu, P, o);
+                Rb += __shfl_xor_sync(0xffffffffu, Rb, o);
+                Pb += __shfl_xor_sync(0xffffffffu, Pb, o);
+            }
+            if (lane == 0) {
+                const ulonglong2 own = __ldcg(&p.tot[(size_t)sq * grid + c]);
+                const bool use_r = k < g && R > 0;  // a vanishing residual (p == q) draws from p
+                const unsigned long long total = use_r ? R : P, below = use_r ? Rb : Pb;
+                const unsigned long long mine = use_r ? own.x : own.y;
+                float u = __ldg(p.u_sample + sq);
+                if (!(u >= 0.f)) u = 0.f;
+                u = fminf(u, 0.99999994f);  // u in [0, 1): the crossing always exists
+                const unsigned long long thr = __umul64hi(__float2ull_rn(u * 18446744073709551616.f), total);
+                int find = 0;
+                if (total == 0) {  // no positive mass at all: report, emit 0
+                    if (c == 0) {
+                        raise_error(p.err, kErrDeviceArg);
+                        p.out_tokens[d0 + sq + k] = 0;
+                    }
+                } else if (below <= thr && thr < below + mine) {
+                    find = 1;
+                    off_sh = thr - below;
+                }
+                find_sh = find;
+                use_r_sh = use_r;
+            }
+        }
+        __syncthreads();
+        if (find_sh && warp >= kVeEpi) {
+            // ---- the crossing is in this slice: chunk masses in entry order, then the entry
+            DrawRow d;
+            d.ct = d0 + sq + k;
+            d.cd = k < g ? p.rows_t + d0 + k : -1;
+            d.Mt = rst[d.ct].x;
+            d.izt = __fdiv_rn(1.f, rst[d.ct].y);
+            d.Md = d.cd >= 0 ? rst[d.cd].x : 0.f;
+            d.izd = d.cd >= 0 ? __fdiv_rn(1.f, rst[d.cd].y) : 0.f;
+            const bool use_r = use_r_sh != 0;
+            if (warp == kVeEpi) {  // one warp scans the chunk masses in entry order (tile, then quarter)
+                const unsigned long long off = off_sh;
+                const int n = ntile * 4, i0 = 2 * lane;  // lane l holds chunks 2l and 2l + 1
+                const ulonglong2 c0 = i0 < n ? chunk[sq * n + i0] : make_ulonglong2(0ull, 0ull);
+                const ulonglong2 c1 = i0 + 1 < n ? chunk[sq * n + i0 + 1] : make_ulonglong2(0ull, 0ull);
+                const unsigned long long x0 = use_r ? c0.x : c0.y, x1 = use_r ? c1.x : c1.y;
+                const unsigned long long incl = warp_incl_scan(x0 + x1, lane);
+                const unsigned long long b0 = incl - x1 - x0, b1 = incl - x1;
+                const bool h0 = x0 > 0 && b0 <= off && off < b1, h1 = x1 > 0 && b1 <= off && off < incl;
+                const unsigned hits = __ballot_sync(0xffffffffu, h0 || h1);  // exactly one with exact sums
+                if (hits == 0u) {
+                    if (lane == 0) sel_sh = -1;
+                } else if (lane == __ffs(hits) - 1) {
+                    sel_sh = h0 ? i0 : i0 + 1;
+                    base_sh = h0 ? b0 : b1;
+                }
+            }
+            named_sync(1, 128);
+            const int sel = sel_sh;
+            if (sel < 0) {  // unreachable with exact sums: report, emit the slice's first entry
+                if (tid == kVeEpi * 32) {
+                    raise_error(p.err, kErrDeviceArg);
+                    p.out_tokens[d0 + sq + k] = v0;
+                }
+            } else if ((sel & 3) == q) {
+                const int t = sel >> 2;
+                const int v = v0 + t * kVeM + q * 32 + lane;
+                const float2 w2 = entry_weights<NP>(tq, t, d, v < v1, p.c2);
+                const float w = use_r ? w2.x : w2.y;
+                // offset of the threshold inside the chunk, back in probability units
+                const float off = __ull2float_rn(off_sh - base_sh) * 2.220446049250313e-16f;
+                const float run = warp_incl_scan_f(w, lane);
+                const unsigned hit = __ballot_sync(0xffffffffu, w > 0.f && run > off);
+                const unsigned pos = __ballot_sync(0xffffffffu, w > 0.f);
+                // fp32 rounding inside the chunk can leave the crossing just past its end: then
+                // the chunk's last entry with positive weight
+                const int ln = hit ? __ffs(hit) - 1 : (pos ? 31 - __clz(pos) : 0);
+                if (lane == 0) p.out_tokens[d0 + sq + k] = v0 + t * kVeM + q * 32 + ln;
+            }
+        }
+        __syncthreads();
     }
 
     // ---- release tensor memory; the last CTA out clears the grid-barrier counters
@@ -729,10 +662,10 @@ size_t ve_smem_bytes() {
 
 struct VeLayout {
     size_t sync_off, part_off, xg_off, tot_off, total;
-    size_t rowst_off, tickets_off, draw_off, logits_off;  // the streamed path (more than 64 rows at T > 0)
+    size_t rowst_off, tickets_off, draw_off, logits_off;  // the streamed path at T > 0 (0: not in this layout)
 };
 int ve_padded(int vocab) { return (int)(((long long)vocab + 7) / 8 * 8); }
-VeLayout ve_layout(int num_seqs, int total_draft, int vocab, bool padded) {
+VeLayout ve_layout(int num_seqs, int total_draft, int vocab, bool full) {
     VeLayout l;
     const int rows = 2 * total_draft + num_seqs;
     l.sync_off = 0;
@@ -741,17 +674,17 @@ VeLayout ve_layout(int num_seqs, int total_draft, int vocab, bool padded) {
     l.tot_off = l.xg_off + align_up((size_t)(total_draft > 0 ? total_draft : 1) * sizeof(float2), 256);
     l.total = l.tot_off + align_up((size_t)(num_seqs > 0 ? num_seqs : 1) * kVeMaxGrid * sizeof(ulonglong2), 256);
     l.rowst_off = l.tickets_off = l.draw_off = l.logits_off = 0;
-    if (rows > kVerifyResidentRows) {
+    if (rows > (full ? kVerifyKeepRows : kVerifyResidentRows)) {
         l.rowst_off = l.total;
         l.tickets_off = l.rowst_off + align_up((size_t)rows * sizeof(float2), 256);
         l.draw_off = l.tickets_off + align_up((size_t)num_seqs * sizeof(int), 256);
         l.logits_off = l.draw_off + align_up(accept_draw_scratch_bytes(num_seqs, vocab), 256);
-        l.total = l.logits_off + align_up((size_t)rows * (size_t)(padded ? ve_padded(vocab) : vocab) * sizeof(float), 256);
+        l.total = l.logits_off + align_up((size_t)rows * (size_t)(full ? ve_padded(vocab) : vocab) * sizeof(float), 256);
     }
     return l;
 }
 
-template <bool GREEDY, int NP, int APS>
+template <int NP, int APS>
 int ve_launch(const CUtensorMap& wmap, const VeParams& p, int grid, const DeviceInfo& dev, cudaStream_t stream) {
     static std::mutex cfg_mu;        // per instantiation (a template's own statics)
     static int configured[64] = {};
@@ -759,11 +692,11 @@ int ve_launch(const CUtensorMap& wmap, const VeParams& p, int grid, const Device
     if (dev.device >= 0 && dev.device < 64) {
         std::lock_guard<std::mutex> cfg_lock(cfg_mu);  // once per device, from any host thread
         if (!configured[dev.device]) {
-            if (cudaFuncSetAttribute(verify_epilogue_kernel<GREEDY, NP, APS>,
+            if (cudaFuncSetAttribute(verify_epilogue_kernel<NP, APS>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
                 return BP_ERR_CUDA;
             int per_sm = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, verify_epilogue_kernel<GREEDY, NP, APS>,
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, verify_epilogue_kernel<NP, APS>,
                                                               kVeThreads, smem) != cudaSuccess ||
                 per_sm < 1)
                 return BP_ERR_UNSUPPORTED;
@@ -780,14 +713,14 @@ int ve_launch(const CUtensorMap& wmap, const VeParams& p, int grid, const Device
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, verify_epilogue_kernel<GREEDY, NP, APS>, wmap, p) == cudaSuccess ? BP_OK
+    return cudaLaunchKernelEx(&cfg, verify_epilogue_kernel<NP, APS>, wmap, p) == cudaSuccess ? BP_OK
                                                                                                : BP_ERR_CUDA;
 }
 
 }  // namespace
 
-size_t verify_epilogue_scratch_bytes(int num_seqs, int total_draft, int vocab, bool padded) {
-    return ve_layout(num_seqs, total_draft, vocab, padded).total;
+size_t verify_epilogue_scratch_bytes(int num_seqs, int total_draft, int vocab, bool full) {
+    return ve_layout(num_seqs, total_draft, vocab, full).total;
 }
 
 int verify_epilogue_config(int rows, int vocab, int hidden, int sm_count, int* grid, int* np, int* tiles_per_cta) {
@@ -808,18 +741,24 @@ int launch_verify_epilogue(const VerifyEpilogueArgs& a, const DeviceInfo& dev, c
     const bool greedy = a.temperature == 0.f;
     const int rows_t = a.total_draft + a.num_seqs;
     const int rows = rows_t + (greedy ? 0 : a.total_draft);
-    const VeLayout l = ve_layout(a.num_seqs, a.total_draft, a.vocab, false);
     uint8_t* ws = static_cast<uint8_t*>(a.scratch);
-    if (rows > kVerifyResidentRows) {
+    // Which path.  Streamed: greedy calls (nothing but statistics leaves the chip; 152 SMs, vocabulary 151936 x
+    // 2560, streamed against resident: 16 rows 119.5 / 121.0 us, 64 rows 121.3 / 154.6 us) and, at T > 0, more
+    // than 32 rows (62 rows 144.8 / 178.0 us: beyond 32 the resident kernel's stages hold half as many W rows
+    // and its epilogue runs twice the columns).  Up to 32 rows at T > 0 the resident kernel's logits never leave
+    // tensor memory (31 rows: 136.7 / 127.1 us).  The streamed path's logits and draw scratch need a workspace
+    // sized for them; from 33 to 64 rows a smaller one keeps the resident kernel.
+    const bool fits = ve_layout(a.num_seqs, a.total_draft, a.vocab, true).total <= a.scratch_bytes;
+    const VeLayout l = ve_layout(a.num_seqs, a.total_draft, a.vocab, fits);
+    if (greedy || (rows > kVerifyKeepRows && l.logits_off != 0)) {
         VerifyStreamScratch s;
-        s.logits = reinterpret_cast<float*>(ws + l.logits_off);
-        // rows that start 16-byte aligned where the workspace has the room (it does when it was sized for this call)
-        const bool pad = a.vocab <= INT_MAX - 8 && ve_layout(a.num_seqs, a.total_draft, a.vocab, true).total <= a.scratch_bytes;
-        s.ld = pad ? ve_padded(a.vocab) : a.vocab;
         s.part = reinterpret_cast<float2*>(ws + l.part_off);
-        s.row_stats = reinterpret_cast<float2*>(ws + l.rowst_off);
+        // (without regions of its own -- greedy, few rows -- the row statistics take the slice masses' place)
+        s.row_stats = reinterpret_cast<float2*>(ws + (l.rowst_off ? l.rowst_off : l.tot_off));
         s.tickets = reinterpret_cast<int*>(ws + l.tickets_off);
         s.draw = ws + l.draw_off;
+        s.logits = reinterpret_cast<float*>(ws + l.logits_off);
+        s.ld = fits ? ve_padded(a.vocab) : a.vocab;  // rows that start 16-byte aligned where there is room
         return launch_verify_stream(a, s, dev, stream);
     }
     int grid = 0, NP = 0, per = 0;
@@ -839,7 +778,7 @@ int launch_verify_epilogue(const VerifyEpilogueArgs& a, const DeviceInfo& dev, c
 
     VeParams p;
     p.h_target = static_cast<const __nv_bfloat16*>(a.h_target);
-    p.h_draft = static_cast<const __nv_bfloat16*>(greedy ? a.h_target : a.h_draft);
+    p.h_draft = static_cast<const __nv_bfloat16*>(a.h_draft);
     p.hidden = a.hidden;
     p.vocab = a.vocab;
     p.atoms = a.hidden / kVeAtom;
@@ -850,7 +789,7 @@ int launch_verify_epilogue(const VerifyEpilogueArgs& a, const DeviceInfo& dev, c
     p.tiles_base = tiles_total / grid;
     p.tiles_extra = tiles_total % grid;
     p.tmem_cols = cols;
-    p.c2 = greedy ? 0.f : 1.4426950408889634f / a.temperature;
+    p.c2 = 1.4426950408889634f / a.temperature;
     p.tokens = a.tokens;
     p.cu_draft = a.cu_draft;
     p.u_accept = a.u_accept;
@@ -865,17 +804,9 @@ int launch_verify_epilogue(const VerifyEpilogueArgs& a, const DeviceInfo& dev, c
     p.sync = reinterpret_cast<unsigned int*>(ws + l.sync_off);
     p.err = a.err_word;
     const bool two = p.atoms % 2 == 0;  // two atoms per stage where the hidden size allows
-    if (greedy && NP == 32)
-        return two ? ve_launch<true, 32, 2>(wmap, p, grid, dev, stream)
-                   : ve_launch<true, 32, 1>(wmap, p, grid, dev, stream);
-    if (greedy)
-        return two ? ve_launch<true, 64, 2>(wmap, p, grid, dev, stream)
-                   : ve_launch<true, 64, 1>(wmap, p, grid, dev, stream);
     if (NP == 32)
-        return two ? ve_launch<false, 32, 2>(wmap, p, grid, dev, stream)
-                   : ve_launch<false, 32, 1>(wmap, p, grid, dev, stream);
-    return two ? ve_launch<false, 64, 2>(wmap, p, grid, dev, stream)
-               : ve_launch<false, 64, 1>(wmap, p, grid, dev, stream);
+        return two ? ve_launch<32, 2>(wmap, p, grid, dev, stream) : ve_launch<32, 1>(wmap, p, grid, dev, stream);
+    return two ? ve_launch<64, 2>(wmap, p, grid, dev, stream) : ve_launch<64, 1>(wmap, p, grid, dev, stream);
 }
 
 }  // namespace bp

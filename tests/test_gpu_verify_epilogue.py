@@ -432,3 +432,23 @@ def test_streamed_rows_padded_or_not(vocab):
     with pytest.raises(bp.BlockPilotError) as e:
         run_gpu(inp, 1.0, ws=bp.workspace(least, dev())[:-1])
     assert e.value.status == 4
+
+
+@pytest.mark.parametrize("vocab", [4000, 5003])
+@pytest.mark.parametrize("blocks", [(17,), (16, 12), (16, 16, 1), (1,) * 33])
+def test_33_to_64_rows_on_either_path(blocks, vocab):
+    """33 to 64 rows at T = 1: streamed in a workspace of the size the library asks for, resident in one that
+    holds no logits; T = 0 streams in both."""
+    w = wl.custom(seed=sum(blocks), ctx=(0,) * len(blocks), block=blocks, vocab=vocab)
+    td, s = sum(blocks) - len(blocks), len(blocks)
+    up = lambda n: -(-n // 256) * 256  # noqa: E731
+    least = 512 + up((2 * td + s) * 160 * 8) + up(max(td, 1) * 8) + up(s * 160 * 16)
+    assert 33 <= 2 * td + s <= 64 and least < bp.verify_epilogue_workspace_size(s, td, vocab)
+    for temp in (1.0, 0.0):
+        inp = wl.lm_head_inputs(w, temp, hidden=192)
+        ref = run_oracle(inp, temp)
+        for ws in (None, bp.workspace(least, dev())):
+            compare(inp, temp, run_gpu(inp, temp, ws=ws), ref)
+    with pytest.raises(bp.BlockPilotError) as e:
+        run_gpu(inp, 0.0, ws=bp.workspace(least, dev())[:-1])
+    assert e.value.status == 4
