@@ -167,6 +167,7 @@ struct PolicyTcParams {
     int num_reqs, d_in, hidden, num_cand;
     int atoms_total, atoms_per_cta, tiles, npad;
     int w_bytes, x_bytes, h_bytes, op_bytes;  // dynamic shared-memory regions
+    int gathered;  // streamed: the gather kernel came before (it releases this one behind its own wait)
     const float* b1;
     const __nv_bfloat16* w2;
     const float* b2;
@@ -185,13 +186,15 @@ __device__ __forceinline__ int atomic_add_acq_rel_gpu(int* addr, int v) {
 }
 
 // Gathers the pooled rows of every request group into a contiguous [groups*64][d_in] buffer (rows
-// past the last request zero), so that the streamed path can load x with TMA like W1.
+// past the last request zero), so that the streamed path can load x with TMA like W1.  (Without a row index
+// the feature rows are loaded where they are and nothing is gathered.)  It releases the streamed kernel behind
+// its own wait, when every earlier kernel is complete, so that one may load what this one does not write.
 __global__ void __launch_bounds__(256) policy_gather_kernel(const __nv_bfloat16* __restrict__ feats,
                                                             int64_t row_stride, const int32_t* __restrict__ row_index,
                                                             int num_reqs, int d_in, int groups, int npad,
                                                             __nv_bfloat16* __restrict__ xg) {
-    griddep_launch_dependents();
     griddep_wait();
+    griddep_launch_dependents();
     const int chunks = d_in / 8;
     const long long total = (long long)groups * npad * chunks;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
@@ -269,15 +272,24 @@ __global__ void __launch_bounds__(kTcThreads) policy_tc_kernel(const __grid_cons
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_sh;
-    griddep_wait();  // inputs may come from the previous kernel on the stream
+    // inputs may come from the previous kernel on the stream; behind the gather kernel only x does
+    const bool early = RING && p.gathered && tid < 32;
+    if (!early) griddep_wait();
     if (RING) {
         static_assert(!RING || (S >= 2 && S <= kTcStages && S <= kTcMaxAtoms), "ring depth");
         const uint32_t stage_bytes = (uint32_t)(kTcAtomBytes + npad * 128);
         if (tid == 0) {  // producer: W1 and x atoms through the ring
-            int j = 0;
+            const int first = min(S, na);
+            for (int i = 0; i < first; ++i) {
+                mbar_arrive_expect_tx(&bar_w[i], stage_bytes);
+                tma_load_2d(sW + i * kTcAtomBytes, &w1map, &bar_w[i], (a0 + i) * kTcAtom, m0);
+            }
+            if (early) griddep_wait();  // the gathered x
+            for (int i = 0; i < first; ++i) tma_load_2d(sX + i * npad * 128, &xmap, &bar_w[i], (a0 + i) * kTcAtom, n0);
+            int j = first;
             for (; j < na; ++j) {
                 const int st = j % S;
-                if (j >= S && !mbar_wait(&bar_empty[st], ((j / S) - 1) & 1, kWaitBudget)) {
+                if (!mbar_wait(&bar_empty[st], ((j / S) - 1) & 1, kWaitBudget)) {
                     raise_error(p.err, kErrTimeout);
                     break;
                 }
@@ -643,11 +655,13 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
                           CU_TENSOR_MAP_SWIZZLE_128B) != BP_OK)
         return -1;
     xmap = w1map;  // not read by the one-shot kernel
-    if (ring) {
-        const cuuint64_t xdims[2] = {(cuuint64_t)a.d_in, (cuuint64_t)groups * kTcMaxN};
+    const bool gather = ring && a.row_index != nullptr;
+    if (ring) {  // the gathered rows, or the feature rows themselves (rows past the last request read zero)
+        const cuuint64_t xdims[2] = {(cuuint64_t)a.d_in, gather ? (cuuint64_t)groups * kTcMaxN : (cuuint64_t)a.num_reqs};
+        const cuuint64_t xstrides[1] = {(cuuint64_t)(gather ? a.d_in : a.row_stride) * 2};
         const cuuint32_t xbox[2] = {(cuuint32_t)kTcAtom, (cuuint32_t)npad};
-        if (encode_tensor_map(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, xg, xdims, strides, xbox,
-                              CU_TENSOR_MAP_SWIZZLE_128B) != BP_OK)
+        if (encode_tensor_map(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, gather ? xg : const_cast<void*>(a.feats),
+                              xdims, xstrides, xbox, CU_TENSOR_MAP_SWIZZLE_128B) != BP_OK)
             return -1;
     }
     PolicyTcParams p;
@@ -666,6 +680,7 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
     p.x_bytes = x_bytes;
     p.h_bytes = h_bytes;
     p.op_bytes = op_bytes;
+    p.gathered = gather;
     p.b1 = a.b1;
     p.w2 = static_cast<const __nv_bfloat16*>(a.w2);
     p.b2 = a.b2;
@@ -678,7 +693,7 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
     cudaLaunchAttribute pdl[1];
     pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     pdl[0].val.programmaticStreamSerializationAllowed = 1;
-    if (ring) {
+    if (gather) {
         const long long total = (long long)groups * npad * (a.d_in / 8);
         long long blocks = (total + 255) / 256;
         const long long cap = 4LL * dev.sm_count;
