@@ -157,7 +157,7 @@ constexpr int kTcMaxAtoms = 8;     // atoms per CTA when all of them are loaded 
 constexpr int kTcStages = 5;       // ring depth at most, when the atoms of a CTA are streamed (large d_in)
 constexpr int kTcMaxKS = 9;        // CTAs per cluster (non-portable above 8)
 constexpr int kTcThreads = 128;    // thread t = tile row t = TMEM lane t
-constexpr uint32_t kTcTmemCols = 64;
+constexpr int kTcIssuers = kTcThreads / 32;  // one-shot: warps that issue MMAs, each into its own accumulator
 constexpr int kTcMaxSmem = 200 * 1024;
 
 struct PolicyTcParams {
@@ -167,6 +167,7 @@ struct PolicyTcParams {
     int num_reqs, d_in, hidden, num_cand;
     int atoms_total, atoms_per_cta, tiles, npad;
     int w_bytes, x_bytes, h_bytes, op_bytes;  // dynamic shared-memory regions
+    uint32_t tmem_cols;
     int gathered;  // streamed: the gather kernel came before (it releases this one behind its own wait)
     const float* b1;
     const __nv_bfloat16* w2;
@@ -259,17 +260,17 @@ __global__ void __launch_bounds__(kTcThreads) policy_tc_kernel(const __grid_cons
         for (int a = 0; a < nb; ++a) mbar_init(&bar_w[a], 1);
         if (RING)
             for (int st = 0; st < S; ++st) mbar_init(&bar_empty[st], 1);
-        mbar_init(&bar_mma, 1);
+        mbar_init(&bar_mma, RING ? 1 : max(1, min(na, kTcIssuers)));  // one commit per issuer
         fence_mbar_init();
     }
     if (warp == 0) {
-        tmem_alloc(&tmem_sh, kTcTmemCols);
+        tmem_alloc(&tmem_sh, p.tmem_cols);
         tmem_relinquish();
     }
-    griddep_launch_dependents();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    griddep_launch_dependents();
     const uint32_t tmem = tmem_sh;
     // inputs may come from the previous kernel on the stream; behind the gather kernel only x does
     const bool early = RING && p.gathered && tid < 32;
@@ -366,7 +367,36 @@ __global__ void __launch_bounds__(kTcThreads) policy_tc_kernel(const __grid_cons
                 cp_async16(dst, src + (valid ? k : 0), valid);
             }
         }
-        // the small operands of the epilogue, read while the copies are in flight
+        cp_async_wait_all();
+        fence_proxy_async_smem();  // the MMAs read x through the async proxy
+        __syncthreads();
+        // A thread of each warp issues the MMAs of atoms warp, warp + 4, ... into the warp's own accumulator: at
+        // N = 32 an MMA runs in a few tens of cycles but takes one thread about 120 to issue, so one issuer
+        // needed 2400 cycles for 5 atoms.  The four accumulators are added when they are read.
+        if ((tid & 31) == 0) {
+            const uint32_t idesc = idesc_bf16_f32(kTcM, npad, false, false);
+            const uint32_t acc = tmem + (uint32_t)(warp * npad);
+            bool ok = true;
+            for (int a = warp; a < na && ok; a += kTcIssuers) {
+                if (!mbar_wait(&bar_w[a], 0, kWaitBudget)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t wa = smem_addr(sW + a * kTcAtomBytes), xa = smem_addr(sX + a * npad * 128);
+#pragma unroll
+                for (int kk = 0; kk < kTcAtom / 16; ++kk)
+                    umma_ss(acc, smem_desc(wa + kk * 32, 16, 1024, kSwizzle128B),
+                            smem_desc(xa + kk * 32, 16, 1024, kSwizzle128B), idesc, (a - warp) | kk ? 1u : 0u);
+            }
+            if (!ok) {  // the warp's W1 atoms land before the CTA moves on
+                raise_error(p.err, kErrTimeout);
+                for (int a = warp; a < na; a += kTcIssuers) mbar_wait(&bar_w[a], 0, kDrainBudget);
+            }
+            if (warp < na) umma_commit(&bar_mma);
+        }
+        __syncwarp();
+        // the small operands of the epilogue, read while the MMAs run
         for (int i = tid; i < C * nr; i += kTcThreads) {
             const int c = i / nr, rr = i % nr;
             const int j = m0 + rb + rr;
@@ -378,30 +408,6 @@ __global__ void __launch_bounds__(kTcThreads) policy_tc_kernel(const __grid_cons
                 b2s[c] = p.b2[c];
                 cands[c] = p.candidates[c];
             }
-        cp_async_wait_all();
-        fence_proxy_async_smem();  // the MMAs read x through the async proxy
-        __syncthreads();
-        if (tid == 0 && na > 0) {
-            const uint32_t idesc = idesc_bf16_f32(kTcM, npad, false, false);
-            bool ok = true;
-            for (int a = 0; a < na && ok; ++a) {
-                if (!mbar_wait(&bar_w[a], 0, kWaitBudget)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                const uint32_t wa = smem_addr(sW + a * kTcAtomBytes), xa = smem_addr(sX + a * npad * 128);
-#pragma unroll
-                for (int kk = 0; kk < kTcAtom / 16; ++kk)
-                    umma_ss(tmem, smem_desc(wa + kk * 32, 16, 1024, kSwizzle128B),
-                            smem_desc(xa + kk * 32, 16, 1024, kSwizzle128B), idesc, (a | kk) ? 1u : 0u);
-            }
-            if (!ok) {  // every W1 atom's copy lands before the CTA moves on
-                raise_error(p.err, kErrTimeout);
-                for (int a = 0; a < na; ++a) mbar_wait(&bar_w[a], 0, kDrainBudget);
-            }
-            umma_commit(&bar_mma);
-        }
     }
     // ---- this CTA's partial tile row (thread = row = TMEM lane)
     float d[kTcMaxN];
@@ -413,11 +419,18 @@ __global__ void __launch_bounds__(kTcThreads) policy_tc_kernel(const __grid_cons
 #pragma unroll
         for (int c0 = 0; c0 < kTcMaxN; c0 += 16) {
             if (c0 < npad) {  // uniform: npad is the same in every thread
-                uint32_t v[16];
-                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+                constexpr int kAcc = RING ? 1 : kTcIssuers;  // accumulators, npad columns apart
+                uint32_t v[kAcc][16];
+#pragma unroll
+                for (int w = 0; w < kAcc; ++w)
+                    if (w < na) tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(w * npad + c0), v[w]);
                 tmem_ld_wait();
 #pragma unroll
-                for (int e = 0; e < 16; ++e) d[c0 + e] = __uint_as_float(v[e]);
+                for (int w = 0; w < kAcc; ++w)
+                    if (w < na) {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) d[c0 + e] += __uint_as_float(v[w][e]);
+                    }
             }
         }
     }
@@ -528,7 +541,7 @@ __global__ void __launch_bounds__(kTcThreads) policy_tc_kernel(const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 0) tmem_dealloc(tmem, kTcTmemCols);
+    if (warp == 0) tmem_dealloc(tmem, p.tmem_cols);
 }
 
 // Scratch of the tensor-core path: partials and tickets (after the CUDA-core path's h buffer).
@@ -655,8 +668,15 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
     const int slots = ring ? kTcKernels[kernel].stages : per;
     const int w_bytes = slots * kTcAtomBytes > pd_bytes ? slots * kTcAtomBytes : pd_bytes;
     const int x_bytes = slots * npad * 128;
-    const int smem = smem_for(slots);
+    int smem = smem_for(slots);
     if (smem > kTcMaxSmem) return -1;
+    // Tensor memory: one accumulator of npad columns, or one per issuer.  A CTA waits for its columns while its
+    // cluster peers wait for it, so no more CTAs may share an SM than its 512 columns serve: the shared memory
+    // of a CTA keeps them to that.
+    uint32_t cols = 32;
+    while ((int)cols < npad * (ring ? 1 : kTcIssuers)) cols <<= 1;
+    const int least = dev.max_smem_optin / (int)(512 / cols + 1) + 1024;
+    smem = smem > least ? smem : least;
 
     CUtensorMap w1map, xmap;
     const cuuint64_t dims[2] = {(cuuint64_t)a.d_in, (cuuint64_t)a.hidden};
@@ -691,6 +711,7 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
     p.x_bytes = x_bytes;
     p.h_bytes = h_bytes;
     p.op_bytes = op_bytes;
+    p.tmem_cols = cols;
     p.gathered = gather;
     p.b1 = a.b1;
     p.w2 = static_cast<const __nv_bfloat16*>(a.w2);
