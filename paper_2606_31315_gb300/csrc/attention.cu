@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (failed) break;
             }
             if (SPREAD) l_run += __shfl_xor_sync(0xffffffffu, l_run, 16);  // the whole row's sum
-            if (!FLAT && CS > 1) {  // the rows' (m, l) for the merge, while the last P V runs
+            if (!FLAT && CS > 1 && !p.part) {  // the rows' (m, l) for the merge, while the last P V runs
                 if (half == 0) row_ml[r] = make_float2(m_run, l_run);
                 __syncwarp();
                 cluster_arrive_release();
@@ -745,23 +745,20 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
             if (g.nt > 0) ++nq;
-            if (FLAT && !g.whole && m_valid > p.slot_rows) {  // a block longer than max_q_len: rows past the slot are dropped
+            const bool partial = FLAT ? !g.whole : CS > 1 && p.part != nullptr;  // goes to a workspace slot
+            if (partial && m_valid > p.slot_rows) {  // a block longer than max_q_len: rows past the slot are dropped
                 if (r == 0 && warp == 2) raise_error(p.err, kErrDeviceArg);
                 row_active = row_active && r < p.slot_rows;
             }
-            if (FLAT && !failed && row_active) {
-                if (g.whole) {
-                    write_row(g);
-                } else {  // the partial (O, m, l) of this stretch's rows, for attn_combine_kernel
-                    float* slot = p.part + (size_t)(2 * blockIdx.x + g.slot) * p.slot_rows * (kD + 2);
-                    float* orow = slot + (size_t)r * kD + half * kOCols;
+            if (FLAT && g.whole) {
+                if (!failed && row_active) write_row(g);
+            } else if (partial && row_active) {  // the partial (O, m, l) of this stretch's rows, for the merge
+                float* slot = p.part + (size_t)(FLAT ? 2 * blockIdx.x + g.slot : blockIdx.x) * p.slot_rows * (kD + 2);
+                float* orow = slot + (size_t)r * kD + half * kOCols;
 #pragma unroll
-                    for (int c = 0; c < kOCols / 4; ++c)
-                        *reinterpret_cast<float4*>(orow + c * 4) =
-                            make_float4(o_acc[c * 4], o_acc[c * 4 + 1], o_acc[c * 4 + 2], o_acc[c * 4 + 3]);
-                    if (half == 0)
-                        *reinterpret_cast<float2*>(slot + (size_t)p.slot_rows * kD + 2 * r) = make_float2(m_run, l_run);
-                }
+                for (int c = 0; c < kOCols / 8; ++c) st_global_f32x8(orow + c * 8, &o_acc[c * 8]);
+                if (half == 0)
+                    *reinterpret_cast<float2*>(slot + (size_t)p.slot_rows * kD + 2 * r) = make_float2(m_run, l_run);
             }
         }
         if (failed) raise_error(p.err, kErrTimeout);
@@ -774,6 +771,74 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (!FLAT) {
         if (CS == 1) {
             if (row_active) write_row(one);
+        } else if (p.part) {
+            // ---- merge of the CS partial (m, l, O) triples through the workspace slots, i.e. through L2: every CTA
+            // has written its own; behind one cluster barrier each CTA loads the rows it owns of all of them, a
+            // warp per row: lane c the 16-byte chunk c of every partial and, c below the cluster size, partial c's
+            // (m, l), whose weights go round the warp by shuffles.  SM to SM a partial crosses at about 14 bytes a
+            // clock, through L2 several times faster: 1 x 2064 keys 8.18 -> 7.92 us in clusters of 9 and 8.31 -> 7.70
+            // in clusters of 11, 1 x 4112 9.24 -> 8.66 us.  With more than two rows a warp (clusters of 2 to 4) the
+            // rounds of loads cost more than the remote stores below (8 x 915 keys 16.4 against 12.8 us).
+            __syncwarp();
+            if (is_softmax) cluster_arrive_release();
+            cluster_wait();
+            m_valid = min(min(kM, one.B * G - one.mt * kM), p.slot_rows);
+            const int row0 = one.mt * kM;
+            const int per = (m_valid + (int)CS - 1) / (int)CS;
+            const int rbeg = (int)crank * per;
+            const int nmy = max(0, min(m_valid, rbeg + per) - rbeg);
+            const size_t slot_floats = (size_t)p.slot_rows * (kD + 2);
+            const float* first = p.part + (size_t)(blockIdx.x - crank) * slot_floats;  // the cluster's first slot
+            // two rows a warp at most (launch_attention_bf16), their loads in flight together
+            constexpr int kRowsPerWarp = 2;
+            float4 v[kRowsPerWarp][kMaxCluster];
+            float2 ml[kRowsPerWarp];
+#pragma unroll
+            for (int k = 0; k < kRowsPerWarp; ++k) {
+                const int j = warp + k * (kThreads / 32), row = rbeg + j;
+                ml[k] = make_float2(-INFINITY, 0.f);
+                if (j < nmy) {
+#pragma unroll
+                    for (int pr = 0; pr < kMaxCluster; ++pr)
+                        if (pr < (int)CS)
+                            v[k][pr] = __ldcg(reinterpret_cast<const float4*>(first + pr * slot_floats + (size_t)row * kD) + lane);
+                    if (lane < (int)CS)
+                        ml[k] = __ldcg(reinterpret_cast<const float2*>(first + lane * slot_floats + (size_t)p.slot_rows * kD + 2 * row));
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < kRowsPerWarp; ++k) {
+                const int j = warp + k * (kThreads / 32);
+                if (j >= nmy) break;
+                float M = ml[k].x;
+#pragma unroll
+                for (int o = kMaxCluster / 2; o >= 1; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+                M = __shfl_sync(0xffffffffu, M, 0);
+                const float w = ml[k].x == -INFINITY ? 0.f : fast_exp2(ml[k].x - M);
+                float L = w * ml[k].y;
+#pragma unroll
+                for (int o = kMaxCluster / 2; o >= 1; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+                L = __shfl_sync(0xffffffffu, L, 0);
+                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int pr = 0; pr < kMaxCluster; ++pr) {
+                    if (pr < (int)CS) {
+                        const float wp = __shfl_sync(0xffffffffu, w, pr);
+                        acc.x += wp * v[k][pr].x;
+                        acc.y += wp * v[k][pr].y;
+                        acc.z += wp * v[k][pr].z;
+                        acc.w += wp * v[k][pr].w;
+                    }
+                }
+                const float inv = L > 0.f ? 1.f / L : 0.f;
+                const int lr = row0 + rbeg + j;
+                const size_t orow = (size_t)(one.q0 + lr / G) * p.num_q_heads + one.h * G + lr % G;
+                uint2 w2;
+                w2.x = pack_bf16x2(acc.x * inv, acc.y * inv);
+                w2.y = pack_bf16x2(acc.z * inv, acc.w * inv);
+                *reinterpret_cast<uint2*>(p.o + orow * kD + lane * 4) = w2;
+                if (p.lse && lane == 0) p.lse[orow] = (M + __log2f(L)) * kLn2;
+            }
         } else {
             // ---- merge of the CS partial (m, l, O) triples through distributed shared memory.  Row r of the
             // unit belongs to CTA r / per.  Behind the first cluster barrier (arrived at when the last weights
@@ -1371,16 +1436,17 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
     // cluster split: a split of each unit's keys for which every unit's cluster is resident in the same
     // wave (a unit left for a second wave would double the time).  The tiles of the longest unit per CTA
     // set the time: minimise them; among equal counts take the smallest cluster whose merge needs the
-    // fewest passes (a pass merges up to 12 owned rows per CTA).  A cluster's barriers and merge cost
-    // about three tiles of one CTA's chain (batch 1, Qwen3-4B heads: 2 tiles 5.3 us alone against
-    // 7.3-9.9 us in clusters; 4 tiles 7.6 us alone, 7.4 us in clusters of 6), so a split that saves
-    // fewer than three tiles stays whole
+    // fewest passes (a pass merges up to 6 owned rows per CTA, one a warp: 1 x 2064 keys in 2 tiles a CTA
+    // take 7.70 us in clusters of 11, 7.92 us in clusters of 9).  A cluster's barriers and merge cost
+    // about three tiles of one CTA's chain (batch 1, Qwen3-4B heads: 2 tiles 5.0 us alone against
+    // 7.0-7.4 us in clusters; 5 tiles 7.2 us in clusters of 5), so a split that saves fewer than three
+    // tiles stays whole
     const int m_rows = std::min(kM, a.max_q_len * G);
     int cs = 1, best = max_tiles, best_pass = 0;
     for (int c = 2; c <= kMaxCluster; ++c) {
         if (c > max_tiles || units > max_active[c] || units * c > dev.sm_count) continue;
         const int per = (max_tiles + c - 1) / c;
-        const int passes = ((m_rows + c - 1) / c + 11) / 12;
+        const int passes = ((m_rows + c - 1) / c + kThreads / 32 - 1) / (kThreads / 32);
         if (per < best || (per == best && cs > 1 && passes < best_pass)) {
             best = per;
             cs = c;
@@ -1447,6 +1513,12 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
     }
 
     cfg.gridDim = dim3((unsigned)(units * cs), 1, 1);
+    // a cluster's partials meet in the workspace where it has the flat split's slots and the rows a CTA owns are
+    // at most two a warp, else in shared memory
+    if (cs > 1 && (p.slot_rows + cs - 1) / cs <= 2 * kThreads / 32 && units * cs <= 2 * kAttnFlatMaxGrid &&
+        a.scratch != nullptr &&
+        a.scratch_bytes >= attention_flat_scratch_bytes(a.max_q_len, G))
+        p.part = static_cast<float*>(a.scratch);
     p.early_release = units <= max_active[cs] && units * cs <= dev.sm_count;  // one wave
     // A CTA's bandwidth is what it keeps in flight; where SMs are idle and each CTA streams a long run, refilling
     // K's stages early (AHEAD) took 16 x 4112 keys (128 CTAs of 33 tiles) from 47.4 to 44.9 us and 4 x 8208
