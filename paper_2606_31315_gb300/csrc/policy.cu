@@ -270,7 +270,10 @@ __global__ void __launch_bounds__(kTcThreads) policy_tc_kernel(const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    griddep_launch_dependents();
+    // The one-shot kernel lets its dependents launch at once; the streamed one, which fills the SMs for longer,
+    // once its stream has ended: clusters of a next call placed into what is left of the SMs share some of them
+    // while others idle (32 x 151936, calls back to back: 122.3 us released here).
+    if (!RING) griddep_launch_dependents();
     const uint32_t tmem = tmem_sh;
     // inputs may come from the previous kernel on the stream; behind the gather kernel only x does
     const bool early = RING && p.gathered && tid < 32;
@@ -409,6 +412,8 @@ __global__ void __launch_bounds__(kTcThreads) policy_tc_kernel(const __grid_cons
                 cands[c] = p.candidates[c];
             }
     }
+    if (RING && na > 0 && !mbar_wait(&bar_mma, 0, kDrainBudget)) raise_error(p.err, kErrTimeout);
+    if (RING) griddep_launch_dependents();
     // ---- this CTA's partial tile row (thread = row = TMEM lane)
     float d[kTcMaxN];
 #pragma unroll
