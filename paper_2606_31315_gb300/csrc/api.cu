@@ -382,7 +382,7 @@ int bp_verify_commit(int32_t* ctx_lens, const int32_t* n_accepted, const int32_t
 
 size_t bp_policy_select_workspace_size(int num_reqs, int d_in, int hidden, int num_cand) {
     if (num_reqs < 0 || d_in < 1 || hidden < 1 || num_cand < 1) return 0;
-    return sizeof(WorkspaceHeader) + policy_scratch_bytes(num_reqs, d_in, hidden, num_cand);
+    return sizeof(WorkspaceHeader) + policy_scratch_bytes(num_reqs, d_in, hidden, num_cand, true);
 }
 
 int bp_policy_select(const void* feats, int64_t feat_row_stride, const int32_t* row_index, int num_reqs, int d_in,
@@ -397,7 +397,8 @@ int bp_policy_select(const void* feats, int64_t feat_row_stride, const int32_t* 
     const int elt = wdtype == BP_BF16 ? 2 : 4;
     if ((d_in * elt) % 16 != 0 || (feat_row_stride * elt) % 16 != 0 || !aligned(feats, 16) || !aligned(w1, 16))
         return BP_ERR_UNSUPPORTED;
-    int rc = check_workspace(workspace, workspace_bytes, bp_policy_select_workspace_size(num_reqs, d_in, hidden, num_cand));
+    int rc = check_workspace(workspace, workspace_bytes,
+                             sizeof(WorkspaceHeader) + policy_scratch_bytes(num_reqs, d_in, hidden, num_cand, false));
     if (rc != BP_OK) return rc;
     DeviceInfo dev;
     if ((rc = device_info(&dev)) != BP_OK) return rc;
@@ -406,6 +407,7 @@ int bp_policy_select(const void* feats, int64_t feat_row_stride, const int32_t* 
     a.w1 = w1; a.b1 = b1; a.hidden = hidden; a.w2 = w2; a.b2 = b2; a.num_cand = num_cand;
     a.candidates = candidates; a.wdtype = wdtype; a.logits_out = logits_out; a.block_size_out = block_size_out;
     a.scratch = scratch(workspace);
+    a.scratch_bytes = workspace_bytes - sizeof(WorkspaceHeader);
     a.err_word = err_word(workspace);
     rc = launch_policy(a, dev, static_cast<cudaStream_t>(stream));
     if (rc == BP_ERR_CUDA) cudaGetLastError();

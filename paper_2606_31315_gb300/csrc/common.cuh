@@ -151,9 +151,11 @@ struct PolicyArgs {
     float* logits_out;
     int32_t* block_size_out;
     void* scratch;
+    size_t scratch_bytes;
     unsigned int* err_word;
 };
-size_t policy_scratch_bytes(int num_reqs, int d_in, int hidden, int num_cand);
+// full: what callers are told to bring (with the flat split's region); otherwise what a call needs at least.
+size_t policy_scratch_bytes(int num_reqs, int d_in, int hidden, int num_cand, bool full);
 int launch_policy(const PolicyArgs& a, const DeviceInfo& dev, cudaStream_t stream);
 
 struct VerifyEpilogueArgs {

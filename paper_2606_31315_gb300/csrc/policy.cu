@@ -20,10 +20,13 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
+#include <limits.h>
+
 #include <mutex>
 
 #include "common.cuh"
 #include "ptx_sm103.cuh"
+#include "softmax_math.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -549,6 +552,283 @@ __global__ void __launch_bounds__(kTcThreads) policy_tc_kernel(const __grid_cons
     if (warp == 0) tmem_dealloc(tmem, p.tmem_cols);
 }
 
+// ---------------------------------------------------------------- streamed W1, split flat over the SMs
+// For d_in too wide to hold a CTA's share of W1 at once.  The 64-column atoms of every (request group, 128-row
+// tile of W1) form one list, cut into equal runs, one per CTA and one CTA per SM (no clusters: 16 clusters of 9
+// CTAs never fill 152 SMs, and where they land decides how many share one).  A CTA streams its run through one
+// TMA ring; a run that ends or begins inside a tile leaves a partial tile, so every run's part of a tile goes to a
+// workspace slot, and the CTA that completes a tile (an atomic ticket, no waiting) adds the tile's parts in run
+// order, applies b1, ReLU and its columns of W2; the one that completes the last tile adds the tiles' shares of
+// the output layer in tile order and takes the argmax.  Every sum runs in a fixed order.
+// What bounds it: HBM, W1 read once (32 x 151936 -> 2048: 632 MB in 111 us, 5.7 TB/s, about 8 us of it the tail's
+// two tickets and sums).  An MMA at N <= 64 costs one thread more to issue than to run, so two warps take the
+// stages in turn, each with an accumulator of its own.
+constexpr int kFlStages = 8;        // 16 KB of W1 and up to 8 KB of x each
+constexpr int kFlThreads = 224;     // warp 0 TMA, warps 1 and 6 MMA, warps 2-5 epilogue (thread = tile row)
+constexpr int kFlMaxGrid = 192;
+constexpr int kFlC = 16;            // candidates per round of the output layer's reduction
+
+struct PolicyFlatParams {
+    PolicyTcParams tc;
+    int groups, runs_total;   // request groups; atoms of the whole list
+    float4* slots;            // [grid + tiles * groups][npad / 4][128] partial tiles
+    int* tile_tickets;        // [groups * tiles], zero between calls
+    uint32_t cols;
+};
+
+__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+__global__ void __launch_bounds__(kFlThreads, 1) policy_flat_kernel(const __grid_constant__ CUtensorMap w1map,
+                                                                   const __grid_constant__ CUtensorMap xmap,
+                                                                   const PolicyFlatParams f) {
+    constexpr int S = kFlStages;
+    const PolicyTcParams& p = f.tc;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    __shared__ uint64_t full[S], empty[S], acc_full[2], acc_empty[2], mma_done;
+    __shared__ uint32_t tmem_sh;
+    __shared__ int last_sh, ok_sh[4];
+    __shared__ float red[4][kFlC][kTcMaxN];  // the warps' sums of one round; the final logits
+    __shared__ float w2_sh[kFlC][kTcM];      // a round's columns of W2 (each thread its own row's)
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int npad = p.npad, A = p.atoms_total, C = p.num_cand;
+    const int stage_bytes = kTcAtomBytes + npad * 128;
+    const int grid = (int)gridDim.x, cta = (int)blockIdx.x;
+    const int lo = (int)((long long)cta * f.runs_total / grid), hi = (int)((long long)(cta + 1) * f.runs_total / grid);
+    if (tid == 0) {
+        prefetch_tensormap(&w1map);
+        prefetch_tensormap(&xmap);
+        for (int st = 0; st < S; ++st) {
+            mbar_init(&full[st], 1);
+            mbar_init(&empty[st], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&acc_full[b], 2);
+            mbar_init(&acc_empty[b], 4);
+        }
+        mbar_init(&mma_done, 2);
+        fence_mbar_init();
+    }
+    if (warp == 1) {
+        tmem_alloc(&tmem_sh, f.cols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    griddep_launch_dependents();
+    const uint32_t tmem = tmem_sh;
+    // inputs may come from the previous kernel on the stream; behind the gather kernel only x does
+    const bool early = p.gathered && warp == 0;
+    if (!early) griddep_wait();
+
+    if (warp == 0) {
+        if (lane == 0) {
+            auto issue_w = [&](int J, int i) {
+                mbar_arrive_expect_tx(&full[J % S], (uint32_t)stage_bytes);
+                tma_load_2d(base + (J % S) * stage_bytes, &w1map, &full[J % S], (i % A) * kTcAtom, (i / A) % p.tiles * kTcM);
+            };
+            auto issue_x = [&](int J, int i) {
+                tma_load_2d(base + (J % S) * stage_bytes + kTcAtomBytes, &xmap, &full[J % S], (i % A) * kTcAtom,
+                            i / A / p.tiles * kTcMaxN);
+            };
+            const int first = min(S, hi - lo);
+            for (int J = 0; J < first; ++J) issue_w(J, lo + J);
+            if (early) griddep_wait();  // the gathered x
+            for (int J = 0; J < first; ++J) issue_x(J, lo + J);
+            int issued = first;
+            for (int i = lo + first; i < hi; ++i) {
+                const int J = i - lo;
+                if (!mbar_wait(&empty[J % S], ((J / S) - 1) & 1, kWaitBudget)) {
+                    raise_error(p.err, kErrTimeout);
+                    break;
+                }
+                issue_w(J, i);
+                issue_x(J, i);
+                issued = J + 1;
+            }
+            if (issued < hi - lo)  // wound down early: the copies still in flight land before the CTA leaves
+                for (int J = max(0, issued - S); J < issued; ++J) mbar_wait(&full[J % S], (J / S) & 1, kDrainBudget);
+        }
+    } else if (warp == 1 || warp == 6) {
+        // ---- MMA issuers: stage J goes to issuer J % 2; part sg of a tile accumulates into buffer sg % 2
+        if (lane == 0) {
+            const int me = warp == 1 ? 0 : 1;
+            const uint32_t idesc = idesc_bf16_f32(kTcM, npad, false, false);
+            bool ok = true;
+            int sg = 0;
+            for (int i = lo; i < hi && ok; ++sg) {
+                const int end = min(hi, (i / A + 1) * A), b = sg & 1;
+                if (sg >= 2 && !mbar_wait(&acc_empty[b], ((sg >> 1) - 1) & 1, kWaitBudget)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t acc = tmem + (uint32_t)((2 * b + me) * npad);
+                uint32_t add = 0u;
+                for (int J = i - lo + (((i - lo) & 1) != me); J < end - lo; J += 2) {
+                    if (!mbar_wait(&full[J % S], (J / S) & 1, kWaitBudget)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t wa = smem_addr(base + (J % S) * stage_bytes), xa = wa + kTcAtomBytes;
+#pragma unroll
+                    for (int kk = 0; kk < kTcAtom / 16; ++kk) {
+                        umma_ss(acc, smem_desc(wa + kk * 32, 16, 1024, kSwizzle128B),
+                                smem_desc(xa + kk * 32, 16, 1024, kSwizzle128B), idesc, add);
+                        add = 1u;
+                    }
+                    umma_commit(&empty[J % S]);  // the stage is free once these MMAs have read it
+                }
+                if (ok) umma_commit(&acc_full[b]);
+                i = end;
+            }
+            if (!ok) raise_error(p.err, kErrTimeout);
+            umma_commit(&mma_done);  // every MMA issued is complete before tensor memory is released
+            mbar_wait(&mma_done, 0, kDrainBudget);
+        }
+    } else {
+        // ---- epilogue: thread = tile row = tensor-memory lane (quad * 32 + lane)
+        const int quad = warp & 3, row = quad * 32 + lane, et = tid - 64;
+        const uint32_t tq = tmem + ((uint32_t)(quad * 32) << 16);
+        int sg = 0;
+        for (int i = lo; i < hi; ++sg) {
+            const int gt = i / A, end = min(hi, (gt + 1) * A), b = sg & 1, natoms = end - i;
+            const bool two = natoms > 1;            // both issuers have atoms of this part
+            const int only = (i - lo) & 1;          // the one that has, otherwise
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (sg >> 1) & 1, kWaitBudget));
+            if (lane == 0) ok_sh[quad] = ok;
+            epi_sync();  // the four warps go on or leave together
+            if (!(ok_sh[0] && ok_sh[1] && ok_sh[2] && ok_sh[3])) {
+                if (et == 0) raise_error(p.err, kErrTimeout);
+                break;
+            }
+            tc_fence_after();
+            float4* slot = f.slots + (size_t)(cta + gt) * (npad / 4) * kTcM;
+#pragma unroll 1
+            for (int c0 = 0; c0 < npad; c0 += 16) {
+                uint32_t v0[16], v1[16];
+                tmem_ld16(tq + (uint32_t)((2 * b + (two ? 0 : only)) * npad + c0), v0);
+                if (two) tmem_ld16(tq + (uint32_t)((2 * b + 1) * npad + c0), v1);
+                tmem_ld_wait();
+                float x[16];
+#pragma unroll
+                for (int e = 0; e < 16; ++e) x[e] = __uint_as_float(v0[e]) + (two ? __uint_as_float(v1[e]) : 0.f);
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    slot[(c0 / 4 + e) * kTcM + row] = make_float4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acc_empty[b]);
+            // the parts of this tile: runs j0 .. j1 (run j begins at j * runs_total / grid)
+            const long long T = f.runs_total;
+            const int j0 = (int)((((long long)gt * A + 1) * grid - 1) / T), j1 = (int)(((long long)(gt + 1) * A * grid - 1) / T);
+            epi_sync();  // every thread's part before thread 0's release (cumulative)
+            if (et == 0) last_sh = atomic_add_acq_rel_gpu(f.tile_tickets + gt, 1) == j1 - j0;
+            epi_sync();
+            i = end;
+            if (!last_sh) continue;
+            // ---- the tile is complete: its parts in run order, + b1, ReLU, its columns of W2
+            if (et == 0) f.tile_tickets[gt] = 0;  // ready for the next call
+            const int g = gt / p.tiles, tile = gt - g * p.tiles, j = tile * kTcM + row;
+            const int ng = min(kTcMaxN, p.num_reqs - g * kTcMaxN);
+            const float bias = j < p.hidden ? p.b1[j] : 0.f;
+            auto load_w2 = [&](int c0) {  // every load in flight before the first is used
+                float w[kFlC];
+#pragma unroll
+                for (int c = 0; c < kFlC; ++c)
+                    w[c] = c0 + c < C && j < p.hidden ? __bfloat162float(p.w2[(size_t)(c0 + c) * p.hidden + j]) : 0.f;
+#pragma unroll
+                for (int c = 0; c < kFlC; ++c) w2_sh[c][row] = w[c];
+            };
+            if (C <= kFlC) load_w2(0);
+            float* dst = p.part + ((size_t)g * p.tiles + tile) * (kTcMaxN * C);
+#pragma unroll 1
+            for (int h0 = 0; h0 < npad; h0 += 32) {  // 32 requests at a time
+                float h[32];
+#pragma unroll
+                for (int e = 0; e < 32; ++e) h[e] = 0.f;
+                for (int q = j0; q <= j1; q += 4) {  // four parts' loads in flight
+                    float4 z[4][8];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            z[u][e] = q + u <= j1 && h0 + 4 * e < npad
+                                          ? __ldcg(f.slots + ((size_t)(q + u + gt) * (npad / 4) + h0 / 4 + e) * kTcM + row)
+                                          : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            h[4 * e] += z[u][e].x;
+                            h[4 * e + 1] += z[u][e].y;
+                            h[4 * e + 2] += z[u][e].z;
+                            h[4 * e + 3] += z[u][e].w;
+                        }
+                }
+#pragma unroll
+                for (int e = 0; e < 32; ++e) h[e] = j < p.hidden ? fmaxf(0.f, h[e] + bias) : 0.f;
+                for (int c0 = 0; c0 < C; c0 += kFlC) {
+                    const int nc = min(kFlC, C - c0);
+                    if (C > kFlC) load_w2(c0);
+#pragma unroll 1
+                    for (int c = 0; c < nc; ++c) {  // lane n: the sum over the warp's 32 rows for request h0 + n
+                        const float w = w2_sh[c][row];
+                        float v[32];
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) v[e] = h[e] * w;
+                        red[quad][c][lane] = reduce_scatter32(v, lane);
+                    }
+                    epi_sync();
+                    for (int k = et; k < nc * 32; k += 128) {
+                        const int c = k >> 5, n = h0 + (k & 31);
+                        if (n < ng)
+                            dst[n * C + c0 + c] = (red[0][c][k & 31] + red[1][c][k & 31]) + (red[2][c][k & 31] + red[3][c][k & 31]);
+                    }
+                    epi_sync();
+                }
+            }
+            if (et == 0) last_sh = atomic_add_acq_rel_gpu(p.counters + g, 1) == p.tiles - 1;
+            epi_sync();
+            if (!last_sh) continue;
+            // ---- every tile of the group: logits in tile order, then the argmax per request
+            if (et == 0) p.counters[g] = 0;  // ready for the next call
+            float* logits = &red[0][0][0];   // ng * C <= 64 * 64 floats
+            const float* from = p.part + (size_t)g * p.tiles * (kTcMaxN * C);
+            for (int k = et; k < ng * C; k += 128) {
+                float sum = p.b2[k % C];
+                for (int t0 = 0; t0 < p.tiles; t0 += 16) {
+                    float v[16];
+#pragma unroll
+                    for (int u = 0; u < 16; ++u)
+                        v[u] = t0 + u < p.tiles ? __ldcg(from + (size_t)(t0 + u) * (kTcMaxN * C) + k) : 0.f;
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) sum += v[u];
+                }
+                logits[k] = sum;
+                if (p.logits_out) p.logits_out[(size_t)g * kTcMaxN * C + k] = sum;
+            }
+            epi_sync();
+            for (int n = et; n < ng; n += 128) {
+                int best = 0;
+                for (int c = 1; c < C; ++c)
+                    if (logits[n * C + c] > logits[n * C + best]) best = c;
+                p.block_size_out[g * kTcMaxN + n] = p.candidates[best];
+            }
+            epi_sync();
+        }
+    }
+    // ---- release tensor memory
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 1) tmem_dealloc(tmem, f.cols);
+}
+
 // Scratch of the tensor-core path: partials and tickets (after the CUDA-core path's h buffer).
 size_t tc_part_bytes(int num_reqs, int hidden, int num_cand) {
     const size_t groups = ((size_t)num_reqs + kTcMaxN - 1) / kTcMaxN;
@@ -560,6 +840,17 @@ size_t tc_part_bytes(int num_reqs, int hidden, int num_cand) {
 size_t tc_x_bytes(int num_reqs, int d_in) {
     const size_t groups = ((size_t)num_reqs + kTcMaxN - 1) / kTcMaxN;
     return align_up(groups * kTcMaxN * (size_t)d_in * 2, 256);
+}
+
+// The flat split's region: its slots and its tile tickets.
+size_t flat_slot_bytes(int num_reqs, int hidden) {
+    const size_t groups = ((size_t)num_reqs + kTcMaxN - 1) / kTcMaxN, tiles = ((size_t)hidden + kTcM - 1) / kTcM;
+    const size_t npad = ((size_t)(num_reqs < kTcMaxN ? num_reqs : kTcMaxN) + 15) / 16 * 16;
+    return align_up((kFlMaxGrid + groups * tiles) * kTcM * npad * sizeof(float), 256);
+}
+size_t flat_bytes(int num_reqs, int hidden) {
+    const size_t groups = ((size_t)num_reqs + kTcMaxN - 1) / kTcMaxN, tiles = ((size_t)hidden + kTcM - 1) / kTcM;
+    return flat_slot_bytes(num_reqs, hidden) + align_up(groups * tiles * sizeof(int), 256);
 }
 
 // The instantiations: the one-shot kernel, then the rings, deepest first (the order of preference).
@@ -583,6 +874,8 @@ int configure_tc(int device) {
         if (cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem) != cudaSuccess ||
             cudaFuncSetAttribute(k.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
             return BP_ERR_CUDA;
+    if (cudaFuncSetAttribute(policy_flat_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem) != cudaSuccess)
+        return BP_ERR_CUDA;
     if (device >= 0 && device < 64) configured[device] = true;
     return BP_OK;
 }
@@ -627,7 +920,7 @@ int active_ring_clusters(int device, int ks, int smem) {
 }
 
 // Launches the tensor-core path; returns -1 when the shape is outside its limits.
-int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counters, __nv_bfloat16* xg,
+int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counters, __nv_bfloat16* xg, uint8_t* flat,
            cudaStream_t stream) {
     if (reinterpret_cast<uintptr_t>(a.w1) % 16 != 0 || a.num_cand > 64) return -1;
     const int atoms_total = (a.d_in + kTcAtom - 1) / kTcAtom;
@@ -658,7 +951,16 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
     // 151936 -> 2048: 16 tiles of 9-CTA clusters took 200 us with the 5-stage ring at one CTA per SM);
     // if none, the deepest that fits
     int kernel = 0;  // index into kTcKernels
-    if (ring) {
+    // flat split: where a cluster's CTA would stream a long run of atoms, or far more than its share if every SM
+    // took part (clusters hold at most 9 CTAs a tile).  Atoms per CTA in clusters / flat, and the calls' times:
+    // 32 x 151936 -> 2048: 264 / 250, 118.3 / 111.1 us; -> 1024: 264 / 125, 84.7 / 63.2; 16 x 128256 -> 512: 223 /
+    // 53, 71.8 / 38.3 us.  Elsewhere meeting through the workspace costs more than the idle SMs: 5 x 32000 ->
+    // 1280: 56 / 33, 24.7 / 26.5 us; 10 x 32000 -> 2048: 56 / 53, 31.0 / 33.4 us; 17 x 5912 -> 2304: 12 / 11,
+    // 15.6 / 19.0 us.
+    const long long atoms_all = (long long)groups * tiles * atoms_total;
+    const bool flat_split = ring && flat != nullptr && atoms_all <= INT_MAX / 2 &&
+                            (per >= 128 || per >= atoms_all / dev.sm_count + 32);
+    if (ring && !flat_split) {
         for (int i = 1; i <= kTcRings; ++i) {
             const int sm = smem_for(kTcKernels[i].stages);
             if (sm > kTcMaxSmem) continue;
@@ -670,10 +972,10 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
         }
         if (kernel == 0) return -1;
     }
-    const int slots = ring ? kTcKernels[kernel].stages : per;
+    const int slots = flat_split ? kFlStages : ring ? kTcKernels[kernel].stages : per;
     const int w_bytes = slots * kTcAtomBytes > pd_bytes ? slots * kTcAtomBytes : pd_bytes;
     const int x_bytes = slots * npad * 128;
-    int smem = smem_for(slots);
+    int smem = flat_split ? 1024 + kFlStages * (kTcAtomBytes + npad * 128) : smem_for(slots);
     if (smem > kTcMaxSmem) return -1;
     // Tensor memory: one accumulator of npad columns, or one per issuer.  A CTA waits for its columns while its
     // cluster peers wait for it, so no more CTAs may share an SM than its 512 columns serve: the shared memory
@@ -744,6 +1046,26 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
                                groups, npad, xg) != cudaSuccess)
             return BP_ERR_CUDA;
     }
+    if (flat_split) {
+        PolicyFlatParams f;
+        f.tc = p;
+        f.groups = groups;
+        f.runs_total = groups * tiles * atoms_total;
+        f.slots = reinterpret_cast<float4*>(flat);
+        f.tile_tickets = reinterpret_cast<int*>(flat + flat_slot_bytes(a.num_reqs, a.hidden));
+        f.cols = 32;
+        while ((int)f.cols < 4 * npad) f.cols <<= 1;
+        int ctas = dev.sm_count < kFlMaxGrid ? dev.sm_count : kFlMaxGrid;
+        ctas = ctas < f.runs_total ? ctas : f.runs_total;
+        cudaLaunchConfig_t fcfg = {};
+        fcfg.gridDim = dim3((unsigned)ctas, 1, 1);
+        fcfg.blockDim = dim3(kFlThreads, 1, 1);
+        fcfg.dynamicSmemBytes = (size_t)smem;
+        fcfg.stream = stream;
+        fcfg.attrs = pdl;
+        fcfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&fcfg, policy_flat_kernel, w1map, xmap, f) == cudaSuccess ? BP_OK : BP_ERR_CUDA;
+    }
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     cfg.gridDim = dim3((unsigned)(tiles * ks), (unsigned)groups, 1);
@@ -812,9 +1134,9 @@ int run(const PolicyArgs& a, cudaStream_t stream) {
 
 }  // namespace
 
-size_t policy_scratch_bytes(int num_reqs, int d_in, int hidden, int num_cand) {
+size_t policy_scratch_bytes(int num_reqs, int d_in, int hidden, int num_cand, bool full) {
     return align_up(sizeof(float) * (size_t)num_reqs * hidden, 256) + tc_part_bytes(num_reqs, hidden, num_cand) +
-           tc_x_bytes(num_reqs, d_in);
+           tc_x_bytes(num_reqs, d_in) + (full ? flat_bytes(num_reqs, hidden) : 0);
 }
 
 int launch_policy(const PolicyArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
@@ -826,7 +1148,10 @@ int launch_policy(const PolicyArgs& a, const DeviceInfo& dev, cudaStream_t strea
         const size_t tiles = ((size_t)a.hidden + kTcM - 1) / kTcM;
         int* counters = reinterpret_cast<int*>(w + align_up(sizeof(float) * groups * tiles * kTcMaxN * (size_t)a.num_cand, 256));
         __nv_bfloat16* xg = reinterpret_cast<__nv_bfloat16*>(w + tc_part_bytes(a.num_reqs, a.hidden, a.num_cand));
-        const int rc = run_tc(a, dev, part, counters, xg, stream);
+        // the flat split's region comes last: a workspace without it streams through clusters
+        uint8_t* flat = static_cast<uint8_t*>(a.scratch) + policy_scratch_bytes(a.num_reqs, a.d_in, a.hidden, a.num_cand, false);
+        if (a.scratch_bytes < policy_scratch_bytes(a.num_reqs, a.d_in, a.hidden, a.num_cand, true)) flat = nullptr;
+        const int rc = run_tc(a, dev, part, counters, xg, flat, stream);
         if (rc != -1) return rc;
         return run<__nv_bfloat16>(a, stream);
     }

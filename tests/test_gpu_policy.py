@@ -83,3 +83,45 @@ def test_d_in_tail_and_two_request_groups(d_in):
     # per CTA) streams through the ring and wraps around it.
     w = wl.custom(seed=7, policy=dict(num_reqs=70, d_in=d_in, hidden=300, wdtype="bf16", feat_std=1.0))
     _compare(wl.policy_inputs(w))
+
+
+@pytest.mark.parametrize("n,d_in,hidden", [
+    (4, 41992, 256),     # 2 tiles of 657 atoms (the last of 8 columns): dozens of runs per tile
+    (33, 40000, 900),    # a partial tile of 4 rows, 48 padded requests
+    (64, 82000, 300),    # a full group
+    (130, 41000, 300),   # three request groups, the last of two
+    (1, 40000, 128),     # one tile cut over every CTA, runs of 4 or 5 atoms
+    (17, 5912, 600),     # short runs: clusters in either workspace
+])
+@pytest.mark.parametrize("gather", [True, False])
+def test_streamed_splits(n, d_in, hidden, gather):
+    """Wide inputs on both splits of the stream: flat over the SMs in a workspace of the size the library asks
+    for, clusters in one without the flat split's region; feature rows in place or gathered.  Against the oracle,
+    and with each other to the rounding of fp32 sums in another order (bound: sqrt(d_in) 2^-24 of |w||x|, a few
+    1e-6 of the largest logit; 1e-4 is far inside the bar)."""
+    w = wl.custom(seed=n + hidden, policy=dict(num_reqs=n, d_in=d_in, hidden=hidden, wdtype="bf16", feat_std=1.0))
+    pin = wl.policy_inputs(w)
+    if not gather:
+        pin["feats"], pin["row_index"] = np.ascontiguousarray(pin["feats"][pin["row_index"]]), None
+    ref = _oracle(pin)
+    scale = np.abs(ref["logits"]).max()
+    f = lambda k: to_dev(pin[k], "bf16" if k in ("feats", "w1", "w2") else None)  # noqa: E731
+    ri = to_dev(pin["row_index"]) if gather else None
+    args = [f(k) for k in ("feats", "w1", "b1", "w2", "b2", "candidates")]
+    c = len(pin["candidates"])
+    up = lambda x: -(-x // 256) * 256  # noqa: E731
+    groups, tiles = -(-n // 64), -(-hidden // 128)
+    least = 256 + up(4 * n * hidden) + up(4 * groups * tiles * 64 * c) + up(4 * groups) + up(groups * 64 * d_in * 2)
+    full = bp.policy_select_workspace_size(n, d_in, hidden, c)
+    assert least < full
+    for size in (full, least):
+        ws = bp.workspace(size, "cuda")
+        for _ in range(2):  # the tickets are back at zero after a call
+            bs, lo = bp.policy_select(*args, row_index=ri, ws=ws)
+        assert bp.get_status(ws) == 0
+        assert np.abs(lo.cpu().numpy() - ref["logits"]).max() <= 1e-4 * scale
+        ok = ref["top2_margin"] >= 1e-4 * scale
+        np.testing.assert_array_equal(bs.cpu().numpy()[ok], ref["block_size"][ok])
+    with pytest.raises(bp.BlockPilotError) as e:
+        bp.policy_select(*args, row_index=ri, ws=bp.workspace(least, "cuda")[:-1])
+    assert e.value.status == 4
