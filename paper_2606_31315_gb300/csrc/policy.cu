@@ -13,10 +13,11 @@
 //   * The cluster's output-layer partials go to the workspace; the last tile to finish (an
 //     atomic ticket, no waiting) adds them in tile order with b2 and takes the argmax (lowest
 //     index on ties).  Every sum runs in a fixed order: the result is deterministic.
-// fp32 weights (and bf16 shapes outside the tensor-core limits) -- CUDA cores:
-//   kernel 1 streams W1 once for a group of up to 32 requests (rows staged in shared memory,
-//   a warp per hidden row, fp32 accumulation, bias and ReLU fused into the store of h);
-//   kernel 2 (one CTA per request) applies the output layer and takes the argmax.
+// fp32 weights -- CUDA cores: register-tiled products with d_in split over a cluster, then (one CTA per
+// request) the output layer and the argmax.
+// bf16 shapes outside the tensor-core limits -- CUDA cores: a kernel that streams W1 once for a group of up
+// to 32 requests (rows staged in shared memory, a warp per hidden row, bias and ReLU fused into the store of
+// h), then the same output layer.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
@@ -52,16 +53,6 @@ struct Vec8<__nv_bfloat16> {
         }
     }
 };
-template <>
-struct Vec8<float> {
-    __device__ __forceinline__ static void load(const float* p, float (&f)[8]) {
-        const float4 a = *reinterpret_cast<const float4*>(p);
-        const float4 b = *reinterpret_cast<const float4*>(p + 4);
-        f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w;
-        f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
-    }
-};
-
 template <typename T>
 __global__ void __launch_bounds__(kThreads1) policy_hidden_kernel(const T* __restrict__ feats, int64_t row_stride,
                                                                   const int32_t* __restrict__ row_index, int n0,
@@ -115,40 +106,135 @@ __global__ void __launch_bounds__(kThreads1) policy_hidden_kernel(const T* __res
     }
 }
 
+// Output layer and argmax of one request per CTA: a warp per candidate (its 8 warps' chains of loads side by side;
+// one candidate after the other over the whole block took 9 us for 9 candidates).
 template <typename T>
 __global__ void __launch_bounds__(256) policy_out_kernel(const float* __restrict__ hbuf, int hidden,
                                                          const T* __restrict__ w2, const float* __restrict__ b2,
                                                          int num_cand, const int32_t* __restrict__ candidates,
                                                          float* __restrict__ logits_out,
                                                          int32_t* __restrict__ block_size_out) {
-    __shared__ float red[8];
     __shared__ float logits[64];
-    const int n = blockIdx.x, tid = threadIdx.x;
+    const int n = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     griddep_launch_dependents();
     griddep_wait();
     const float* h = hbuf + (size_t)n * hidden;
-    for (int c = 0; c < num_cand; ++c) {
-        float acc = 0.f;
-        for (int j = tid; j < hidden; j += 256) acc = fmaf(static_cast<float>(w2[(size_t)c * hidden + j]), h[j], acc);
+    for (int c = tid >> 5; c < num_cand; c += 8) {
+        const T* w = w2 + (size_t)c * hidden;
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        int j = lane;
+        for (; j + 96 < hidden; j += 128)
 #pragma unroll
-        for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if ((tid & 31) == 0) red[tid >> 5] = acc;
-        __syncthreads();
-        if (tid == 0) {
-            float t = 0.f;
-            for (int w = 0; w < 8; ++w) t += red[w];
-            logits[c] = t + b2[c];
-        }
-        __syncthreads();
+            for (int u = 0; u < 4; ++u) acc[u] = fmaf(static_cast<float>(w[j + 32 * u]), h[j + 32 * u], acc[u]);
+        for (; j < hidden; j += 32) acc[0] = fmaf(static_cast<float>(w[j]), h[j], acc[0]);
+        float sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+        for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0) logits[c] = sum + b2[c];
     }
+    __syncthreads();
     if (tid == 0) {
         int best = 0;
         for (int c = 1; c < num_cand; ++c)
             if (logits[c] > logits[best]) best = c;
         block_size_out[n] = candidates[best];
-        if (logits_out)
-            for (int c = 0; c < num_cand; ++c) logits_out[(size_t)n * num_cand + c] = logits[c];
     }
+    if (logits_out)
+        for (int c = tid; c < num_cand; c += 256) logits_out[(size_t)n * num_cand + c] = logits[c];
+}
+
+// ---------------------------------------------------------------- hidden layer, fp32 weights
+// A cluster of up to 8 CTAs takes a tile of 64 hidden rows x 32 requests and splits d_in; a CTA streams its
+// 32-column chunks of W1 and of the pooled rows through a 4-stage cp.async ring and keeps 4 x 2 outputs per thread
+// (fp32 FFMA, in order along its columns).  The partial tiles are summed in rank order through distributed shared
+// memory, with b1 and ReLU.  What bounds it: for a few requests the stream of W1, for many the shared-memory reads
+// of the products (11 wavefronts a warp for 32 FFMAs).  A warp per hidden row, its requests' rows read whole from
+// shared memory for every row of W1, took 8 wavefronts for 8 FFMAs on part of the SMs: with the output layer 20 x
+// 4000 -> 1024 went from 83.6 to 29.8 us, 1 x 1024 -> 256 from 13.3 to 7.4, 128 x 8192 -> 3072 from 3410 to 629.
+constexpr int kPfRows = 64, kPfReqs = 32, kPfK = 32, kPfStages = 4, kPfMaxKS = 8;
+constexpr int kPfLd = kPfK + 4;  // 16-byte reads of 8 consecutive rows fall on distinct banks
+constexpr int kPfStageFloats = (kPfRows + kPfReqs) * kPfLd;
+constexpr size_t kPfSmem = sizeof(float) * kPfStages * kPfStageFloats;
+
+__global__ void __launch_bounds__(256) policy_f32_hidden_kernel(const float* __restrict__ feats, int64_t row_stride,
+                                                                const int32_t* __restrict__ row_index, int num_reqs,
+                                                                int d_in, const float* __restrict__ w1,
+                                                                const float* __restrict__ b1, int hidden, int g0,
+                                                                float* __restrict__ hbuf) {
+    extern __shared__ float4 pf_smem[];
+    float* ring = reinterpret_cast<float*>(pf_smem);
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;  // rows tx + 16 i, requests 2 ty and 2 ty + 1
+    griddep_launch_dependents();
+    griddep_wait();
+    cg::cluster_group cluster = cg::this_cluster();
+    const int KS = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int j0 = (blockIdx.x / KS) * kPfRows, n0 = (g0 + (int)blockIdx.y) * kPfReqs;
+    const int nr = min(kPfRows, hidden - j0), ng = min(kPfReqs, num_reqs - n0);
+    const int chunks = (d_in + kPfK - 1) / kPfK;
+    const int c0 = (int)((long long)rank * chunks / KS), nc = (int)((long long)(rank + 1) * chunks / KS) - c0;
+    // copies of a chunk: thread t's 16 bytes (t % 8) of W1 rows t / 8 and t / 8 + 32 and of request t / 8
+    const int lr = tid >> 3, lk = 4 * (tid & 7);
+    const bool va = lr < nr, vb = lr + 32 < nr, vx = lr < ng;
+    const float* wa = w1 + (size_t)(j0 + (va ? lr : 0)) * d_in;
+    const float* wb = w1 + (size_t)(j0 + (vb ? lr + 32 : 0)) * d_in;
+    const float* xr = feats + (vx ? (row_index ? (long long)row_index[n0 + lr] : (long long)(n0 + lr)) : 0ll) * row_stride;
+    auto load = [&](int c) {
+        if (c < nc) {
+            const int k = (c0 + c) * kPfK + lk;
+            const bool in = k < d_in;
+            float* st = ring + (c % kPfStages) * kPfStageFloats + lr * kPfLd + lk;
+            cp_async16(st, wa + (in ? k : 0), in && va);
+            cp_async16(st + 32 * kPfLd, wb + (in ? k : 0), in && vb);
+            cp_async16(st + kPfRows * kPfLd, xr + (in ? k : 0), in && vx);
+        }
+        cp_async_commit();
+    };
+    for (int c = 0; c < kPfStages - 1; ++c) load(c);
+    float acc[4][2] = {};
+    const bool active = 4 * (tid >> 5) < ng;  // the warp's four requests
+    for (int c = 0; c < nc; ++c) {
+        cp_async_wait_group<kPfStages - 2>();
+        __syncthreads();  // chunk c has landed everywhere, and everyone is done with chunk c - 1
+        load(c + kPfStages - 1);
+        if (active) {
+            const float* w = ring + (c % kPfStages) * kPfStageFloats + tx * kPfLd;
+            const float* x = ring + (c % kPfStages) * kPfStageFloats + (kPfRows + 2 * ty) * kPfLd;
+#pragma unroll
+            for (int k = 0; k < kPfK; k += 4) {
+                const float4 xa = *reinterpret_cast<const float4*>(x + k);
+                const float4 xb = *reinterpret_cast<const float4*>(x + kPfLd + k);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 v = *reinterpret_cast<const float4*>(w + 16 * i * kPfLd + k);
+                    acc[i][0] = fmaf(v.w, xa.w, fmaf(v.z, xa.z, fmaf(v.y, xa.y, fmaf(v.x, xa.x, acc[i][0]))));
+                    acc[i][1] = fmaf(v.w, xb.w, fmaf(v.z, xb.z, fmaf(v.y, xb.y, fmaf(v.x, xb.x, acc[i][1]))));
+                }
+            }
+        }
+    }
+    cp_async_wait_group<0>();
+    __syncthreads();
+    // the partial tile [request][row], then each CTA its share of the rows
+    float* part = ring;
+    constexpr int kLdP = kPfRows + 1;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        part[(2 * ty) * kLdP + tx + 16 * i] = acc[i][0];
+        part[(2 * ty + 1) * kLdP + tx + 16 * i] = acc[i][1];
+    }
+    cluster.sync();
+    const int per = (kPfRows + KS - 1) / KS, r0 = rank * per, rows = min(nr, r0 + per) - r0;
+    for (int item = tid; item < rows * ng; item += 256) {
+        const int r = r0 + item % rows, n = item / rows;
+        float v[kPfMaxKS];
+#pragma unroll
+        for (int q = 0; q < kPfMaxKS; ++q) v[q] = q < KS ? *cluster.map_shared_rank(part + n * kLdP + r, q) : 0.f;
+        float sum = 0.f;
+#pragma unroll
+        for (int q = 0; q < kPfMaxKS; ++q) sum += v[q];
+        hbuf[(size_t)(n0 + n) * hidden + j0 + r] = fmaxf(0.f, sum + b1[j0 + r]);
+    }
+    cluster.sync();  // no CTA leaves while a peer may still read its shared memory
 }
 
 // ---------------------------------------------------------------- tensor-core path (bf16)
@@ -1083,8 +1169,27 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
     return e == cudaSuccess ? BP_OK : BP_ERR_CUDA;
 }
 
+// The output layer behind a hidden layer in hbuf.
 template <typename T>
-int run(const PolicyArgs& a, cudaStream_t stream) {
+int run_out(const PolicyArgs& a, const float* hbuf, cudaStream_t stream) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)a.num_reqs, 1, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, policy_out_kernel<T>, hbuf, a.hidden, static_cast<const T*>(a.w2), a.b2, a.num_cand,
+                              a.candidates, a.logits_out, a.block_size_out) == cudaSuccess
+               ? BP_OK
+               : BP_ERR_CUDA;
+}
+
+// bf16 shapes outside the tensor-core limits.
+int run_bf16(const PolicyArgs& a, cudaStream_t stream) {
+    using T = __nv_bfloat16;
     float* hbuf = static_cast<float*>(a.scratch);
     const int max_group = kSmemBudget / (a.d_in * (int)sizeof(T));
     if (max_group < 1) return BP_ERR_UNSUPPORTED;
@@ -1100,8 +1205,6 @@ int run(const PolicyArgs& a, cudaStream_t stream) {
         if (cudaFuncSetAttribute(policy_hidden_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget) !=
                 cudaSuccess ||
             cudaFuncSetAttribute(policy_hidden_kernel<T>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 cudaSharedmemCarveoutMaxShared) != cudaSuccess ||
-            cudaFuncSetAttribute(policy_out_kernel<T>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  cudaSharedmemCarveoutMaxShared) != cudaSuccess)
             return BP_ERR_CUDA;
         configured[dev] = true;
@@ -1123,13 +1226,52 @@ int run(const PolicyArgs& a, cudaStream_t stream) {
                                hbuf) != cudaSuccess)
             return BP_ERR_CUDA;
     }
-    cfg.gridDim = dim3((unsigned)a.num_reqs, 1, 1);
+    return run_out<T>(a, hbuf, stream);
+}
+
+int run_f32(const PolicyArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
+    if (a.d_in * (long long)sizeof(float) > kSmemBudget) return BP_ERR_UNSUPPORTED;  // the entry point's limit
+    float* hbuf = static_cast<float*>(a.scratch);
+    static std::mutex cfg_mu;
+    static bool configured[64] = {};
+    if (dev.device < 0 || dev.device >= 64) return BP_ERR_CUDA;
+    {
+        std::lock_guard<std::mutex> cfg_lock(cfg_mu);  // once per device, from any host thread
+        if (!configured[dev.device]) {
+            if (cudaFuncSetAttribute(policy_f32_hidden_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)kPfSmem) != cudaSuccess)
+                return BP_ERR_CUDA;
+            configured[dev.device] = true;
+        }
+    }
+    const int tiles = (a.hidden + kPfRows - 1) / kPfRows, groups = (a.num_reqs + kPfReqs - 1) / kPfReqs;
+    const int chunks = (a.d_in + kPfK - 1) / kPfK;
+    // d_in split so that about two CTAs reach every SM, with at least two chunks each
+    const long long want = 2LL * dev.sm_count / ((long long)tiles * groups);
+    int ks = (int)(want < kPfMaxKS ? want : kPfMaxKS);
+    ks = ks < chunks / 2 ? ks : chunks / 2;
+    ks = ks < 1 ? 1 : ks;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
     cfg.blockDim = dim3(256, 1, 1);
-    cfg.dynamicSmemBytes = 0;
-    if (cudaLaunchKernelEx(&cfg, policy_out_kernel<T>, (const float*)hbuf, a.hidden, static_cast<const T*>(a.w2), a.b2,
-                           a.num_cand, a.candidates, a.logits_out, a.block_size_out) != cudaSuccess)
-        return BP_ERR_CUDA;
-    return BP_OK;
+    cfg.dynamicSmemBytes = kPfSmem;
+    cfg.stream = stream;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)ks;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    for (int g0 = 0; g0 < groups; g0 += 65535) {  // the grid's y limit
+        cfg.gridDim = dim3((unsigned)(tiles * ks), (unsigned)(groups - g0 < 65535 ? groups - g0 : 65535), 1);
+        if (cudaLaunchKernelEx(&cfg, policy_f32_hidden_kernel, static_cast<const float*>(a.feats), a.row_stride,
+                               a.row_index, a.num_reqs, a.d_in, static_cast<const float*>(a.w1), a.b1, a.hidden, g0,
+                               hbuf) != cudaSuccess)
+            return BP_ERR_CUDA;
+    }
+    return run_out<float>(a, hbuf, stream);
 }
 
 }  // namespace
@@ -1153,9 +1295,9 @@ int launch_policy(const PolicyArgs& a, const DeviceInfo& dev, cudaStream_t strea
         if (a.scratch_bytes < policy_scratch_bytes(a.num_reqs, a.d_in, a.hidden, a.num_cand, true)) flat = nullptr;
         const int rc = run_tc(a, dev, part, counters, xg, flat, stream);
         if (rc != -1) return rc;
-        return run<__nv_bfloat16>(a, stream);
+        return run_bf16(a, stream);
     }
-    return run<float>(a, stream);
+    return run_f32(a, dev, stream);
 }
 
 }  // namespace bp

@@ -125,3 +125,22 @@ def test_streamed_splits(n, d_in, hidden, gather):
     with pytest.raises(bp.BlockPilotError) as e:
         bp.policy_select(*args, row_index=ri, ws=bp.workspace(least, "cuda")[:-1])
     assert e.value.status == 4
+
+
+@pytest.mark.parametrize("n,d_in,hidden", [
+    (1, 4, 1),          # one copy, one row
+    (33, 36, 65),       # a request and a row past a tile, a chunk of 4 columns
+    (32, 1000, 64),     # exactly one tile
+    (70, 4100, 300),    # three request tiles, d_in split over a cluster
+    (5, 40960, 130),    # the widest input the fp32 path takes
+])
+def test_fp32_tiles(n, d_in, hidden):
+    """fp32 sums of d_in and hidden terms: errors of a few sqrt(length) 2^-24 of the terms, 1e-6 of the logits."""
+    w = wl.custom(seed=n + hidden, policy=dict(num_reqs=n, d_in=d_in, hidden=hidden, wdtype="f32", feat_std=1.0))
+    pin = wl.policy_inputs(w)
+    bs, lo = _run(pin)
+    ref = _oracle(pin)
+    scale = np.abs(ref["logits"]).max()
+    assert np.abs(lo - ref["logits"]).max() <= 1e-5 * scale
+    ok = ref["top2_margin"] >= 1e-4 * scale
+    np.testing.assert_array_equal(bs[ok], ref["block_size"][ok])
