@@ -966,21 +966,22 @@ int configure_tc(int device) {
     return BP_OK;
 }
 
-// Clusters of ks streaming CTAs with smem bytes of dynamic shared memory each that the device holds at
-// once (cached per device, cluster size and size).  The occupancy query counts clusters at one CTA per
-// SM (on this GB300 it answers 15 nine-CTA clusters at every size); clusters also share SMs when the
+// Clusters of ks CTAs of an instantiation with smem bytes of dynamic shared memory each that the device holds at
+// once (cached per device, instantiation, cluster size and size).  The occupancy query counts clusters at one CTA
+// per SM (on this GB300 it answers 15 nine-CTA clusters at every size); clusters also share SMs when the
 // shared memory lets several CTAs fit, so its count is scaled by the CTAs per SM (measured: 16 such
 // clusters ran at once at two CTAs per SM, not at one).
-int active_ring_clusters(int device, int ks, int smem) {
+int active_clusters(int device, int kernel, int ks, int smem) {
     struct Entry {
-        int device, ks, smem, n;
+        int device, kernel, ks, smem, n;
     };
     static std::mutex mu;
-    static Entry cache[64];
-    static int used = 0;
+    static Entry cache[256];
+    static int used = 0, next = 0;
     std::lock_guard<std::mutex> lock(mu);
     for (int i = 0; i < used; ++i)
-        if (cache[i].device == device && cache[i].ks == ks && cache[i].smem == smem) return cache[i].n;
+        if (cache[i].device == device && cache[i].kernel == kernel && cache[i].ks == ks && cache[i].smem == smem)
+            return cache[i].n;
     cudaLaunchConfig_t probe = {};
     cudaLaunchAttribute pa[1];
     probe.gridDim = dim3((unsigned)ks, 1, 1);
@@ -993,7 +994,7 @@ int active_ring_clusters(int device, int ks, int smem) {
     probe.attrs = pa;
     probe.numAttrs = 1;
     int n = 0, per_sm = 0, reserved = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kTcKernels[1].fn, &probe) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveClusters(&n, kTcKernels[kernel].fn, &probe) != cudaSuccess ||
         cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device) != cudaSuccess ||
         cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, device) != cudaSuccess) {
         cudaGetLastError();
@@ -1001,7 +1002,9 @@ int active_ring_clusters(int device, int ks, int smem) {
     }
     const int ctas_per_sm = per_sm / (smem + reserved);
     n *= ctas_per_sm > 1 ? ctas_per_sm : 1;
-    if (used < 64) cache[used++] = Entry{device, ks, smem, n};
+    cache[next] = Entry{device, kernel, ks, smem, n};  // the oldest entry makes room
+    next = (next + 1) % 256;
+    used = used < 256 ? used + 1 : 256;
     return n;
 }
 
@@ -1018,20 +1021,41 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
     ks = ks < 1 ? 1 : ks;
     ks = ks > kTcMaxKS ? kTcMaxKS : ks;
     ks = ks > atoms_total ? atoms_total : ks;
-    const int per = (atoms_total + ks - 1) / ks;
-    const bool ring = per > kTcMaxAtoms;  // too many atoms to hold at once: stream them
+    const bool ring = (atoms_total + ks - 1) / ks > kTcMaxAtoms;  // too many atoms to hold at once: stream them
     const int pd_bytes = kTcM * (npad + 4) * 4;
-    const int rpr = (kTcM + ks - 1) / ks;
-    int h_bytes = rpr * npad * 4;
     const int lg_bytes = kTcMaxN * a.num_cand * 4;  // the last tile's logits reuse the h region
-    h_bytes = h_bytes > lg_bytes ? h_bytes : lg_bytes;
     const int op_bytes = kTcMaxN * a.num_cand * 4;
-    const int w2s_bytes = a.num_cand * rpr * 4;
-    const auto smem_for = [&](int slots) {  // atoms held at once
+    const auto h_for = [&](int k) {  // h of the rows a CTA of k owns
+        const int h = (kTcM + k - 1) / k * npad * 4;
+        return h > lg_bytes ? h : lg_bytes;
+    };
+    const auto smem_for = [&](int slots, int k) {  // slots: atoms held at once
         const int wb = slots * kTcAtomBytes > pd_bytes ? slots * kTcAtomBytes : pd_bytes;
-        return 1024 + wb + slots * npad * 128 + h_bytes + op_bytes + w2s_bytes;
+        return 1024 + wb + slots * npad * 128 + h_for(k) + op_bytes + a.num_cand * ((kTcM + k - 1) / k) * 4;
+    };
+    // Tensor memory: one accumulator of npad columns, or one per issuer.  A CTA waits for its columns while its
+    // cluster peers wait for it, so no more CTAs may share an SM than its 512 columns serve: the shared memory
+    // of a CTA keeps them to that.
+    uint32_t cols = 32;
+    while ((int)cols < npad * (ring ? 1 : kTcIssuers)) cols <<= 1;
+    const int least = dev.max_smem_optin / (int)(512 / cols + 1) + 1024;
+    const auto launch_smem = [&](int slots, int k) {
+        const int sm = smem_for(slots, k);
+        return sm > least ? sm : least;
     };
     if (configure_tc(dev.device) != BP_OK) return BP_ERR_CUDA;
+    // one-shot: the widest split whose clusters are all resident at once, while a CTA still holds its atoms (a
+    // cluster left for a second wave doubles the call: 60 x 2000 -> 3000, 24 tiles, clusters of 6: 27.0 us)
+    if (!ring)
+        for (int k = ks; k >= 1 && (atoms_total + k - 1) / k <= kTcMaxAtoms; --k) {
+            const int sm = launch_smem((atoms_total + k - 1) / k, k);
+            if (sm <= kTcMaxSmem && active_clusters(dev.device, 0, k, sm) >= tiles * groups) {
+                ks = k;
+                break;
+            }
+        }
+    const int per = (atoms_total + ks - 1) / ks;
+    const int h_bytes = h_for(ks);
     // ring: the deepest under which every cluster of the grid is resident at once -- a cluster left for
     // a second wave streams its tile alone at a fraction of the bandwidth (measured at 64 requests x
     // 151936 -> 2048: 16 tiles of 9-CTA clusters took 200 us with the 5-stage ring at one CTA per SM);
@@ -1048,10 +1072,10 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
                             (per >= 128 || per >= atoms_all / dev.sm_count + 32);
     if (ring && !flat_split) {
         for (int i = 1; i <= kTcRings; ++i) {
-            const int sm = smem_for(kTcKernels[i].stages);
+            const int sm = launch_smem(kTcKernels[i].stages, ks);
             if (sm > kTcMaxSmem) continue;
             if (kernel == 0) kernel = i;
-            if (active_ring_clusters(dev.device, ks, sm) >= tiles * groups) {
+            if (active_clusters(dev.device, i, ks, sm) >= tiles * groups) {
                 kernel = i;
                 break;
             }
@@ -1061,15 +1085,8 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
     const int slots = flat_split ? kFlStages : ring ? kTcKernels[kernel].stages : per;
     const int w_bytes = slots * kTcAtomBytes > pd_bytes ? slots * kTcAtomBytes : pd_bytes;
     const int x_bytes = slots * npad * 128;
-    int smem = flat_split ? 1024 + kFlStages * (kTcAtomBytes + npad * 128) : smem_for(slots);
+    const int smem = flat_split ? 1024 + kFlStages * (kTcAtomBytes + npad * 128) : launch_smem(slots, ks);
     if (smem > kTcMaxSmem) return -1;
-    // Tensor memory: one accumulator of npad columns, or one per issuer.  A CTA waits for its columns while its
-    // cluster peers wait for it, so no more CTAs may share an SM than its 512 columns serve: the shared memory
-    // of a CTA keeps them to that.
-    uint32_t cols = 32;
-    while ((int)cols < npad * (ring ? 1 : kTcIssuers)) cols <<= 1;
-    const int least = dev.max_smem_optin / (int)(512 / cols + 1) + 1024;
-    smem = smem > least ? smem : least;
 
     CUtensorMap w1map, xmap;
     const cuuint64_t dims[2] = {(cuuint64_t)a.d_in, (cuuint64_t)a.hidden};
