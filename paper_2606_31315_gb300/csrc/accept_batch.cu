@@ -41,6 +41,7 @@ constexpr int kBChunk = 16384;                 // vocabulary entries per chunk
 constexpr int kBVec = kBChunk / 4 / kBThreads;  // 16-byte groups per thread: 16 (64 entries)
 constexpr int kBSegs = kBVec;                  // 128-entry segments per warp of a chunk
 constexpr int kMaxDrawSplit = 4;               // parts a draw chunk may be cut into
+constexpr int kKeep = 2;                       // part totals a lane of the crossing search keeps
 
 struct BatchParams {
     const float* target;  // [rows_t][ld], vocab entries each
@@ -179,15 +180,21 @@ __device__ __forceinline__ void load_row_parts(const BatchParams& p, int r, int 
 }
 template <bool GREEDY>
 __device__ __forceinline__ void merge_parts(float2& acc, const float2 (&x)[kMergeBatch]) {
+    if (GREEDY) {
 #pragma unroll
-    for (int q = 0; q < kMergeBatch; ++q) {
-        if (GREEDY) {
+        for (int q = 0; q < kMergeBatch; ++q) {
             int ai = __float_as_int(acc.y);
             amax_merge(acc.x, ai, x[q].x, __float_as_int(x[q].y));
             acc.y = __int_as_float(ai);
-        } else {
-            lse_merge(acc.x, acc.y, x[q].x, x[q].y);
         }
+    } else {  // the largest maximum first, then every sum scaled to it: no exponential waits for another
+        float m = acc.x;
+#pragma unroll
+        for (int q = 0; q < kMergeBatch; ++q) m = fmaxf(m, x[q].x);
+        float s = acc.y * ex2d(acc.x, m);
+#pragma unroll
+        for (int q = 0; q < kMergeBatch; ++q) s = __fmaf_rn(x[q].y, ex2d(x[q].x, m), s);
+        acc = make_float2(m, s);
     }
 }
 // Both rows r1, r2 (r2 < 0: none) at once: every load of the first batch is issued before any merge.
@@ -483,7 +490,18 @@ __global__ void __launch_bounds__(kBThreads, SPLIT > 1 ? 2 : PH) batch_draw_kern
     // ---- every part is in: the distribution, the threshold and the crossing part (exact sums)
     if (warp == 0) {
         unsigned long long R = 0, P = 0;
-        for (int c = lane; c < units; c += 32) {
+        ulonglong2 keep[kKeep];  // the lane's first parts, for the search below
+#pragma unroll
+        for (int q = 0; q < kKeep; ++q) {
+            const int c = lane + 32 * q;
+            keep[q] = c < units ? __ldcg(&p.ctot[(size_t)s * units + c]) : make_ulonglong2(0ull, 0ull);
+        }
+#pragma unroll
+        for (int q = 0; q < kKeep; ++q) {
+            R += keep[q].x;
+            P += keep[q].y;
+        }
+        for (int c = lane + 32 * kKeep; c < units; c += 32) {
             const ulonglong2 x = __ldcg(&p.ctot[(size_t)s * units + c]);
             R += x.x;
             P += x.y;
@@ -501,13 +519,8 @@ __global__ void __launch_bounds__(kBThreads, SPLIT > 1 ? 2 : PH) batch_draw_kern
         const unsigned long long thr = __umul64hi(__float2ull_rn(u * 18446744073709551616.f), total);
         int cstar = -1;
         unsigned long long below = 0;
-        for (int c0 = 0; c0 < units && cstar < 0; c0 += 32) {  // parts in entry order, 32 at a time
-            const int c = c0 + lane;
-            unsigned long long x = 0;
-            if (c < units) {
-                const ulonglong2 t = __ldcg(&p.ctot[(size_t)s * units + c]);
-                x = use_r ? t.x : t.y;
-            }
+        // parts in entry order, 32 at a time; the first ones from registers (a second round trip took 0.6 us)
+        auto search = [&](int c0, unsigned long long x) {
             const unsigned long long incl = warp_incl_scan(x, lane) + below;
             const unsigned long long excl = incl - x;
             const unsigned hit = __ballot_sync(0xffffffffu, x > 0 && excl <= thr && thr < incl);
@@ -518,6 +531,17 @@ __global__ void __launch_bounds__(kBThreads, SPLIT > 1 ? 2 : PH) batch_draw_kern
             } else {
                 below = __shfl_sync(0xffffffffu, incl, 31);
             }
+        };
+#pragma unroll
+        for (int q = 0; q < kKeep; ++q)
+            if (cstar < 0 && 32 * q < units) search(32 * q, use_r ? keep[q].x : keep[q].y);
+        for (int c0 = 32 * kKeep; c0 < units && cstar < 0; c0 += 32) {
+            unsigned long long x = 0;
+            if (c0 + lane < units) {
+                const ulonglong2 t = __ldcg(&p.ctot[(size_t)s * units + c0 + lane]);
+                x = use_r ? t.x : t.y;
+            }
+            search(c0, x);
         }
         if (lane == 0) {
             if (total == 0 || cstar < 0) {  // no positive mass (or unreachable with exact sums): report
