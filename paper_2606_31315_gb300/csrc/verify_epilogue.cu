@@ -12,7 +12,7 @@
 // acceptance has used them, so the only HBM stream is W itself (read once).
 //
 // One persistent cooperative launch, one CTA per SM (every CTA co-resident):
-//   * CTA c owns a contiguous slice of the vocabulary, at most 16 tiles of 128 LM-head rows.  Its
+//   * CTA c owns a contiguous slice of the vocabulary, at most 16 tiles of up to 128 LM-head rows.  Its
 //     W rows stream once through an 8-stage TMA ring (one 128 x 64 bf16 box per stage, 128-byte
 //     swizzle); warp 2 gathers the same 64 columns of every state row (target rows, then drafter
 //     rows, zero rows up to NP) into the stage with 16-byte cp.async copies; one thread of warp 1
@@ -63,7 +63,7 @@ struct VeParams {
     const __nv_bfloat16* h_draft;   // [rows - rows_t][hidden]
     int hidden, vocab, atoms;
     int num_seqs, total_draft, rows_t, rows;
-    int tiles_base, tiles_extra;    // CTA c: tiles_base + (c < tiles_extra) tiles
+    int slice, tail;                // CTA c: entries from c * slice on; rows of a slice's last tile (a multiple of 8)
     uint32_t tmem_cols;
     float c2;                       // log2(e) / T
     const int32_t* tokens;
@@ -176,7 +176,8 @@ __device__ __forceinline__ float2 entry_weights(uint32_t tmem_q, int t, const Dr
 
 template <int NP, int APS>
 __global__ void __launch_bounds__(kVeThreads, 1)
-    verify_epilogue_kernel(const __grid_constant__ CUtensorMap wmap, const VeParams p) {
+    verify_epilogue_kernel(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap wtail,
+                           const VeParams p) {
     constexpr int STG = ve_stages(NP, APS);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sW = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -195,10 +196,9 @@ __global__ void __launch_bounds__(kVeThreads, 1)
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int c = (int)blockIdx.x, grid = (int)gridDim.x;
-    const int ntile = p.tiles_base + (c < p.tiles_extra ? 1 : 0);
-    const int tile0 = c * p.tiles_base + min(c, p.tiles_extra);
-    const int v0 = tile0 * kVeM;                        // first vocabulary entry of the slice
-    const int v1 = min(p.vocab, v0 + ntile * kVeM);
+    const int v0 = c * p.slice;                         // the slice's vocabulary entries [v0, v1)
+    const int v1 = min(p.vocab, v0 + p.slice);
+    const int ntile = (v1 - v0 + kVeM - 1) / kVeM, tail_tile = (p.slice - 1) / kVeM;
     const int spt = p.atoms / APS;                   // ring stages per tile
     const int J = ntile * spt;                          // ring stages of this CTA
     const int S = p.num_seqs;
@@ -206,14 +206,18 @@ __global__ void __launch_bounds__(kVeThreads, 1)
     // stage j of the ring: atoms a0 .. a0 + APS - 1 of tile t, both found from j
     auto issue_w = [&](int j) {
         const int st = j % STG, t = j / spt, a0 = (j - t * spt) * APS;
-        mbar_arrive_expect_tx(&wfull[st], APS * kVeWBytes);
+        // the slice's last tile has `tail` rows; the rest of its stage keeps older rows, whose lanes nobody reads
+        const bool last = t == tail_tile;
+        mbar_arrive_expect_tx(&wfull[st], (uint32_t)(APS * (last ? p.tail : kVeM) * 128));
 #pragma unroll
         for (int u = 0; u < APS; ++u)
-            tma_load_2d(sW + (st * APS + u) * kVeWBytes, &wmap, &wfull[st], (a0 + u) * kVeAtom, (tile0 + t) * kVeM);
+            tma_load_2d(sW + (st * APS + u) * kVeWBytes, last ? &wtail : &wmap, &wfull[st], (a0 + u) * kVeAtom,
+                        v0 + t * kVeM);
     };
     const int j_first = min(STG, J);  // stages issued before the block-wide set-up completes
     if (tid == 0) {
         prefetch_tensormap(&wmap);
+        prefetch_tensormap(&wtail);
         for (int st = 0; st < STG; ++st) {
             mbar_init(&wfull[st], 1);
             mbar_init(&hfull[st], 1);
@@ -434,15 +438,18 @@ __global__ void __launch_bounds__(kVeThreads, 1)
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
             const int r = r0 + b * (kVeThreads / 32);
-            float a0 = -INFINITY, a1 = 0.f;
+            // the largest maximum first, then every sum scaled to it: no exponential waits for another
+            float mx = x[b][0].x;
 #pragma unroll
-            for (int m = 0; m < kVeMaxGrid / 32; ++m) lse_merge(a0, a1, x[b][m].x, x[b][m].y);
+            for (int m = 1; m < kVeMaxGrid / 32; ++m) mx = fmaxf(mx, x[b][m].x);
 #pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) {
-                const float b0 = __shfl_xor_sync(0xffffffffu, a0, o);
-                lse_merge(a0, a1, b0, __shfl_xor_sync(0xffffffffu, a1, o));
-            }
-            if (lane == 0 && r < p.rows) rst[r] = make_float2(a0, a1);
+            for (int o = 16; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            float sum = 0.f;
+#pragma unroll
+            for (int m = 0; m < kVeMaxGrid / 32; ++m) sum = __fmaf_rn(x[b][m].y, ex2d(x[b][m].x, mx), sum);
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (lane == 0 && r < p.rows) rst[r] = make_float2(mx, sum);
         }
     }
     __syncthreads();
@@ -679,13 +686,14 @@ VeLayout ve_layout(int num_seqs, int total_draft, int vocab, bool full) {
         l.tickets_off = l.rowst_off + align_up((size_t)rows * sizeof(float2), 256);
         l.draw_off = l.tickets_off + align_up((size_t)num_seqs * sizeof(int), 256);
         l.logits_off = l.draw_off + align_up(accept_draw_scratch_bytes(num_seqs, vocab), 256);
-        l.total = l.logits_off + align_up((size_t)rows * (size_t)(full ? ve_padded(vocab) : vocab) * sizeof(float), 256);
+        l.total = l.logits_off + align_up((size_t)rows * (full ? ve_padded(vocab) : vocab) * sizeof(float), 256);
     }
     return l;
 }
 
 template <int NP, int APS>
-int ve_launch(const CUtensorMap& wmap, const VeParams& p, int grid, const DeviceInfo& dev, cudaStream_t stream) {
+int ve_launch(const CUtensorMap& wmap, const CUtensorMap& wtail, const VeParams& p, int grid, const DeviceInfo& dev,
+              cudaStream_t stream) {
     static std::mutex cfg_mu;        // per instantiation (a template's own statics)
     static int configured[64] = {};
     const size_t smem = ve_smem_bytes<NP, APS>();
@@ -713,8 +721,8 @@ int ve_launch(const CUtensorMap& wmap, const VeParams& p, int grid, const Device
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, verify_epilogue_kernel<NP, APS>, wmap, p) == cudaSuccess ? BP_OK
-                                                                                               : BP_ERR_CUDA;
+    return cudaLaunchKernelEx(&cfg, verify_epilogue_kernel<NP, APS>, wmap, wtail, p) == cudaSuccess ? BP_OK
+                                                                                                     : BP_ERR_CUDA;
 }
 
 }  // namespace
@@ -722,6 +730,12 @@ int ve_launch(const CUtensorMap& wmap, const VeParams& p, int grid, const Device
 size_t verify_epilogue_scratch_bytes(int num_seqs, int total_draft, int vocab, bool full) {
     return ve_layout(num_seqs, total_draft, vocab, full).total;
 }
+
+// Entries per CTA: equal shares of the vocabulary, in eights (the swizzle's rows).  With whole tiles, of 151,936
+// entries 123 CTAs had 8 and 29 had 7, done 12 us before the others; HBM was still nearly busy, so the gain is small
+// there (31 rows, hidden 2560: 126.1 -> 125.7 us) and grows where a tile is more of a share (50,257 entries: 56.7 ->
+// 55.4 us; 32,000: 42.9 -> 41.6 us).
+static int ve_slice(int vocab, int grid) { return (int)(((long long)vocab + grid * 8 - 1) / (grid * 8) * 8); }
 
 int verify_epilogue_config(int rows, int vocab, int hidden, int sm_count, int* grid, int* np, int* tiles_per_cta) {
     if (hidden % kVeAtom != 0) return BP_ERR_UNSUPPORTED;
@@ -731,9 +745,10 @@ int verify_epilogue_config(int rows, int vocab, int hidden, int sm_count, int* g
     const int NP = rows <= 32 ? 32 : 64;
     const int per = (tiles_total + g - 1) / g;
     if (per > kVeMaxTiles || per * NP > 512) return BP_ERR_UNSUPPORTED;
-    *grid = g;
+    const int slice = ve_slice(vocab, g);  // at most per tiles
+    *grid = (vocab + slice - 1) / slice;
     *np = NP;
-    *tiles_per_cta = per;
+    *tiles_per_cta = (slice + kVeM - 1) / kVeM;
     return BP_OK;
 }
 
@@ -764,16 +779,20 @@ int launch_verify_epilogue(const VerifyEpilogueArgs& a, const DeviceInfo& dev, c
     int grid = 0, NP = 0, per = 0;
     int rc = verify_epilogue_config(rows, a.vocab, a.hidden, dev.sm_count, &grid, &NP, &per);
     if (rc != BP_OK) return rc;
-    const int tiles_total = (a.vocab + kVeM - 1) / kVeM;
     uint32_t cols = 32;
     while (cols < (uint32_t)(per * NP)) cols <<= 1;
 
-    CUtensorMap wmap;
+    const int slice = ve_slice(a.vocab, min(min(dev.sm_count, kVeMaxGrid), (a.vocab + kVeM - 1) / kVeM));
+    const int tail = slice - (slice - 1) / kVeM * kVeM;
+    CUtensorMap wmap, wtail;
     const cuuint64_t dims[2] = {(cuuint64_t)a.hidden, (cuuint64_t)a.vocab};
     const cuuint64_t strides[1] = {(cuuint64_t)a.hidden * 2};
     const cuuint32_t box[2] = {(cuuint32_t)kVeAtom, (cuuint32_t)kVeM};
+    const cuuint32_t box_tail[2] = {(cuuint32_t)kVeAtom, (cuuint32_t)tail};
     if (encode_tensor_map(&wmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(a.lm_head), dims, strides, box,
-                          CU_TENSOR_MAP_SWIZZLE_128B) != BP_OK)
+                          CU_TENSOR_MAP_SWIZZLE_128B) != BP_OK ||
+        encode_tensor_map(&wtail, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(a.lm_head), dims, strides,
+                          box_tail, CU_TENSOR_MAP_SWIZZLE_128B) != BP_OK)
         return BP_ERR_CUDA;
 
     VeParams p;
@@ -786,8 +805,8 @@ int launch_verify_epilogue(const VerifyEpilogueArgs& a, const DeviceInfo& dev, c
     p.total_draft = a.total_draft;
     p.rows_t = rows_t;
     p.rows = rows;
-    p.tiles_base = tiles_total / grid;
-    p.tiles_extra = tiles_total % grid;
+    p.slice = slice;
+    p.tail = tail;
     p.tmem_cols = cols;
     p.c2 = 1.4426950408889634f / a.temperature;
     p.tokens = a.tokens;
@@ -805,8 +824,10 @@ int launch_verify_epilogue(const VerifyEpilogueArgs& a, const DeviceInfo& dev, c
     p.err = a.err_word;
     const bool two = p.atoms % 2 == 0;  // two atoms per stage where the hidden size allows
     if (NP == 32)
-        return two ? ve_launch<32, 2>(wmap, p, grid, dev, stream) : ve_launch<32, 1>(wmap, p, grid, dev, stream);
-    return two ? ve_launch<64, 2>(wmap, p, grid, dev, stream) : ve_launch<64, 1>(wmap, p, grid, dev, stream);
+        return two ? ve_launch<32, 2>(wmap, wtail, p, grid, dev, stream)
+                   : ve_launch<32, 1>(wmap, wtail, p, grid, dev, stream);
+    return two ? ve_launch<64, 2>(wmap, wtail, p, grid, dev, stream)
+               : ve_launch<64, 1>(wmap, wtail, p, grid, dev, stream);
 }
 
 }  // namespace bp

@@ -7,8 +7,8 @@
 // over the whole vocabulary.  The resident kernel (verify_epilogue.cu) keeps a batch's whole
 // [rows, V] accumulator in tensor memory, which bounds it to 64 rows: the GPU's tensor memory holds
 // about 39 MB, and 248 rows of a 151,936-entry vocabulary take 151 MB in fp32.  Here:
-//   1. lm_head_stream_kernel: one CTA per SM owns a contiguous run of 256-entry passes of the
-//      vocabulary.  Per pass, its W rows (256 entries x 64 hidden columns per stage) and the states of
+//   1. lm_head_stream_kernel: one CTA per SM owns an equal contiguous share of the vocabulary,
+//      streamed in passes of 256 entries and a last pass of what is left.  Per pass, its W rows (256 entries x 64 hidden columns per stage) and the states of
 //      up to 256 rows stream through a TMA ring; one thread issues M=128 (state rows) x N=256 (entries)
 //      x K=16 tcgen05 MMAs, one per 128-row half of the states.  Tensor-memory lane = state row, so each
 //      epilogue thread owns one row and folds the pass's 256 logits into its row's running (max, sum of
@@ -63,7 +63,7 @@ constexpr size_t vs_smem_bytes() {
 
 struct VsParams {
     int vocab, atoms;
-    int passes_base, passes_extra;  // CTA c: passes_base + (c < passes_extra) passes of 256 entries
+    int slice, tail;                // CTA c: entries from c * slice on; entries of a slice's last pass (multiples of 8)
     int nt, nt8, nd;                // the group's target rows, nt rounded up to 8, its drafter rows
     int ht0, hd0;                   // first target / drafter state of the group (TMA row coordinates)
     int row_t0, row_d0;             // their stacked rows (target rows first, then the drafter's)
@@ -142,10 +142,10 @@ __device__ __forceinline__ void store_chunk(uint8_t* stage, const uint32_t (&r)[
     for (int i = 0; i < 8; ++i)
         *reinterpret_cast<uint4*>(stage + lane * 128 + ((i ^ (lane & 7)) << 4)) =
             make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
-    if (p.tma_store) {
+    if (p.tma_store && n == 32) {
         fence_proxy_async_smem();  // the copy reads the buffer through the async proxy
         __syncwarp();
-        if (lane == 0 && srow0 < p.grows) {  // rows past the group, entries past the vocabulary: clipped
+        if (lane == 0 && srow0 < p.grows) {  // rows past the group: clipped
             tma_store_2d(lmap, stage, v0, srow0);
             bulk_commit_group();
         }
@@ -175,9 +175,9 @@ __device__ __forceinline__ void store_chunk(uint8_t* stage, const uint32_t (&r)[
 
 template <bool GREEDY, int MT, bool WRITE>
 __global__ void __launch_bounds__(kVsThreads, 1)
-    lm_head_stream_kernel(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap htmap,
-                          const __grid_constant__ CUtensorMap hdmap, const __grid_constant__ CUtensorMap lmap,
-                          const VsParams p) {
+    lm_head_stream_kernel(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap wtail,
+                          const __grid_constant__ CUtensorMap htmap, const __grid_constant__ CUtensorMap hdmap,
+                          const __grid_constant__ CUtensorMap lmap, const VsParams p) {
     constexpr int STG = vs_stages(MT);
     constexpr int NB = 2 / MT;                     // accumulator buffers of MT x 256 columns
     constexpr int STAGE = kVsWBytes + MT * kVsHBytes;
@@ -191,13 +191,13 @@ __global__ void __launch_bounds__(kVsThreads, 1)
     griddep_launch_dependents();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int c = (int)blockIdx.x;
-    const int npass = p.passes_base + (c < p.passes_extra ? 1 : 0);
-    const int pass0 = c * p.passes_base + min(c, p.passes_extra);
+    const int e0 = c * p.slice, e1 = min(p.vocab, e0 + p.slice);  // the slice's entries [e0, e1)
+    const int npass = (e1 - e0 + kVsN - 1) / kVsN, tail_pass = (p.slice - 1) / kVsN;
     const int J = npass * p.atoms;  // ring stages of this CTA
-    const uint32_t stage_tx = (uint32_t)(kVsWBytes + (p.nt + p.nd) * 128);
 
     if (tid == 0) {
         prefetch_tensormap(&wmap);
+        prefetch_tensormap(&wtail);
         if (p.nt) prefetch_tensormap(&htmap);
         if (p.nd) prefetch_tensormap(&hdmap);
         if (WRITE && p.tma_store) prefetch_tensormap(&lmap);
@@ -236,8 +236,11 @@ __global__ void __launch_bounds__(kVsThreads, 1)
                 const int pp = j / p.atoms, a = j - pp * p.atoms;
                 uint8_t* sw = sbase + st * STAGE;
                 uint8_t* sh = sw + kVsWBytes;
-                mbar_arrive_expect_tx(&full[st], stage_tx);
-                tma_load_2d_hint(sw, &wmap, &full[st], a * kVsAtom, (pass0 + pp) * kVsN, pol);
+                // a slice's last pass has `tail` entries; the rest of its stage keeps older rows, whose columns of
+                // the accumulator nobody reads
+                const bool last = pp == tail_pass;
+                mbar_arrive_expect_tx(&full[st], (uint32_t)(((last ? p.tail : kVsN) + p.nt + p.nd) * 128));
+                tma_load_2d_hint(sw, last ? &wtail : &wmap, &full[st], a * kVsAtom, e0 + pp * kVsN, pol);
                 if (p.nt) tma_load_2d(sh, &htmap, &full[st], a * kVsAtom, p.ht0);
                 if (p.nd) tma_load_2d(sh + p.nt8 * 128, &hdmap, &full[st], a * kVsAtom, p.hd0);
                 issued = j + 1;
@@ -249,7 +252,8 @@ __global__ void __launch_bounds__(kVsThreads, 1)
     } else if (warp == kVsIssuer) {
         // ---- MMA issuer: pass pp accumulates into buffer pp % NB; half m of the states into its own 256 columns
         if (lane == 0) {
-            const uint32_t idesc = idesc_bf16_f32(kVsM, kVsN, false, false);
+            const uint32_t idesc_full = idesc_bf16_f32(kVsM, kVsN, false, false);
+            const uint32_t idesc_tail = idesc_bf16_f32(kVsM, (p.tail + 15) / 16 * 16, false, false);
             bool ok = true;
             int j = 0;
             for (int pp = 0; pp < npass && ok; ++pp) {
@@ -259,6 +263,7 @@ __global__ void __launch_bounds__(kVsThreads, 1)
                     break;
                 }
                 tc_fence_after();
+                const uint32_t idesc = pp == tail_pass ? idesc_tail : idesc_full;
                 const uint32_t dcol = tmem + (uint32_t)(b * MT * kVsN);
                 for (int a = 0; a < p.atoms; ++a, ++j) {
                     const int st = j % STG;
@@ -299,14 +304,14 @@ __global__ void __launch_bounds__(kVsThreads, 1)
             ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (pp / NB) & 1, kWaitBudget));
             if (!ok) break;
             tc_fence_after();
-            const int vb = (pass0 + pp) * kVsN + cb;  // entry of the warp's first column
+            const int vb = e0 + pp * kVsN + cb;  // entry of the warp's first column
 #pragma unroll 1
             for (int c0 = 0; c0 < CW; c0 += 64) {  // two chunks of 32 columns per wait
                 uint32_t r0[32], r1[32];
                 tmem_ld32(tq + (uint32_t)(b * MT * kVsN + c0), r0);
                 tmem_ld32(tq + (uint32_t)(b * MT * kVsN + c0 + 32), r1);
                 tmem_ld_wait();
-                const int v0 = vb + c0, n0 = min(32, p.vocab - v0), n1 = min(32, p.vocab - v0 - 32);
+                const int v0 = vb + c0, n0 = min(32, e1 - v0), n1 = min(32, e1 - v0 - 32);
                 if (n0 > 0) {
                     if (WRITE) store_chunk(stage, r0, lane, srow0, p, &lmap, v0, n0);
                     if (row >= 0) fold_chunk<GREEDY>(r0, n0, v0, p.c2, a0, a1);
@@ -386,8 +391,8 @@ __global__ void __launch_bounds__(256) lm_head_row_merge_kernel(const float2* __
 }
 
 template <bool GREEDY, int MT, bool WRITE>
-int vs_launch(const CUtensorMap& wmap, const CUtensorMap& htmap, const CUtensorMap& hdmap, const CUtensorMap& lmap,
-              const VsParams& p, int grid, const DeviceInfo& dev, cudaStream_t stream) {
+int vs_launch(const CUtensorMap& wmap, const CUtensorMap& wtail, const CUtensorMap& htmap, const CUtensorMap& hdmap,
+              const CUtensorMap& lmap, const VsParams& p, int grid, const DeviceInfo& dev, cudaStream_t stream) {
     static std::mutex cfg_mu;  // per instantiation (a template's own statics)
     static int configured[64] = {};
     const size_t smem = vs_smem_bytes<MT, WRITE>();
@@ -410,20 +415,21 @@ int vs_launch(const CUtensorMap& wmap, const CUtensorMap& htmap, const CUtensorM
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, lm_head_stream_kernel<GREEDY, MT, WRITE>, wmap, htmap, hdmap, lmap, p) ==
+    return cudaLaunchKernelEx(&cfg, lm_head_stream_kernel<GREEDY, MT, WRITE>, wmap, wtail, htmap, hdmap, lmap, p) ==
                    cudaSuccess
                ? BP_OK
                : BP_ERR_CUDA;
 }
 
 template <bool GREEDY>
-int vs_dispatch(int mt, bool write, const CUtensorMap& wmap, const CUtensorMap& htmap, const CUtensorMap& hdmap,
-                const CUtensorMap& lmap, const VsParams& p, int grid, const DeviceInfo& dev, cudaStream_t stream) {
+int vs_dispatch(int mt, bool write, const CUtensorMap& wmap, const CUtensorMap& wtail, const CUtensorMap& htmap,
+                const CUtensorMap& hdmap, const CUtensorMap& lmap, const VsParams& p, int grid, const DeviceInfo& dev,
+                cudaStream_t stream) {
     if (mt == 2)
-        return write ? vs_launch<GREEDY, 2, true>(wmap, htmap, hdmap, lmap, p, grid, dev, stream)
-                     : vs_launch<GREEDY, 2, false>(wmap, htmap, hdmap, lmap, p, grid, dev, stream);
-    return write ? vs_launch<GREEDY, 1, true>(wmap, htmap, hdmap, lmap, p, grid, dev, stream)
-                 : vs_launch<GREEDY, 1, false>(wmap, htmap, hdmap, lmap, p, grid, dev, stream);
+        return write ? vs_launch<GREEDY, 2, true>(wmap, wtail, htmap, hdmap, lmap, p, grid, dev, stream)
+                     : vs_launch<GREEDY, 2, false>(wmap, wtail, htmap, hdmap, lmap, p, grid, dev, stream);
+    return write ? vs_launch<GREEDY, 1, true>(wmap, wtail, htmap, hdmap, lmap, p, grid, dev, stream)
+                 : vs_launch<GREEDY, 1, false>(wmap, wtail, htmap, hdmap, lmap, p, grid, dev, stream);
 }
 
 int encode_rows(CUtensorMap* map, const void* base, int hidden, int rows, int box_rows) {
@@ -436,9 +442,16 @@ int encode_rows(CUtensorMap* map, const void* base, int hidden, int rows, int bo
 
 }  // namespace
 
+// Entries per CTA: equal shares of the vocabulary, in eights (the swizzle's rows).  Runs of whole passes left SMs idle at the end: of 151,936 entries 138 CTAs had 4 passes and 14 had 3
+// (8 x 16 rows, hidden 2560, T = 0: 122.2 -> 116.5 us), of 50,257 entries 45 had 2 and 107 had 1 (8 x 31 rows, T = 1:
+// 82.4 -> 77.0 us).
+static int verify_stream_slice(int vocab, int sm_count) {
+    const int ctas = min(min(sm_count, kVsMaxSlices), (vocab + kVsN - 1) / kVsN);
+    return ctas < 1 ? 0 : (int)(((long long)vocab + ctas * 8 - 1) / (ctas * 8) * 8);
+}
 int verify_stream_grid(int vocab, int sm_count) {
-    const int passes = (vocab + kVsN - 1) / kVsN;
-    return min(min(sm_count, kVsMaxSlices), passes);
+    const int slice = verify_stream_slice(vocab, sm_count);
+    return slice < 1 ? 0 : (vocab + slice - 1) / slice;
 }
 
 int launch_verify_stream(const VerifyEpilogueArgs& a, const VerifyStreamScratch& s, const DeviceInfo& dev,
@@ -451,14 +464,15 @@ int launch_verify_stream(const VerifyEpilogueArgs& a, const VerifyStreamScratch&
     const int grid = verify_stream_grid(a.vocab, dev.sm_count);
     if (grid < 1 || a.hidden % kVsAtom != 0) return BP_ERR_UNSUPPORTED;
 
-    const int passes = (a.vocab + kVsN - 1) / kVsN;
-    CUtensorMap wmap, htmap, hdmap, lmap;
-    if (encode_rows(&wmap, a.lm_head, a.hidden, a.vocab, kVsN) != BP_OK) return BP_ERR_CUDA;
+    CUtensorMap wmap, wtail, htmap, hdmap, lmap;
     VsParams p;
     p.vocab = a.vocab;
     p.atoms = a.hidden / kVsAtom;
-    p.passes_base = passes / grid;
-    p.passes_extra = passes % grid;
+    p.slice = verify_stream_slice(a.vocab, dev.sm_count);
+    p.tail = p.slice - (p.slice - 1) / kVsN * kVsN;
+    if (encode_rows(&wmap, a.lm_head, a.hidden, a.vocab, kVsN) != BP_OK ||
+        encode_rows(&wtail, a.lm_head, a.hidden, a.vocab, p.tail) != BP_OK)
+        return BP_ERR_CUDA;
     p.c2 = greedy ? 0.f : 1.4426950408889634f / a.temperature;
     p.logits = logits;
     // the path's own rows are padded to 16-byte boundaries where the workspace has the room (8 x 31 rows of a
@@ -501,8 +515,8 @@ int launch_verify_stream(const VerifyEpilogueArgs& a, const VerifyStreamScratch&
         const CUtensorMap& ht = p.nt ? htmap : wmap;  // an unused map slot holds any valid map
         const CUtensorMap& hd = p.nd ? hdmap : wmap;
         const CUtensorMap& lm = p.tma_store ? lmap : wmap;
-        const int rc = greedy ? vs_dispatch<true>(mt, write, wmap, ht, hd, lm, p, grid, dev, stream)
-                              : vs_dispatch<false>(mt, write, wmap, ht, hd, lm, p, grid, dev, stream);
+        const int rc = greedy ? vs_dispatch<true>(mt, write, wmap, wtail, ht, hd, lm, p, grid, dev, stream)
+                              : vs_dispatch<false>(mt, write, wmap, wtail, ht, hd, lm, p, grid, dev, stream);
         if (rc != BP_OK) return rc;
         r0 = r1;
     }

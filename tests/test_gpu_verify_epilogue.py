@@ -452,3 +452,15 @@ def test_33_to_64_rows_on_either_path(blocks, vocab):
     with pytest.raises(bp.BlockPilotError) as e:
         run_gpu(inp, 0.0, ws=bp.workspace(least, dev())[:-1])
     assert e.value.status == 4
+
+
+@pytest.mark.parametrize("vocab", [19459, 39000, 50257])
+@pytest.mark.parametrize("blocks", [(4,), (16, 16, 9)])
+def test_vocabulary_in_equal_shares(blocks, vocab):
+    """Shares of the vocabulary that are no whole tiles (resident kernel, few rows) or passes (streamed kernel): a last
+    tile or pass of 8 entries up, and a last CTA with less than a share."""
+    w = wl.custom(seed=vocab + len(blocks), ctx=(0,) * len(blocks), block=blocks, vocab=vocab)
+    for temp in (1.0, 0.0):
+        inp = wl.lm_head_inputs(w, temp, hidden=128)
+        compare(inp, temp, run_gpu(inp, temp, want_logits=True), run_oracle(inp, temp))
+        compare(inp, temp, run_gpu(inp, temp), run_oracle(inp, temp))
