@@ -442,11 +442,15 @@ int encode_rows(CUtensorMap* map, const void* base, int hidden, int rows, int bo
 
 }  // namespace
 
-// Entries per CTA: equal shares of the vocabulary, in eights (the swizzle's rows).  Runs of whole passes left SMs idle at the end: of 151,936 entries 138 CTAs had 4 passes and 14 had 3
-// (8 x 16 rows, hidden 2560, T = 0: 122.2 -> 116.5 us), of 50,257 entries 45 had 2 and 107 had 1 (8 x 31 rows, T = 1:
-// 82.4 -> 77.0 us).
+// Entries per CTA: equal shares of the vocabulary, in eights (the swizzle's rows).  Runs of whole passes left SMs idle
+// at the end: of 151,936 entries 138 CTAs had 4 passes and 14 had 3 (8 x 16 rows, hidden 2560, T = 0: 122.2 -> 116.5
+// us), of 50,257 entries 45 had 2 and 107 had 1 (8 x 31 rows, T = 1: 82.4 -> 77.0 us).  Shares are a pass at least
+// where that gives three quarters of the SMs one -- every CTA reads all states, so more CTAs cost L2 traffic (8 x 31
+// rows, T = 1, 32,000 entries: 125 CTAs 50.2, 152 CTAs 50.9 us; 28,000: 110 CTAs 47.7, 152 CTAs 45.5) -- and go down
+// to 64 entries below that (8,192: 32 CTAs 39.3, 128 CTAs 30.7 us).
 static int verify_stream_slice(int vocab, int sm_count) {
-    const int ctas = min(min(sm_count, kVsMaxSlices), (vocab + kVsN - 1) / kVsN);
+    const int sms = min(sm_count, kVsMaxSlices), passes = (vocab + kVsN - 1) / kVsN;
+    const int ctas = min(sms, 4 * passes > 3 * sms ? passes : (vocab + 63) / 64);
     return ctas < 1 ? 0 : (int)(((long long)vocab + ctas * 8 - 1) / (ctas * 8) * 8);
 }
 int verify_stream_grid(int vocab, int sm_count) {

@@ -454,7 +454,7 @@ def test_33_to_64_rows_on_either_path(blocks, vocab):
     assert e.value.status == 4
 
 
-@pytest.mark.parametrize("vocab", [19459, 39000, 50257])
+@pytest.mark.parametrize("vocab", [70, 19459, 32000, 39000, 50257])
 @pytest.mark.parametrize("blocks", [(4,), (16, 16, 9)])
 def test_vocabulary_in_equal_shares(blocks, vocab):
     """Shares of the vocabulary that are no whole tiles (resident kernel, few rows) or passes (streamed kernel): a last
