@@ -11,10 +11,10 @@
 //      streamed in passes of 256 entries and a last pass of what is left.  Per pass, its W rows (256 entries x 64 hidden columns per stage) and the states of
 //      up to 256 rows stream through a TMA ring; one thread issues M=128 (state rows) x N=256 (entries)
 //      x K=16 tcgen05 MMAs, one per 128-row half of the states.  Tensor-memory lane = state row, so each
-//      epilogue thread owns one row and folds the pass's 256 logits into its row's running (max, sum of
+//      epilogue thread owns part of one row's entries and folds their logits into a running (max, sum of
 //      2^(l*log2e/T - max)) -- at T = 0 its (max, lowest index) -- with one exponential per logit and no
-//      exchange between threads.  At T > 0 it also writes the logits once (each warp's 32 x 32 chunk
-//      staged in shared memory and sent by one TMA store): the draw at the first rejection needs a
+//      exchange between threads until the end.  At T > 0 it also writes the logits once (each warp's 32 x 16
+//      half chunk staged in shared memory and sent by one TMA store): the draw at the first rejection needs a
 //      whole row pair again, and no on-chip store can hold every row until the decisions are known.
 //      At T = 0 nothing but the statistics leaves the chip.  Each CTA writes its slice's statistics
 //      of every row.
@@ -44,9 +44,12 @@ constexpr int kVsWBytes = kVsN * 128;    // W of one stage: 256 entries x 128 by
 constexpr int kVsM = 128;                // state rows per half: the MMA M, tensor-memory lanes
 constexpr int kVsAtom = 64;              // hidden columns per 128-byte swizzle atom
 constexpr int kVsHBytes = kVsM * 128;    // states of one stage and half: 128 rows x 128 bytes
-constexpr int kVsThreads = 320;          // warps 0-7 epilogue, 8 TMA producer, 9 MMA issuer
-constexpr int kVsEpiWarps = 8;
-constexpr int kVsProducer = 8, kVsIssuer = 9;
+// Warps 0-15 epilogue, 16 TMA producer, 17 MMA issuer.  Sixteen epilogue warps with 2 KB of staging each hide one
+// another's waits for tensor memory and for the stores' reads a little better than eight with 4 KB (hidden 2560,
+// 151,936 entries, T = 1: 248 rows 183.1 -> 181.4 us, 62 rows 145.1 -> 143.8).
+constexpr int kVsThreads = 576;
+constexpr int kVsEpiWarps = 16;
+constexpr int kVsProducer = 16, kVsIssuer = 17;
 constexpr int kVsMaxSlices = 160;        // slices (CTAs) per row in the statistics array
 
 // MT halves of 128 state rows.  Tensor memory (512 columns) holds two passes' accumulators with one
@@ -55,10 +58,11 @@ constexpr int kVsMaxSlices = 160;        // slices (CTAs) per row in the statist
 // fills then ask more of shared memory per entry than it serves: measured slower.)  Stages
 // of W and states together: 4 x 48 KB with one half, 3 x 64 KB with two; then the store staging.
 __host__ __device__ constexpr int vs_stages(int MT) { return MT == 2 ? 3 : 4; }
-constexpr int kVsStageBytes = 32 * 128;  // per epilogue warp: one chunk of 32 rows x 32 fp32 logits
+// Per epilogue warp: half a chunk of logits (32 rows x 16) where they are written, and at the end its rows' statistics.
+__host__ __device__ constexpr int vs_warp_bytes(bool write) { return write ? 32 * 64 : 32 * (int)sizeof(float2); }
 template <int MT, bool WRITE>
 constexpr size_t vs_smem_bytes() {
-    return 1024 + (size_t)vs_stages(MT) * (kVsWBytes + MT * kVsHBytes) + (WRITE ? kVsEpiWarps * kVsStageBytes : 0);
+    return 1024 + (size_t)vs_stages(MT) * (kVsWBytes + MT * kVsHBytes) + kVsEpiWarps * vs_warp_bytes(WRITE);
 }
 
 struct VsParams {
@@ -124,25 +128,25 @@ __device__ __forceinline__ void fold_chunk(const uint32_t (&r)[32], int n, int v
     }
 }
 
-// The warp's 32 rows x 32 entries of one chunk written to the logits.  Each lane puts its row into the
-// warp's 4 KB staging buffer, 16-byte chunk i of row l at chunk i ^ (l & 7) -- the 128-byte swizzle of
-// a TMA box of 32 rows x 32 fp32, and a layout in which neither row-wise writes nor column-wise reads
+// Half a chunk, the warp's 32 rows x 16 entries, written to the logits.  Each lane puts its row into the
+// warp's 2 KB staging buffer, 16-byte chunk i of row l at chunk i ^ ((l >> 1) & 3) -- the 64-byte swizzle of
+// a TMA box of 32 rows x 16 fp32, and a layout in which neither row-wise writes nor column-wise reads
 // conflict.  Where the group's rows are contiguous stacked rows (lmap: the group's rows of the logits),
-// one TMA store sends the box and the warp goes on (it waits only, before the next chunk, until the
-// copy has read the buffer); otherwise every store instruction covers whole 128-byte rows: four rows
-// per 16-byte store, one per 4-byte store where rows are not 16-byte aligned.  srow0: the state-tile
+// one TMA store sends the box and the warp goes on (it waits only, before the next half, until the
+// copy has read the buffer); otherwise every store instruction covers whole 64-byte pieces of rows: eight rows
+// per 16-byte store, two per 4-byte store where rows are not 16-byte aligned.  srow0: the state-tile
 // row of lane 0; n valid entries from v0.  Warp-collective.
-__device__ __forceinline__ void store_chunk(uint8_t* stage, const uint32_t (&r)[32], int lane, int srow0,
-                                            const VsParams& p, const CUtensorMap* lmap, int v0, int n) {
+__device__ __forceinline__ void store_half(uint8_t* stage, const uint32_t* r, int lane, int srow0, const VsParams& p,
+                                           const CUtensorMap* lmap, int v0, int n) {
     if (p.tma_store) {
-        if (lane == 0) bulk_wait_group_read<0>();  // the previous chunk's copy has read the buffer
+        if (lane == 0) bulk_wait_group_read<0>();  // the previous half's copy has read the buffer
         __syncwarp();
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-        *reinterpret_cast<uint4*>(stage + lane * 128 + ((i ^ (lane & 7)) << 4)) =
+    for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<uint4*>(stage + lane * 64 + ((i ^ ((lane >> 1) & 3)) << 4)) =
             make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
-    if (p.tma_store && n == 32) {
+    if (p.tma_store && n == 16) {
         fence_proxy_async_smem();  // the copy reads the buffer through the async proxy
         __syncwarp();
         if (lane == 0 && srow0 < p.grows) {  // rows past the group: clipped
@@ -152,25 +156,27 @@ __device__ __forceinline__ void store_chunk(uint8_t* stage, const uint32_t (&r)[
         return;
     }
     __syncwarp();
-    if (p.vec && n == 32) {
-        const int c = lane & 7;
+    if (p.vec && n == 16) {
+        const int c = lane & 3;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int j = 4 * k + (lane >> 3);
+        for (int k = 0; k < 4; ++k) {
+            const int j = 8 * k + (lane >> 2);
             const int row = stacked_row(p, srow0 + j);
-            const float4 x = *reinterpret_cast<const float4*>(stage + j * 128 + ((c ^ (j & 7)) << 4));
+            const float4 x = *reinterpret_cast<const float4*>(stage + j * 64 + ((c ^ ((j >> 1) & 3)) << 4));
             if (row >= 0) __stcs(reinterpret_cast<float4*>(p.logits + (size_t)row * p.ld + v0) + c, x);
         }
     } else {
+        const int e = lane & 15;
 #pragma unroll 4
-        for (int j = 0; j < 32; ++j) {
+        for (int k = 0; k < 16; ++k) {
+            const int j = 2 * k + (lane >> 4);
             const int row = stacked_row(p, srow0 + j);
             const float x =
-                *reinterpret_cast<const float*>(stage + j * 128 + (((lane >> 2) ^ (j & 7)) << 4) + ((lane & 3) << 2));
-            if (row >= 0 && lane < n) __stcs(p.logits + (size_t)row * p.ld + v0 + lane, x);
+                *reinterpret_cast<const float*>(stage + j * 64 + (((e >> 2) ^ ((j >> 1) & 3)) << 4) + ((e & 3) << 2));
+            if (row >= 0 && e < n) __stcs(p.logits + (size_t)row * p.ld + v0 + e, x);
         }
     }
-    __syncwarp();  // the buffer is free for the next chunk
+    __syncwarp();  // the buffer is free for the next half
 }
 
 template <bool GREEDY, int MT, bool WRITE>
@@ -181,12 +187,11 @@ __global__ void __launch_bounds__(kVsThreads, 1)
     constexpr int STG = vs_stages(MT);
     constexpr int NB = 2 / MT;                     // accumulator buffers of MT x 256 columns
     constexpr int STAGE = kVsWBytes + MT * kVsHBytes;
-    constexpr int CW = MT == 2 ? kVsN : kVsN / 2;  // columns (entries) per epilogue warp and pass
+    constexpr int PARTS = 4 / MT, CW = kVsN / PARTS;  // column parts of a half's epilogue; columns of a warp per pass
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sbase = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ uint64_t full[STG], empty[STG], acc_full[NB], acc_empty[NB], mma_done;
     __shared__ uint32_t tmem_sh;
-    __shared__ float2 half_sh[kVsM];              // MT = 1: the second column half's statistics per row
 
     griddep_launch_dependents();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -290,14 +295,13 @@ __global__ void __launch_bounds__(kVsThreads, 1)
         }
     } else {
         // ---- epilogue: thread = state row (tensor-memory lane); warp w reads lane quarter w % 4 of half
-        // w / 4 (MT = 2: all 256 columns of a pass) or of the only half (MT = 1: column half w / 4)
-        const int q = warp & 3, h = warp >> 2;
-        const int m = MT == 2 ? h : 0, cb = MT == 2 ? 0 : h * CW;
+        // (w / 4) % MT, and of its columns part w / (4 MT)
+        const int q = warp & 3, m = (warp >> 2) % MT, part = (warp >> 2) / MT, cb = part * CW;
         const int srow0 = m * kVsM + q * 32;  // state-tile row of lane 0
         const int row = stacked_row(p, srow0 + lane);
         float a0 = -INFINITY, a1 = GREEDY ? __int_as_float(INT_MAX) : 0.f;
         const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(m * kVsN + cb);
-        uint8_t* stage = sbase + STG * STAGE + warp * kVsStageBytes;  // WRITE only
+        uint8_t* stage = sbase + STG * STAGE + warp * vs_warp_bytes(WRITE);
         bool ok = true;
         for (int pp = 0; pp < npass; ++pp) {
             const int b = pp % NB;
@@ -306,20 +310,15 @@ __global__ void __launch_bounds__(kVsThreads, 1)
             tc_fence_after();
             const int vb = e0 + pp * kVsN + cb;  // entry of the warp's first column
 #pragma unroll 1
-            for (int c0 = 0; c0 < CW; c0 += 64) {  // two chunks of 32 columns per wait
-                uint32_t r0[32], r1[32];
-                tmem_ld32(tq + (uint32_t)(b * MT * kVsN + c0), r0);
-                tmem_ld32(tq + (uint32_t)(b * MT * kVsN + c0 + 32), r1);
+            for (int c0 = 0; c0 < CW; c0 += 32) {
+                const int v0 = vb + c0, n = min(32, e1 - v0);
+                if (n <= 0) break;
+                uint32_t r[32];
+                tmem_ld32(tq + (uint32_t)(b * MT * kVsN + c0), r);
                 tmem_ld_wait();
-                const int v0 = vb + c0, n0 = min(32, e1 - v0), n1 = min(32, e1 - v0 - 32);
-                if (n0 > 0) {
-                    if (WRITE) store_chunk(stage, r0, lane, srow0, p, &lmap, v0, n0);
-                    if (row >= 0) fold_chunk<GREEDY>(r0, n0, v0, p.c2, a0, a1);
-                }
-                if (n1 > 0) {
-                    if (WRITE) store_chunk(stage, r1, lane, srow0, p, &lmap, v0 + 32, n1);
-                    if (row >= 0) fold_chunk<GREEDY>(r1, n1, v0 + 32, p.c2, a0, a1);
-                }
+                if (WRITE) store_half(stage, r, lane, srow0, p, &lmap, v0, min(n, 16));
+                if (row >= 0) fold_chunk<GREEDY>(r, n, v0, p.c2, a0, a1);
+                if (WRITE && n > 16) store_half(stage, r + 16, lane, srow0, p, &lmap, v0 + 16, n - 16);
             }
             tc_fence_before();
             __syncwarp();
@@ -327,11 +326,14 @@ __global__ void __launch_bounds__(kVsThreads, 1)
         }
         if (WRITE && p.tma_store && lane == 0) bulk_wait_group<0>();  // this warp's logits are written
         if (!ok && lane == 0) raise_error(p.err, kErrTimeout);
-        if (MT == 1) {  // the two column halves of a row, merged in entry order
-            if (h == 1) half_sh[q * 32 + lane] = make_float2(a0, a1);
-            named_barrier_sync(1, kVsEpiWarps * 32);
-            if (h == 0) {
-                const float2 o = half_sh[q * 32 + lane];
+        // the column parts of a row, merged in entry order
+        __syncwarp();
+        reinterpret_cast<float2*>(stage)[lane] = make_float2(a0, a1);
+        named_barrier_sync(1, kVsEpiWarps * 32);
+        if (part == 0 && row >= 0) {
+#pragma unroll
+            for (int k = 1; k < PARTS; ++k) {
+                const float2 o = reinterpret_cast<const float2*>(stage + k * 4 * MT * vs_warp_bytes(WRITE))[lane];
                 if (GREEDY) {
                     int bi = __float_as_int(a1);
                     amax_merge(a0, bi, o.x, __float_as_int(o.y));
@@ -340,8 +342,8 @@ __global__ void __launch_bounds__(kVsThreads, 1)
                     lse_merge(a0, a1, o.x, o.y);
                 }
             }
+            p.part[(size_t)row * p.nslices + c] = make_float2(a0, a1);
         }
-        if (row >= 0 && (MT == 2 || h == 0)) p.part[(size_t)row * p.nslices + c] = make_float2(a0, a1);
     }
 
     // ---- release tensor memory
@@ -511,9 +513,9 @@ int launch_verify_stream(const VerifyEpilogueArgs& a, const VerifyStreamScratch&
         if (p.tma_store) {
             const cuuint64_t dims[2] = {(cuuint64_t)a.vocab, (cuuint64_t)(r1 - r0)};
             const cuuint64_t strides[1] = {(cuuint64_t)ld * 4};
-            const cuuint32_t box[2] = {32, 32};
+            const cuuint32_t box[2] = {16, 32};
             if (encode_tensor_map(&lmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, logits + (size_t)r0 * ld, dims,
-                                  strides, box, CU_TENSOR_MAP_SWIZZLE_128B) != BP_OK)
+                                  strides, box, CU_TENSOR_MAP_SWIZZLE_64B) != BP_OK)
                 return BP_ERR_CUDA;
         }
         const CUtensorMap& ht = p.nt ? htmap : wmap;  // an unused map slot holds any valid map
