@@ -101,6 +101,7 @@ typedef enum { BP_F32 = 0, BP_BF16 = 1 } bp_dtype;
  *   softmax_scale  0 selects 1/sqrt(head_dim)
  * Limits: 1 <= num_kv_heads, num_q_heads % num_kv_heads == 0, max_q_len <= 64,
  * max_q_len <= max_kv_len.  Every key row must be finite (bf16 or fp32 values).
+ * A workspace of 256 bytes is accepted too: keys are then split over clusters only, merged on chip.
  * ------------------------------------------------------------------------------- */
 BP_API size_t bp_block_attention_workspace_size(int num_seqs, int max_q_len, int num_q_heads, int num_kv_heads,
                                          int head_dim);
@@ -233,7 +234,8 @@ BP_API int bp_spec_accept_noalloc(const float* target_logits, const float* draft
  * Limits: d_in % 8 == 0 and 16-byte aligned rows for bf16 (d_in % 4 == 0 for fp32),
  * num_cand <= 64.  Any d_in: wide inputs (such as the V-sized logit vector of Section 3.1) are
  * streamed; the workspace then also holds the gathered bf16 rows (num_reqs rounded up to 64) x d_in,
- * which is why its size depends on d_in.
+ * which is why its size depends on d_in, and the partial products of W1 rows whose d_in is cut between
+ * SMs.  A workspace without the latter is accepted: clusters then split d_in, which is slower on long rows.
  * ------------------------------------------------------------------------------- */
 BP_API size_t bp_policy_select_workspace_size(int num_reqs, int d_in, int hidden, int num_cand);
 BP_API int bp_policy_select(const void* feats, int64_t feat_row_stride, const int32_t* row_index, int num_reqs, int d_in,
@@ -243,9 +245,9 @@ BP_API int bp_policy_select(const void* feats, int64_t feat_row_stride, const in
 
 /* ---------------------------------------------------------------------------------
  * Verify epilogue: the LM-head projection of the final hidden states fused with the lossless
- * acceptance of bp_spec_accept; up to 32 rows (and at T = 0) without writing the logits to memory.  Section 2.1 and the
- * Figure 1 caption: the target scores every position of the drafted block in one pass and
- * keeps the longest accepted prefix; the distributions it compares are
+ * acceptance of bp_spec_accept; up to 32 rows (and at T = 0) without writing the logits to
+ * memory.  Section 2.1 and the Figure 1 caption: the target scores every position of the drafted
+ * block in one pass and keeps the longest accepted prefix; the distributions it compares are
  *
  *   p_i = softmax(W h_target_i / T),  q_i = softmax(W h_draft_i / T)
  *
@@ -266,8 +268,8 @@ BP_API int bp_policy_select(const void* feats, int64_t feat_row_stride, const in
  *   rows <= 32 at T > 0 (and up to 64 in a workspace without the room below): one cooperative launch of one
  *     CTA per SM keeps every logit in tensor memory; the logits never reach memory unless logits_out asks
  *     for them (then for testing: it adds the write traffic the fusion exists to avoid).
- *   more rows, and T = 0: the LM head is streamed in 256-entry passes, groups of at most 256 rows per pass
- *     over W, and every row's statistics are formed in the projection's epilogue.  At T = 0 only the
+ *   more rows, and T = 0: the LM head is streamed in passes of up to 256 entries, groups of at most 256 rows
+ *     per pass over W, and every row's statistics are formed in the projection's epilogue.  At T = 0 only the
  *     statistics leave the chip.  At T > 0 the logits are written once (into logits_out if given, else into
  *     the workspace) and only the draw's row pair of each sequence and the logits at the drafted tokens are
  *     read back.  Any vocabulary beyond 64 rows; W is read once per group of 256 rows.

@@ -11,9 +11,12 @@
 //     share of 128-key K/V tiles through a 3-stage TMA ring (SWIZZLE_128B), computes
 //     S = Q K^T into tensor memory, runs an online softmax (fp32, exp2 domain, lazy
 //     rescale of the TMEM accumulator when the row max grows by more than 2^8),
-//     writes P (bf16) back into tensor memory and accumulates O += P V with P as the
-//     TMEM A operand.  The CS partial results are merged through distributed shared
-//     memory -- no global scratch, one launch.
+//     writes P (bf16) back into tensor memory (three S/P buffers) and accumulates O += P V
+//     with P as the TMEM A operand.  Every CTA scales its partial result and pushes each row to
+//     the CTA that owns it, which adds them up: through distributed shared memory, or, where a
+//     CTA owns few rows (wide clusters) and the workspace has the room, through L2.
+//   * The flat split (below) cuts the tiles of all units evenly over the CTAs instead; a second
+//     kernel merges the units that were cut.
 //   * Units are issued longest-first so that ragged batches finish together.
 //   Warp roles: warp 0 = TMA producer + TMEM allocator, warp 1 = MMA issuer,
 //   warps 2..5 = softmax / epilogue (one query row per thread, TMEM lane = row).  Units of at

@@ -1,11 +1,11 @@
 // Block-size policy head (Sections 2.3-2.4 of the BlockPilot paper): once per request,
 //   h = max(0, W1 x + b1),  o = W2 h + b2,  block size = candidates[argmax o].
 //
-// bf16 weights -- tensor cores (sm_103a), one launch:
+// bf16 weights -- tensor cores (sm_103a).  Inputs of up to 8 atoms per CTA, one launch (policy_tc_kernel):
 //   * W1 [hidden x d_in] is cut into 128-row tiles; a thread-block cluster of KS CTAs splits one
 //     tile's d_in into 64-column swizzle atoms.  Each CTA brings its W1 atoms in with TMA
 //     (SWIZZLE_128B), gathers the requests' pooled rows x (row_index) into the matching
-//     K-major layout, and one thread issues M=128 x N=requests tcgen05 MMAs (bf16 in, fp32
+//     K-major layout, and four threads issue M=128 x N=requests tcgen05 MMAs (bf16 in, fp32
 //     accumulated in tensor memory): W1 is read from HBM exactly once for up to 64 requests.
 //   * The KS partial tiles are summed through distributed shared memory; each CTA takes a
 //     share of the rows, adds b1 and applies ReLU, and folds its rows of h straight into the
@@ -13,6 +13,9 @@
 //   * The cluster's output-layer partials go to the workspace; the last tile to finish (an
 //     atomic ticket, no waiting) adds them in tile order with b2 and takes the argmax (lowest
 //     index on ties).  Every sum runs in a fixed order: the result is deterministic.
+// Wider inputs stream W1 and x through a TMA ring: in the same kernel with one issuing thread, or, where a CTA's share
+// is long (policy_flat_kernel), with the atoms of all tiles cut evenly over the SMs.  Pooled rows that row_index picks
+// are first gathered into contiguous rows; without row_index the features are read in place.
 // fp32 weights -- CUDA cores: register-tiled products with d_in split over a cluster, then (one CTA per
 // request) the output layer and the argmax.
 // bf16 shapes outside the tensor-core limits -- CUDA cores: a kernel that streams W1 once for a group of up
