@@ -1458,16 +1458,23 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
     }
     if (cs > 1 && max_tiles - best < 3) cs = 1;
 
+    // AHEAD: a CTA's bandwidth is what it keeps in flight; where SMs are idle and each CTA streams a long run,
+    // refilling K's stages early took 8 x 32784 keys (128 CTAs of 129 tiles) from 163.9 to 153.6 us, 16 x 4112 (128
+    // of 33) from 48.8 to 46.5, 3 x 8208 (clusters of 5, 13 tiles a CTA) from 25.7 to 24.7.  With nearly every SM
+    // streaming, HBM is the bound and the freer order of requests costs more than it hides (144 CTAs: 18 x 16400
+    // keys 178.3 without, 187.8 with; pages of 64 94.8 and 94.0); it loses too in wide clusters (1 x 65552: 54.5
+    // and 55.3), on short runs (4 tiles: 13.2 and 13.4) and with 16-key pages (8 x 32784: 246 and 260).
+    const auto ahead_for = [&](int c) {
+        const long long ctas = units * c;
+        return (paged ? a.page_size >= 32 && ctas < dev.sm_count : ctas * 10 <= 9LL * dev.sm_count) && c <= 5 &&
+               max_tiles >= 12 * c;
+    };
+
     // flat split: the tiles of every sequence's query tiles cut evenly over groups of CTAs, one CTA per KV
     // head and per SM (at most kAttnFlatMaxGrid in all, and no more groups than one head has tiles); units
     // cut between groups are merged by a second kernel.  It needs the Q tile by TMA, the sequences'
-    // offsets in shared memory and the workspace's partial slots and work entries.  Measured on this GPU,
-    // it gains where the cluster split leaves SMs idle while every CTA of the flat split streams a long
-    // run (8 x 32K keys: 170 vs 175 us), and where the cluster split needs three or more waves (64 x 528
-    // keys: 46 vs 50 us); elsewhere the second kernel and the stretch boundaries cost more than the idle
-    // SMs (1 x 2K keys: 13.8 vs 9.3 us; 16 x 4K: 60 vs 52 us; the ragged 32: 109 vs 100 us).
-    // BP_ATTENTION_SPLIT=flat or =cluster overrides the choice, =cluster:N also the cluster size (for tests
-    // and measurements).
+    // offsets in shared memory and the workspace's partial slots and work entries.  BP_ATTENTION_SPLIT=flat or
+    // =cluster overrides the choice, =cluster:N also the cluster size (for tests and measurements).
     const long long tiles_bound = (long long)a.num_seqs * m_tiles * max_tiles;
     const int ngroups = (int)std::min<long long>(std::min(dev.sm_count, kAttnFlatMaxGrid) / a.num_kv_heads,
                                                  tiles_bound);
@@ -1475,17 +1482,31 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
     const bool flat_ok = q_tma && a.num_seqs <= kMaxOrderedSeqs && a.scratch != nullptr &&
                          a.scratch_bytes >= attention_flat_scratch_bytes(a.max_q_len, G) && ngroups >= 1;
     const long long cluster_ctas = units * cs;
-    // and where whole units per CTA leave the longest one far above the average: a CTA streams a tile in about
-    // 1.35 us, 152 of them together at HBM's rate one each 1.48 us, and the flat split adds about 4.2 us for
-    // each stretch of a CTA and 8 us for the second kernel.  20 sequences of 339-5425 keys (longest unit 38
-    // tiles, 19.7 on average): 49.3 against 52.6 us; 25 of up to 10412 (73, 49.3): 90.8 against 96.5 us; the
-    // ragged 32 (62, 54.3): 99 against 89 us.
     const double avg_tiles = (double)a.num_kv_heads * m_tiles * ((double)a.total_kv / kTileN + 0.5 * a.num_seqs) /
                              dev.sm_count;
-    const bool uneven = cs == 1 && flat_ok &&
-                        1.35 * max_tiles > 1.48 * avg_tiles + 4.2 * (1.0 + (double)a.num_seqs / ngroups) + 8.0;
-    bool flat = flat_ok && ((cluster_ctas * 10 <= 9LL * dev.sm_count && tiles_bound >= 64LL * ngroups) ||
-                            cluster_ctas >= 3LL * dev.sm_count || uneven);
+    const double flat_stretches = 4.2 * (1.0 + (double)a.num_seqs / (ngroups > 0 ? ngroups : 1));
+    bool flat;
+    if (cluster_ctas <= dev.sm_count) {
+        // One wave of clusters: the smaller of two estimates (us), fitted to 70 shapes of 1-18 sequences of 2-160K
+        // keys in both splits.  Where they differ by more than 2 % the choice is the faster one, both ways: flat
+        // for 1 x 65552 keys (50.5 against 54.5 us), 7 x 32784 (145 against 151), 10 x 16400 (110 against 146);
+        // clusters for 8 x 32784 (153.6 against 163), 16 x 16400 (152 against 168), 5 x 8208 (34.4 against 38.4).
+        // us per key tile of a CTA: AHEAD, clusters of up to 5, wider clusters, flat (all SMs together then)
+        const double big[4] = {1.10, 1.32, 1.41, 1.39}, p32[4] = {1.26, 1.37, 1.62, 1.45},
+                     p16[4] = {1.83, 1.83, 2.42, 1.70};
+        const double* us = paged && a.page_size < 64 ? (a.page_size < 32 ? p16 : p32) : big;
+        const double est_cluster = us[ahead_for(cs) ? 0 : cs <= 5 ? 1 : 2] * ((max_tiles + cs - 1) / cs) +
+                                   (cs == 1 ? 7.0 : cs <= 5 ? 10.0 : 8.0);
+        flat = flat_ok && us[3] * avg_tiles + flat_stretches + 10.0 < est_cluster;
+    } else {
+        // Several waves of whole units: flat from three waves on (64 x 528 keys: 42.7 against 47.7 us), and where
+        // the longest unit is far above the average.  A CTA streams a tile in about 1.35 us, 152 of them together
+        // at HBM's rate one each 1.48 us: 20 sequences of 339-5425 keys (longest unit 38 tiles, 19.7 on average)
+        // 49.0 against 52.6 us, 25 of up to 10412 (73, 49.3) 90.8 against 97.3; the ragged 32 (62, 54.3) stay in
+        // clusters, 89.8 against 99.1.
+        flat = flat_ok && (cluster_ctas >= 3LL * dev.sm_count ||
+                           1.35 * max_tiles > 1.48 * avg_tiles + flat_stretches + 8.0);
+    }
     if (const char* force = getenv("BP_ATTENTION_SPLIT")) {
         if (strcmp(force, "flat") == 0) {
             flat = flat_ok;
@@ -1523,19 +1544,13 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
         a.scratch_bytes >= attention_flat_scratch_bytes(a.max_q_len, G))
         p.part = static_cast<float*>(a.scratch);
     p.early_release = units <= max_active[cs] && units * cs <= dev.sm_count;  // one wave
-    // A CTA's bandwidth is what it keeps in flight; where SMs are idle and each CTA streams a long run, refilling
-    // K's stages early (AHEAD) took 16 x 4112 keys (128 CTAs of 33 tiles) from 47.4 to 44.9 us and 4 x 8208
-    // (clusters of 4, 17 tiles a CTA) from 29.9 to 28.9 us.  With every SM streaming, HBM is the bound and the
-    // freer order of requests costs more than it hides (the ragged 32 lost 2 us); on short runs (4 tiles: 13.4
-    // against 13.2 us) and in wide clusters (1 x 32784 keys: 31.7 against 30.9 us) it loses too.
-    const bool ahead = units * cs < dev.sm_count && cs <= 4 && max_tiles >= 16 * cs;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cs;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    e = cudaLaunchKernelEx(&cfg, kAttnKernels[4 * ahead + 2 * spread + paged], qmap, kmap, vmap, p);
+    e = cudaLaunchKernelEx(&cfg, kAttnKernels[4 * ahead_for(cs) + 2 * spread + paged], qmap, kmap, vmap, p);
     if (e != cudaSuccess) return BP_ERR_CUDA;
     return BP_OK;
 }

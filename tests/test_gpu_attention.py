@@ -112,6 +112,17 @@ def test_split_choice():
     assert err <= ATTN_TOL and lerr <= LSE_TOL
 
 
+@pytest.mark.parametrize("n, ctx, flat", [(1, 70000, True), (10, 9000, True), (8, 12000, False), (9, 5000, False)])
+def test_split_of_one_wave(n, ctx, flat):
+    """One wave of clusters against the flat split, by the library's estimates: wide clusters or few SMs on long
+    runs go flat, nearly full grids stay in clusters (128 CTAs: K's ring ahead; 144: not)."""
+    a = wl.attention_inputs(wl.custom(seed=n, ctx=(ctx,) * n, block=(16,) * n, num_q_heads=32, num_kv_heads=8))
+    _attn_kernels(a, "auto")
+    assert any("attn_combine_kernel" in x for x in _attn_kernels(a, "auto")) == flat
+    err, lerr = attention_errors(*run_attention(a, CAUSAL), a, CAUSAL, [n // 2])
+    assert err <= ATTN_TOL and lerr <= LSE_TOL
+
+
 def test_qwen3_4b_full():
     a = wl.attention_inputs(wl.get("qwen3_4b"))
     _check(a, CAUSAL)
