@@ -78,7 +78,7 @@ struct AttnParams {
     float* part;
     int4* work;
     int slot_rows;
-    int early_release;  // the grid runs in one wave: dependents may launch as soon as every CTA has started
+    int early_release;  // the grid is one wave of short runs: dependents may launch as soon as every CTA has started
     unsigned int* err;
 };
 constexpr int kMaxSub = kTileN / 16;  // sub-boxes per K/V tile at the smallest page size (16 keys)
@@ -920,8 +920,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     tc_fence_after();
     if (warp == 1) tmem_dealloc(tmem, kTmemCols);
-    // A grid of one wave lets its dependents launch from its start (their prologues overlap it: batch-1
-    // calls back to back, 9.25 against 9.87 us each); otherwise they launch once every CTA is here or has
+    // A grid of one wave of short runs lets its dependents launch from its start (their prologues overlap it:
+    // batch-1 calls back to back, 9.25 against 9.87 us each); otherwise they launch once every CTA is here or has
     // left.  Released at the start, a grid of two waves followed by the acceptance's statistics (thousands
     // of CTAs, chained by programmatic launch) made a step of the ragged batch take 720-820 us instead of
     // 195, and the flat split's step took 206.8 us instead of 200.3.
@@ -1543,7 +1543,11 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
         a.scratch != nullptr &&
         a.scratch_bytes >= attention_flat_scratch_bytes(a.max_q_len, G))
         p.part = static_cast<float*>(a.scratch);
-    p.early_release = units <= max_active[cs] && units * cs <= dev.sm_count;  // one wave
+    // one wave of short runs: dependents start their prologues at once.  Behind a long run an early acceptance waits
+    // on the SMs for nothing and its thousands of CTAs start worse for it: 8 x 32784 keys (129 tiles a CTA) with
+    // the T = 1 acceptance took 194.2 us a step released at the start and 189.7 at the end; alone, 33 tiles a CTA
+    // take 44.8 us either way, 17 tiles 28.0 and 28.4
+    p.early_release = units <= max_active[cs] && units * cs <= dev.sm_count && max_tiles < 24 * cs;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cs;
     attr[0].val.clusterDim.y = 1;
