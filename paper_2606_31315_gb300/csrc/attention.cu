@@ -1484,29 +1484,40 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
     const long long cluster_ctas = units * cs;
     const double avg_tiles = (double)a.num_kv_heads * m_tiles * ((double)a.total_kv / kTileN + 0.5 * a.num_seqs) /
                              dev.sm_count;
-    const double flat_stretches = 4.2 * (1.0 + (double)a.num_seqs / (ngroups > 0 ? ngroups : 1));
-    bool flat;
+    // Estimates (us) of both splits, fitted to 100 shapes timed in both (1-128 sequences of 200-160K keys).
+    // us per key tile of a CTA: AHEAD, clusters of up to 5, wider clusters, flat (all SMs together then)
+    const double big[4] = {1.10, 1.32, 1.41, 1.39}, p32[4] = {1.26, 1.37, 1.62, 1.45}, p16[4] = {1.83, 1.83, 2.42, 1.70};
+    const double* us = paged && a.page_size < 64 ? (a.page_size < 32 ? p16 : p32) : big;
+    // A sequence's query tiles read the same K and V, which its units of one wave share in L2 (16 x 4112 keys, blocks
+    // of 40 -- two tiles: clusters 79.2, flat 103.5 us; 12: 77.9 and 70.9).
+    const bool shared = m_tiles > 1;
+    double est_flat = (shared ? 1.2 : 1.0) * us[3] * avg_tiles + 10.0 + std::min(4.2 * (1.0 + (double)a.num_seqs / std::max(ngroups, 1)), 11.0);
+    double est_cluster;
     if (cluster_ctas <= dev.sm_count) {
-        // One wave of clusters: the smaller of two estimates (us), fitted to 70 shapes of 1-18 sequences of 2-160K
-        // keys in both splits.  Where they differ by more than 2 % the choice is the faster one, both ways: flat
-        // for 1 x 65552 keys (50.5 against 54.5 us), 7 x 32784 (145 against 151), 10 x 16400 (110 against 146);
-        // clusters for 8 x 32784 (153.6 against 163), 16 x 16400 (152 against 168), 5 x 8208 (34.4 against 38.4).
-        // us per key tile of a CTA: AHEAD, clusters of up to 5, wider clusters, flat (all SMs together then)
-        const double big[4] = {1.10, 1.32, 1.41, 1.39}, p32[4] = {1.26, 1.37, 1.62, 1.45},
-                     p16[4] = {1.83, 1.83, 2.42, 1.70};
-        const double* us = paged && a.page_size < 64 ? (a.page_size < 32 ? p16 : p32) : big;
-        const double est_cluster = us[ahead_for(cs) ? 0 : cs <= 5 ? 1 : 2] * ((max_tiles + cs - 1) / cs) +
-                                   (cs == 1 ? 7.0 : cs <= 5 ? 10.0 : 8.0);
-        flat = flat_ok && us[3] * avg_tiles + flat_stretches + 10.0 < est_cluster;
+        // One wave.  Flat for 1 x 65552 keys (50.5 against 54.5 us), 7 x 32784 (145 against 151), 10 x 16400 (110
+        // against 146); clusters for 8 x 32784 (153.6 against 163), 16 x 16400 (152 against 168), 5 x 8208 (34.4
+        // against 38.4).
+        est_cluster = us[ahead_for(cs) ? 0 : cs <= 5 ? 1 : 2] * ((max_tiles + cs - 1) / cs) +
+                      (cs == 1 ? 7.0 : cs <= 5 ? 10.0 : 8.0);
     } else {
-        // Several waves of whole units: flat from three waves on (64 x 528 keys: 42.7 against 47.7 us), and where
-        // the longest unit is far above the average.  A CTA streams a tile in about 1.35 us, 152 of them together
-        // at HBM's rate one each 1.48 us: 20 sequences of 339-5425 keys (longest unit 38 tiles, 19.7 on average)
-        // 49.0 against 52.6 us, 25 of up to 10412 (73, 49.3) 90.8 against 97.3; the ragged 32 (62, 54.3) stay in
-        // clusters, 89.8 against 99.1.
-        flat = flat_ok && (cluster_ctas >= 3LL * dev.sm_count ||
-                           1.35 * max_tiles > 1.48 * avg_tiles + flat_stretches + 8.0);
+        // Several waves of whole units, longest first.  With lengths spread evenly between 2 mean - max and max, the
+        // units of the last wave (at most `last` tiles) land on the shortest of the wave before, which pairs up
+        // to 2 last.  The tiles then stream at HBM's rate where every SM has a unit and faster where some have
+        // none.  20 x 8208 keys: 114.6 flat against 158.6 us; 39 x 4112 113.9 against 136.9; 32 x 4112 98.2 against
+        // 95.1; 20 x 528 23.7 against 19.2.  Batches of mixed lengths pack better than that and cut worse.
+        const int waves = (int)((units + dev.sm_count - 1) / dev.sm_count);
+        const double mean = std::min(avg_tiles * dev.sm_count / units, (double)max_tiles);
+        const double least = std::max(2.0 * mean - max_tiles, 0.0);
+        const double last = least + (max_tiles - least) * (units - (waves - 1.0) * dev.sm_count) / units;
+        const double chain = std::max((double)max_tiles, (waves - 2.0) * max_tiles + 2.0 * last);
+        const double mixed = 1.0 - mean / max_tiles;
+        est_cluster = (shared ? us[0] * chain : (0.86 * chain + 0.48 * avg_tiles) * us[0] / big[0]) +
+                      (shared ? 6.0 : 5.0 + 5.0 * units / dev.sm_count) - 8.0 * mixed;
+        est_flat += 6.0 * mixed;
+        // many waves: flat (57 x 528 keys 33.1 against 39.6 us; blocks of 40, 64 x 1040 102.8 against 106.0)
+        if (cluster_ctas >= (shared ? 5LL : 3LL) * dev.sm_count) est_cluster = est_flat + 1.0;
     }
+    bool flat = flat_ok && est_flat < est_cluster;
     if (const char* force = getenv("BP_ATTENTION_SPLIT")) {
         if (strcmp(force, "flat") == 0) {
             flat = flat_ok;

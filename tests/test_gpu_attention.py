@@ -112,11 +112,14 @@ def test_split_choice():
     assert err <= ATTN_TOL and lerr <= LSE_TOL
 
 
-@pytest.mark.parametrize("n, ctx, flat", [(1, 70000, True), (10, 9000, True), (8, 12000, False), (9, 5000, False)])
-def test_split_of_one_wave(n, ctx, flat):
-    """One wave of clusters against the flat split, by the library's estimates: wide clusters or few SMs on long
-    runs go flat, nearly full grids stay in clusters (128 CTAs: K's ring ahead; 144: not)."""
-    a = wl.attention_inputs(wl.custom(seed=n, ctx=(ctx,) * n, block=(16,) * n, num_q_heads=32, num_kv_heads=8))
+@pytest.mark.parametrize("n, ctx, block, flat", [
+    (1, 70000, 16, True), (10, 9000, 16, True), (8, 12000, 16, False), (9, 5000, 16, False),
+    (20, 4000, 16, True), (32, 1500, 16, False), (10, 4096, 40, True), (16, 1200, 40, False)])
+def test_split_by_estimate(n, ctx, block, flat):
+    """Clusters against the flat split, by the library's estimates.  One wave: wide clusters or few SMs on long
+    runs go flat, nearly full grids stay in clusters (128 CTAs: K's ring ahead; 144: not).  Two waves: flat where the
+    second is nearly empty.  Blocks of 40 have two query tiles, whose clusters share K and V."""
+    a = wl.attention_inputs(wl.custom(seed=n, ctx=(ctx,) * n, block=(block,) * n, num_q_heads=32, num_kv_heads=8))
     _attn_kernels(a, "auto")
     assert any("attn_combine_kernel" in x for x in _attn_kernels(a, "auto")) == flat
     err, lerr = attention_errors(*run_attention(a, CAUSAL), a, CAUSAL, [n // 2])
@@ -247,5 +250,5 @@ def test_uneven_batch_takes_the_flat_split():
     assert any("attn_combine_kernel" in x for x in _attn_kernels(uneven, "auto"))
     err, lerr = attention_errors(*run_attention(uneven, BIDIR), uneven, BIDIR, [0, 1, 10, 19, 20])
     assert err <= ATTN_TOL and lerr <= LSE_TOL
-    even = wl.attention_inputs(wl.custom(seed=8, ctx=(1500,) * 21, block=(16,) * 21, num_q_heads=32, num_kv_heads=8))
+    even = wl.attention_inputs(wl.custom(seed=8, ctx=(1500,) * 32, block=(16,) * 32, num_q_heads=32, num_kv_heads=8))
     assert not any("attn_combine_kernel" in x for x in _attn_kernels(even, "auto"))
