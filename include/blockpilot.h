@@ -245,7 +245,7 @@ BP_API int bp_policy_select(const void* feats, int64_t feat_row_stride, const in
 
 /* ---------------------------------------------------------------------------------
  * Verify epilogue: the LM-head projection of the final hidden states fused with the lossless
- * acceptance of bp_spec_accept; up to 32 rows (and at T = 0) without writing the logits to
+ * acceptance of bp_spec_accept; for few rows (and at T = 0) without writing the logits to
  * memory.  Section 2.1 and the Figure 1 caption: the target scores every position of the drafted
  * block in one pass and keeps the longest accepted prefix; the distributions it compares are
  *
@@ -265,8 +265,8 @@ BP_API int bp_policy_select(const void* feats, int64_t feat_row_stride, const in
  *   logits_out   [rows][vocab] fp32, may be NULL: if given, the logits are also written (rows:
  *                the target rows, then at T > 0 the drafter rows)
  * Two paths, chosen by rows = total_draft + num_seqs (+ total_draft at T > 0):
- *   rows <= 32 at T > 0 (and up to 64 in a workspace without the room below): one cooperative launch of one
- *     CTA per SM keeps every logit in tensor memory; the logits never reach memory unless logits_out asks
+ *   rows <= 32 and num_seqs <= vocab / 40000 at T > 0 (and up to 64 rows in a workspace without the room
+ *     below): one cooperative launch of one CTA per SM keeps every logit in tensor memory; the logits never reach memory unless logits_out asks
  *     for them (then for testing: it adds the write traffic the fusion exists to avoid).
  *   more rows, and T = 0: the LM head is streamed in passes of up to 256 entries, groups of at most 256 rows
  *     per pass over W, and every row's statistics are formed in the projection's epilogue.  At T = 0 only the
@@ -277,8 +277,9 @@ BP_API int bp_policy_select(const void* feats, int64_t feat_row_stride, const in
  *     128 entries and tiles x (32 if rows <= 32 else 64) <= 512 tensor-memory columns (152 SMs: vocab <=
  *     155,648 at rows <= 64, 311,296 at rows <= 32).
  * Limits (else BP_ERR_UNSUPPORTED): hidden % 64 == 0; the rows <= 64 limits above.
- * Workspace: bp_verify_epilogue_workspace_size(num_seqs, total_draft, vocab), sized for T > 0 (beyond 32 rows
- * it holds the fp32 logits, rows padded to a multiple of 8 entries; logits_out given, that part is unused).
+ * Workspace: bp_verify_epilogue_workspace_size(num_seqs, total_draft, vocab), sized for T > 0 (where
+ * the calls stream it holds the fp32 logits, rows padded to a multiple of 8 entries; logits_out given, that part
+ * is unused).
  * A smaller one is accepted: without the padding, and up to 64 rows without the logits.
  * ------------------------------------------------------------------------------- */
 BP_API size_t bp_verify_epilogue_workspace_size(int num_seqs, int total_draft, int vocab);

@@ -177,9 +177,9 @@ struct VerifyEpilogueArgs {
     unsigned int* err_word;
 };
 // Rows (target + drafter) that the verify epilogue's resident kernel (verify_epilogue.cu: every logit kept in
-// tensor memory) can take, and up to which it is chosen at T > 0; others stream (verify_stream.cu).
+// tensor memory) can take, and those it is chosen for at T > 0; others stream (verify_stream.cu).
 constexpr int kVerifyResidentRows = 64;
-constexpr int kVerifyKeepRows = 32;
+inline bool verify_keeps(int rows, int num_seqs, int vocab) { return rows <= 32 && num_seqs <= vocab / 40000; }
 // full: what callers are told to bring (the streamed path's regions wherever it is chosen, its logits rows padded
 // to a multiple of 8); otherwise what a call needs at least.
 size_t verify_epilogue_scratch_bytes(int num_seqs, int total_draft, int vocab, bool full);

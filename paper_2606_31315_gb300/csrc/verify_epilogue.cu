@@ -681,7 +681,7 @@ VeLayout ve_layout(int num_seqs, int total_draft, int vocab, bool full) {
     l.tot_off = l.xg_off + align_up((size_t)(total_draft > 0 ? total_draft : 1) * sizeof(float2), 256);
     l.total = l.tot_off + align_up((size_t)(num_seqs > 0 ? num_seqs : 1) * kVeMaxGrid * sizeof(ulonglong2), 256);
     l.rowst_off = l.tickets_off = l.draw_off = l.logits_off = 0;
-    if (rows > (full ? kVerifyKeepRows : kVerifyResidentRows)) {
+    if (full ? !verify_keeps(rows, num_seqs, vocab) : rows > kVerifyResidentRows) {
         l.rowst_off = l.total;
         l.tickets_off = l.rowst_off + align_up((size_t)rows * sizeof(float2), 256);
         l.draw_off = l.tickets_off + align_up((size_t)num_seqs * sizeof(int), 256);
@@ -761,11 +761,14 @@ int launch_verify_epilogue(const VerifyEpilogueArgs& a, const DeviceInfo& dev, c
     // 2560, streamed against resident: 16 rows 119.5 / 121.0 us, 64 rows 121.3 / 154.6 us) and, at T > 0, more
     // than 32 rows (62 rows 144.8 / 178.0 us: beyond 32 the resident kernel's stages hold half as many W rows
     // and its epilogue runs twice the columns).  Up to 32 rows at T > 0 the resident kernel's logits never leave
-    // tensor memory (31 rows: 136.7 / 127.1 us).  The streamed path's logits and draw scratch need a workspace
-    // sized for them; from 33 to 64 rows a smaller one keeps the resident kernel.
+    // tensor memory (31 rows: 135.7 / 129.2 us), but its draws take their turns (about 2 us for each sequence more)
+    // and its barriers count for more on a small head: it is chosen for up to one sequence per 40,000 entries
+    // (streamed / resident, us: 151,936 entries, 1 sequence 131.0 / 125.9, 4 133.9 / 136.0; 50,257, 1 56.8 / 55.0,
+    // 2 57.8 / 58.5, 4 57.5 / 62.8; 32,000, 1 39.0 / 41.4, 4 39.4 / 48.2).  The streamed path's logits and draw
+    // scratch need a workspace sized for them; up to 64 rows a smaller one keeps the resident kernel.
     const bool fits = ve_layout(a.num_seqs, a.total_draft, a.vocab, true).total <= a.scratch_bytes;
     const VeLayout l = ve_layout(a.num_seqs, a.total_draft, a.vocab, fits);
-    if (greedy || (rows > kVerifyKeepRows && l.logits_off != 0)) {
+    if (greedy || (!verify_keeps(rows, a.num_seqs, a.vocab) && l.logits_off != 0)) {
         VerifyStreamScratch s;
         s.part = reinterpret_cast<float2*>(ws + l.part_off);
         // (without regions of its own -- greedy, few rows -- the row statistics take the slice masses' place)

@@ -455,12 +455,18 @@ def test_33_to_64_rows_on_either_path(blocks, vocab):
 
 
 @pytest.mark.parametrize("vocab", [70, 19459, 32000, 39000, 50257])
-@pytest.mark.parametrize("blocks", [(4,), (16, 16, 9)])
+@pytest.mark.parametrize("blocks", [(4,), (16, 16, 9), (4, 1, 8)])
 def test_vocabulary_in_equal_shares(blocks, vocab):
     """Shares of the vocabulary that are no whole tiles (resident kernel, few rows) or passes (streamed kernel): a last
-    tile or pass of 8 entries up, and a last CTA with less than a share."""
+    tile or pass of 8 entries up, and a last CTA with less than a share.  Up to 32 rows both kernels, the resident
+    one by a workspace that holds no logits."""
     w = wl.custom(seed=vocab + len(blocks), ctx=(0,) * len(blocks), block=blocks, vocab=vocab)
+    td, s = sum(blocks) - len(blocks), len(blocks)
+    up = lambda n: -(-n // 256) * 256  # noqa: E731
+    least = 512 + up((2 * td + s) * 160 * 8) + up(max(td, 1) * 8) + up(s * 160 * 16)
     for temp in (1.0, 0.0):
         inp = wl.lm_head_inputs(w, temp, hidden=128)
-        compare(inp, temp, run_gpu(inp, temp, want_logits=True), run_oracle(inp, temp))
-        compare(inp, temp, run_gpu(inp, temp), run_oracle(inp, temp))
+        ref = run_oracle(inp, temp)
+        compare(inp, temp, run_gpu(inp, temp, want_logits=True), ref)
+        for ws in (None, bp.workspace(least, dev())) if 2 * td + s <= 32 else (None,):
+            compare(inp, temp, run_gpu(inp, temp, ws=ws), ref)
