@@ -692,8 +692,7 @@ def run_ours(args):
             unfused_us=round(t_unfused * 1e6, 3),
             unfused="cuBLAS bf16 GEMM to logits + fp32 cast + accept_kernel"),
         "next1_fused_verify_epilogue_long_context_t1": dict(
-            row(t_ve5, ve5_bytes, ["lm_head_stream_kernel<false,2,true>", "lm_head_row_merge_kernel",
-                                   "batch_draw_kernel"]),
+            row(t_ve5, ve5_bytes, ["lm_head_stream_kernel<false,2,true>", "batch_draw_kernel"]),
             traffic=committed_traffic("lm_head_stream_kernel"),
             rows=int(rows5), design_hbm_bytes=ve5_hbm,
             design_frac=round(ve5_hbm / t_ve5 / 1e9 / peak, 4),

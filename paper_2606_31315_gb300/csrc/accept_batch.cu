@@ -50,7 +50,7 @@ struct BatchParams {
     const int32_t* tokens;
     const int32_t* cu_draft;
     int num_seqs, total_draft, rows_t, vocab, chunks;
-    int nparts;           // statistics per row in part: the chunks, or 1 for rows merged beforehand
+    int nparts;           // statistics per row in part: the chunks, or the LM head's slices (at most kMaxSlices)
     float c2;  // log2(e) / T; 0 at T = 0
     const float* u_accept;
     const float* u_sample;
@@ -197,12 +197,79 @@ __device__ __forceinline__ void merge_parts(float2& acc, const float2 (&x)[kMerg
         acc = make_float2(m, s);
     }
 }
-// Both rows r1, r2 (r2 < 0: none) at once: every load of the first batch is issued before any merge.
+// The streamed LM head's statistics, many slices per row: the CTA's warps (but the one that decides) merge the rows
+// of a sequence's first kShRows positions into shared memory, a warp per row and every load of kMergeRows rows in
+// flight.  In a kernel of their own between the projection and the decisions the same loads cost a launch and a
+// round trip more (hidden 2560, T = 1: 248 rows of 151,936 entries 180.9 -> 179.5 us, 62 rows 143.4 -> 141.9; 60 rows
+// of 4,000 24.9 -> 24.3).
+constexpr int kShRows = 64;
+constexpr int kMergeRows = 5;
+struct SliceRows {
+    float2 target[kShRows], draft[kShRows];  // the merged statistics of positions 0 .. kShRows - 1
+};
 template <bool GREEDY>
-__device__ __forceinline__ void merge_rows(const BatchParams& p, int r1, int r2, float2& a1, float2& a2) {
+__device__ __forceinline__ void merge_slices(const BatchParams& p, int s, int w, int lane, SliceRows* sh) {
+    constexpr int W = kBThreads / 32 - 1, K = kMaxSlices / 32;
+    const int d0 = p.cu_draft[s], g = p.cu_draft[s + 1] - d0;
+    const int nt = min(g + 1, kShRows), n = nt + (GREEDY ? 0 : min(g, kShRows));
+    for (int r0 = w; r0 < n; r0 += kMergeRows * W) {
+        float2 x[kMergeRows][K];
+#pragma unroll
+        for (int b = 0; b < kMergeRows; ++b) {
+            const int r = r0 + b * W;
+            const float2* src = p.part + (size_t)(r < nt ? d0 + s + r : p.rows_t + d0 + r - nt) * p.nparts;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const int i = lane + 32 * k;
+                x[b][k] = r < n && i < p.nparts ? __ldcg(src + i)
+                                                : make_float2(-INFINITY, GREEDY ? __int_as_float(INT_MAX) : 0.f);
+            }
+        }
+#pragma unroll
+        for (int b = 0; b < kMergeRows; ++b) {
+            const int r = r0 + b * W;
+            float2 a = x[b][0];
+            if (GREEDY) {
+                int ai = __float_as_int(a.y);
+#pragma unroll
+                for (int k = 1; k < K; ++k) amax_merge(a.x, ai, x[b][k].x, __float_as_int(x[b][k].y));
+#pragma unroll
+                for (int o = 16; o >= 1; o >>= 1) {
+                    const float m = __shfl_xor_sync(0xffffffffu, a.x, o);
+                    amax_merge(a.x, ai, m, __shfl_xor_sync(0xffffffffu, ai, o));
+                }
+                a.y = __int_as_float(ai);
+            } else {  // the largest maximum first, then every sum scaled to it
+                float m = a.x;
+#pragma unroll
+                for (int k = 1; k < K; ++k) m = fmaxf(m, x[b][k].x);
+#pragma unroll
+                for (int o = 16; o >= 1; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                float t = 0.f;
+#pragma unroll
+                for (int k = 0; k < K; ++k) t = __fmaf_rn(x[b][k].y, ex2d(x[b][k].x, m), t);
+#pragma unroll
+                for (int o = 16; o >= 1; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+                a = make_float2(m, t);
+            }
+            if (lane == 0 && r < n) (r < nt ? sh->target[r] : sh->draft[r - nt]) = a;
+        }
+    }
+}
+
+// Both rows r1, r2 (negative: none) of position i at once, from shared memory where merge_slices left them, else
+// every load of the first batch issued before any merge.
+template <bool GREEDY>
+__device__ __forceinline__ void merge_rows(const BatchParams& p, int r1, int r2, float2& a1, float2& a2,
+                                           const SliceRows* sh, int i) {
     const float2 ident = make_float2(-INFINITY, GREEDY ? __int_as_float(INT_MAX) : 0.f);
     a1 = ident;
     a2 = ident;
+    if (sh != nullptr && i < kShRows) {
+        if (r1 >= 0) a1 = sh->target[i];
+        if (r2 >= 0) a2 = sh->draft[i];
+        return;
+    }
     for (int c0 = 0; c0 < p.nparts; c0 += kMergeBatch) {
         float2 x1[kMergeBatch], x2[kMergeBatch];
         load_row_parts<GREEDY>(p, r1, c0, x1);
@@ -244,14 +311,15 @@ __device__ __forceinline__ DecideIn decide_inputs(const BatchParams& p, int s, i
 // i <= gamma merges target row i's (max, lowest index) from its chunks' and compares drafted token i
 // with it; the first mismatch k by ballot; the emitted token is row k's argmax (the bonus row's when
 // every draft matches).
-__device__ __forceinline__ void decide_greedy(const BatchParams& p, int s, int lane, const DecideIn& in) {
+__device__ __forceinline__ void decide_greedy(const BatchParams& p, int s, int lane, const DecideIn& in,
+                                              const SliceRows* sh) {
     const int d0 = in.d0, g = in.g, t0 = d0 + s;
     int k = g, emitted = 0, bonus = 0;
     for (int i0 = 0; i0 <= g; i0 += 32) {
         const int i = i0 + lane;
         const int x = i0 == 0 ? in.x : (i < g ? p.tokens[d0 + i] : -1);
         float2 st, none;
-        merge_rows<true>(p, i <= g ? t0 + i : -1, -1, st, none);
+        merge_rows<true>(p, i <= g ? t0 + i : -1, -1, st, none, sh, i);
         int am = __float_as_int(st.y);
         if (am >= p.vocab) am = 0;  // every entry -inf: index 0
         bool rej = false;
@@ -286,7 +354,7 @@ __device__ __forceinline__ void decide_greedy(const BatchParams& p, int s, int l
 // token's, and reports draft tokens outside the vocabulary; the others stop at the first block of 32
 // positions that holds a rejection.
 __device__ __forceinline__ void decide_draw(const BatchParams& p, int s, int lane, bool writer, DrawPair* d,
-                                            const DecideIn& in) {
+                                            const DecideIn& in, const SliceRows* sh) {
     const int d0 = in.d0, g = in.g, t0 = d0 + s;
     int k = g;
     float2 stk = make_float2(-INFINITY, 0.f), sdk = stk, bonus = stk;
@@ -297,7 +365,7 @@ __device__ __forceinline__ void decide_draw(const BatchParams& p, int s, int lan
         const int x = i0 == 0 ? in.x : (draft ? p.tokens[d0 + i] : -1);
         const float u = i0 == 0 ? in.u : (draft ? p.u_accept[d0 + i] : 1.f);
         float2 st, sd;
-        merge_rows<false>(p, i <= g ? t0 + i : -1, draft ? p.rows_t + d0 + i : -1, st, sd);
+        merge_rows<false>(p, i <= g ? t0 + i : -1, draft ? p.rows_t + d0 + i : -1, st, sd, sh, i);
         bool rej = false;
         if (draft) {
             const bool valid = x >= 0 && x < p.vocab;
@@ -354,16 +422,29 @@ __device__ __forceinline__ void decide_draw(const BatchParams& p, int s, int lan
     }
 }
 
-// ---- 2. greedy decisions (T = 0): one warp per sequence.  (At T > 0 the draw kernel decides.)
+// ---- 2. greedy decisions (T = 0): one warp per sequence, or, from an LM head's slices, a CTA whose first warp decides.
+// (At T > 0 the draw kernel decides.)
+template <bool SLICES>
 __global__ void __launch_bounds__(kBThreads) batch_decide_kernel(const BatchParams p) {
     griddep_launch_dependents();
+    if (SLICES) {
+        __shared__ SliceRows sh;
+        const int s = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        DecideIn in = {};
+        griddep_wait();
+        if (warp == 0) in = decide_inputs<true>(p, s, lane);
+        else merge_slices<true>(p, s, warp - 1, lane, &sh);
+        __syncthreads();
+        if (warp == 0) decide_greedy(p, s, lane, in, &sh);
+        return;
+    }
     const int s = blockIdx.x * (kBThreads / 32) + (threadIdx.x >> 5);
     DecideIn in = {};
     if (p.inputs_early && s < p.num_seqs) in = decide_inputs<true>(p, s, threadIdx.x & 31);
     griddep_wait();
     if (s >= p.num_seqs) return;
     if (!p.inputs_early) in = decide_inputs<true>(p, s, threadIdx.x & 31);
-    decide_greedy(p, s, threadIdx.x & 31, in);
+    decide_greedy(p, s, threadIdx.x & 31, in, nullptr);
 }
 
 // Weights of four entries: (r = max(0, p - q), p) with p = 2^(l*c2 - Mt) / Zt (r = 0 without a draft row).
@@ -436,8 +517,9 @@ __device__ __forceinline__ unsigned long long chunk_masses(const BatchParams& p,
 // ---- 3. the draw (T > 0): the sequence's decisions, chunk-part masses, then the last part of the
 // sequence finds the entry.  One CTA per (sequence, chunk, part): SPLIT parts of 16384 / SPLIT entries
 // per chunk when the sequences' chunks alone would leave SMs idle.
-template <bool VEC, int PH, int SPLIT>
+template <bool VEC, int PH, int SPLIT, bool SLICES>
 __global__ void __launch_bounds__(kBThreads, SPLIT > 1 ? 2 : PH) batch_draw_kernel(const BatchParams p) {
+    __shared__ SliceRows rows_sh[1];  // SLICES only
     __shared__ unsigned long long segR[kBThreads / 32][kBSegs], segP[kBThreads / 32][kBSegs];
     __shared__ int last_sh, cstar_sh, jstar_sh, wstar_sh, use_r_sh;
     __shared__ unsigned long long off_sh, base_sh;
@@ -450,9 +532,14 @@ __global__ void __launch_bounds__(kBThreads, SPLIT > 1 ? 2 : PH) batch_draw_kern
     DecideIn in = {};
     if (p.inputs_early && warp == 0) in = decide_inputs<false>(p, s, lane);
     griddep_wait();
-    if (warp == 0) {
+    if (SLICES) {
+        if (warp == 0) in = decide_inputs<false>(p, s, lane);
+        else merge_slices<false>(p, s, warp - 1, lane, &rows_sh[0]);
+        __syncthreads();
+        if (warp == 0) decide_draw(p, s, lane, unit == 0, &d_sh, in, &rows_sh[0]);
+    } else if (warp == 0) {
         if (!p.inputs_early) in = decide_inputs<false>(p, s, lane);
-        decide_draw(p, s, lane, unit == 0, &d_sh, in);
+        decide_draw(p, s, lane, unit == 0, &d_sh, in, nullptr);
     }
     __syncthreads();
     const DrawPair d = d_sh;
@@ -679,18 +766,21 @@ int launch_pdl(Kernel kernel, unsigned blocks, const BatchParams& p, cudaStream_
 }
 
 // The decisions (and at T > 0 the draw) once p.part holds the rows' statistics.
-template <bool GREEDY, bool VEC>
+template <bool GREEDY, bool VEC, bool SLICES>
 int run_decisions(const BatchParams& p, int sm_count, cudaStream_t stream) {
-    if (GREEDY)
-        return launch_pdl(batch_decide_kernel, (unsigned)((p.num_seqs + kBThreads / 32 - 1) / (kBThreads / 32)), p,
-                          stream);
+    if (GREEDY) {
+        const int per = SLICES ? 1 : kBThreads / 32;  // sequences per CTA
+        return launch_pdl(batch_decide_kernel<SLICES>, (unsigned)((p.num_seqs + per - 1) / per), p, stream);
+    }
     // the draw (with the decisions): its chunks cut into 4 or 2 parts while every CTA stays in the first
     // wave (two CTAs per SM: the sequences' chunks alone would leave SMs idle), else whole chunks
     const long long draw = (long long)p.num_seqs * p.chunks;
-    if (draw * 4 <= 2LL * sm_count) return launch_pdl(batch_draw_kernel<VEC, 1, 4>, (unsigned)(draw * 4), p, stream);
-    if (draw * 2 <= 2LL * sm_count) return launch_pdl(batch_draw_kernel<VEC, 1, 2>, (unsigned)(draw * 2), p, stream);
-    return draw > sm_count ? launch_pdl(batch_draw_kernel<VEC, 2, 1>, (unsigned)draw, p, stream)
-                           : launch_pdl(batch_draw_kernel<VEC, 1, 1>, (unsigned)draw, p, stream);
+    if (draw * 4 <= 2LL * sm_count)
+        return launch_pdl(batch_draw_kernel<VEC, 1, 4, SLICES>, (unsigned)(draw * 4), p, stream);
+    if (draw * 2 <= 2LL * sm_count)
+        return launch_pdl(batch_draw_kernel<VEC, 1, 2, SLICES>, (unsigned)(draw * 2), p, stream);
+    return draw > sm_count ? launch_pdl(batch_draw_kernel<VEC, 2, 1, SLICES>, (unsigned)draw, p, stream)
+                           : launch_pdl(batch_draw_kernel<VEC, 1, 1, SLICES>, (unsigned)draw, p, stream);
 }
 
 template <bool GREEDY, bool VEC>
@@ -700,7 +790,7 @@ int run_batch(const BatchParams& p, int sm_count, cudaStream_t stream) {
     // T = 0, where the statistics CTAs are small enough to sit eight to an SM, plain order (184.5 against
     // 187.1 us chained)
     const int rc = launch_pdl(batch_stats_kernel<GREEDY, VEC>, (unsigned)(rows * p.chunks), p, stream, !GREEDY);
-    return rc != BP_OK ? rc : run_decisions<GREEDY, VEC>(p, sm_count, stream);
+    return rc != BP_OK ? rc : run_decisions<GREEDY, VEC, false>(p, sm_count, stream);
 }
 
 BatchParams batch_params(const AcceptArgs& a, int ld, int* tickets, void* draw_scratch) {
@@ -749,14 +839,16 @@ int launch_accept_batch(const AcceptArgs& a, int sm_count, int* tickets, void* s
     return vec ? run_batch<false, true>(p, sm_count, stream) : run_batch<false, false>(p, sm_count, stream);
 }
 
-int launch_accept_rows(const AcceptArgs& a, int ld, const float2* row_stats, int sm_count, int* tickets,
-                       void* draw_scratch, cudaStream_t stream) {
+int launch_accept_slices(const AcceptArgs& a, int ld, const float2* part, int slices, int sm_count, int* tickets,
+                         void* draw_scratch, cudaStream_t stream) {
+    if (slices > kMaxSlices) return BP_ERR_UNSUPPORTED;
     BatchParams p = batch_params(a, ld, tickets, draw_scratch);
-    p.part = const_cast<float2*>(row_stats);
-    p.nparts = 1;
+    p.part = const_cast<float2*>(part);
+    p.nparts = slices;
     const bool greedy = a.temperature == 0.f, vec = batch_vec(a, greedy);
-    if (greedy) return run_decisions<true, true>(p, sm_count, stream);  // reads no logits
-    return vec ? run_decisions<false, true>(p, sm_count, stream) : run_decisions<false, false>(p, sm_count, stream);
+    if (greedy) return run_decisions<true, true, true>(p, sm_count, stream);  // reads no logits
+    return vec ? run_decisions<false, true, true>(p, sm_count, stream)
+               : run_decisions<false, false, true>(p, sm_count, stream);
 }
 
 }  // namespace bp

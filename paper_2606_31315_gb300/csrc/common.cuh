@@ -125,13 +125,14 @@ inline bool accept_may_batch(int num_seqs, int total_draft, int vocab) {
 }
 size_t accept_batch_scratch_bytes(int num_seqs, int total_draft, int vocab);
 int launch_accept_batch(const AcceptArgs& a, int sm_count, int* tickets, void* scratch, cudaStream_t stream);
-// The throughput path's decisions and draw alone, from statistics merged beforehand: row_stats[r] is row
-// r's (scaled max, sum of 2^(l*log2e/T - max)) over the whole vocabulary, at T = 0 its (max, lowest
-// index bits); rows in the stacked order (target rows, then the drafter's), ld floats apart.  At T = 0 no
-// logits are read.
+// The throughput path's decisions and draw alone, from statistics of `slices` parts of the vocabulary:
+// part[r * slices + c] is row r's (scaled max, sum of 2^(l*log2e/T - max)) over slice c, at T = 0 its (max,
+// lowest index bits); rows in the stacked order (target rows, then the drafter's), ld floats apart.  At T = 0
+// no logits are read.
+constexpr int kMaxSlices = 160;
 size_t accept_draw_scratch_bytes(int num_seqs, int vocab);
-int launch_accept_rows(const AcceptArgs& a, int ld, const float2* row_stats, int sm_count, int* tickets,
-                       void* draw_scratch, cudaStream_t stream);
+int launch_accept_slices(const AcceptArgs& a, int ld, const float2* part, int slices, int sm_count, int* tickets,
+                         void* draw_scratch, cudaStream_t stream);
 // Same kernel, scratch taken from the library's own static device array (no workspace).
 int launch_accept_noalloc(const AcceptArgs& a, const DeviceInfo& dev, cudaStream_t stream);
 
@@ -191,7 +192,6 @@ struct VerifyStreamScratch {
     float* logits;      // [rows][ld] fp32: the logits at T > 0 when the caller gives no logits_out
     int ld;             // floats from one of those rows to the next: the vocabulary, rounded up to 8 if it fits
     float2* part;       // [rows][slices] slice statistics
-    float2* row_stats;  // [rows] merged statistics
     int* tickets;       // [num_seqs], zero between calls
     void* draw;         // accept_draw_scratch_bytes(num_seqs, vocab)
 };

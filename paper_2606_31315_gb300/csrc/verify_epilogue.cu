@@ -669,7 +669,7 @@ size_t ve_smem_bytes() {
 
 struct VeLayout {
     size_t sync_off, part_off, xg_off, tot_off, total;
-    size_t rowst_off, tickets_off, draw_off, logits_off;  // the streamed path at T > 0 (0: not in this layout)
+    size_t tickets_off, draw_off, logits_off;  // the streamed path at T > 0 (0: not in this layout)
 };
 int ve_padded(int vocab) { return (int)(((long long)vocab + 7) / 8 * 8); }
 VeLayout ve_layout(int num_seqs, int total_draft, int vocab, bool full) {
@@ -680,10 +680,9 @@ VeLayout ve_layout(int num_seqs, int total_draft, int vocab, bool full) {
     l.xg_off = l.part_off + align_up((size_t)(rows > 0 ? rows : 1) * kVeMaxGrid * sizeof(float2), 256);
     l.tot_off = l.xg_off + align_up((size_t)(total_draft > 0 ? total_draft : 1) * sizeof(float2), 256);
     l.total = l.tot_off + align_up((size_t)(num_seqs > 0 ? num_seqs : 1) * kVeMaxGrid * sizeof(ulonglong2), 256);
-    l.rowst_off = l.tickets_off = l.draw_off = l.logits_off = 0;
+    l.tickets_off = l.draw_off = l.logits_off = 0;
     if (full ? !verify_keeps(rows, num_seqs, vocab) : rows > kVerifyResidentRows) {
-        l.rowst_off = l.total;
-        l.tickets_off = l.rowst_off + align_up((size_t)rows * sizeof(float2), 256);
+        l.tickets_off = l.total;
         l.draw_off = l.tickets_off + align_up((size_t)num_seqs * sizeof(int), 256);
         l.logits_off = l.draw_off + align_up(accept_draw_scratch_bytes(num_seqs, vocab), 256);
         l.total = l.logits_off + align_up((size_t)rows * (full ? ve_padded(vocab) : vocab) * sizeof(float), 256);
@@ -771,8 +770,6 @@ int launch_verify_epilogue(const VerifyEpilogueArgs& a, const DeviceInfo& dev, c
     if (greedy || (!verify_keeps(rows, a.num_seqs, a.vocab) && l.logits_off != 0)) {
         VerifyStreamScratch s;
         s.part = reinterpret_cast<float2*>(ws + l.part_off);
-        // (without regions of its own -- greedy, few rows -- the row statistics take the slice masses' place)
-        s.row_stats = reinterpret_cast<float2*>(ws + (l.rowst_off ? l.rowst_off : l.tot_off));
         s.tickets = reinterpret_cast<int*>(ws + l.tickets_off);
         s.draw = ws + l.draw_off;
         s.logits = reinterpret_cast<float*>(ws + l.logits_off);

@@ -18,9 +18,9 @@
 //      whole row pair again, and no on-chip store can hold every row until the decisions are known.
 //      At T = 0 nothing but the statistics leaves the chip.  Each CTA writes its slice's statistics
 //      of every row.
-//   2. lm_head_row_merge_kernel: one warp per row merges the slices' statistics in a fixed order.
-//   3. The decisions and the draw of accept_batch.cu on those row statistics: only the draw's row pair
-//      per sequence (and the logits at the drafted tokens) is read back.
+//   2. The decisions and the draw of accept_batch.cu, whose CTAs first merge the slices' statistics of their
+//      sequence's rows in a fixed order: only the draw's row pair per sequence (and the logits at the drafted
+//      tokens) is read back.
 // Rows beyond 256 go in groups of at most 256, one projection launch per group (W is read once per
 // group).  Every wait is bounded; an expired wait sets the workspace error word and the kernel winds
 // down after its own copies and MMAs have completed.
@@ -50,7 +50,6 @@ constexpr int kVsHBytes = kVsM * 128;    // states of one stage and half: 128 ro
 constexpr int kVsThreads = 576;
 constexpr int kVsEpiWarps = 16;
 constexpr int kVsProducer = 16, kVsIssuer = 17;
-constexpr int kVsMaxSlices = 160;        // slices (CTAs) per row in the statistics array
 
 // MT halves of 128 state rows.  Tensor memory (512 columns) holds two passes' accumulators with one
 // half -- the epilogue of one pass overlaps the MMAs of the next -- or one pass with two.  (Passes of
@@ -355,43 +354,6 @@ __global__ void __launch_bounds__(kVsThreads, 1)
     }
 }
 
-// One warp per stacked row: the slices' statistics merged in a fixed order (each lane its slices in
-// increasing order, then a butterfly), so every call gives bit-identical row statistics.
-template <bool GREEDY>
-__global__ void __launch_bounds__(256) lm_head_row_merge_kernel(const float2* __restrict__ part, int nslices,
-                                                                int rows, float2* __restrict__ out) {
-    griddep_launch_dependents();
-    griddep_wait();
-    const int r = (int)blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (r >= rows) return;
-    constexpr int K = kVsMaxSlices / 32;
-    float2 x[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const int i = lane + 32 * k;
-        x[k] = i < nslices ? __ldcg(&part[(size_t)r * nslices + i])
-                           : make_float2(-INFINITY, GREEDY ? __int_as_float(INT_MAX) : 0.f);
-    }
-    float a0 = x[0].x, a1 = x[0].y;
-    int ai = __float_as_int(a1);
-#pragma unroll
-    for (int k = 1; k < K; ++k) {
-        if (GREEDY) amax_merge(a0, ai, x[k].x, __float_as_int(x[k].y));
-        else lse_merge(a0, a1, x[k].x, x[k].y);
-    }
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-        const float b0 = __shfl_xor_sync(0xffffffffu, a0, o);
-        if (GREEDY) {
-            amax_merge(a0, ai, b0, __shfl_xor_sync(0xffffffffu, ai, o));
-        } else {
-            const float b1 = __shfl_xor_sync(0xffffffffu, a1, o);
-            lse_merge(a0, a1, b0, b1);
-        }
-    }
-    if (lane == 0) out[r] = make_float2(a0, GREEDY ? __int_as_float(ai) : a1);
-}
-
 template <bool GREEDY, int MT, bool WRITE>
 int vs_launch(const CUtensorMap& wmap, const CUtensorMap& wtail, const CUtensorMap& htmap, const CUtensorMap& hdmap,
               const CUtensorMap& lmap, const VsParams& p, int grid, const DeviceInfo& dev, cudaStream_t stream) {
@@ -451,7 +413,7 @@ int encode_rows(CUtensorMap* map, const void* base, int hidden, int rows, int bo
 // rows, T = 1, 32,000 entries: 125 CTAs 50.2, 152 CTAs 50.9 us; 28,000: 110 CTAs 47.7, 152 CTAs 45.5) -- and go down
 // to 64 entries below that (8,192: 32 CTAs 39.3, 128 CTAs 30.7 us).
 static int verify_stream_slice(int vocab, int sm_count) {
-    const int sms = min(sm_count, kVsMaxSlices), passes = (vocab + kVsN - 1) / kVsN;
+    const int sms = min(sm_count, kMaxSlices), passes = (vocab + kVsN - 1) / kVsN;
     const int ctas = min(sms, 4 * passes > 3 * sms ? passes : (vocab + 63) / 64);
     return ctas < 1 ? 0 : (int)(((long long)vocab + ctas * 8 - 1) / (ctas * 8) * 8);
 }
@@ -527,21 +489,6 @@ int launch_verify_stream(const VerifyEpilogueArgs& a, const VerifyStreamScratch&
         r0 = r1;
     }
 
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((rows + 7) / 8));
-    cfg.blockDim = dim3(256);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const float2* part = s.part;
-    const cudaError_t e = greedy ? cudaLaunchKernelEx(&cfg, lm_head_row_merge_kernel<true>, part, grid, rows, s.row_stats)
-                                 : cudaLaunchKernelEx(&cfg, lm_head_row_merge_kernel<false>, part, grid, rows,
-                                                      s.row_stats);
-    if (e != cudaSuccess) return BP_ERR_CUDA;
-
     AcceptArgs aa;
     aa.target = logits;
     aa.draft = logits ? logits + (size_t)rows_t * ld : nullptr;
@@ -558,7 +505,7 @@ int launch_verify_stream(const VerifyEpilogueArgs& a, const VerifyStreamScratch&
     aa.accept_prob = a.accept_prob;
     aa.scratch = nullptr;
     aa.err_word = a.err_word;
-    return launch_accept_rows(aa, ld, s.row_stats, dev.sm_count, s.tickets, s.draw, stream);
+    return launch_accept_slices(aa, ld, s.part, grid, dev.sm_count, s.tickets, s.draw, stream);
 }
 
 }  // namespace bp

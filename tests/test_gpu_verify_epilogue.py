@@ -470,3 +470,12 @@ def test_vocabulary_in_equal_shares(blocks, vocab):
         compare(inp, temp, run_gpu(inp, temp, want_logits=True), ref)
         for ws in (None, bp.workspace(least, dev())) if 2 * td + s <= 32 else (None,):
             compare(inp, temp, run_gpu(inp, temp, ws=ws), ref)
+
+
+@pytest.mark.parametrize("temp", [1.0, 0.0])
+@pytest.mark.parametrize("blocks", [(66,), (64, 65, 3), (100, 1)])
+def test_streamed_long_blocks(blocks, temp):
+    """Sequences around and beyond the 64 positions whose slice statistics the decisions hold in shared memory."""
+    w = wl.custom(seed=sum(blocks), ctx=(0,) * len(blocks), block=blocks, vocab=9001)
+    inp = wl.lm_head_inputs(w, temp, hidden=128)
+    compare(inp, temp, run_gpu(inp, temp), run_oracle(inp, temp))
