@@ -53,6 +53,7 @@ constexpr int kStageBytes = 2 * kKVBytes;       // 64 KB
 constexpr int kDynSmem = kQBytes + kStages * kStageBytes + 1024;
 constexpr int kThreads = 192;
 constexpr uint32_t kTmemCols = 512;
+static_assert(kDynSmem >= tmem_smem_share((int)kTmemCols, 228 * 1024), "leaves no other CTA's tensor memory room");
 constexpr uint32_t kColO = 384;
 constexpr int kMaxOrderedSeqs = 256;  // longest-first ordering for batches up to this size
 constexpr int kMaxCluster = 16;

@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include "../../include/blockpilot.h"
+#include "tmem_share.h"
 
 namespace bp {
 
@@ -45,8 +46,14 @@ struct DeviceInfo {
     int sm_count = 0;
     int cc_major = 0, cc_minor = 0;
     int max_smem_optin = 0;
+    int sm_smem = 0, block_smem = 0;  // shared memory of an SM; the system's share of it per CTA
 };
 int device_info(DeviceInfo* out);  // BP_OK or BP_ERR_CUDA
+// The dynamic shared memory of a CTA that needs `bytes` and holds `columns` of tensor memory (tmem_share.h).
+inline size_t tmem_smem(const DeviceInfo& dev, int columns, size_t bytes) {
+    const size_t share = (size_t)(tmem_smem_share(columns, dev.sm_smem) - dev.block_smem);
+    return bytes > share ? bytes : share;
+}
 
 // Encodes a tiled TMA descriptor (driver entry point resolved once).
 int encode_tensor_map(CUtensorMap* map, CUtensorMapDataType dt, cuuint32_t rank, void* base, const cuuint64_t* dims,

@@ -1037,15 +1037,9 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
         return 1024 + wb + slots * npad * 128 + h_for(k) + op_bytes + a.num_cand * ((kTcM + k - 1) / k) * 4;
     };
     // Tensor memory: one accumulator of npad columns, or one per issuer.  A CTA waits for its columns while its
-    // cluster peers wait for it, so no more CTAs may share an SM than its 512 columns serve: the shared memory
-    // of a CTA keeps them to that.
-    uint32_t cols = 32;
-    while ((int)cols < npad * (ring ? 1 : kTcIssuers)) cols <<= 1;
-    const int least = dev.max_smem_optin / (int)(512 / cols + 1) + 1024;
-    const auto launch_smem = [&](int slots, int k) {
-        const int sm = smem_for(slots, k);
-        return sm > least ? sm : least;
-    };
+    // cluster peers wait for it: its shared memory keeps what meets on an SM to the columns there are (tmem_share.h).
+    const int cols = tmem_columns(npad * (ring ? 1 : kTcIssuers));
+    const auto launch_smem = [&](int slots, int k) { return (int)tmem_smem(dev, cols, (size_t)smem_for(slots, k)); };
     if (configure_tc(dev.device) != BP_OK) return BP_ERR_CUDA;
     // one-shot: the widest split whose clusters are all resident at once, while a CTA still holds its atoms (a
     // cluster left for a second wave doubles the call: 60 x 2000 -> 3000, 24 tiles, clusters of 6: 27.0 us)
@@ -1088,7 +1082,9 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
     const int slots = flat_split ? kFlStages : ring ? kTcKernels[kernel].stages : per;
     const int w_bytes = slots * kTcAtomBytes > pd_bytes ? slots * kTcAtomBytes : pd_bytes;
     const int x_bytes = slots * npad * 128;
-    const int smem = flat_split ? 1024 + kFlStages * (kTcAtomBytes + npad * 128) : launch_smem(slots, ks);
+    const int flat_cols = tmem_columns(4 * npad);
+    const int smem = flat_split ? (int)tmem_smem(dev, flat_cols, 1024 + kFlStages * (kTcAtomBytes + (size_t)npad * 128))
+                                : launch_smem(slots, ks);
     if (smem > kTcMaxSmem) return -1;
 
     CUtensorMap w1map, xmap;
@@ -1124,7 +1120,7 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
     p.x_bytes = x_bytes;
     p.h_bytes = h_bytes;
     p.op_bytes = op_bytes;
-    p.tmem_cols = cols;
+    p.tmem_cols = (uint32_t)cols;
     p.gathered = gather;
     p.b1 = a.b1;
     p.w2 = static_cast<const __nv_bfloat16*>(a.w2);
@@ -1159,8 +1155,7 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
         f.runs_total = groups * tiles * atoms_total;
         f.slots = reinterpret_cast<float4*>(flat);
         f.tile_tickets = reinterpret_cast<int*>(flat + flat_slot_bytes(a.num_reqs, a.hidden));
-        f.cols = 32;
-        while ((int)f.cols < 4 * npad) f.cols <<= 1;
+        f.cols = (uint32_t)flat_cols;
         int ctas = dev.sm_count < kFlMaxGrid ? dev.sm_count : kFlMaxGrid;
         ctas = ctas < f.runs_total ? ctas : f.runs_total;
         cudaLaunchConfig_t fcfg = {};

@@ -695,16 +695,18 @@ int ve_launch(const CUtensorMap& wmap, const CUtensorMap& wtail, const VeParams&
               cudaStream_t stream) {
     static std::mutex cfg_mu;        // per instantiation (a template's own statics)
     static int configured[64] = {};
-    const size_t smem = ve_smem_bytes<NP, APS>();
+    // (the CTAs wait for one another at the grid barriers with their tensor memory held)
+    const size_t smem = tmem_smem(dev, (int)p.tmem_cols, ve_smem_bytes<NP, APS>());
+    const size_t most = tmem_smem(dev, kTmemColumns, ve_smem_bytes<NP, APS>());
     if (dev.device >= 0 && dev.device < 64) {
         std::lock_guard<std::mutex> cfg_lock(cfg_mu);  // once per device, from any host thread
         if (!configured[dev.device]) {
             if (cudaFuncSetAttribute(verify_epilogue_kernel<NP, APS>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess)
                 return BP_ERR_CUDA;
             int per_sm = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, verify_epilogue_kernel<NP, APS>,
-                                                              kVeThreads, smem) != cudaSuccess ||
+                                                              kVeThreads, most) != cudaSuccess ||
                 per_sm < 1)
                 return BP_ERR_UNSUPPORTED;
             configured[dev.device] = 1;
@@ -779,8 +781,6 @@ int launch_verify_epilogue(const VerifyEpilogueArgs& a, const DeviceInfo& dev, c
     int grid = 0, NP = 0, per = 0;
     int rc = verify_epilogue_config(rows, a.vocab, a.hidden, dev.sm_count, &grid, &NP, &per);
     if (rc != BP_OK) return rc;
-    uint32_t cols = 32;
-    while (cols < (uint32_t)(per * NP)) cols <<= 1;
 
     const int slice = ve_slice(a.vocab, min(min(dev.sm_count, kVeMaxGrid), (a.vocab + kVeM - 1) / kVeM));
     const int tail = slice - (slice - 1) / kVeM * kVeM;
@@ -807,7 +807,7 @@ int launch_verify_epilogue(const VerifyEpilogueArgs& a, const DeviceInfo& dev, c
     p.rows = rows;
     p.slice = slice;
     p.tail = tail;
-    p.tmem_cols = cols;
+    p.tmem_cols = (uint32_t)tmem_columns(per * NP);
     p.c2 = 1.4426950408889634f / a.temperature;
     p.tokens = a.tokens;
     p.cu_draft = a.cu_draft;

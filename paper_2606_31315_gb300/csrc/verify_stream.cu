@@ -359,7 +359,7 @@ int vs_launch(const CUtensorMap& wmap, const CUtensorMap& wtail, const CUtensorM
               const CUtensorMap& lmap, const VsParams& p, int grid, const DeviceInfo& dev, cudaStream_t stream) {
     static std::mutex cfg_mu;  // per instantiation (a template's own statics)
     static int configured[64] = {};
-    const size_t smem = vs_smem_bytes<MT, WRITE>();
+    const size_t smem = tmem_smem(dev, kTmemColumns, vs_smem_bytes<MT, WRITE>());
     if (dev.device >= 0 && dev.device < 64) {
         std::lock_guard<std::mutex> cfg_lock(cfg_mu);  // once per device, from any host thread
         if (!configured[dev.device]) {
