@@ -7,7 +7,7 @@
 #include <stdint.h>
 
 #include "../../include/blockpilot.h"
-#include "tmem_share.h"
+#include "tmem_share.cuh"
 
 namespace bp {
 
@@ -49,7 +49,7 @@ struct DeviceInfo {
     int sm_smem = 0, block_smem = 0;  // shared memory of an SM; the system's share of it per CTA
 };
 int device_info(DeviceInfo* out);  // BP_OK or BP_ERR_CUDA
-// The dynamic shared memory of a CTA that needs `bytes` and holds `columns` of tensor memory (tmem_share.h).
+// The dynamic shared memory of a CTA that needs `bytes` and holds `columns` of tensor memory (tmem_share.cuh).
 inline size_t tmem_smem(const DeviceInfo& dev, int columns, size_t bytes) {
     const size_t share = (size_t)(tmem_smem_share(columns, dev.sm_smem) - dev.block_smem);
     return bytes > share ? bytes : share;

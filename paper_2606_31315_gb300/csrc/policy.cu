@@ -1037,7 +1037,7 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
         return 1024 + wb + slots * npad * 128 + h_for(k) + op_bytes + a.num_cand * ((kTcM + k - 1) / k) * 4;
     };
     // Tensor memory: one accumulator of npad columns, or one per issuer.  A CTA waits for its columns while its
-    // cluster peers wait for it: its shared memory keeps what meets on an SM to the columns there are (tmem_share.h).
+    // cluster peers wait for it: its shared memory keeps what meets on an SM to the columns there are (tmem_share.cuh).
     const int cols = tmem_columns(npad * (ring ? 1 : kTcIssuers));
     const auto launch_smem = [&](int slots, int k) { return (int)tmem_smem(dev, cols, (size_t)smem_for(slots, k)); };
     if (configure_tc(dev.device) != BP_OK) return BP_ERR_CUDA;

@@ -1,4 +1,4 @@
-"""Tensor memory shared by CTAs of different launches (csrc/tmem_share.h), checked on the host: whatever CTAs fit an
+"""Tensor memory shared by CTAs of different launches (csrc/tmem_share.cuh), checked on the host: whatever CTAs fit an
 SM's shared memory, their tensor-memory columns fit too, so that no allocation waits for columns held by a CTA that
 itself waits for cluster or grid peers (two policy calls on two streams)."""
 import ctypes
@@ -18,7 +18,7 @@ BLOCK = 1024     # the system's share per CTA
 def rule(tmp_path_factory):
     d = tmp_path_factory.mktemp("tmem_share")
     src, lib = d / "rule.cc", d / "rule.so"
-    src.write_text('#include "tmem_share.h"\n'
+    src.write_text('#include "tmem_share.cuh"\n'
                    'extern "C" int columns(int n) { return bp::tmem_columns(n); }\n'
                    'extern "C" int share(int c, int sm) { return bp::tmem_smem_share(c, sm); }\n')
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", f"-I{_build.CSRC}", str(src), "-o", str(lib)], check=True)
