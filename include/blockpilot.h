@@ -141,7 +141,8 @@ BP_API int bp_block_attention_paged(const void* q, const void* k_cache, const vo
  *   k_new, v_new  [total_new][num_kv_heads][head_dim] dtype (bf16 or fp32),
  *                 head_dim * element size a multiple of 16 bytes
  *   k_cache, v_cache, block_table, pages_per_seq, page_size as bp_block_attention_paged
- * The pages that receive the rows must already be in the block table.  No workspace. */
+ * The pages that receive the rows must already be in the block table.  total_new may exceed cu_new[num_seqs] (a
+ * padded k_new): the rows past it go behind the last sequence's keys, where its pages must have room.  No workspace. */
 BP_API int bp_kv_append(void* k_cache, void* v_cache, const void* k_new, const void* v_new, const int32_t* cu_new,
                         const int32_t* cu_kv, const int32_t* block_table, int pages_per_seq, int page_size,
                         int num_pages, int num_seqs, int total_new, int num_kv_heads, int head_dim, int dtype,

@@ -1683,11 +1683,11 @@ __global__ void __launch_bounds__(256) kv_append_kernel(uint8_t* __restrict__ kc
     uint4 first = make_uint4(0u, 0u, 0u, 0u);
     if (lane < 2 * n16) first = *from(lane);
     int s = 0, pos, page0 = 0, page1 = 0;
-    const bool one = num_seqs == 1;  // offsets 0 and total_new
+    const bool one = num_seqs == 1;
     if (one) {
         if (lane < pages_per_seq) page0 = __ldg(bt + lane);
         if (lane + 32 < pages_per_seq) page1 = __ldg(bt + lane + 32);
-        pos = __ldg(cu_kv + 1) - __ldg(cu_kv) - total_new + t;
+        pos = __ldg(cu_kv + 1) - __ldg(cu_kv) - __ldg(cu_new + 1) + t;
     } else if (num_seqs <= 32) {  // the sequences after the first that start at or before row t, counted
         const int begin = lane < num_seqs ? __ldg(cu_new + lane) : 0, end = lane < num_seqs ? __ldg(cu_new + lane + 1) : 0;
         const int len = lane < num_seqs ? __ldg(cu_kv + lane + 1) - __ldg(cu_kv + lane) : 0;

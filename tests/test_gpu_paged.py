@@ -85,3 +85,28 @@ def test_append_block_then_attend(page_size):
     o, lse = _run_paged(a, pk, bp.MASK_CAUSAL)
     err, lerr = attention_errors(o, lse, a, bp.MASK_CAUSAL, range(len(blocks)))
     assert err <= ATTN_TOL and lerr <= LSE_TOL, (err, lerr)
+
+
+@pytest.mark.parametrize("blocks, pad", [((5,), 3), ((1,), 15), ((4, 9), 3), ((3,) * 40, 7)])
+def test_append_of_padded_rows(blocks, pad):
+    """k_new with rows past cu_new[num_seqs]: the block's rows go to the keys that end the sequence, by cu_new and not
+    by the number of rows, for one sequence, up to 32 and more; the padding lands behind the last sequence's keys."""
+    page, ctx = 16, 37
+    lens = [ctx + b for b in blocks]
+    per_seq = (ctx + max(blocks) + pad + page - 1) // page  # pages with room for the padding
+    s = len(blocks)
+    gen = torch.Generator().manual_seed(pad)
+    new = [torch.randn(sum(blocks) + pad, 2, 64, generator=gen).to(torch.bfloat16) for _ in range(2)]
+    table = torch.randperm(s * per_seq, generator=gen).to(torch.int32).view(s, per_seq)
+    caches = [torch.zeros(s * per_seq * page, 2, 64, dtype=torch.bfloat16, device=dev()) for _ in range(2)]
+    cu_new = torch.tensor([0, *np.cumsum(blocks)], dtype=torch.int32)
+    cu_kv = torch.tensor([0, *np.cumsum(lens)], dtype=torch.int32)
+    bp.kv_append(caches[0], caches[1], new[0].to(dev()), new[1].to(dev()), cu_new.to(dev()), cu_kv.to(dev()),
+                 table.to(dev()), page)
+    for cache, rows in zip(caches, new):
+        want = torch.zeros(s * per_seq * page, 2, 64, dtype=torch.bfloat16)
+        for t in range(len(rows)):
+            i = min(int(np.searchsorted(cu_new.numpy(), t, side="right")) - 1, s - 1)
+            key = ctx + t - int(cu_new[i])
+            want[int(table[i, key // page]) * page + key % page] = rows[t]
+        assert torch.equal(cache.cpu(), want)
