@@ -33,8 +33,9 @@
  *     another entry point) may lie where that data is: zero-fill the workspace again before
  *     such a call (spec_accept's per-sequence tickets come first, in 256-byte units of 64
  *     sequences, so there only a call with more of those units than an earlier one needs
- *     this).  Its first 16 bytes hold a sticky device error word read by bp_get_status.  Two
- *     calls that may run concurrently need distinct workspaces.
+ *     this; verify_epilogue's counters too, 2 + num_seqs of them, in a workspace as large as
+ *     the largest call's size).  Its first 16 bytes hold a sticky device error word read by
+ *     bp_get_status.  Two calls that may run concurrently need distinct workspaces.
  *   - Host-checkable problems (NULL pointers, unsupported shapes, a workspace that is too
  *     small) return an error code immediately and enqueue nothing.  Problems only the GPU
  *     sees (a draft token id outside [0, V), a bounded wait that timed out) set the

@@ -667,23 +667,30 @@ size_t ve_smem_bytes() {
     return 1024 + (size_t)ve_stages(NP, APS) * APS * (kVeWBytes + NP * 128);
 }
 
+// What has to be zero between calls comes first, at places that do not depend on the draft: the grid barrier's two
+// words and then the streamed draw's ticket per sequence.  So calls with other block sizes (and, within a 256-byte
+// unit of counters, another number of sequences) can share a workspace: behind statistics sized by the rows, a
+// call's tickets would lie where an earlier call left data, no part of a draw would come last, and the emitted token
+// would not be written.
 struct VeLayout {
-    size_t sync_off, part_off, xg_off, tot_off, total;
-    size_t tickets_off, draw_off, logits_off;  // the streamed path at T > 0 (0: not in this layout)
+    size_t sync_off, tickets_off, part_off, xg_off, tot_off, total;
+    size_t draw_off, logits_off;  // the streamed path at T > 0 (0: not in this layout)
 };
+constexpr size_t kVeSyncBytes = 2 * sizeof(unsigned int);
 int ve_padded(int vocab) { return (int)(((long long)vocab + 7) / 8 * 8); }
 VeLayout ve_layout(int num_seqs, int total_draft, int vocab, bool full) {
     VeLayout l;
     const int rows = 2 * total_draft + num_seqs;
+    const bool streams = full ? !verify_keeps(rows, num_seqs, vocab) : rows > kVerifyResidentRows;
     l.sync_off = 0;
-    l.part_off = 256;
+    l.tickets_off = kVeSyncBytes;
+    l.part_off = streams ? align_up(l.tickets_off + (size_t)num_seqs * sizeof(int), 256) : 256;
     l.xg_off = l.part_off + align_up((size_t)(rows > 0 ? rows : 1) * kVeMaxGrid * sizeof(float2), 256);
     l.tot_off = l.xg_off + align_up((size_t)(total_draft > 0 ? total_draft : 1) * sizeof(float2), 256);
     l.total = l.tot_off + align_up((size_t)(num_seqs > 0 ? num_seqs : 1) * kVeMaxGrid * sizeof(ulonglong2), 256);
-    l.tickets_off = l.draw_off = l.logits_off = 0;
-    if (full ? !verify_keeps(rows, num_seqs, vocab) : rows > kVerifyResidentRows) {
-        l.tickets_off = l.total;
-        l.draw_off = l.tickets_off + align_up((size_t)num_seqs * sizeof(int), 256);
+    l.draw_off = l.logits_off = 0;
+    if (streams) {
+        l.draw_off = l.total;
         l.logits_off = l.draw_off + align_up(accept_draw_scratch_bytes(num_seqs, vocab), 256);
         l.total = l.logits_off + align_up((size_t)rows * (full ? ve_padded(vocab) : vocab) * sizeof(float), 256);
     }

@@ -479,3 +479,20 @@ def test_streamed_long_blocks(blocks, temp):
     w = wl.custom(seed=sum(blocks), ctx=(0,) * len(blocks), block=blocks, vocab=9001)
     inp = wl.lm_head_inputs(w, temp, hidden=128)
     compare(inp, temp, run_gpu(inp, temp), run_oracle(inp, temp))
+
+
+@pytest.mark.parametrize("vocab, sets", [
+    (4000, [(21, 20), (31, 32), (23, 23), (40, 9), (2, 2), (31, 32)]),        # streamed, 33 to 97 rows and 6
+    (40064, [(24,), (16,), (32,), (4,), (24,), (50,), (17,)]),                # one sequence: either path
+    (5003, [(1,) * 62, (2, 1) * 20, (3,) * 60, (1,) * 40, (2,) * 62]),        # as many sequences as a unit of counters
+])
+def test_one_workspace_for_varying_blocks(vocab, sets):
+    """Block sizes chosen per step: a workspace of the largest call's size serves every smaller draft, in any order and
+    without being cleared (the counters lie in front of everything whose place depends on the draft)."""
+    sizes = [bp.verify_epilogue_workspace_size(len(b), sum(b) - len(b), vocab) for b in sets]
+    ws = bp.workspace(max(sizes), dev())
+    for k, blocks in enumerate(sets):
+        w = wl.custom(seed=k, ctx=(0,) * len(blocks), block=blocks, vocab=vocab)
+        for temp in (1.0, 0.0):
+            inp = wl.lm_head_inputs(w, temp, hidden=64)
+            compare(inp, temp, run_gpu(inp, temp, ws=ws), run_oracle(inp, temp))
