@@ -1098,7 +1098,8 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
     const bool gather = ring && a.row_index != nullptr;
     if (ring) {  // the gathered rows, or the feature rows themselves (rows past the last request read zero)
         const cuuint64_t xdims[2] = {(cuuint64_t)a.d_in, gather ? (cuuint64_t)groups * kTcMaxN : (cuuint64_t)a.num_reqs};
-        const cuuint64_t xstrides[1] = {(cuuint64_t)(gather ? a.d_in : a.row_stride) * 2};
+        // (a single request's stride is not used and may be any, also more than a map can hold)
+        const cuuint64_t xstrides[1] = {(cuuint64_t)(gather || a.num_reqs == 1 ? a.d_in : a.row_stride) * 2};
         const cuuint32_t xbox[2] = {(cuuint32_t)kTcAtom, (cuuint32_t)npad};
         if (encode_tensor_map(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, gather ? xg : const_cast<void*>(a.feats),
                               xdims, xstrides, xbox, CU_TENSOR_MAP_SWIZZLE_128B) != BP_OK)

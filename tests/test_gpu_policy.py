@@ -144,3 +144,15 @@ def test_fp32_tiles(n, d_in, hidden):
     assert np.abs(lo - ref["logits"]).max() <= 1e-5 * scale
     ok = ref["top2_margin"] >= 1e-4 * scale
     np.testing.assert_array_equal(bs[ok], ref["block_size"][ok])
+
+
+def test_one_wide_request_of_any_row_stride():
+    """The stride of a single row is not used: one wider than a tensor map can hold is taken too."""
+    w = wl.custom(seed=3, policy=dict(num_reqs=1, d_in=98304, hidden=64, wdtype="bf16", feat_std=1.0))
+    pin = wl.policy_inputs(w)
+    f = lambda k: to_dev(pin[k], "bf16" if k in ("feats", "w1", "w2") else None)  # noqa: E731
+    rest = [f(k) for k in ("w1", "b1", "w2", "b2", "candidates")]
+    feats = f("feats")[:1]
+    bs, lo = bp.policy_select(feats, *rest)
+    bs1, lo1 = bp.policy_select(feats.as_strided((1, 98304), (1 << 40, 1)), *rest)
+    assert torch.equal(bs, bs1) and torch.equal(lo, lo1)
