@@ -1058,15 +1058,22 @@ int run_tc(const PolicyArgs& a, const DeviceInfo& dev, float* part, int* counter
     // 151936 -> 2048: 16 tiles of 9-CTA clusters took 200 us with the 5-stage ring at one CTA per SM);
     // if none, the deepest that fits
     int kernel = 0;  // index into kTcKernels
-    // flat split: where a cluster's CTA would stream a long run of atoms, or far more than its share if every SM
-    // took part (clusters hold at most 9 CTAs a tile).  Atoms per CTA in clusters / flat, and the calls' times:
-    // 32 x 151936 -> 2048: 264 / 250, 118.3 / 111.1 us; -> 1024: 264 / 125, 84.7 / 63.2; 16 x 128256 -> 512: 223 /
-    // 53, 71.8 / 38.3 us.  Elsewhere meeting through the workspace costs more than the idle SMs: 5 x 32000 ->
-    // 1280: 56 / 33, 24.7 / 26.5 us; 10 x 32000 -> 2048: 56 / 53, 31.0 / 33.4 us; 17 x 5912 -> 2304: 12 / 11,
-    // 15.6 / 19.0 us.
-    const long long atoms_all = (long long)groups * tiles * atoms_total;
-    const bool flat_split = ring && flat != nullptr && atoms_all <= INT_MAX / 2 &&
-                            (per >= 128 || per >= atoms_all / dev.sm_count + 32);
+    // flat split: where a cluster's CTA would stream far more atoms than its share if every SM took part (clusters
+    // hold at most 9 CTAs a tile).  Meeting through the workspace costs the equivalent of about 32 atoms, more the
+    // more runs meet in a tile (one CTA adds them), and beyond 32 requests the sums' second round.  Fitted to 330
+    // shapes timed both ways; atoms per CTA in clusters / flat, and the times in clusters / flat: 4 x 151936 -> 700:
+    // 264 / 94, 82.5 / 46.5 us; 17 x 84288 -> 1280: 147 / 87, 51.2 / 47.6; 64 x 151936 -> 700: 264 / 94, 86.6 / 63.4;
+    // 64 x 151936 -> 1700: 264 / 219, 96.3 / 107.8; 40 x 50304 -> 256: 88 / 10, 33.5 / 39.5; 40 x 84288 -> 2048: 147 /
+    // 139, 65.4 / 71.8; 5 x 32000 -> 1280: 56 / 33, 24.7 / 26.5.
+    // And for long runs in place where the clusters outnumber those that get SMs of their own: where they land then
+    // decides the time (32 x 151936 -> 2048, 16 clusters of 9: 109 to 121 us, flat 111).  Behind a gather kernel
+    // clusters stay the better half (40 x 151936 -> 2048 122.9 and 126.5, 32 -> 2650 144.9 and 152.1).
+    const long long atoms_all = (long long)groups * tiles * atoms_total, share = atoms_all / dev.sm_count;
+    const long long meet = atoms_total / (share > 0 ? share : 1);  // runs of a tile
+    const bool flat_split =
+        ring && flat != nullptr && atoms_all <= INT_MAX / 2 &&
+        (per >= share + 32 + 3 * meet * npad / 640 + (npad > 32 ? 48 : 0) ||
+         (a.row_index == nullptr && per >= 240 && tiles * groups > active_clusters(dev.device, 1, ks, kTcMaxSmem)));
     if (ring && !flat_split) {
         for (int i = 1; i <= kTcRings; ++i) {
             const int sm = launch_smem(kTcKernels[i].stages, ks);

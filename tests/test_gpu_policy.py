@@ -91,6 +91,8 @@ def test_d_in_tail_and_two_request_groups(d_in):
     (64, 82000, 300),    # a full group
     (130, 41000, 300),   # three request groups, the last of two
     (1, 40000, 128),     # one tile cut over every CTA, runs of 4 or 5 atoms
+    (33, 120000, 900),   # 48 padded requests on runs long enough for the flat split
+    (130, 130000, 300),  # so are these three groups
     (17, 5912, 600),     # short runs: clusters in either workspace
 ])
 @pytest.mark.parametrize("gather", [True, False])
