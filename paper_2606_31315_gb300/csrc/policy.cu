@@ -109,33 +109,61 @@ __global__ void __launch_bounds__(kThreads1) policy_hidden_kernel(const T* __res
     }
 }
 
-// Output layer and argmax of one request per CTA: a warp per candidate (its 8 warps' chains of loads side by side;
-// one candidate after the other over the whole block took 9 us for 9 candidates).
+// Output layer and argmax of one request per CTA.  Every thread takes the hidden units 256 apart for up to kOutC
+// candidates at a time, kOutUnroll units' loads in flight: what bounds it is the number of round trips to L2.  (fp32,
+// 1 x 64 -> 3262 -> 9: 23.2 us a call with a warp per candidate and hidden / 128 rounds, 16.3 with the block on one
+// candidate after the other, 8.2 here.)  Dependents launch behind the wait: released at the start, calls back to back
+// took 92 us instead of 58 at 32 x 16000 -> 512 and 145 instead of 101 at 64.
+constexpr int kOutC = 16, kOutUnroll = 4;
 template <typename T>
 __global__ void __launch_bounds__(256) policy_out_kernel(const float* __restrict__ hbuf, int hidden,
                                                          const T* __restrict__ w2, const float* __restrict__ b2,
                                                          int num_cand, const int32_t* __restrict__ candidates,
                                                          float* __restrict__ logits_out,
                                                          int32_t* __restrict__ block_size_out) {
-    __shared__ float logits[64];
-    const int n = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
-    griddep_launch_dependents();
+    __shared__ float red[8][kOutC], logits[64];
+    const int n = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     griddep_wait();
+    griddep_launch_dependents();  // (before its wait, a next call's hidden layer settles on the SMs this one's runs on)
     const float* h = hbuf + (size_t)n * hidden;
-    for (int c = tid >> 5; c < num_cand; c += 8) {
-        const T* w = w2 + (size_t)c * hidden;
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        int j = lane;
-        for (; j + 96 < hidden; j += 128)
+    for (int c0 = 0; c0 < num_cand; c0 += kOutC) {
+        const int nc = min(kOutC, num_cand - c0);
+        const T* w = w2 + (size_t)c0 * hidden;
+        float acc[kOutC];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) acc[u] = fmaf(static_cast<float>(w[j + 32 * u]), h[j + 32 * u], acc[u]);
-        for (; j < hidden; j += 32) acc[0] = fmaf(static_cast<float>(w[j]), h[j], acc[0]);
-        float sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+        for (int c = 0; c < kOutC; ++c) acc[c] = 0.f;
+        for (int j0 = tid; j0 < hidden; j0 += 256 * kOutUnroll) {
+            float hv[kOutUnroll], wv[kOutUnroll][kOutC];
 #pragma unroll
-        for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        if (lane == 0) logits[c] = sum + b2[c];
+            for (int u = 0; u < kOutUnroll; ++u) {
+                const int j = j0 + 256 * u;
+                hv[u] = j < hidden ? h[j] : 0.f;
+#pragma unroll
+                for (int c = 0; c < kOutC; ++c)
+                    wv[u][c] = c < nc && j < hidden ? static_cast<float>(w[(size_t)c * hidden + j]) : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < kOutUnroll; ++u)
+#pragma unroll
+                for (int c = 0; c < kOutC; ++c) acc[c] = fmaf(wv[u][c], hv[u], acc[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < kOutC; ++c) {
+            if (c < nc) {
+#pragma unroll
+                for (int o = 16; o; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+                if (lane == 0) red[warp][c] = acc[c];
+            }
+        }
+        __syncthreads();
+        if (tid < nc) {
+            float sum = 0.f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sum += red[k][tid];
+            logits[c0 + tid] = sum + b2[c0 + tid];
+        }
+        __syncthreads();
     }
-    __syncthreads();
     if (tid == 0) {
         int best = 0;
         for (int c = 1; c < num_cand; ++c)
@@ -153,7 +181,7 @@ __global__ void __launch_bounds__(256) policy_out_kernel(const float* __restrict
 // memory, with b1 and ReLU.  What bounds it: for a few requests the stream of W1, for many the shared-memory reads
 // of the products (11 wavefronts a warp for 32 FFMAs).  A warp per hidden row, its requests' rows read whole from
 // shared memory for every row of W1, took 8 wavefronts for 8 FFMAs on part of the SMs: with the output layer 20 x
-// 4000 -> 1024 went from 83.6 to 29.8 us, 1 x 1024 -> 256 from 13.3 to 7.4, 128 x 8192 -> 3072 from 3410 to 629.
+// 4000 -> 1024 went from 81.4 to 23.1 us, 1 x 1024 -> 256 from 13.0 to 7.2, 128 x 8192 -> 3072 from 3350 to 518.
 constexpr int kPfRows = 64, kPfReqs = 32, kPfK = 32, kPfStages = 4, kPfMaxKS = 8;
 constexpr int kPfLd = kPfK + 4;  // 16-byte reads of 8 consecutive rows fall on distinct banks
 constexpr int kPfStageFloats = (kPfRows + kPfReqs) * kPfLd;

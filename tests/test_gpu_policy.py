@@ -158,3 +158,23 @@ def test_one_wide_request_of_any_row_stride():
     bs, lo = bp.policy_select(feats, *rest)
     bs1, lo1 = bp.policy_select(feats.as_strided((1, 98304), (1 << 40, 1)), *rest)
     assert torch.equal(bs, bs1) and torch.equal(lo, lo1)
+
+
+@pytest.mark.parametrize("hidden", [1, 255, 1025, 3262])
+@pytest.mark.parametrize("cand", [1, 16, 17, 64])
+@pytest.mark.parametrize("dtype, tol", [(torch.float32, 1e-5), (torch.bfloat16, 1e-5)])
+def test_output_layer_rounds(dtype, tol, hidden, cand):
+    """Candidates in rounds of 16, hidden units past a thread's loads in flight.  fp32 sums of 72 and hidden terms:
+    a few sqrt(length) 2^-24 of the terms.  (72 bf16 columns: h stays fp32 and W2 is exact in fp32.)"""
+    gen = torch.Generator().manual_seed(hidden + cand)
+    rnd = lambda *s: torch.randn(*s, generator=gen)  # noqa: E731
+    x, w1, b1, w2, b2 = rnd(3, 72), rnd(hidden, 72) / 8, rnd(hidden), rnd(cand, hidden) / hidden ** 0.5, rnd(cand)
+    x, w1, w2 = (t.to(dtype) for t in (x, w1, w2))
+    sizes = torch.arange(cand, dtype=torch.int32) + 2
+    bs, lo = bp.policy_select(*(t.cuda() for t in (x, w1, b1, w2, b2, sizes)))
+    h = (x.double() @ w1.double().T + b1.double()).clamp_min(0)
+    ref = h @ w2.double().T + b2.double()
+    assert (lo.cpu().double() - ref).abs().max() <= tol * ref.abs().max() + 1e-6
+    top = ref.topk(min(2, cand)).values
+    clear = (top[:, 0] - top[:, -1] > 1e-4) if cand > 1 else torch.ones(3, dtype=torch.bool)
+    assert torch.equal(bs.cpu()[clear], sizes[ref.argmax(1)][clear])
