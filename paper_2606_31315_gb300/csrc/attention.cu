@@ -24,7 +24,8 @@
 //   16 lanes of each TMEM sub-partition and each half-warp takes one 64-key half of a row, so
 //   all four softmax warps share the exp2 work.
 //
-// fp32 path (CUDA cores): register-tiled online softmax, keys split over a thread-block cluster.
+// fp32 path (CUDA cores): register-tiled online softmax, keys split over a thread-block cluster; contexts of a few
+// keys: a warp per row.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
@@ -1297,6 +1298,82 @@ __global__ void __launch_bounds__(kFThreads) attn_f32_kernel(const F32Params p) 
     }
 }
 
+// Contexts of a few keys: one warp per (query row, query head), online softmax over the row's visible keys in chunks
+// of 32 (lane = key), lane d-slices of the output.  Its chain grows with the keys, but it needs no shared memory to
+// speak of: thousands of short rows run at once where the tiled kernel takes one wave of two CTAs an SM after
+// another (8 heads of 64: 256 sequences of 5 keys 8.6 against 31.3 us, of 17 keys 20.1 and 31.4, of 41 48.4 and 32.0;
+// one of 5 keys and heads of 32 3.4 and 4.3).
+__global__ void __launch_bounds__(128) attn_f32_row_kernel(const float* __restrict__ q, const float* __restrict__ k,
+                                                            const float* __restrict__ v, float* __restrict__ o,
+                                                            float* __restrict__ lse, const int32_t* __restrict__ cu_q,
+                                                            const int32_t* __restrict__ cu_kv, int num_seqs,
+                                                            int total_q, int hq, int hkv, int D, int causal,
+                                                            float scale) {
+    __shared__ float qs[4][kF32MaxD];
+    griddep_launch_dependents();
+    griddep_wait();
+    const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long row = (long long)blockIdx.x * 4 + wib;
+    if (row >= (long long)total_q * hq) return;
+    const int t = (int)(row / hq), h = (int)(row % hq);
+    const int g = hq / hkv, kvh = h / g;
+    int lo = 0, hi = num_seqs;  // sequence containing query t: cu_q[s] <= t < cu_q[s+1]
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (cu_q[mid] <= t) lo = mid; else hi = mid;
+    }
+    const int s = lo;
+    const int B = cu_q[s + 1] - cu_q[s];
+    const int i = t - cu_q[s];
+    const int kv0 = cu_kv[s];
+    const int n = cu_kv[s + 1] - kv0;
+    const int L = n - B;
+    const int nk = causal ? L + i + 1 : n;
+    for (int d = lane; d < D; d += 32) qs[wib][d] = q[((size_t)t * hq + h) * D + d];
+    __syncwarp();
+    float m = -INFINITY, l = 0.f;
+    float acc[kF32MaxD / 32];
+#pragma unroll
+    for (int e = 0; e < kF32MaxD / 32; ++e) acc[e] = 0.f;
+    for (int j0 = 0; j0 < nk; j0 += 32) {
+        const int j = j0 + lane;
+        float sc = -INFINITY;
+        if (j < nk) {
+            const float* kr = k + ((size_t)(kv0 + j) * hkv + kvh) * D;
+            float dot = 0.f;
+            for (int d = 0; d < D; ++d) dot = fmaf(qs[wib][d], kr[d], dot);
+            sc = dot * scale;
+        }
+        float cm = sc;
+        for (int off = 16; off; off >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, off));
+        const float m_new = fmaxf(m, cm);
+        const float alpha = (m == -INFINITY) ? 0.f : expf(m - m_new);
+        const float pj = (j < nk) ? expf(sc - m_new) : 0.f;
+        float ps = pj;
+        for (int off = 16; off; off >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, off);
+        l = l * alpha + ps;
+#pragma unroll
+        for (int e = 0; e < kF32MaxD / 32; ++e) acc[e] *= alpha;
+        const int cnt = min(32, nk - j0);
+        for (int jj = 0; jj < cnt; ++jj) {
+            const float pjj = __shfl_sync(0xffffffffu, pj, jj);
+            const float* vr = v + ((size_t)(kv0 + j0 + jj) * hkv + kvh) * D;
+#pragma unroll
+            for (int e = 0; e < kF32MaxD / 32; ++e) {
+                const int d = lane + e * 32;
+                if (d < D) acc[e] = fmaf(pjj, vr[d], acc[e]);
+            }
+        }
+        m = m_new;
+    }
+#pragma unroll
+    for (int e = 0; e < kF32MaxD / 32; ++e) {
+        const int d = lane + e * 32;
+        if (d < D) o[((size_t)t * hq + h) * D + d] = acc[e] / l;
+    }
+    if (lse && lane == 0) lse[(size_t)t * hq + h] = m + logf(l);
+}
+
 }  // namespace
 
 namespace {
@@ -1643,8 +1720,34 @@ int launch_attention_f32(const AttentionArgs& a, const DeviceInfo& dev, cudaStre
     p.causal = a.mask == BP_MASK_CAUSAL_BLOCK;
     p.scale = a.scale;
     const long long units = (long long)a.num_seqs * a.num_kv_heads * p.m_tiles;
-    if (units > INT32_MAX) return BP_ERR_UNSUPPORTED;
     const int chunks = (a.max_kv_len + kFK - 1) / kFK;
+    // Up to one chunk of keys: a warp per row where that is faster, by estimates (us) fitted to 360 shapes timed both
+    // ways (1-256 sequences of 5-258 keys, blocks of 1-8, head_dim 32-128): a row's chain and the keys all rows read,
+    // against waves of tiles.
+    if (chunks <= 1) {
+        const double n = std::min(a.max_kv_len, a.total_kv), D = a.head_dim, rows = (double)a.total_q * a.num_q_heads;
+        const long long at_once = (a.head_dim <= 64 ? 2LL : 1LL) * dev.sm_count, waves = (units + at_once - 1) / at_once;
+        const double filled = std::min((long long)kFR, (long long)a.max_q_len * G) / (double)kFR;
+        const double est_rows = 2.0 + (0.19 + 0.002 * D) * n + 4.2e-6 * rows * n * D;
+        const double est_tiles =
+            waves * (a.head_dim <= 64 ? (waves == 1 ? 4.5 : 4.85) + 1.9 * filled : 5.3 + 3.9 * filled);
+        if (est_rows < est_tiles) {
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute attr[1];
+            cfg.gridDim = dim3((unsigned)(((long long)a.total_q * a.num_q_heads + 3) / 4), 1, 1);
+            cfg.blockDim = dim3(128, 1, 1);
+            cfg.stream = stream;
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            return cudaLaunchKernelEx(&cfg, attn_f32_row_kernel, p.q, p.k, p.v, p.o, p.lse, p.cu_q, p.cu_kv, a.num_seqs,
+                                      a.total_q, p.hq, p.hkv, p.D, p.causal, p.scale) == cudaSuccess
+                       ? BP_OK
+                       : BP_ERR_CUDA;
+        }
+    }
+    if (units > INT32_MAX) return BP_ERR_UNSUPPORTED;
     const auto aligned16 = [](const void* x) { return (reinterpret_cast<uintptr_t>(x) & 15) == 0; };
     const bool vec = a.head_dim % 4 == 0 && aligned16(a.q) && aligned16(a.k) && aligned16(a.v) && aligned16(a.o);
     if (a.head_dim <= 64)

@@ -213,6 +213,22 @@ def test_fp32_shapes(ctx, block, hq, hkv, d):
         assert err <= 1e-5 and lerr <= 1e-5, (err, lerr)
 
 
+@pytest.mark.parametrize("hq,hkv,d", [(8, 8, 32), (8, 2, 128), (6, 2, 33), (4, 1, 64)])
+@pytest.mark.parametrize("ctx,block", [
+    ((4,), (1,)), ((0,), (8,)), ((31,), (1,)), ((55,), (9,)),                 # one sequence, up to a chunk of keys
+    ((4, 0, 2, 16, 9) * 40, (1, 8, 0, 2, 3) * 40),                            # hundreds of short ones, some empty
+    ((40, 30, 0, 50) * 60, (1, 2, 8, 13) * 60),                               # on either side of the line by head_dim
+])
+def test_fp32_short_contexts(ctx, block, hq, hkv, d):
+    """Contexts of at most one 64-key chunk, by the row kernel or the tiled one.  Bars as test_fp32_shapes."""
+    w = wl.custom(seed=d + len(ctx), ctx=ctx, block=block, num_q_heads=hq, num_kv_heads=hkv, head_dim=d, dtype="f32")
+    a = wl.attention_inputs(w)
+    for mask in (CAUSAL, BIDIR):
+        o, lse = run_attention(a, mask)
+        err, lerr = attention_errors(o, lse, a, mask, range(0, len(ctx), max(1, len(ctx) // 8)))
+        assert err <= 1e-5 and lerr <= 1e-5, (err, lerr)
+
+
 def test_fp32_unaligned_bases():
     """Tensors that start off a 16-byte boundary give the same values as aligned ones (same order of sums)."""
     a = wl.attention_inputs(wl.custom(seed=3, ctx=(200, 30), block=(8, 5), num_q_heads=4, num_kv_heads=2, head_dim=64,
