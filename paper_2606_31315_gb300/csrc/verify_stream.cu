@@ -76,6 +76,7 @@ struct VsParams {
     int vec;                        // logits rows start 16-byte aligned
     int tma_store;                  // the group's rows are contiguous stacked rows: chunks go out by TMA
     int grows;                      // stacked rows of the group
+    int w_first;                    // W is loaded to leave L2 first
     float2* part;                   // [rows][nslices] slice statistics
     int nslices;
     unsigned int* err;
@@ -230,7 +231,7 @@ __global__ void __launch_bounds__(kVsThreads, 1)
         // ---- TMA producer: stage j = (pass j / atoms, hidden atom j % atoms): 256 W rows, the group's states
         if (lane == 0) {
             int issued = 0;
-            const uint64_t pol = l2_policy_evict_first();  // W is read once: it leaves L2 to the states and the logits
+            const uint64_t pol = p.w_first ? l2_policy_evict_first() : l2_policy_normal();
             for (int j = 0; j < J; ++j) {
                 const int st = j % STG;
                 if (j >= STG && !mbar_wait(&empty[st], ((j / STG) - 1) & 1, kWaitBudget)) {
@@ -422,6 +423,20 @@ int verify_stream_grid(int vocab, int sm_count) {
     return slice < 1 ? 0 : (vocab + slice - 1) / slice;
 }
 
+// When W is loaded to leave L2 first.  Without logits to write, in the last group of rows, which reads W for the last
+// time (64 rows, 128,256 x 1024: 46.8 us with, 47.8 without; 320 rows, 100,352 x 1024 in two groups: 78.3 in both, 75.9
+// in the last, 79.7 in none).  With logits, where a CTA has one or two passes: the group's logits wait in L2 for their
+// way to memory (120 rows, 40,000 x 1536: 39.7 and 43.2; 620 rows, 50,257 x 2560 192.8 and 200.4); with more passes the
+// write-back keeps up and the hint costs second reads of W (120 rows, 151,936 x 896: 71.3 and 67.5; 128,256 x 1024 68.2
+// and 65.3; 100,352 x 1024 53.5 and 53.2), but for two halves of rows on a head several times their logits (248 rows,
+// 151,936 x 2560: 184.3 and 186.1).  And not where W and the logits stay in L2 from call to call (120 rows, 32,000
+// x 1024: 24.2 and 19.6; 40,000 x 896 29.2 and 25.4).  Timed over 260 shapes of 48 to 1240 rows.
+static bool w_leaves_first(bool write, bool last_group, int rows, int slice, long long w_bytes, long long logits_bytes) {
+    if (!write) return last_group;
+    return w_bytes + logits_bytes > (95LL << 20) &&
+           (slice <= 2 * kVsN || (rows > kVsM && w_bytes >= 4 * logits_bytes));
+}
+
 int launch_verify_stream(const VerifyEpilogueArgs& a, const VerifyStreamScratch& s, const DeviceInfo& dev,
                          cudaStream_t stream) {
     const bool greedy = a.temperature == 0.f;
@@ -472,6 +487,8 @@ int launch_verify_stream(const VerifyEpilogueArgs& a, const VerifyStreamScratch&
         // TMA stores where state-tile row i is stacked row r0 + i for every row the group holds
         p.tma_store = p.vec && (p.nt % 8 == 0 || p.nd == 0);
         p.grows = r1 - r0;
+        p.w_first = w_leaves_first(write, r1 >= rows, r1 - r0, p.slice, (long long)a.vocab * a.hidden * 2,
+                                   (long long)(r1 - r0) * ld * 4);
         if (p.tma_store) {
             const cuuint64_t dims[2] = {(cuuint64_t)a.vocab, (cuuint64_t)(r1 - r0)};
             const cuuint64_t strides[1] = {(cuuint64_t)ld * 4};
