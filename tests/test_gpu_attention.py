@@ -3,8 +3,9 @@
 Tolerance: max |O - O_ref| / max |O_ref| <= 2e-2 per (sequence, query head) slice (bf16 inputs,
 fp32 accumulation); log-sum-exp within 2e-3.  Small ragged cases are compared in full, on both
 splits of the keys (the flat split and the cluster split, each forced, the cluster split also in
-clusters of 3: contexts this short stay in one CTA per unit when the library chooses, so the forced
-clusters keep the distributed-shared-memory merge covered at every group size); the full-size workloads run
+clusters of 3: contexts this short stay in one CTA per unit when the library chooses; those clusters
+merge through distributed shared memory, or through the workspace where a unit has at most 34 rows --
+test_cluster_merges takes both merges at other sizes); the full-size workloads run
 exactly as the benchmark launches them (the library's own choice of split) and are compared on
 sampled sequences (and KV heads for the 32K-context case).
 """
@@ -268,3 +269,48 @@ def test_uneven_batch_takes_the_flat_split():
     assert err <= ATTN_TOL and lerr <= LSE_TOL
     even = wl.attention_inputs(wl.custom(seed=8, ctx=(1500,) * 32, block=(16,) * 32, num_q_heads=32, num_kv_heads=8))
     assert not any("attn_combine_kernel" in x for x in _attn_kernels(even, "auto"))
+
+
+def _run(a, mask, split="auto", ws_bytes=None, max_kv=None, page=0):
+    """run_attention with a workspace of ws_bytes, another max_kv_len or a paged cache."""
+    from _gpu import attention_ws, forced_split
+
+    q, cu_q, cu_kv = to_dev(a["q"], "bf16"), to_dev(a["cu_q"]), to_dev(a["cu_kv"])
+    lse = torch.empty(q.shape[0], q.shape[1], device="cuda")
+    ws = attention_ws(a) if ws_bytes is None else bp.workspace(ws_bytes, "cuda")
+    max_kv = max_kv or a["max_kv_len"]
+    with forced_split(split):
+        if page:
+            pk = wl.paged_kv(a["k"], a["v"], a["cu_kv"], page, seed=page)
+            bt = np.zeros((len(a["cu_q"]) - 1, max(pk["block_table"].shape[1], -(-max_kv // page))), dtype=np.int32)
+            bt[:, :pk["block_table"].shape[1]] = pk["block_table"]
+            o, _ = bp.block_attention_paged(q, to_dev(pk["k_cache"], "bf16"), to_dev(pk["v_cache"], "bf16"), cu_q, cu_kv,
+                                            to_dev(bt), page, int(a["cu_kv"][-1]), a["max_q_len"], max_kv, mask=mask,
+                                            lse=lse, ws=ws)
+        else:
+            o, _ = bp.block_attention(q, to_dev(a["k"], "bf16"), to_dev(a["v"], "bf16"), cu_q, cu_kv, a["max_q_len"],
+                                      max_kv, mask=mask, lse=lse, ws=ws)
+    assert bp.get_status(ws) == 0
+    return o.float().cpu().numpy(), lse.cpu().numpy()
+
+
+@pytest.mark.parametrize("n", [4, 5, 8, 11, 16])
+@pytest.mark.parametrize("ctx,block,page", [
+    ((2100,), (1,), 0), ((2100,), (9,), 64), ((3000,), (12,), 0), ((2050,), (16,), 16), ((2500,), (24,), 0),
+    ((2080,), (32,), 128), ((2600, 200), (16, 3), 0), ((300, 2300), (24, 32), 64),
+])
+def test_cluster_merges(n, ctx, block, page):
+    """Clusters of n on both row layouts, merged through the workspace (where a CTA owns few rows) and, without the
+    workspace, through distributed shared memory: one sequence, or two of which one has fewer tiles than CTAs; owners
+    with fewer rows than others or none; 2 KV heads, so that clusters of 16 are resident.  Both merges add the same
+    partials in fp32, in another order: they differ by bf16 roundings of the output, 2^-8 of its size at most."""
+    a = wl.attention_inputs(wl.custom(seed=n + ctx[0], ctx=ctx, block=block, num_q_heads=8, num_kv_heads=2))
+    for mask in (CAUSAL, BIDIR):
+        full = _run(a, mask, f"cluster:{n}", page=page)
+        chip = _run(a, mask, f"cluster:{n}", ws_bytes=256, page=page)
+        for o, lse in (full, chip):
+            err, lerr = attention_errors(o, lse, a, mask, range(len(ctx)))
+            assert err <= ATTN_TOL and lerr <= LSE_TOL
+        assert np.abs(full[0] - chip[0]).max() <= 2 ** -8 * max(1.0, np.abs(full[0]).max())
+        np.testing.assert_allclose(full[1], chip[1], rtol=0, atol=1e-5)
+
