@@ -33,6 +33,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 
 #include "common.cuh"
@@ -57,6 +58,7 @@ constexpr uint32_t kTmemCols = 512;
 static_assert(kDynSmem >= tmem_smem_share((int)kTmemCols, 228 * 1024), "leaves no other CTA's tensor memory room");
 constexpr uint32_t kColO = 384;
 constexpr int kMaxOrderedSeqs = 256;  // longest-first ordering for batches up to this size
+constexpr int kMaxDealtSeqs = 64;     // flat split: batches whose units may be dealt out instead of cut evenly
 constexpr int kMaxCluster = 16;
 
 struct AttnParams {
@@ -76,10 +78,13 @@ struct AttnParams {
     int pages_per_seq, page_shift;
     // flat split: partial (O, m, l) slots in the workspace, two per CTA, slot_rows rows each; and one
     // work entry (two int4) per CTA for the merge: (first tile, end tile, all tiles, rows) and (first
-    // query row, query tile) of the cut unit whose first tile the CTA holds, or first tile -1
+    // query row, query tile, parts) of the cut unit whose first tile the CTA holds, or first tile -1; parts > 0:
+    // the unit lies in the first slots of that many CTA groups from this one on
     float* part;
     int4* work;
     int slot_rows;
+    float us_whole, us_part, us_cut;  // flat split: us per key tile of whole units, of parts, with every SM streaming
+    int sm_count, ahead_ok;  // flat split: may K's ring refill ahead of V's (pages of at least 32 keys)
     int early_release;  // the grid is one wave of short runs: dependents may launch as soon as every CTA has started
     unsigned int* err;
 };
@@ -114,6 +119,7 @@ struct Seg {
     int jt0, nt;        // first tile of the stretch within the unit, tiles in it
     int whole;          // flat split: the stretch is the whole unit (the CTA writes the output)
     int slot;           // flat split, part of a unit: the CTA's partial slot (0 first stretch, 1 last)
+    int parts;          // flat split, units dealt out: the parts the unit is cut into (0: cut evenly with the others)
 };
 
 // Flat split: key tiles of every sequence over its 128-row query tiles, counted once for all KV heads
@@ -123,35 +129,42 @@ __device__ __forceinline__ int flat_seq_tiles(int B, int n, int G) {
     return B > 0 ? cdiv(B * G, kM) * cdiv(n, kTileN) : 0;
 }
 
-// Flat split: the prefix sums of the sequences' tile counts into pre[0..S] (S <= kMaxOrderedSeqs), by one
-// warp: each lane sums 8 consecutive sequences, then an exclusive scan of the lane sums.
-__device__ __forceinline__ void flat_prefix(const AttnParams& p, int32_t* pre, int lane) {
-    constexpr int kPer = (kMaxOrderedSeqs + 31) / 32;
-    int loc[kPer];
-    int run = 0;
+// Flat split: the prefix sums of the sequences' tile counts into pre[0..S] (S <= kMaxOrderedSeqs), by the whole CTA:
+// every thread loads its own sequences' offsets (one round trip), then one warp's lanes sum 8 consecutive counts and
+// scan the lane sums.
+__device__ __forceinline__ void flat_prefix(const AttnParams& p, int32_t* pre, int tid) {
+    constexpr int kPer = kMaxOrderedSeqs / 32;
+    static_assert(kPer * 32 == kMaxOrderedSeqs, "whole lanes");
+    for (int s = tid; s < p.num_seqs; s += kThreads) {
+        const int B = __ldg(p.cu_q + s + 1) - __ldg(p.cu_q + s);
+        const int n = __ldg(p.cu_kv + s + 1) - __ldg(p.cu_kv + s);
+        pre[s + 1] = flat_seq_tiles(B, n, p.group);
+    }
+    __syncthreads();
+    if (tid < 32) {
+        int loc[kPer];
+        int run = 0;
 #pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        const int s = lane * kPer + k;
-        if (s < p.num_seqs) {
-            const int B = __ldg(p.cu_q + s + 1) - __ldg(p.cu_q + s);
-            const int n = __ldg(p.cu_kv + s + 1) - __ldg(p.cu_kv + s);
-            run += flat_seq_tiles(B, n, p.group);
+        for (int k = 0; k < kPer; ++k) {
+            const int s = tid * kPer + k;
+            if (s < p.num_seqs) run += pre[s + 1];
+            loc[k] = run;
         }
-        loc[k] = run;
-    }
-    int incl = run;
+        int incl = run;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const int excl = incl - run;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (tid >= o) incl += y;
+        }
+        const int excl = incl - run;
 #pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        const int s = lane * kPer + k;
-        if (s < p.num_seqs) pre[s + 1] = excl + loc[k];
+        for (int k = 0; k < kPer; ++k) {
+            const int s = tid * kPer + k;
+            if (s < p.num_seqs) pre[s + 1] = excl + loc[k];
+        }
+        if (tid == 0) pre[0] = 0;
     }
-    if (lane == 0) pre[0] = 0;
+    __syncthreads();
 }
 
 // Flat split: the stretch that starts at global tile t of a CTA (KV head h) whose range ends at t_end
@@ -181,6 +194,37 @@ __device__ __forceinline__ Seg flat_seg(const AttnParams& p, const int32_t* pre,
     g.nt = min(ntu - g.jt0, t_end - t);
     g.whole = g.jt0 == 0 && g.nt == ntu;
     g.slot = first ? 0 : 1;
+    g.parts = 0;
+    return g;
+}
+
+// Flat split, units dealt out: the parts of a unit of L tiles where c groups of CTAs are free for each (the cluster
+// split's rule: a merge costs about three tiles of one CTA's chain).
+__device__ __forceinline__ int dealt_parts(int L, int c) { return L - cdiv(L, c) >= 3 ? min(c, L) : 1; }
+
+// Flat split, units dealt out: the rank (longest first) of the t-th unit of CTA group grp of ng, S sequences: c = ng / S
+// groups a unit, or rounds there and back over the groups.
+__device__ __forceinline__ int dealt_rank(int t, int grp, int ng, int c) {
+    return c >= 1 ? grp / c : t * ng + ((t & 1) ? ng - 1 - grp : grp);
+}
+
+// ... and its stretch (order: the sequences by rank).
+__device__ __forceinline__ Seg dealt_seg(const AttnParams& p, const uint8_t* order, int t, int grp, int ng, int c, int h) {
+    Seg g;
+    g.s = order[dealt_rank(t, grp, ng, c)];
+    g.q0 = __ldg(p.cu_q + g.s);
+    g.B = __ldg(p.cu_q + g.s + 1) - g.q0;
+    g.kv0 = __ldg(p.cu_kv + g.s);
+    g.n = __ldg(p.cu_kv + g.s + 1) - g.kv0;
+    g.h = h;
+    g.mt = 0;
+    const int L = cdiv(g.n, kTileN);
+    g.parts = c >= 1 ? dealt_parts(L, c) : 1;
+    const int part = c >= 1 ? grp - grp / c * c : 0;
+    g.jt0 = part * L / g.parts;
+    g.nt = (part + 1) * L / g.parts - g.jt0;
+    g.whole = g.parts == 1;
+    g.slot = 0;
     return g;
 }
 
@@ -192,15 +236,16 @@ __device__ __forceinline__ Seg flat_seg(const AttnParams& p, const int32_t* pre,
 // 64-column halves of a row (tcgen05 16x32bx2 accesses), combining row statistics by shuffle.
 // FLAT: the flat split.  The key tiles of all units, in order, are cut into gridDim.x equal ranges,
 // one per CTA (no clusters); a CTA works through the stretches of its range one after another with
-// one pipeline (K/V ring, S double buffer, O accumulator) and writes a unit it covers whole straight
-// to the output, a partial stretch to its workspace slot for attn_combine_kernel.  Otherwise the
-// cluster split: a unit per cluster, its tiles cut into CS ranges, partials merged through
-// distributed shared memory.
+// one pipeline (K/V ring, S/P buffers, O accumulator) and writes a unit it covers whole straight
+// to the output, a partial stretch to its workspace slot for attn_combine_kernel.  FLAT == 2: where the lengths turn
+// out even (the host knows only a bound and their sum), the CTAs deal the units out instead, longest first, whole
+// or in equal parts.  Otherwise the cluster split: a unit per cluster, its tiles cut into CS ranges, partials merged
+// through distributed shared memory or the workspace.
 // AHEAD (cluster split): K and V are separate rings.  K's stage is free after Q K^T, a softmax and a P V before
 // V's, and refills then, V a tile behind (the order in which the stages come free); with the rings joined both
 // wait for the tile's P V and only one of the three stages is in flight.  Where the line lies:
 // launch_attention_bf16.
-template <bool PAGED, bool SPREAD, bool FLAT, bool AHEAD>
+template <bool PAGED, bool SPREAD, int FLAT, bool AHEAD>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_bf16_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
                         const __grid_constant__ CUtensorMap vmap, const AttnParams p) {
@@ -221,6 +266,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     __shared__ int unit_seq_sh;
     // cluster split: the sequences' key offsets (longest-first order); flat split: their tile prefix sums
     __shared__ int32_t seq_sh[kMaxOrderedSeqs + 1];
+    __shared__ uint8_t order_sh[FLAT == 2 ? kMaxDealtSeqs : 1];  // units dealt out: the sequences, longest first
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
@@ -237,19 +283,76 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     // ---- work assignment.  Flat split: global tiles [t_lo, t_hi).  Cluster split: one stretch, `one`.
     int t_lo = 0, t_hi = 0, T = 0;
+    bool dealt = false;
+    bool ahead = AHEAD && !FLAT;  // (flat split: where every CTA has one stretch)
     Seg one{};
+    const int ngroups = FLAT ? gridDim.x / p.num_kv_heads : 1, grp = FLAT ? blockIdx.x / p.num_kv_heads : 0;
+    const int free_groups = FLAT == 2 ? ngroups / p.num_seqs : 0;  // groups of CTAs per unit, if at least one
     if (FLAT) {
         if (p.num_seqs > 1) {
-            if (warp == 0) flat_prefix(p, seq_sh, lane);
-            __syncthreads();
+            flat_prefix(p, seq_sh, tid);
             T = seq_sh[p.num_seqs];
         } else {
             T = flat_seq_tiles(p.total_q, p.total_kv, G);
         }
         // CTAs come in groups of one per KV head; group j has tiles [t_lo, t_hi) of every head
-        const int ngroups = gridDim.x / p.num_kv_heads, grp = blockIdx.x / p.num_kv_heads;
         t_lo = (int)((long long)grp * T / ngroups);
         t_hi = (int)((long long)(grp + 1) * T / ngroups);
+        // Lengths the host could only bound: even cuts, or the units dealt out -- by the host's estimates, on the
+        // lengths as they are.  Every CTA decides the same.  (16 x 2016 keys in a cache of 8192: 37.0 us cut evenly,
+        // 29.7 dealt out, 26.9 in clusters.)
+        const int S = p.num_seqs;
+        if constexpr (FLAT == 2) {  // (1 < S <= kMaxDealtSeqs, one query tile)
+            if (tid == 0) unit_seq_sh = 0;
+            if (tid < S) {
+                const int len = seq_sh[tid + 1] - seq_sh[tid];
+                int rank = 0;
+                for (int u = 0; u < S; ++u) {
+                    const int lu = seq_sh[u + 1] - seq_sh[u];
+                    rank += (lu > len) || (lu == len && u < tid);
+                }
+                order_sh[rank] = (uint8_t)tid;
+            }
+            __syncthreads();
+            const auto tiles_of = [&](int rank) { return seq_sh[order_sh[rank] + 1] - seq_sh[order_sh[rank]]; };
+            const int rounds = cdiv(S, ngroups), longest = tiles_of(0);
+            int chain;  // key tiles of the busiest CTA
+            if (free_groups >= 1) {
+                chain = cdiv(longest, dealt_parts(longest, free_groups));
+            } else {
+                for (int g = tid; g < ngroups; g += kThreads) {
+                    int sum = 0;
+                    for (int t = 0; t < rounds; ++t) {
+                        const int rank = dealt_rank(t, g, ngroups, 0);
+                        if (rank < S) sum += tiles_of(rank);
+                    }
+                    atomicMax(&unit_seq_sh, sum);
+                }
+                __syncthreads();
+                chain = unit_seq_sh;
+            }
+            const float even = p.us_cut * (float)T / (float)ngroups;
+            const float est_cut = even + 10.f + fminf(4.2f * (1.f + (float)S / (float)ngroups), 11.f);
+            const float est_dealt = free_groups >= 1 && chain < longest
+                                        ? fmaxf(p.us_part * (float)chain, even) + 10.5f
+                                        : fmaxf(p.us_whole * (float)chain, even) + 9.5f + 4.f * (float)(rounds - 1);
+            dealt = est_dealt < est_cut;
+            if (dealt) {
+                const int parts = free_groups >= 1 ? dealt_parts(longest, free_groups) : 0;
+                ahead = AHEAD && p.ahead_ok && parts >= 1 && parts <= 5 && chain >= 6 &&
+                        S * parts * p.num_kv_heads * 10 <= 9 * p.sm_count;
+                t_lo = 0;
+                t_hi = 0;
+                if (free_groups >= 1) {
+                    const int rank = grp / free_groups, part = grp - rank * free_groups;
+                    t_hi = rank < S && tiles_of(rank) > 0 && part < dealt_parts(tiles_of(rank), free_groups) ? 1 : 0;
+                } else {
+                    while (t_hi < rounds && dealt_rank(t_hi, grp, ngroups, 0) < S &&
+                           tiles_of(dealt_rank(t_hi, grp, ngroups, 0)) > 0)
+                        ++t_hi;
+                }
+            }
+        }
     } else {
         const int unit_rank = blockIdx.x / CS;
         const int units_per_seq = p.num_kv_heads * p.m_tiles;
@@ -292,14 +395,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         one.nt = (int)((long long)(crank + 1) * tiles / CS) - one.jt0;
         one.whole = 0;
         one.slot = 0;
+        one.parts = 0;
     }
     // The stretches of this CTA, in order: `first` is the CTA's first one; t advances past each.
     auto seg_at = [&](int t, bool first) -> Seg {
-        return FLAT ? flat_seg(p, seq_sh, t, t_hi, (int)(blockIdx.x % p.num_kv_heads), first) : one;
+        if (!FLAT) return one;
+        const int h = (int)(blockIdx.x % p.num_kv_heads);
+        return FLAT == 2 && dealt ? dealt_seg(p, order_sh, t, grp, ngroups, free_groups, h)
+                                  : flat_seg(p, seq_sh, t, t_hi, h, first);
     };
     const int t_begin = FLAT ? t_lo : 0;
     const int t_end = FLAT ? t_hi : 1;
-    auto seg_len = [&](const Seg& g) { return FLAT ? g.nt : 1; };
+    auto seg_len = [&](const Seg& g) { return FLAT && !(FLAT == 2 && dealt) ? g.nt : 1; };
 
     // ---- Q tile -> shared memory, SWIZZLE_128B K-major (two 64-column halves).  With a TMA map the
     // 128/G block positions x G heads box lands exactly as rows r = i*G + j; otherwise (cluster split
@@ -360,13 +467,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
     auto issue_k = [&](int J, const Seg& g, int jl, const int (&row)[kMaxSub]) {
         const int st = J % kStages;
-        uint64_t* bar = AHEAD ? &bar_k_full[st] : &bar_kv_full[st];
-        mbar_arrive_expect_tx(bar, AHEAD ? kKVBytes : kStageBytes);  // not AHEAD: V's bytes too
+        uint64_t* bar = ahead ? &bar_k_full[st] : &bar_kv_full[st];
+        mbar_arrive_expect_tx(bar, ahead ? kKVBytes : kStageBytes);  // not ahead: V's bytes too
         load_rows(sKV + st * kStageBytes, &kmap, bar, g, jl, row);
     };
     auto issue_v = [&](int J, const Seg& g, int jl, const int (&row)[kMaxSub]) {
         const int st = J % kStages;
-        if (AHEAD) mbar_arrive_expect_tx(&bar_kv_full[st], kKVBytes);
+        if (ahead) mbar_arrive_expect_tx(&bar_kv_full[st], kKVBytes);
         load_rows(sKV + st * kStageBytes + kKVBytes, &vmap, &bar_kv_full[st], g, jl, row);
     };
     // the Q tile of stretch g (producer thread only)
@@ -431,13 +538,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int jl = 0; jl < g.nt; ++jl, ++J) {
                     int rows[kMaxSub];
                     tile_rows(g, jl, rows);  // page lookups in flight while the stage drains
-                    if (J >= kStages && !mbar_wait(AHEAD ? &bar_k_empty[J % kStages] : &bar_done[J % kStages],
+                    if (J >= kStages && !mbar_wait(ahead ? &bar_k_empty[J % kStages] : &bar_done[J % kStages],
                                                    ((J / kStages) - 1) & 1, kWaitBudget)) {
                         ok = false;
                         break;
                     }
                     issue_k(J, g, jl, rows);
-                    if (AHEAD) {  // one stretch: tile J - 1's V, once its stage is free
+                    if (ahead) {  // one stretch: tile J - 1's V, once its stage is free
                         if (J > 0) {
                             if (jv >= kStages &&
                                 !mbar_wait(&bar_done[jv % kStages], ((jv / kStages) - 1) & 1, kWaitBudget)) {
@@ -466,7 +573,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         ++nq;
                     }
                 }
-                if (AHEAD && ok) {  // the last tile's V
+                if (ahead && ok) {  // the last tile's V
                     ok = jv < kStages || mbar_wait(&bar_done[jv % kStages], ((jv / kStages) - 1) & 1, kWaitBudget);
                     if (ok) {
                         issue_v(jv, g, jv, rows_v);
@@ -476,10 +583,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             if (!ok) raise_error(p.err, kErrTimeout);
             // no copy may still be in flight when the CTA leaves
-            const int nv = AHEAD ? jv : J;
+            const int nv = ahead ? jv : J;
             for (int j = max(0, nv - kStages); j < nv; ++j)
                 if (!mbar_wait(&bar_kv_full[j % kStages], (j / kStages) & 1, kDrainBudget)) raise_error(p.err, kErrTimeout);
-            if (AHEAD)
+            if (ahead)
                 for (int j = max(0, J - kStages); j < J; ++j)
                     if (!mbar_wait(&bar_k_full[j % kStages], (j / kStages) & 1, kDrainBudget)) raise_error(p.err, kErrTimeout);
             if (nq > 0 && !mbar_wait(&bar_q_full, (nq - 1) & 1, kDrainBudget)) raise_error(p.err, kErrTimeout);
@@ -494,7 +601,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             bool ok = true;
             auto issue_pv = [&](int Jx, bool first) {
                 const int st = Jx % kStages;
-                if (AHEAD && !mbar_wait(&bar_kv_full[st], (Jx / kStages) & 1, kWaitBudget)) return false;
+                if (ahead && !mbar_wait(&bar_kv_full[st], (Jx / kStages) & 1, kWaitBudget)) return false;
                 if (!mbar_wait(&bar_p_full[st], (Jx / kStages) & 1, kWaitBudget)) return false;
                 tc_fence_after();
                 const uint32_t v_addr = smem_addr(sKV + st * kStageBytes + kKVBytes);
@@ -517,8 +624,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int jl = 0; jl < g.nt; ++jl, ++J) {
                     // (the stage was refilled after the P V of tile J - kStages, so its S buffer is free too)
                     const int st = J % kStages;
-                    if (!mbar_wait(AHEAD ? &bar_k_full[st] : &bar_kv_full[st], (J / kStages) & 1, kWaitBudget)) { ok = false; break; }
-                    if (AHEAD && J >= kStages && !mbar_wait(&bar_done[st], ((J / kStages) - 1) & 1, kWaitBudget)) { ok = false; break; }
+                    if (!mbar_wait(ahead ? &bar_k_full[st] : &bar_kv_full[st], (J / kStages) & 1, kWaitBudget)) { ok = false; break; }
+                    if (ahead && J >= kStages && !mbar_wait(&bar_done[st], ((J / kStages) - 1) & 1, kWaitBudget)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t k_addr = smem_addr(sKV + st * kStageBytes);
 #pragma unroll
@@ -529,7 +636,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         umma_ss(tmem + col_s(st), adesc, bdesc, id_s, kk > 0 ? 1u : 0u);
                     }
                     umma_commit(&bar_s_full[st]);
-                    if (AHEAD) umma_commit(&bar_k_empty[st]);
+                    if (ahead) umma_commit(&bar_k_empty[st]);
                     if (jl == g.nt - 1) umma_commit(&bar_q_empty);  // the last read of this stretch's Q
                     if (jl >= 1 && !issue_pv(J - 1, jl == 1)) { ++J; ok = false; break; }
                 }
@@ -594,7 +701,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const Seg g = seg_at(t, t == t_begin);
             if (FLAT && !g.whole && g.jt0 == 0) {  // a cut unit that starts here
                 entry = make_int4(t, t + cdiv(g.n, kTileN), T, min(min(kM, g.B * G - g.mt * kM), p.slot_rows));
-                entry2 = make_int4(g.q0, g.mt, 0, 0);
+                entry2 = make_int4(g.q0, g.mt, g.parts, 0);
             }
             t += seg_len(g);
             const int row0 = g.mt * kM;
@@ -931,37 +1038,29 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // Flat split, second kernel: the units whose tiles were cut between CTA groups.  The CTA of the main
-// kernel that holds a cut unit's first tile names it in its work entry; CTA (c, r) here takes work entry
-// c and its rows [r * kCombRows, (r + 1) * kCombRows).  Thread (row, 16-byte chunk) merges the partial
+// kernel that holds a cut unit's first tile names it in its work entry.  Thread (row, 16-byte chunk) merges the partial
 // (O, m, l) of the unit's CTAs in order -- O = sum_j 2^(m_j - M) O_j / sum_j 2^(m_j - M) l_j, M the
 // largest m_j, as a running merge over batches of kCombBatch partials whose loads are all in flight --
 // and writes the bf16 output chunk (and the row's log-sum-exp).
 constexpr int kCombRows = 8;
 constexpr int kCombThreads = kCombRows * kD / 4;  // 256: one 16-byte chunk of a row each
 constexpr int kCombBatch = 8;
-__global__ void __launch_bounds__(kCombThreads) attn_combine_kernel(const AttnParams p, int grid_main) {
-    __shared__ int32_t gstart[kAttnFlatMaxGrid + 1];  // the CTA groups' ranges: group j has [gstart[j], gstart[j+1])
-    griddep_launch_dependents();
-    griddep_wait();  // the partials and work entries of the main kernel
-    const int tid = threadIdx.x;
-    const int G = p.group;
-    const int chunks = (p.slot_rows + kCombRows - 1) / kCombRows;
-    const int c = blockIdx.x / chunks, r = blockIdx.x - c * chunks;
-    const int4 wk = __ldcg(p.work + 2 * c), wk2 = __ldcg(p.work + 2 * c + 1);
-    if (wk.x < 0) return;  // CTA c holds no cut unit's first tile (uniform per CTA)
-    const int U0 = wk.x, U1 = wk.y, T = wk.z, rows = wk.w, q0 = wk2.x, mt = wk2.y;
+
+// Rows [r * kCombRows, (r + 1) * kCombRows) of the cut unit of work entry (wk, wk2) of CTA c; gstart: the CTA groups'
+// ranges, group j has [gstart[j], gstart[j + 1]) (not read for a unit dealt out).
+__device__ __forceinline__ void combine_rows(const AttnParams& p, const int32_t* gstart, int ngroups, const int4& wk,
+                                             const int4& wk2, int c, int r) {
+    const int tid = threadIdx.x, G = p.group;
+    const int U0 = wk.x, U1 = wk.y, rows = wk.w, q0 = wk2.x, mt = wk2.y;
+    const int parts = wk2.z;  // dealt out: the first slots of this many groups
     const int h = c % p.num_kv_heads;
-    if (r * kCombRows >= rows) return;  // uniform per CTA
-    const int ngroups = grid_main / p.num_kv_heads;
-    for (int j = tid; j <= ngroups; j += kCombThreads) gstart[j] = (int)((long long)j * T / ngroups);
-    __syncthreads();
-    // the group whose range holds the unit's last tile: the last j with gstart[j] <= U1 - 1
     int lo = c / p.num_kv_heads, hi = ngroups;
-    while (hi - lo > 1) {
+    // the group whose range holds the unit's last tile: the last j with gstart[j] <= U1 - 1
+    while (parts == 0 && hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
         if (gstart[mid] <= U1 - 1) lo = mid; else hi = mid;
     }
-    const int j0 = c / p.num_kv_heads, j1 = lo;
+    const int j0 = c / p.num_kv_heads, j1 = parts > 0 ? j0 + parts - 1 : lo;
     const int rl = r * kCombRows + tid / (kD / 4);  // the row within the unit
     const int c4 = tid % (kD / 4);                  // its 16-byte chunk
     if (rl >= rows) return;
@@ -977,10 +1076,10 @@ __global__ void __launch_bounds__(kCombThreads) attn_combine_kernel(const AttnPa
             const int j = jb + k;
             ml[k] = make_float2(-INFINITY, 0.f);
             v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (j <= j1 && gstart[j] < gstart[j + 1]) {
+            if (j <= j1 && (parts > 0 || gstart[j] < gstart[j + 1])) {
                 // CTA (group j, head h): its first stretch (slot 0) unless its range began before the unit
-                const float* sp =
-                    p.part + (size_t)(2 * (j * p.num_kv_heads + h) + (gstart[j] >= U0 ? 0 : 1)) * slot_floats;
+                const float* sp = p.part + (size_t)(2 * (j * p.num_kv_heads + h) +
+                                                    (parts > 0 || gstart[j] >= U0 ? 0 : 1)) * slot_floats;
                 ml[k] = __ldcg(reinterpret_cast<const float2*>(sp + ml_off));
                 v[k] = __ldcg(reinterpret_cast<const float4*>(sp + (size_t)rl * kD + c4 * 4));
             }
@@ -1013,6 +1112,60 @@ __global__ void __launch_bounds__(kCombThreads) attn_combine_kernel(const AttnPa
     w2.y = pack_bf16x2(acc.z * inv, acc.w * inv);
     *reinterpret_cast<uint2*>(p.o + orow * kD + c4 * 4) = w2;
     if (p.lse && c4 == 0) p.lse[orow] = (M + __log2f(Lsum)) * 0.6931471805599453f;
+}
+
+// LIST = false: CTA (c, r) takes work entry c and its piece r.  LIST = true, behind the kernel that may have dealt the
+// units out so that few or none were cut: three CTAs an SM list the cut units and take their pieces in turn.  (A CTA
+// for every piece there could be takes 2.6 us where nothing was cut, the list 1.5; where most units were cut both take
+// the same, and with one unit per head the list 0.5 us more.)
+constexpr int kCombPerSm = 3;
+static_assert(kCombThreads >= kAttnFlatMaxGrid, "a thread per work entry");
+template <bool LIST>
+__global__ void __launch_bounds__(kCombThreads, kCombPerSm) attn_combine_kernel(const AttnParams p, int grid_main) {
+    __shared__ int32_t gstart[kAttnFlatMaxGrid + 1];
+    griddep_launch_dependents();
+    griddep_wait();  // the partials and work entries of the main kernel
+    const int tid = threadIdx.x, ngroups = grid_main / p.num_kv_heads;
+    const int chunks = (p.slot_rows + kCombRows - 1) / kCombRows;
+    auto ranges = [&](int T) {
+        for (int j = tid; j <= ngroups; j += kCombThreads) gstart[j] = (int)((long long)j * T / ngroups);
+        __syncthreads();
+    };
+    if constexpr (!LIST) {
+        const int c = blockIdx.x / chunks, r = blockIdx.x - c * chunks;
+        const int4 wk = __ldcg(p.work + 2 * c), wk2 = __ldcg(p.work + 2 * c + 1);
+        if (wk.x < 0 || r * kCombRows >= wk.w) return;  // CTA c holds no cut unit's first tile, or it has no such rows
+        ranges(wk.z);
+        combine_rows(p, gstart, ngroups, wk, wk2, c, r);
+    } else {
+        __shared__ int4 unit[kAttnFlatMaxGrid], unit2[kAttnFlatMaxGrid];  // the cut units' entries; their CTA in .w
+        __shared__ int cuts[kCombThreads / 32];
+        int4 mine = make_int4(-1, 0, 0, 0), mine2 = mine;
+        if (tid < grid_main) {
+            mine = __ldcg(p.work + 2 * tid);
+            mine2 = __ldcg(p.work + 2 * tid + 1);
+        }
+        const unsigned ball = __ballot_sync(0xffffffffu, mine.x >= 0);
+        if ((tid & 31) == 0) cuts[tid >> 5] = __popc(ball);
+        __syncthreads();
+        int n = 0, at = __popc(ball & ((1u << (tid & 31)) - 1u));
+#pragma unroll
+        for (int w = 0; w < kCombThreads / 32; ++w) {
+            if (w < (tid >> 5)) at += cuts[w];
+            n += cuts[w];
+        }
+        if (n == 0) return;
+        if (mine.x >= 0) {
+            unit[at] = mine;
+            unit2[at] = make_int4(mine2.x, mine2.y, mine2.z, tid);
+        }
+        __syncthreads();
+        if (unit2[0].z == 0) ranges(unit[0].z);  // cut evenly: every entry names the same number of tiles
+        for (int piece = blockIdx.x; piece < n * chunks; piece += gridDim.x) {
+            const int4 wk2 = unit2[piece / chunks];
+            combine_rows(p, gstart, ngroups, unit[piece / chunks], wk2, wk2.w, piece % chunks);
+        }
+    }
 }
 
 // --------------------------------------------------------------------------- fp32 path
@@ -1392,15 +1545,18 @@ size_t attention_flat_scratch_bytes(int max_q_len, int group) {
 }
 
 namespace {
-// The instantiations: [variant][spread][paged], variants cluster split, cluster split AHEAD, flat split.
+// The instantiations: [variant][spread][paged], variants cluster split, cluster split AHEAD, flat split, flat split or
+// dealt out.
 using AttnKernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, AttnParams);
-const AttnKernel kAttnKernels[12] = {
-    attn_bf16_tc_kernel<false, false, false, false>, attn_bf16_tc_kernel<true, false, false, false>,
-    attn_bf16_tc_kernel<false, true, false, false>,  attn_bf16_tc_kernel<true, true, false, false>,
-    attn_bf16_tc_kernel<false, false, false, true>,  attn_bf16_tc_kernel<true, false, false, true>,
-    attn_bf16_tc_kernel<false, true, false, true>,   attn_bf16_tc_kernel<true, true, false, true>,
-    attn_bf16_tc_kernel<false, false, true, false>,  attn_bf16_tc_kernel<true, false, true, false>,
-    attn_bf16_tc_kernel<false, true, true, false>,   attn_bf16_tc_kernel<true, true, true, false>};
+const AttnKernel kAttnKernels[16] = {
+    attn_bf16_tc_kernel<false, false, 0, false>, attn_bf16_tc_kernel<true, false, 0, false>,
+    attn_bf16_tc_kernel<false, true, 0, false>,  attn_bf16_tc_kernel<true, true, 0, false>,
+    attn_bf16_tc_kernel<false, false, 0, true>,  attn_bf16_tc_kernel<true, false, 0, true>,
+    attn_bf16_tc_kernel<false, true, 0, true>,   attn_bf16_tc_kernel<true, true, 0, true>,
+    attn_bf16_tc_kernel<false, false, 1, false>, attn_bf16_tc_kernel<true, false, 1, false>,
+    attn_bf16_tc_kernel<false, true, 1, false>,  attn_bf16_tc_kernel<true, true, 1, false>,
+    attn_bf16_tc_kernel<false, false, 2, true>,  attn_bf16_tc_kernel<true, false, 2, true>,
+    attn_bf16_tc_kernel<false, true, 2, true>,   attn_bf16_tc_kernel<true, true, 2, true>};
 }  // namespace
 
 int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStream_t stream) {
@@ -1505,7 +1661,7 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
     for (int c = 0; c <= kMaxCluster; ++c) max_active[c] = max_active_dev[dev.device][c];
     cfg_lock.unlock();
 
-    const int max_tiles = (a.max_kv_len + kTileN - 1) / kTileN;
+    const int max_tiles = (std::min(a.max_kv_len, a.total_kv) + kTileN - 1) / kTileN;  // of the longest, at most
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     cfg.blockDim = dim3(kThreads, 1, 1);
@@ -1552,7 +1708,8 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
     // head and per SM (at most kAttnFlatMaxGrid in all, and no more groups than one head has tiles); units
     // cut between groups are merged by a second kernel.  It needs the Q tile by TMA, the sequences'
     // offsets in shared memory and the workspace's partial slots and work entries.  BP_ATTENTION_SPLIT=flat or
-    // =cluster overrides the choice, =cluster:N also the cluster size (for tests and measurements).
+    // =cluster overrides the choice, =cluster:N also the cluster size, =dealt lets the kernel choose between cuts and
+    // dealing (for tests and measurements).
     const long long tiles_bound = (long long)a.num_seqs * m_tiles * max_tiles;
     const int ngroups = (int)std::min<long long>(std::min(dev.sm_count, kAttnFlatMaxGrid) / a.num_kv_heads,
                                                  tiles_bound);
@@ -1562,43 +1719,86 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
     const long long cluster_ctas = units * cs;
     const double avg_tiles = (double)a.num_kv_heads * m_tiles * ((double)a.total_kv / kTileN + 0.5 * a.num_seqs) /
                              dev.sm_count;
-    // Estimates (us) of both splits, fitted to 100 shapes timed in both (1-128 sequences of 200-160K keys).
+    // Estimates (us) of both splits, fitted to 100 shapes timed in both (1-128 sequences of 200-160K keys) and checked
+    // against 260 more (1 to 32 KV heads, blocks of 1 to 64, pages of 16 to 64).
     // us per key tile of a CTA: AHEAD, clusters of up to 5, wider clusters, flat (all SMs together then)
-    const double big[4] = {1.10, 1.32, 1.41, 1.39}, p32[4] = {1.26, 1.37, 1.62, 1.45}, p16[4] = {1.83, 1.83, 2.42, 1.70};
-    const double* us = paged && a.page_size < 64 ? (a.page_size < 32 ? p16 : p32) : big;
+    const double big[4] = {1.10, 1.32, 1.41, 1.39}, p32[4] = {1.26, 1.37, 1.62, 1.45};
+    const double p16[4] = {1.83, 1.83, 2.42, 1.70};
+    const bool page16 = paged && a.page_size < 32;
+    const double* us = page16 ? p16 : paged && a.page_size < 64 ? p32 : big;
     // A sequence's query tiles read the same K and V, which its units of one wave share in L2 (16 x 4112 keys, blocks
     // of 40 -- two tiles: clusters 79.2, flat 103.5 us; 12: 77.9 and 70.9).
     const bool shared = m_tiles > 1;
-    double est_flat = (shared ? 1.2 : 1.0) * us[3] * avg_tiles + 10.0 + std::min(4.2 * (1.0 + (double)a.num_seqs / std::max(ngroups, 1)), 11.0);
-    double est_cluster;
-    if (cluster_ctas <= dev.sm_count) {
-        // One wave.  Flat for 1 x 65552 keys (50.5 against 54.5 us), 7 x 32784 (145 against 151), 10 x 16400 (110
-        // against 146); clusters for 8 x 32784 (153.6 against 163), 16 x 16400 (152 against 168), 5 x 8208 (34.4
-        // against 38.4).
-        est_cluster = us[ahead_for(cs) ? 0 : cs <= 5 ? 1 : 2] * ((max_tiles + cs - 1) / cs) +
-                      (cs == 1 ? 7.0 : cs <= 5 ? 10.0 : 8.0);
-    } else {
-        // Several waves of whole units, longest first.  With lengths spread evenly between 2 mean - max and max, the
-        // units of the last wave (at most `last` tiles) land on the shortest of the wave before, which pairs up
+    // flat: the second kernel merges eight partials a round, and with few KV heads a unit is cut over many groups (16 / 2
+    // heads, 1 x 16016 keys, 76 parts: 21.8 us, in clusters 15.4)
+    const double cut_parts = (double)ngroups / ((double)a.num_seqs * m_tiles);
+    const double est_flat =
+        (shared ? 1.2 : 1.0) * us[3] * avg_tiles + 10.0 +
+        std::min(4.2 * (1.0 + (double)a.num_seqs / std::max(ngroups, 1)), 11.0) +
+        0.7 * std::max(0.0, std::ceil(cut_parts / 8.0) - 3.0);
+    // clusters, the longest unit of `longest` key tiles; mixed: how far the others fall short of it
+    double mixed = 0.0;
+    const auto est_cluster_for = [&](int longest) {
+        if (cluster_ctas <= dev.sm_count) {
+            // One wave.  Flat for 1 x 65552 keys (50.5 against 54.5 us), 7 x 32784 (145 against 151), 10 x 16400 (110
+            // against 146); clusters for 8 x 32784 (153.6 against 163), 16 x 16400 (152 against 168), 5 x 8208 (34.4
+            // against 38.4).  Wide clusters stream as fast as HBM lets so many CTAs, down to a CTA's own chain (16 / 2
+            // heads, 1 x 16016 keys: 32 CTAs of 8 tiles, 15.4 us); with small pages the chain alone counts.
+            const double wide = us == big ? std::max(0.68, (double)cluster_ctas / 128.0) * us[2] : us[2];
+            mixed = 0.0;
+            return (ahead_for(cs) ? us[0] : cs <= 5 ? us[1] : wide) * ((longest + cs - 1) / cs) +
+                   (cs == 1 ? 7.0 : cs <= 5 ? 10.0 : 8.0);
+        }
+        // Several waves of whole units, longest first.  With lengths spread evenly between 2 mean - longest and longest,
+        // the units of the last wave (at most `last` tiles) land on the shortest of the wave before, which pairs up
         // to 2 last.  The tiles then stream at HBM's rate where every SM has a unit and faster where some have
         // none.  20 x 8208 keys: 114.6 flat against 158.6 us; 39 x 4112 113.9 against 136.9; 32 x 4112 98.2 against
         // 95.1; 20 x 528 23.7 against 19.2.  Batches of mixed lengths pack better than that and cut worse.
         const int waves = (int)((units + dev.sm_count - 1) / dev.sm_count);
-        const double mean = std::min(avg_tiles * dev.sm_count / units, (double)max_tiles);
-        const double least = std::max(2.0 * mean - max_tiles, 0.0);
-        const double last = least + (max_tiles - least) * (units - (waves - 1.0) * dev.sm_count) / units;
-        const double chain = std::max((double)max_tiles, (waves - 2.0) * max_tiles + 2.0 * last);
-        const double mixed = 1.0 - mean / max_tiles;
-        est_cluster = (shared ? us[0] * chain : (0.86 * chain + 0.48 * avg_tiles) * us[0] / big[0]) +
-                      (shared ? 6.0 : 5.0 + 5.0 * units / dev.sm_count) - 8.0 * mixed;
-        est_flat += 6.0 * mixed;
-        // many waves: flat (57 x 528 keys 33.1 against 39.6 us; blocks of 40, 64 x 1040 102.8 against 106.0)
-        if (cluster_ctas >= (shared ? 5LL : 3LL) * dev.sm_count) est_cluster = est_flat + 1.0;
-    }
-    bool flat = flat_ok && est_flat < est_cluster;
+        const double mean = std::min(avg_tiles * dev.sm_count / units, (double)longest);
+        const double least = std::max(2.0 * mean - longest, 0.0);
+        const double last = least + (longest - least) * (units - (waves - 1.0) * dev.sm_count) / units;
+        const double chain = std::max((double)longest, (waves - 2.0) * longest + 2.0 * last);
+        mixed = 1.0 - mean / longest;
+        return (shared ? us[0] * chain : (0.86 * chain + 0.48 * avg_tiles) * us[0] / big[0]) +
+               (shared ? 6.0 : 5.0 + 5.0 * units / dev.sm_count) - 8.0 * mixed;
+    };
+    // The longest sequence may have max_kv_len keys, or under a loose bound (a captured loop's cache capacity) all of
+    // them total_kv / num_seqs.  Flat where it is the faster split either way.  Where only the bound says so, the
+    // kernel looks at the lengths and, if they are even, deals the units out as clusters would have them, about 3 us
+    // slower (the second launch): worth the risk where the even lengths take 20 us in clusters, or 25 if the bound is
+    // so far above the mean that it is more likely loose.  us dealt or cut by the kernel / in clusters / always cut:
+    // 12 x 4016 keys, bound 8192, 43.9 / 40.9 / 44.5; 16 x 2016, bound 8192, 29.7 / 26.9 / 36.2; 16 x 1016 20.0 / 17.1 /
+    // 26.4; 10 of 512 to 8192 keys 41.6 / 75.3 / 40.8.  And flat by the simple rule: many waves (57 x 528 keys 33.1
+    // against 39.6 us; blocks of 40, 64 x 1040 102.8 against 106.0, pages of 16, 40 x 1540 118.3 against 144.2), and
+    // where clusters leave SMs idle on long runs, unless they are clearly the faster.
+    const long long mean_kv = ((long long)a.total_kv + a.num_seqs - 1) / a.num_seqs;
+    const int even_tiles = std::min(max_tiles, (int)((mean_kv + kTileN - 1) / kTileN));
+    const bool many = cluster_ctas >= (shared && !page16 ? 5LL : 3LL) * dev.sm_count;
+    const bool simple = (cluster_ctas * 10 <= 9LL * dev.sm_count && tiles_bound >= 64LL * ngroups) ||
+                        cluster_ctas >= 3LL * dev.sm_count;
+    const double est_even = est_cluster_for(even_tiles), flat_even = est_flat + 6.0 * mixed;
+    const double est_cluster = est_cluster_for(max_tiles), flat_bound = est_flat + 6.0 * mixed;
+    const bool deals = m_tiles == 1 && a.num_seqs > 1 && a.num_seqs <= kMaxDealtSeqs;
+    const double risk = cluster_ctas > dev.sm_count || max_tiles <= 2.4 * even_tiles ? 20.0 : 25.0;
+    bool flat = flat_ok && (many || (flat_bound < est_cluster
+                                         ? simple || flat_even < est_even || (deals && est_even >= risk)
+                                         : simple && est_cluster > 0.97 * flat_bound));
+    // (where cutting evenly is the faster either way the kernel is spared the choice: 10 x 16400 keys 110.3 us, 111.9
+    // with it)
+    bool deal = deals && flat_even >= est_even;
+    p.sm_count = dev.sm_count;
+    p.ahead_ok = !page16;
+    p.us_whole = (float)us[0];
+    p.us_part = (float)us[1];
+    p.us_cut = (float)us[3];
     if (const char* force = getenv("BP_ATTENTION_SPLIT")) {
         if (strcmp(force, "flat") == 0) {
             flat = flat_ok;
+            deal = false;
+        } else if (strcmp(force, "dealt") == 0) {  // flat with the choice left to the kernel
+            flat = flat_ok;
+            deal = deals;
         } else if (strncmp(force, "cluster", 7) == 0) {
             flat = false;
             // cluster:N forces clusters of N CTAs when every unit's cluster is then resident in one wave
@@ -1613,16 +1813,18 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
         cfg.gridDim = dim3((unsigned)flat_grid, 1, 1);
         cfg.attrs = &attr[1];
         cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, kAttnKernels[8 + 2 * spread + paged], qmap, kmap, vmap, p);
+        e = cudaLaunchKernelEx(&cfg, kAttnKernels[(deal ? 12 : 8) + 2 * spread + paged], qmap, kmap, vmap, p);
         if (e != cudaSuccess) return BP_ERR_CUDA;
-        if (max_tiles <= 1) return BP_OK;  // every unit is one tile: none is cut between CTAs
+        if (a.max_kv_len <= kTileN) return BP_OK;  // every unit is one tile: none is cut between CTAs
         cudaLaunchConfig_t cc = {};
-        cc.gridDim = dim3((unsigned)(flat_grid * ((p.slot_rows + kCombRows - 1) / kCombRows)), 1, 1);
+        const int pieces = flat_grid * ((p.slot_rows + kCombRows - 1) / kCombRows);
+        cc.gridDim = dim3((unsigned)(deal ? std::min(pieces, kCombPerSm * dev.sm_count) : pieces), 1, 1);
         cc.blockDim = dim3(kCombThreads, 1, 1);
         cc.stream = stream;
         cc.attrs = &attr[1];
         cc.numAttrs = 1;
-        return cudaLaunchKernelEx(&cc, attn_combine_kernel, p, flat_grid) == cudaSuccess ? BP_OK : BP_ERR_CUDA;
+        e = cudaLaunchKernelEx(&cc, deal ? attn_combine_kernel<true> : attn_combine_kernel<false>, p, flat_grid);
+        return e == cudaSuccess ? BP_OK : BP_ERR_CUDA;
     }
 
     cfg.gridDim = dim3((unsigned)(units * cs), 1, 1);
@@ -1636,7 +1838,7 @@ int launch_attention_bf16(const AttentionArgs& a, const DeviceInfo& dev, cudaStr
     // on the SMs for nothing and its thousands of CTAs start worse for it: 8 x 32784 keys (129 tiles a CTA) with
     // the T = 1 acceptance took 194.2 us a step released at the start and 189.7 at the end; alone, 33 tiles a CTA
     // take 44.8 us either way, 17 tiles 28.0 and 28.4
-    p.early_release = units <= max_active[cs] && units * cs <= dev.sm_count && max_tiles < 24 * cs;
+    p.early_release = units <= max_active[cs] && units * cs <= dev.sm_count && even_tiles < 24 * cs;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cs;
     attr[0].val.clusterDim.y = 1;

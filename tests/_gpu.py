@@ -41,9 +41,10 @@ def attention_ws(a: dict, split: str = "auto"):
 def forced_split(split: str):
     """The library's choice between the flat and the cluster split of the keys ("auto"), or one of them
     forced through BP_ATTENTION_SPLIT, which the library reads at every call ("cluster3": the cluster
-    split in clusters of 3, so that short contexts too are merged; "cluster:N" of N)."""
+    split in clusters of 3, so that short contexts too are merged; "cluster:N" of N; "dealt": the flat split
+    whose kernel may deal the units out)."""
     old = os.environ.get("BP_ATTENTION_SPLIT")
-    if split in ("flat", "cluster") or split.startswith("cluster:"):
+    if split in ("flat", "cluster", "dealt") or split.startswith("cluster:"):
         os.environ["BP_ATTENTION_SPLIT"] = split
     elif split == "cluster3":
         os.environ["BP_ATTENTION_SPLIT"] = "cluster:3"

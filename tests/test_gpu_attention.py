@@ -314,3 +314,60 @@ def test_cluster_merges(n, ctx, block, page):
         assert np.abs(full[0] - chip[0]).max() <= 2 ** -8 * max(1.0, np.abs(full[0]).max())
         np.testing.assert_allclose(full[1], chip[1], rtol=0, atol=1e-5)
 
+
+@pytest.mark.parametrize("ctx,block,hq,hkv", [
+    ((2000,) * 2, (16, 12), 32, 8),                                           # equal parts, 9 groups of CTAs a unit
+    ((1500, 1400, 90, 0, 3), (16, 9, 1, 0, 24), 32, 8),                       # parts; few tiles, none, an empty block
+    ((700,) * 12, (16, 3) * 6, 32, 8),                                        # a group a unit, K's ring ahead
+    ((300, 290, 310, 20) * 10, (9, 16, 1, 24) * 10, 32, 8),                   # rounds there and back over the groups
+    ((130,) * 64, (4,) * 64, 16, 16),                                         # as many sequences as are dealt; 9 groups
+    ((5000,) + (200,) * 11, (8,) * 12, 32, 8),                                # one long among short: cut evenly
+    ((900,) * 5, (16,) * 5, 8, 1),                                            # one KV head: dozens of parts
+    ((260, 250, 240), (32, 31, 30), 32, 32),                                  # four groups for three sequences
+])
+@pytest.mark.parametrize("page", [0, 16, 64])
+def test_units_dealt_out(ctx, block, hq, hkv, page):
+    """The flat split whose kernel may deal the units out, whole or in equal parts, by the lengths it finds."""
+    a = wl.attention_inputs(wl.custom(seed=len(ctx) + hkv, ctx=ctx, block=block, num_q_heads=hq, num_kv_heads=hkv))
+    seqs = range(0, len(ctx), max(1, len(ctx) // 6))
+    for mask in (CAUSAL, BIDIR):
+        o, lse = _run(a, mask, "dealt", page=page)
+        err, lerr = attention_errors(o, lse, a, mask, seqs)
+        assert err <= ATTN_TOL and lerr <= LSE_TOL, (err, lerr)
+
+
+def _merges(a, **kw):
+    from torch.profiler import ProfilerActivity, profile
+
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        _run(a, CAUSAL, **kw)
+        torch.cuda.synchronize()
+    return any("attn_combine_kernel" in e.name for e in prof.events())
+
+
+@pytest.mark.parametrize("n, ctx, bound, flat", [
+    (2, 500, 8192, False), (4, 2000, 32768, False), (8, 1000, 8192, False), (12, 500, 8192, False),
+    (16, 2000, 8192, False), (16, 4000, 16384, True), (24, 2000, 8192, True)])
+@pytest.mark.parametrize("page", [0, 64])
+def test_loose_bound_on_the_lengths(n, ctx, bound, flat, page):
+    """max_kv_len as a capacity far above the lengths: the values of the exact bound (to the rounding of another
+    split), and where equal lengths take less than about 25 us the clusters an exact bound gets."""
+    a = wl.attention_inputs(wl.custom(seed=n, ctx=(ctx,) * n, block=(16,) * n, num_q_heads=32, num_kv_heads=8))
+    _merges(a)
+    assert _merges(a, max_kv=bound, page=page) == flat
+    o, lse = _run(a, CAUSAL, max_kv=bound, page=page)
+    err, lerr = attention_errors(o, lse, a, CAUSAL, [0, n - 1])
+    assert err <= ATTN_TOL and lerr <= LSE_TOL
+
+
+@pytest.mark.parametrize("n, ctx, hq, hkv, flat", [
+    (1, 16000, 16, 2, False), (1, 16000, 32, 4, False), (24, 16000, 32, 1, True), (4, 4000, 32, 1, False),
+    (24, 16000, 16, 2, True), (10, 4000, 32, 16, True), (4, 4000, 32, 16, False), (10, 4000, 32, 32, True)])
+def test_split_by_estimate_other_head_counts(n, ctx, hq, hkv, flat):
+    """The faster split as timed, for 1 to 32 KV heads."""
+    a = wl.attention_inputs(wl.custom(seed=n + hkv, ctx=(ctx,) * n, block=(16,) * n, num_q_heads=hq, num_kv_heads=hkv))
+    _merges(a)
+    assert _merges(a) == flat
+    o, lse = _run(a, CAUSAL)
+    err, lerr = attention_errors(o, lse, a, CAUSAL, [n - 1], 0)
+    assert err <= ATTN_TOL and lerr <= LSE_TOL
