@@ -97,7 +97,8 @@ typedef enum { BP_F32 = 0, BP_BF16 = 1 } bp_dtype;
  *            scores of each output row; may be NULL
  *   cu_q, cu_kv  [num_seqs+1] int32 device arrays, non-decreasing, cu_*[0] = 0,
  *            cu_q[num_seqs] = total_q, cu_kv[num_seqs] = total_kv
- *   max_q_len, max_kv_len  host-side upper bounds of B_s and L_s+B_s
+ *   max_q_len, max_kv_len  host-side upper bounds of B_s and L_s+B_s (max_kv_len may be a cache's capacity; the
+ *            nearer to the longest sequence, the better the split of the keys is chosen)
  *   dtype    BP_BF16 (tensor-core path, head_dim 128) or BP_F32 (head_dim <= 128)
  *   softmax_scale  0 selects 1/sqrt(head_dim)
  * Limits: 1 <= num_kv_heads, num_q_heads % num_kv_heads == 0, max_q_len <= 64,
@@ -267,9 +268,11 @@ BP_API int bp_policy_select(const void* feats, int64_t feat_row_stride, const in
  *   logits_out   [rows][vocab] fp32, may be NULL: if given, the logits are also written (rows:
  *                the target rows, then at T > 0 the drafter rows)
  * Two paths, chosen by rows = total_draft + num_seqs (+ total_draft at T > 0):
- *   rows <= 32 and num_seqs <= vocab / 40000 at T > 0 (and up to 64 rows in a workspace without the room
- *     below): one cooperative launch of one CTA per SM keeps every logit in tensor memory; the logits never reach memory unless logits_out asks
- *     for them (then for testing: it adds the write traffic the fusion exists to avoid).
+ *   rows <= 32 and num_seqs <= vocab / 40000 at T > 0: one cooperative launch of one CTA per SM keeps every
+ *     logit in tensor memory; the logits never reach memory unless logits_out asks for them (then for
+ *     testing: it adds the write traffic the fusion exists to avoid).  Other calls of up to 64 rows at T > 0 take
+ *     this path too in a workspace without the room below, of a size asked for formerly: accepted for
+ *     compatibility, slower than streaming.
  *   more rows, and T = 0: the LM head is streamed in passes of up to 256 entries, groups of at most 256 rows
  *     per pass over W, and every row's statistics are formed in the projection's epilogue.  At T = 0 only the
  *     statistics leave the chip.  At T > 0 the logits are written once (into logits_out if given, else into

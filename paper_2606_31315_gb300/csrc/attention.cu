@@ -12,11 +12,12 @@
 //     S = Q K^T into tensor memory, runs an online softmax (fp32, exp2 domain, lazy
 //     rescale of the TMEM accumulator when the row max grows by more than 2^8),
 //     writes P (bf16) back into tensor memory (three S/P buffers) and accumulates O += P V
-//     with P as the TMEM A operand.  Every CTA scales its partial result and pushes each row to
-//     the CTA that owns it, which adds them up: through distributed shared memory, or, where a
-//     CTA owns few rows (wide clusters) and the workspace has the room, through L2.
-//   * The flat split (below) cuts the tiles of all units evenly over the CTAs instead; a second
-//     kernel merges the units that were cut.
+//     with P as the TMEM A operand.  The partial results are merged by the CTAs that own the rows:
+//     every CTA scales its rows and pushes them to their owners through distributed shared memory,
+//     or, where a CTA owns few rows (wide clusters) and the workspace has the room, leaves them as
+//     they are in its own slot there, and the owner loads and weighs them.
+//   * The flat split (below) cuts the tiles of all units evenly over the CTAs instead, or deals the
+//     units out; a second kernel merges the units that were cut.
 //   * Units are issued longest-first so that ragged batches finish together.
 //   Warp roles: warp 0 = TMA producer + TMEM allocator, warp 1 = MMA issuer,
 //   warps 2..5 = softmax / epilogue (one query row per thread, TMEM lane = row).  Units of at
@@ -241,7 +242,7 @@ __device__ __forceinline__ Seg dealt_seg(const AttnParams& p, const uint8_t* ord
 // out even (the host knows only a bound and their sum), the CTAs deal the units out instead, longest first, whole
 // or in equal parts.  Otherwise the cluster split: a unit per cluster, its tiles cut into CS ranges, partials merged
 // through distributed shared memory or the workspace.
-// AHEAD (cluster split): K and V are separate rings.  K's stage is free after Q K^T, a softmax and a P V before
+// AHEAD (cluster split; FLAT == 2 where every CTA has one stretch): K and V are separate rings.  K's stage is free after Q K^T, a softmax and a P V before
 // V's, and refills then, V a tile behind (the order in which the stages come free); with the rings joined both
 // wait for the tile's P V and only one of the three stages is in flight.  Where the line lies:
 // launch_attention_bf16.
@@ -1180,7 +1181,7 @@ __global__ void __launch_bounds__(kCombThreads, kCombPerSm) attn_combine_kernel(
 // merge.  Within a chunk, the 10 shared-memory wavefronts a warp needs for its 32 FFMAs.  The kernel it
 // replaces (a warp per output row, a key per lane, each lane walking its key row alone) read 32 rows per load
 // instruction and put the whole context into one warp's chain: 4 sequences x 1008 keys x 8 positions, 4 / 2
-// heads of 64, took 322.7 us a call and takes 13.9 us here; the error against 64-bit sums went from 6.3e-7
+// heads of 64, took 322.7 us a call and takes 10.2 us here; the error against 64-bit sums went from 6.3e-7
 // to 3.3e-7 (shorter chains).
 constexpr int kF32MaxD = 128;
 constexpr int kFR = 32;         // query rows per tile

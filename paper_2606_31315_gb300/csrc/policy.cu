@@ -677,7 +677,7 @@ __global__ void __launch_bounds__(kTcThreads) policy_tc_kernel(const __grid_cons
 // workspace slot, and the CTA that completes a tile (an atomic ticket, no waiting) adds the tile's parts in run
 // order, applies b1, ReLU and its columns of W2; the one that completes the last tile adds the tiles' shares of
 // the output layer in tile order and takes the argmax.  Every sum runs in a fixed order.
-// What bounds it: HBM, W1 read once (32 x 151936 -> 2048: 632 MB in 111 us, 5.7 TB/s, about 8 us of it the tail's
+// What bounds it: HBM, W1 read once (32 x 151936 -> 2048: 632 MB in 108 to 111 us, 5.8 TB/s, about 8 us of it the tail's
 // two tickets and sums).  An MMA at N <= 64 costs one thread more to issue than to run, so two warps take the
 // stages in turn, each with an accumulator of its own.
 constexpr int kFlStages = 8;        // 16 KB of W1 and up to 8 KB of x each

@@ -8,7 +8,8 @@
 // [rows, V] accumulator in tensor memory, which bounds it to 64 rows: the GPU's tensor memory holds
 // about 39 MB, and 248 rows of a 151,936-entry vocabulary take 151 MB in fp32.  Here:
 //   1. lm_head_stream_kernel: one CTA per SM owns an equal contiguous share of the vocabulary,
-//      streamed in passes of 256 entries and a last pass of what is left.  Per pass, its W rows (256 entries x 64 hidden columns per stage) and the states of
+//      streamed in passes of 256 entries and a last pass of what is left.  Per pass, its W rows (256 entries x 64
+//      hidden columns per stage) and the states of
 //      up to 256 rows stream through a TMA ring; one thread issues M=128 (state rows) x N=256 (entries)
 //      x K=16 tcgen05 MMAs, one per 128-row half of the states.  Tensor-memory lane = state row, so each
 //      epilogue thread owns part of one row's entries and folds their logits into a running (max, sum of
