@@ -19,6 +19,8 @@ CASE is one of:
                       contexts 562..8118 (576 MB of K/V)
   attention_c5        causal verify attention over the long-context batch: 8 sequences of 32768 + 16
                       keys (1.07 GB of K/V)
+  attention_flat      causal verify attention that takes the flat split: 20 sequences of 8192 + 16 keys (672 MB)
+  attention_f32       fp32 attention, 4 sequences of 1000 + 8 keys, 4 / 2 heads, D = 64
   accept_c5_t1        acceptance of the long-context batch at T = 1: 8 x 16 target and 8 x 15 draft
                       rows over 151936 (150.7 MB): the three throughput kernels
   step_c5             one long-context verify step: attention_c5, then accept_c5_t1
@@ -118,6 +120,17 @@ def _batch_attention(dev, gen, ctx, block):
     return lambda: bp.block_attention(q, k, v, cu_q, cu_kv, max(block), max(kv), mask=bp.MASK_CAUSAL, ws=ws)
 
 
+def _attention_f32(dev, gen):
+    n, ctx, block, hq, hkv, d = 4, 1000, 8, 4, 2, 64
+    q = torch.randn(n * block, hq, d, device=dev, generator=gen)
+    k = torch.randn(n * (ctx + block), hkv, d, device=dev, generator=gen)
+    v = torch.randn(n * (ctx + block), hkv, d, device=dev, generator=gen)
+    cu_q = torch.arange(0, n * block + 1, block, dtype=torch.int32, device=dev)
+    cu_kv = torch.arange(0, n * (ctx + block) + 1, ctx + block, dtype=torch.int32, device=dev)
+    ws = bp.workspace(bp.block_attention_workspace_size(n, block, hq, hkv, d), dev)
+    return lambda: bp.block_attention(q, k, v, cu_q, cu_kv, block, ctx + block, ws=ws)
+
+
 def _accept_c5(dev, gen):
     s, td = 8, 8 * (B - 1)
     t = torch.randn(td + s, V, device=dev, generator=gen) * 3
@@ -180,6 +193,8 @@ CASES = {
     "attention": _attention,
     "attention_c3": lambda dev, gen: _batch_attention(dev, gen, *_ragged_shapes()),
     "attention_c5": lambda dev, gen: _batch_attention(dev, gen, [32768] * 8, [B] * 8),
+    "attention_flat": lambda dev, gen: _batch_attention(dev, gen, [8192] * 20, [B] * 20),
+    "attention_f32": _attention_f32,
     "accept_c5_t1": _accept_c5,
     "step_c5": _step_c5,
     "policy": lambda dev, gen: _policy(dev, gen, 2560),
